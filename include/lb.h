@@ -48,7 +48,10 @@ typedef enum {
 } lb_status;
 
 typedef enum {
-    LB_FP64 = 0,         /* distributions stored and updated in IEEE double */
+    LB_FP64 = 0,         /* distributions stored in IEEE double; for d > 1 a
+                            collision forms its sums exactly on the integer
+                            pipes where the node's values allow it and rounds
+                            each result once, else in double arithmetic */
     LB_FP32_SHIFTED = 1, /* stored and updated in float as f - w*theta_ref */
     LB_FX64 = 2          /* stored as 64-bit fixed point round(f * 2^F), with F
                             chosen by lb_set_theta0 so that max|theta0| * 2^F <

@@ -131,7 +131,7 @@ __device__ __forceinline__ void gather_rev_walls(const A *__restrict__ src, cons
 
 // The periodic two-phase gather split in two calls, so that a kernel can
 // issue the vector loads of two fields before it shuffles either (the same
-// loads and halo scalars as gather_two_phase).  REV pulls from x + e_i, the
+// loads and halo scalars as gather).  REV pulls from x + e_i, the
 // adjoint's reverse pull, instead of x - e_i.  gather_late_finish shifts by
 // e_x and reads the row-end wrap of the lane holding the row's last node.
 template <class L, typename T, int V, bool REV>

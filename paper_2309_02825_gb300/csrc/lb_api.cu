@@ -238,7 +238,7 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     // Layout.
     const int V = (precision == LB_FP32_SHIFTED) ? lbk::Vec<float>::V : lbk::Vec<double>::V;
     c->elem = (precision == LB_FP32_SHIFTED) ? 4 : 8;
-    const int W = lbk::lane_width(c->d, c->elem, precision == LB_FP64);
+    const int W = lbk::lane_width(c->d, c->elem);
     c->geom = lbk::make_geom(c->N[0], c->N[1], c->N[2], c->N[3], V, W);
     const lbk::Geom &g = c->geom;
 

@@ -26,6 +26,9 @@ namespace lbk {
 template <typename T> struct CollOf {
     using type = Coll<T>;
 };
+template <> struct CollOf<double> {
+    using type = CollF64;
+};
 template <> struct CollOf<long long> {
     using type = CollFx;
 };
@@ -445,6 +448,8 @@ template <typename T> cudaError_t upload_desc(lb_batch *b)
         h[j].g = b->inst[j].geom;
         if constexpr (std::is_same<T, long long>::value)
             h[j].k = lbk::make_coll_fx(&b->inst[j]);
+        else if constexpr (std::is_same<T, double>::value)
+            h[j].k = lbk::make_coll_f64(b->inst[j]);
         else
             h[j].k = lbk::make_coll<T>(b->inst[j]);
         h[j].off = b->off[j];
@@ -714,13 +719,13 @@ template <typename T> static cudaError_t upload_single_desc(lb_ctx *c)
     h.g = c->geom;
     if constexpr (std::is_same<T, long long>::value)
         h.k = make_coll_fx(c);
+    else if constexpr (std::is_same<T, double>::value)
+        h.k = make_coll_f64(*c);
     else
         h.k = make_coll<T>(*c);
     h.off = 0;
     cudaError_t e = cudaSuccess;
-    if (!c->tb_desc) e = cudaMalloc(&c->tb_desc, sizeof(InstDesc<long long>) > sizeof(InstDesc<double>)
-                                                       ? sizeof(InstDesc<long long>)
-                                                       : sizeof(InstDesc<double>));
+    if (!c->tb_desc) e = cudaMalloc(&c->tb_desc, std::max(sizeof(InstDesc<long long>), sizeof(InstDesc<double>)));
     if (e == cudaSuccess) e = cudaMemcpy(c->tb_desc, &h, sizeof(h), cudaMemcpyHostToDevice);
     return e;
 }

@@ -2,7 +2,7 @@
 // batched and adjoint kernels: compile-time loops, periodic wrap, vector
 // access, the fixed-point products, the shifted pull of one
 // population along x, where a pull reads from on periodic and mirror-wall
-// grids (pop_source), the two gather orders, and the closed-form
+// grids (pop_source), the gathers, and the closed-form
 // moment-space collision for D1Q3, D2Q9, D3Q19 and D4Q33
 // (Eq. (distribution-f)) with the sweep kernel built from them.
 #pragma once
@@ -353,37 +353,13 @@ __device__ __forceinline__ PopSrc pop_source(const Geom &g, const RowPos &r)
     return p;
 }
 
-// Gather the pre-collision f(x, n) for the V nodes of this lane, one
-// population at a time (each shifted pull right after its load).  Used for
-// FP64 storage, whose sweep is bound by the FP64 pipe: the lower register
-// count keeps more warps resident to hide FP64 latency.
+// Gather the pre-collision f(x, n) for the V nodes of this lane in two
+// phases: every 16-byte vector load of every population, and the one halo
+// scalar a warp edge needs, is issued before any shuffle consumes a loaded
+// value, so a warp has all q rows in flight at once.
 template <class L, typename T, int V = Vec<T>::V, bool MIR = false>
-__device__ __forceinline__ void gather_interleaved(const T *__restrict__ src, const Geom &g, int64_t row, int x0,
-                                                   int lane, T (&f)[L::Q][V])
-{
-    const RowPos rpos = row_pos<L::D>(g, row);
-    const bool mx = MIR && (g.mirror & 1u);
-    static_for<0, L::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        constexpr int ex = L::E[i][0];
-        const PopSrc ps = pop_source<L, i, MIR>(g, rpos);
-        const T *rp = src + (int64_t)ps.pop * g.slab + ps.row * g.pitch;
-        if (!MIR || !mx) {
-            pull_row<T, ex, V>(rp, x0, lane, g.N0, f[i], rp, g.N0 - 1, 0);
-        } else {
-            const T *rx = src + (int64_t)ps.popx * g.slab + ps.row * g.pitch;
-            pull_row<T, ex, V>(rp, x0, lane, g.N0, f[i], rx, 1, g.N0 - 2);
-        }
-    });
-}
-
-// Gather in two phases: every 16-byte vector load of every population, and
-// the one halo scalar a warp edge needs, is issued before any shuffle
-// consumes a loaded value, so a warp has all q rows in flight at once.  Used
-// for the HBM-bound storage types (FP32, 64-bit fixed point).
-template <class L, typename T, int V = Vec<T>::V, bool MIR = false>
-__device__ __forceinline__ void gather_two_phase(const T *__restrict__ src, const Geom &g, int64_t row, int x0,
-                                                 int lane, T (&f)[L::Q][V])
+__device__ __forceinline__ void gather(const T *__restrict__ src, const Geom &g, int64_t row, int x0, int lane,
+                                       T (&f)[L::Q][V])
 {
     const RowPos rpos = row_pos<L::D>(g, row);
     const int xb = x0 + V * lane;
@@ -459,17 +435,6 @@ __device__ __forceinline__ void gather_flat(const T *__restrict__ src, const Geo
         const T *rp = src + (int64_t)i * g.slab + src_row<L::D, ey, ez, ew>(g, rpos) * g.pitch;
         f[i] = __ldg(rp + (ex == 1 ? xl : (ex == -1 ? xr : x)));
     });
-}
-
-template <class L, typename T, int V = Vec<T>::V, bool MIR = false>
-__device__ __forceinline__ void gather(const T *__restrict__ src, const Geom &g, int64_t row, int x0, int lane,
-                                       T (&f)[L::Q][V])
-{
-    // two-phase unless FP64 (FP64-pipe bound) or too many values to keep in flight
-    if constexpr (std::is_same<T, double>::value || L::Q * V > 80)
-        gather_interleaved<L, T, V, MIR>(src, g, row, x0, lane, f);
-    else
-        gather_two_phase<L, T, V, MIR>(src, g, row, x0, lane, f);
 }
 
 // The rest population is formed as theta minus all the others when the
@@ -819,9 +784,87 @@ __device__ __forceinline__ void collide(D4Q33, long long *f, const CollFx &k)
 }
 
 
-// Threads per block of the sweep: 128 for the HBM-bound storage types
-// (more, smaller blocks balance the SMs better), 256 for FP64.
-template <typename T> __host__ __device__ constexpr int sweep_threads() { return std::is_same<T, double>::value ? 256 : 128; }
+// FP64 collisions on the integer pipes.  GB300 issues FP64 at 1/64 of the
+// FP32 and integer rates, so the 31.5 (D2Q9) FP64 operations of the direct
+// collision bind the sweep (85 % of that pipe) at a third of the HBM rate.
+// Here a node's q doubles are aligned to their largest exponent as int64:
+// a double is m 2^(e - 1075) with a 53-bit m, held as m 2^(PB + e - emax).
+// When every exponent lies within PB of the largest, no bit is dropped: the
+// moment sums are exact, each product with a 64-fraction-bit constant is
+// rounded once at 2^-(52 + PB) of the largest value (mulfx_c), and every
+// result is rounded once to FP64 (to nearest, ties to even), where the direct
+// form rounds after each operation.  PB is as large as keeps the sum of the
+// magnitudes below 2^62 for the weights in use: 7 for D2Q9 (the largest
+// population is about half of theta), 5 for D3Q19 and D4Q33 (about 1/8, 1/12);
+// a node whose magnitudes sum to 2^62 or more, whose exponents spread wider
+// (a population near zero, a relaxation set with tiny weights) or that holds
+// a zero, subnormal, infinity, NaN or an exponent at the ends of the range
+// takes the direct form.  The host takes the integer form only where the
+// constants lie in mulfx_c's range and bound the rest population
+// (make_coll_f64).  Per sweep, direct -> integer form: D2Q9 4096^2 997 -> 358
+// us (6.74 TB/s, the copy rate), 512^2 22.7 -> 10.0; D3Q19 256^3 2158 -> 785;
+// D4Q33 50^4 1452 -> 608.
+template <class L> __host__ __device__ constexpr int f64_align_bit() { return L::Q <= 9 ? 7 : 5; }
+
+// s 2^(emax - 1075 - PB) rounded to nearest, ties to even, for
+// 100 <= emax <= 2000 (every nonzero result is a normal number).  The hardware
+// conversion rounds; the power of two goes onto the exponent field.  It issues
+// at the FP64 rate, but one per result (7 for D2Q9) leaves that pipe under half
+// busy, while assembling the double in integers costs 24 instructions each on
+// the pipes that bind the sweep: 4096^2 358 us with all results converted by
+// hardware, 385 with three of seven, 410 with none.
+template <int PB> __device__ __forceinline__ double f64_from_aligned(long long s, unsigned emax)
+{
+    const double r = (double)s;
+    return s == 0 ? 0.0 : __hiloint2double(__double2hiint(r) + (int)((emax - 1075u - (unsigned)PB) << 20), __double2loint(r));
+}
+
+template <class L> __device__ __forceinline__ void collide(L, double *f, const CollF64 &k)
+{
+    constexpr int Q = L::Q, PB = f64_align_bit<L>(), B0 = 1 + 2 * L::D;
+    if (k.ints) {
+        unsigned e[Q], mx = 0u, mn = 0x7ff00000u;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            e[i] = (unsigned)__double2hiint(f[i]) & 0x7ff00000u;
+            mx = max(mx, e[i]);
+            mn = min(mn, e[i]);
+        }
+        if (mx - mn <= ((unsigned)PB << 20) && mx - (100u << 20) <= (1900u << 20)) {
+            long long v[Q];
+            unsigned sum = 0u;  // of the magnitudes' high words (each below 2^(21 + PB))
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
+                const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+                const unsigned sh = (unsigned)PB - ((mx - e[i]) >> 20);  // 0 .. PB
+                const unsigned vh = __funnelshift_l(lo, mh, sh), vl = lo << sh;
+                sum += vh;
+                const unsigned s = (unsigned)((int)hi >> 31);
+                v[i] = (long long)((((unsigned long long)(vh ^ s) << 32) | (vl ^ s)) - (((unsigned long long)s << 32) | s));
+            }
+            if (sum < 0x3fffffc0u) {  // magnitudes sum below 2^62
+                const unsigned emax = mx >> 20;
+                collide(L{}, v, k.x);
+                // the two velocities of a diagonal pair hold equal values
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    if (i >= B0 && ((i - B0) & 3) >= 2)
+                        f[i] = f[i - 2];
+                    else
+                        f[i] = f64_from_aligned<PB>(v[i], emax);
+                }
+                return;
+            }
+        }
+    }
+    collide(L{}, f, k.k);
+}
+// One axis: three populations, nine FP64 operations; the direct form.
+__device__ __forceinline__ void collide(D1Q3, double *f, const CollF64 &k) { collide(D1Q3{}, f, k.k); }
+
+// Threads per block of the sweep: more, smaller blocks balance the SMs better.
+template <typename T> __host__ __device__ constexpr int sweep_threads() { return 128; }
 
 // K is the collision-constant type; the matching collide() overload (float,
 // double or 64-bit fixed point) is picked by overload resolution.

@@ -44,6 +44,15 @@ bool fx_constants_ok(const lb_ctx &c)
     return true;
 }
 
+CollF64 make_coll_f64(const lb_ctx &c)
+{
+    CollF64 r;
+    r.k = make_coll<double>(c);
+    r.ints = fx_constants_ok(c) && fabs(r.k.c0) + 4.0 * fabs(r.k.k2) < 1.9;
+    r.x = r.ints ? make_coll_fx(&c) : CollFx{};
+    return r;
+}
+
 // The constants with the context's range flag, for the single-grid sweeps.
 static CollFxR make_coll_fxr(lb_ctx *c)
 {

@@ -67,14 +67,14 @@ template <> struct Vec<long long> { using type = longlong2; static constexpr int
 // One 16-byte vector, except in 4D: with q = 33 populations two-phase
 // gathers of one 16-byte vector per population need more registers than
 // keep enough warps resident, so the 4D sweep narrows the lane to 8 bytes
-// (one int64, two floats); FP64, bound by the FP64 pipe, keeps the vector.
-__host__ __device__ inline constexpr int lane_width(int d, int elem_bytes, bool fp64)
+// (one int64, one double, two floats).
+__host__ __device__ inline constexpr int lane_width(int d, int elem_bytes)
 {
-    return (d == 4 && !fp64) ? 8 / elem_bytes : 16 / elem_bytes;
+    return d == 4 ? 8 / elem_bytes : 16 / elem_bytes;
 }
 template <class L, typename T> __host__ __device__ constexpr int lane_width()
 {
-    return lane_width(L::D, (int)sizeof(T), std::is_same<T, double>::value);
+    return lane_width(L::D, (int)sizeof(T));
 }
 
 // Grid geometry of one padded state array.
@@ -171,6 +171,13 @@ struct CollFx {
 struct CollFxR : CollFx {
     int *range;
 };
+// FP64 storage: the constants as doubles, and with 64 fraction bits for the
+// collision formed on the integer pipes (used where ints != 0).
+struct CollF64 {
+    Coll<double> k;
+    CollFx x;
+    int ints;
+};
 constexpr int kFxCoefBits = 62;  // initialisation and adjoint constants
 constexpr int kFxCollBits = 64;  // collision constants (CollFx)
 
@@ -258,6 +265,11 @@ CollFx make_coll_fx(const lb_ctx *c);  // the same constants in 64-bit fixed poi
 // and |k3| < 1/4; wd and cA grow with the weights (the paper's set leaves
 // the range only for eps above 1.66 in 2D, 0.88 in 3D and 0.61 in 4D).
 bool fx_constants_ok(const lb_ctx &c);
+// The FP64 collision's constants.  Its integer form is taken (ints = 1) for
+// constants that fx_constants_ok admits and whose rest population
+// c0 theta - 2 k2 sum P_aa stays below 2^63 for magnitudes that sum below 2^62
+// (|c0| + 4 |k2| < 1.9: the paper's set at every eps of its examples).
+CollF64 make_coll_f64(const lb_ctx &c);
 // Device flags of a context (ctx->dflag): 0 initialisation, 1 recovery
 // (bit 0: theta <= 0 or non-finite, bit 2: a staging wait timed out),
 // 2 fixed-point sweep range (CollFxR).

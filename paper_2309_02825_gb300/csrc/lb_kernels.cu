@@ -500,24 +500,35 @@ template Coll<double> make_coll<double>(const lb_ctx &);
 template Coll<float> make_coll<float>(const lb_ctx &);
 
 
+template <typename T> struct SweepK {
+    using type = Coll<T>;
+    static type make(const lb_ctx &c) { return make_coll<T>(c); }
+};
+template <> struct SweepK<double> {
+    using type = CollF64;
+    static type make(const lb_ctx &c) { return make_coll_f64(c); }
+};
+
 template <class L, typename T> static cudaError_t sweep_t(lb_ctx *c, const void *src, void *dst)
 {
+    using K = typename SweepK<T>::type;
+    const K k = SweepK<T>::make(*c);
     constexpr int TH = sweep_threads<T>();
     const bool flat = sweep_flat(c->geom, L::D, (int)sizeof(T));
     const unsigned nb = (unsigned)(((flat ? c->geom.fseg : c->geom.nseg) + TH / 32 - 1) / (TH / 32));
     if constexpr (L::D == 4 && sizeof(T) == 8) {
         if (flat) {
-            sweep_flat_kernel<L, T, Coll<T>><<<nb, TH, 0, c->stream>>>((const T *)src, (T *)dst, c->geom,
-                                                                       make_coll<T>(*c));
+            sweep_flat_kernel<L, T, K><<<nb, TH, 0, c->stream>>>((const T *)src, (T *)dst, c->geom,
+                                                                       k);
             return cudaGetLastError();
         }
     }
     if (c->geom.mirror)
-        sweep_kernel<L, T, Coll<T>, true><<<nb, TH, 0, c->stream>>>(
-            (const T *)src, (T *)dst, c->geom, make_coll<T>(*c));
+        sweep_kernel<L, T, K, true><<<nb, TH, 0, c->stream>>>(
+            (const T *)src, (T *)dst, c->geom, k);
     else
-        sweep_kernel<L, T, Coll<T>><<<nb, TH, 0, c->stream>>>(
-            (const T *)src, (T *)dst, c->geom, make_coll<T>(*c));
+        sweep_kernel<L, T, K><<<nb, TH, 0, c->stream>>>(
+            (const T *)src, (T *)dst, c->geom, k);
     return cudaGetLastError();
 }
 
