@@ -196,18 +196,21 @@ lb_status lb_set_theta0(lb_ctx *ctx, const double *theta0, const double *grad_th
 lb_status lb_step(lb_ctx *ctx, int64_t nsteps);
 
 /*
- * Temporally blocked sweeps (periodic 2D grids).  The sweep of lb_step reads
- * and writes the whole state every step, so it is bound by HBM bandwidth.
- * With blocking, each launch advances K steps: a block loads one tile of
+ * Schedule of the sweeps.  A sweep of one step per launch reads and writes the
+ * whole state every step, so it is bound by HBM bandwidth.  A new context runs
+ * the library's own choice: on periodic 2D and 3D grids large enough to fill
+ * the device, launches of two to five steps that march windows of the grid
+ * along its slowest axis; one sweep per launch elsewhere.  This call selects
+ * one sweep per launch or, on periodic 2D grids, launches of K steps on square
+ * tiles: a block loads one tile of
  * the grid with a K-node periodic halo into shared memory, runs the same
  * pull + collide K times there (one shared buffer, updated in place: steps
  * alternate between pulling from the neighbours' slots and updating a
  * node's own slots, and each node reads exactly the slots it writes) and
  * stores the tile, so HBM is read and written once per K steps; the halo
- * nodes are recomputed.  Results are bit-identical to lb_step's one sweep per
- * launch.  For LB_FX64 the range check (|f| < 2^61) covers the values
- * stored at the end of every launch.
- *   steps_per_launch  K in 1..64, or 0 for one sweep per launch (default).
+ * nodes are recomputed.  Every schedule gives the same bits, and for LB_FX64
+ * the range check (|f| < 2^61) covers the values of every step.
+ *   steps_per_launch  K in 1..64, or 0 for one sweep per launch.
  *   tile     each axis of N nodes is cut into ceil(N / tile) near-equal tiles;
  *            the largest tile plus its halo, 9 values per node, must fit the
  *            device's shared memory per block.
@@ -218,19 +221,23 @@ lb_status lb_step(lb_ctx *ctx, int64_t nsteps);
  */
 lb_status lb_set_blocking(lb_ctx *ctx, int steps_per_launch, int tile, int threads);
 
-/* Current blocking, info[0..3] (host): {steps per launch (0: none), tile, threads, tiles}. */
+/*
+ * Schedule set by lb_set_blocking or lb_autotune, info[0..3] (host): {steps per
+ * launch, tile edge (marching windows: columns per window), threads, blocks per
+ * launch}; zeros for one sweep per launch and for the library's own choice.
+ */
 lb_status lb_get_blocking(const lb_ctx *ctx, int *info);
 
 /*
  * Times about trial_steps steps (rounded up to whole launches) for one sweep
- * per launch and for blocked sweeps (K = 2, 3, 4, 5, 6, 8, 12 x the largest
+ * per launch, for marching windows and for square tiles (K = 2, 3, 4, 5, 6, 8, 12 x the largest
  * square tile that fits one to four blocks per SM and that tile less 4 nodes
  * x 256, 512, 1024 threads) on this
  * grid and keeps the fastest (lb_set_blocking).  The trials overwrite the
- * state: call lb_set_theta0 afterwards.  A grid that blocking does not cover
- * (d != 2, walls) keeps one sweep per launch.  choice (host, may be NULL)
- * receives {steps per launch (0: one sweep per launch), tile, threads,
- * microseconds per step of the winner}.  Synchronises the stream.
+ * state: call lb_set_theta0 afterwards.  A grid that tiles do not cover
+ * (d != 2, walls) keeps its schedule.  choice (host, may be NULL) receives
+ * {steps per launch (0: one sweep per launch), tile (or columns per marching
+ * window), threads, microseconds per step of the winner}.  Synchronises the stream.
  * Errors: LB_EINVAL, LB_ECUDA.
  */
 lb_status lb_autotune(lb_ctx *ctx, int trial_steps, double *choice);

@@ -141,6 +141,28 @@ cudaError_t record_blocked(lb_ctx *c, int from)
     return e;
 }
 
+// The schedule lb_step runs when the caller has set none (kSchedAuto).  On
+// periodic 2D and 3D grids large enough to fill the chip, marching sweeps
+// (lb_march.cu); on small 2D grids, whose single sweeps last about as long as
+// their launch, several steps per launch on square tiles; else one sweep per
+// launch.  Every choice gives the same bits.
+cudaError_t choose_schedule(lb_ctx *c)
+{
+    if (c->sched != lbk::kSchedAuto) return cudaSuccess;
+    c->run = lbk::kSchedSweeps;
+    lbk::blocked_release(c);
+    c->march = lbk::MarchPlan{};
+    if (c->geom.mirror) return cudaSuccess;
+    bool worth = false;
+    cudaError_t e = lbk::march_setup(c, &c->march, &worth);
+    if (e != cudaSuccess) return e;
+    if (worth) {
+        c->run = lbk::kSchedMarch;
+        return cudaSuccess;
+    }
+    return cudaSuccess;
+}
+
 bool capturing(cudaStream_t s)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -258,13 +280,18 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     }
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    c->scratch_blocks = (sms > 0 ? sms : 148) * 4;
+    if (sms > 0) c->sms = sms;
+    c->scratch_blocks = c->sms * 4;
     if ((e = cudaMalloc(&c->scratch, sizeof(double) * lbk::kRedSlots * c->scratch_blocks)) != cudaSuccess ||
         (e = cudaMalloc(&c->dout, sizeof(double) * 64)) != cudaSuccess ||
         (e = cudaMalloc(&c->dflag, sizeof(int) * 4)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 4, c->stream)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: scratch allocation");
+    }
+    if ((e = choose_schedule(c)) != cudaSuccess) {
+        free_ctx(c);
+        return cuda_fail(nullptr, e, "lb_create: schedule");
     }
     *out = c;
     return LB_OK;
@@ -314,8 +341,12 @@ lb_status lb_set_boundary(lb_ctx *c, const int *kind)
         }
     c->geom.mirror = mask;
     c->initialized = false;  // the stored state follows the old walls: initialise again
-    if (mask) lbk::blocked_release(c);  // blocked sweeps are periodic only
     ++c->gen;
+    if (mask && c->sched != lbk::kSchedAuto) {  // sweeps of several steps per launch are periodic only
+        lbk::blocked_release(c);
+        c->sched = c->run = lbk::kSchedSweeps;
+    }
+    if ((e = choose_schedule(c)) != cudaSuccess) return cuda_fail(c, e, "lb_set_boundary: schedule");
     return LB_OK;
 }
 
@@ -356,11 +387,11 @@ lb_status lb_set_viscosity(lb_ctx *c, double nu)
     c->sigma = trial.sigma;
     c->cs2 = trial.cs2;
     ++c->gen;
-    if (c->tb_k > 0) {  // the blocked descriptor carries the collision constants
-        bool fits = true;
-        if ((e = lbk::blocked_setup(c, c->tb_k, c->tb_tile, c->tb_threads, &fits)) != cudaSuccess)
-            return cuda_fail(c, e, "lb_set_viscosity: blocked sweeps");
-    }
+    for (auto &g : c->tb_graph)
+        if (g) {
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
     return LB_OK;
 }
 
@@ -379,6 +410,7 @@ lb_status lb_set_blocking(lb_ctx *c, int steps_per_launch, int tile, int threads
     bool fits = true;
     if ((e = lbk::blocked_setup(c, steps_per_launch, tile, threads, &fits)) != cudaSuccess)
         return cuda_fail(c, e, "lb_set_blocking");
+    c->sched = c->run = c->tb_k ? lbk::kSchedTiles : lbk::kSchedSweeps;
     if (!fits) return fail(c, LB_EINVAL, "lb_set_blocking: tile plus halo exceeds the shared memory per block");
     return LB_OK;
 }
@@ -386,10 +418,18 @@ lb_status lb_set_blocking(lb_ctx *c, int steps_per_launch, int tile, int threads
 lb_status lb_get_blocking(const lb_ctx *c, int *info)
 {
     if (!c || !info) return LB_EINVAL;
-    info[0] = c->tb_k;
-    info[1] = c->tb_tile;
-    info[2] = c->tb_threads;
-    info[3] = c->tb_ntiles;
+    info[0] = info[1] = info[2] = info[3] = 0;
+    if (c->sched == lbk::kSchedTiles) {
+        info[0] = c->tb_k;
+        info[1] = c->tb_tile;
+        info[2] = c->tb_threads;
+        info[3] = c->tb_ntiles;
+    } else if (c->sched == lbk::kSchedMarch) {
+        info[0] = c->march.steps;
+        info[1] = c->march.bx;
+        info[2] = c->march.threads;
+        info[3] = c->march.nx * c->march.ny * c->march.nc;
+    }
     return LB_OK;
 }
 
@@ -408,9 +448,14 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_autotune");
     struct Cand {
-        int K, tile, threads;
+        int sched, K, tile, threads;
     };
-    std::vector<Cand> cands = {{0, 0, 0}};
+    std::vector<Cand> cands = {{lbk::kSchedSweeps, 0, 0, 0}};
+    lbk::MarchPlan plan{};
+    bool worth = false;
+    if ((e = lbk::march_setup(c, &plan, &worth)) != cudaSuccess) return cuda_fail(c, e, "lb_autotune");
+    if (plan.steps) cands.push_back({lbk::kSchedMarch, plan.steps, plan.bx, plan.threads});
+    c->march = plan;
     int optin = 0;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device)) != cudaSuccess)
         return cuda_fail(c, e, "lb_autotune");
@@ -423,7 +468,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
             // the largest square tile for this many blocks per SM, and one 4 nodes smaller (less work per block)
             for (int tile : {edge - 2 * K, edge - 2 * K - 4}) {
                 if (tile < 8) continue;
-                for (int th : {256, 512, 1024}) cands.push_back({K, tile, th});
+                for (int th : {256, 512, 1024}) cands.push_back({lbk::kSchedTiles, K, tile, th});
             }
         }
     const bool was_init = c->initialized;
@@ -436,11 +481,12 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
     lb_status st = LB_OK;
     for (const Cand &cd : cands) {
         bool fits = true;
-        if ((e = lbk::blocked_setup(c, cd.K, cd.tile, cd.threads, &fits)) != cudaSuccess) {
+        if ((e = lbk::blocked_setup(c, cd.sched == lbk::kSchedTiles ? cd.K : 0, cd.tile, cd.threads, &fits)) != cudaSuccess) {
             st = cuda_fail(c, e, "lb_autotune");
             break;
         }
         if (!fits) continue;
+        c->sched = c->run = cd.sched;
         const int64_t n = cd.K ? (trial_steps + cd.K - 1) / cd.K * cd.K : trial_steps;
         if ((st = lb_step(c, n)) != LB_OK) break;  // warm-up
         if ((e = cudaEventRecord(e0, c->stream)) != cudaSuccess) {
@@ -465,10 +511,12 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
     c->initialized = false;  // the trials overwrote the state: set it again
     c->step = 0;
     (void)was_init;
-    if (st != LB_OK) return st;
+    if (st != LB_OK) win = cands[0];
     bool fits = true;
-    if ((e = lbk::blocked_setup(c, win.K, win.tile, win.threads, &fits)) != cudaSuccess)
+    if ((e = lbk::blocked_setup(c, win.sched == lbk::kSchedTiles ? win.K : 0, win.tile, win.threads, &fits)) != cudaSuccess)
         return cuda_fail(c, e, "lb_autotune");
+    c->sched = c->run = win.sched;
+    if (st != LB_OK) return st;
     if (choice) {
         choice[0] = win.K;
         choice[1] = win.tile;
@@ -552,7 +600,17 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     // directly so that they land in the caller's graph.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
-    if (c->tb_k > 0) {
+    if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps) {
+        // marching launches; the remainder below, one sweep per launch
+        while (nsteps >= c->march.steps) {
+            cudaError_t e = lbk::march_launch(c, c->f[c->cur], c->f[c->cur ^ 1], c->stream);
+            if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: marching launch");
+            c->cur ^= 1;
+            c->step += c->march.steps;
+            nsteps -= c->march.steps;
+        }
+    }
+    if (c->run == lbk::kSchedTiles && c->tb_k > 0) {
         // blocked: launches of tb_k steps (recorded in graphs), then one launch for the remainder
         int64_t launches = nsteps / c->tb_k;
         const int rem = (int)(nsteps % c->tb_k);

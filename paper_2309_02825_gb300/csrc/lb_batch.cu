@@ -160,17 +160,33 @@ __host__ __device__ inline size_t tb_smem_bytes(int q, int elem, int W, int H)
     return (size_t)q * W * H * elem;
 }
 
-template <class L, typename T, int TH>
+// One grid's tiles, numbered row by row: tx x ty nodes each, the last of a row
+// or column smaller.
+template <typename T> struct OneGrid {
+    InstDesc<T> d;
+    int tx, ty, ntx;
+};
+
+// ONE: the tiles of a single grid, its descriptor a kernel argument and each
+// tile's place found from the block's number; else instances and tiles from
+// the tables of a batch.
+template <class L, typename T, int TH, bool ONE>
 __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const InstDesc<T> *__restrict__ inst,
                                                                      const TileDesc *__restrict__ tiles,
                                                                      const T *__restrict__ src, T *__restrict__ dst,
-                                                                     int K, int *__restrict__ range)
+                                                                     int K, int *__restrict__ range, OneGrid<T> one)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int Q = L::Q, NW = TH / 32;
     constexpr int E = (int)sizeof(T), NB = Q * E;  // bytes per value, per node
-    const TileDesc t = tiles[blockIdx.x];
-    const InstDesc<T> D = inst[t.inst];
+    TileDesc t;
+    if constexpr (ONE) {
+        const int by = (int)blockIdx.x / one.ntx, bx = (int)blockIdx.x - by * one.ntx;
+        t = {0, bx * one.tx, by * one.ty, min(one.tx, one.d.g.N0 - bx * one.tx), min(one.ty, one.d.g.N1 - by * one.ty)};
+    } else {
+        t = tiles[blockIdx.x];
+    }
+    const InstDesc<T> D = ONE ? one.d : inst[t.inst];
     const int W = t.tx + 2 * K, H = t.ty + 2 * K;
     const int gx0 = t.x0 - K;  // global column of tile column 0 (may be < 0)
     const unsigned smA = (unsigned)__cvta_generic_to_shared(smem_raw);
@@ -196,7 +212,16 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    // K steps in place, alternating pull and local.
+    // K steps in place, alternating pull and local.  acc: OR of the high words +
+    // 2^29 of the fixed-point values of every step (|v| < 2^61 check; a
+    // diagonal pair's two values are equal).
+    unsigned acc = 0u;
+    const auto check = [&](const T(&f)[Q]) {
+        if constexpr (std::is_same<T, long long>::value) {
+#pragma unroll
+            for (int i = 0; i < 7; ++i) acc |= (unsigned)((unsigned long long)f[i] >> 32) + 0x20000000u;
+        }
+    };
     for (int st = 0; st < K; ++st) {
         // this thread's nodes of the RW x RH region: flat indices tid, tid + TH,
         // ... walked as (row, column) without a division per node
@@ -219,6 +244,7 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
                     f[i] = lds<T, (-ex * Q + o) * E>(rb[1 - ey]);
                 });
                 collide(L{}, f, D.k);
+                check(f);
                 static_for<0, Q>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     constexpr int ex = L::E[i][0], ey = L::E[i][1];
@@ -239,6 +265,7 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
                     f[i] = lds<T, i * E>(nb);
                 });
                 collide(L{}, f, D.k);
+                check(f);
                 static_for<0, Q>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     sts<reflect_pop<L>(i, 3) * E>(nb, f[i]);
@@ -252,7 +279,6 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
     // from slot opp(i) of z, after an odd number from slot i of z + e_i.
     T *d = dst + D.off;
     const bool odd = (K & 1) != 0;
-    unsigned acc = 0u;  // fixed point: OR of the high words + 2^29 of the stored values (|v| < 2^61 check)
     for (int r = warp; r < t.ty; r += NW) {
         T *grow = d + (int64_t)(t.y0 + r) * D.g.pitch + t.x0;
         const unsigned rb[3] = {smA + (unsigned)(r + K - 1) * rowB, smA + (unsigned)(r + K) * rowB,
@@ -263,8 +289,6 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
                 constexpr int i = decltype(I)::value;
                 constexpr int ex = L::E[i][0], ey = L::E[i][1], o = reflect_pop<L>(i, 3);
                 const T v = odd ? lds<T, (ex * Q + i) * E>(rb[1 + ey] + cb) : lds<T, o * E>(rb[1] + cb);
-                if constexpr (std::is_same<T, long long>::value)
-                    acc |= (unsigned)((unsigned long long)v >> 32) + 0x20000000u;
                 grow[(int64_t)i * D.g.slab + c] = v;
             });
         }
@@ -492,24 +516,21 @@ void append_tiles(std::vector<lbk::TileDesc> &tv, int inst, int n0, int n1, int 
 
 constexpr int kTbGraphLaunches = 16;  // blocked launches per recorded graph (even)
 
-template <typename T, int TH> const void *tb_kernel()
+template <typename T, bool ONE> const void *tb_kernel_for(int threads)
 {
-    return (const void *)lbk::batch_tb_kernel<lbk::D2Q9, T, TH>;
+    return threads == 256   ? (const void *)lbk::batch_tb_kernel<lbk::D2Q9, T, 256, ONE>
+           : threads == 512 ? (const void *)lbk::batch_tb_kernel<lbk::D2Q9, T, 512, ONE>
+                            : (const void *)lbk::batch_tb_kernel<lbk::D2Q9, T, 1024, ONE>;
 }
 
-template <typename T> const void *tb_kernel_for(int threads)
+template <bool ONE> const void *tb_kernel_prec(int precision, int threads)
 {
-    return threads == 256 ? tb_kernel<T, 256>() : (threads == 512 ? tb_kernel<T, 512>() : tb_kernel<T, 1024>());
+    if (precision == LB_FP64) return tb_kernel_for<double, ONE>(threads);
+    if (precision == LB_FX64) return tb_kernel_for<long long, ONE>(threads);
+    return tb_kernel_for<float, ONE>(threads);
 }
 
-const void *tb_kernel_prec(int precision, int threads)
-{
-    if (precision == LB_FP64) return tb_kernel_for<double>(threads);
-    if (precision == LB_FX64) return tb_kernel_for<long long>(threads);
-    return tb_kernel_for<float>(threads);
-}
-
-const void *tb_kernel_of(const lb_batch *b, int threads) { return tb_kernel_prec(b->precision, threads); }
+const void *tb_kernel_of(const lb_batch *b, int threads) { return tb_kernel_prec<false>(b->precision, threads); }
 
 size_t tb_smem(const lb_batch *b, int K)
 {
@@ -520,7 +541,11 @@ size_t tb_smem(const lb_batch *b, int K)
 cudaError_t launch_tb(lb_batch *b, int from, int K, cudaStream_t s)
 {
     int *range = nullptr;
-    void *args[] = {&b->d_desc, &b->d_tiles, &b->buf[from], &b->buf[from ^ 1], &K, &range};
+    lbk::OneGrid<double> unused{};  // at least as large as the other types' (the kernel does not read it)
+    static_assert(sizeof(lbk::OneGrid<double>) >= sizeof(lbk::OneGrid<long long>) &&
+                      sizeof(lbk::OneGrid<double>) >= sizeof(lbk::OneGrid<float>),
+                  "argument size");
+    void *args[] = {&b->d_desc, &b->d_tiles, &b->buf[from], &b->buf[from ^ 1], &K, &range, &unused};
     return cudaLaunchKernel(tb_kernel_of(b, b->tb_threads), dim3((unsigned)b->ntiles), dim3((unsigned)b->tb_threads),
                             args, tb_smem(b, K), s);
 }
@@ -544,8 +569,9 @@ lb_status build_tiles(lb_batch *b, int K, int tile, int threads)
     const size_t need = lbk::tb_smem_bytes(9, (int)b->elem, maxw + 2 * K, maxh + 2 * K);
     if (need > (size_t)optin)
         return bfail(b, LB_EINVAL, "lb_batch_set_blocking: tile plus halo exceeds the shared memory per block");
-    if ((e = cudaFuncSetAttribute(tb_kernel_of(b, threads), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)need)) != cudaSuccess ||
+    // the attribute belongs to the kernel, which every batch shares: allow the device's limit
+    if ((e = cudaFuncSetAttribute(tb_kernel_of(b, threads), cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) !=
+            cudaSuccess ||
         (e = cudaMalloc(&b->d_tiles, sizeof(lbk::TileDesc) * tv.size())) != cudaSuccess ||
         (e = cudaMemcpy(b->d_tiles, tv.data(), sizeof(lbk::TileDesc) * tv.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
@@ -709,25 +735,29 @@ cudaError_t run_steps(lb_batch *b, int64_t n)
 
 // ---------------------------------------------------------------------------
 // Blocked sweeps of a single 2D periodic grid: the batched blocked kernel on
-// a batch of one instance (the context's own buffers, offset 0).
+// one instance (the context's own buffers, offset 0).
 // ---------------------------------------------------------------------------
 namespace lbk {
 
-template <typename T> static cudaError_t upload_single_desc(lb_ctx *c)
+template <typename T> static cudaError_t blocked_launch_t(lb_ctx *c, const void *src, void *dst, int K, cudaStream_t s)
 {
-    InstDesc<T> h;
-    h.g = c->geom;
+    OneGrid<T> one{};
+    one.d.g = c->geom;
     if constexpr (std::is_same<T, long long>::value)
-        h.k = make_coll_fx(c);
+        one.d.k = make_coll_fx(c);
     else if constexpr (std::is_same<T, double>::value)
-        h.k = make_coll_f64(*c);
+        one.d.k = make_coll_f64(*c);
     else
-        h.k = make_coll<T>(*c);
-    h.off = 0;
-    cudaError_t e = cudaSuccess;
-    if (!c->tb_desc) e = cudaMalloc(&c->tb_desc, std::max(sizeof(InstDesc<long long>), sizeof(InstDesc<double>)));
-    if (e == cudaSuccess) e = cudaMemcpy(c->tb_desc, &h, sizeof(h), cudaMemcpyHostToDevice);
-    return e;
+        one.d.k = make_coll<T>(*c);
+    one.tx = c->tb_tx;
+    one.ty = c->tb_ty;
+    one.ntx = ((int)c->N[0] + c->tb_tx - 1) / c->tb_tx;
+    const void *none = nullptr;
+    int *range = c->precision == LB_FX64 ? c->dflag + kFlagRange : nullptr;
+    void *args[] = {&none, &none, (void *)&src, &dst, &K, &range, &one};
+    const size_t smem = tb_smem_bytes(9, (int)c->elem, c->tb_tx + 2 * K, c->tb_ty + 2 * K);
+    return cudaLaunchKernel(tb_kernel_for<T, true>(c->tb_threads), dim3((unsigned)c->tb_ntiles),
+                            dim3((unsigned)c->tb_threads), args, smem, s);
 }
 
 void blocked_release(lb_ctx *c)
@@ -737,10 +767,6 @@ void blocked_release(lb_ctx *c)
             cudaGraphExecDestroy(ge);
             ge = nullptr;
         }
-    cudaFree(c->tb_tiles);
-    cudaFree(c->tb_desc);
-    c->tb_tiles = nullptr;
-    c->tb_desc = nullptr;
     c->tb_k = c->tb_tile = c->tb_threads = c->tb_ntiles = 0;
 }
 
@@ -749,42 +775,38 @@ cudaError_t blocked_setup(lb_ctx *c, int K, int tile, int threads, bool *fits)
     *fits = true;
     blocked_release(c);
     if (K == 0) return cudaSuccess;
-    std::vector<TileDesc> tv;
-    int maxw = 0, maxh = 0;
-    append_tiles(tv, 0, (int)c->N[0], (int)c->N[1], tile, maxw, maxh);
+    const int n0 = (int)c->N[0], n1 = (int)c->N[1];
+    const int ntx = (n0 + tile - 1) / tile, nty = (n1 + tile - 1) / tile;
+    const int tx = (n0 + ntx - 1) / ntx, ty = (n1 + nty - 1) / nty;
+    const int64_t ntiles = (int64_t)((n0 + tx - 1) / tx) * ((n1 + ty - 1) / ty);
     int optin = 0;
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     if (e != cudaSuccess) return e;
-    const size_t need = tb_smem_bytes(9, (int)c->elem, maxw + 2 * K, maxh + 2 * K);
-    if (need > (size_t)optin || tv.size() > 0x7fffffff) {
+    const size_t need = tb_smem_bytes(9, (int)c->elem, tx + 2 * K, ty + 2 * K);
+    if (need > (size_t)optin || ntiles > 0x7fffffff) {
         *fits = false;
         return cudaSuccess;
     }
-    if ((e = cudaFuncSetAttribute(tb_kernel_prec(c->precision, threads), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)need)) != cudaSuccess)
+    // the attribute belongs to the kernel, which every context shares: allow the device's limit
+    if ((e = cudaFuncSetAttribute(tb_kernel_prec<true>(c->precision, threads), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  optin)) != cudaSuccess)
         return e;
-    if ((e = cudaMalloc(&c->tb_tiles, sizeof(TileDesc) * tv.size())) != cudaSuccess ||
-        (e = cudaMemcpy(c->tb_tiles, tv.data(), sizeof(TileDesc) * tv.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return e;
-    e = c->precision == LB_FP64 ? upload_single_desc<double>(c)
-                                : (c->precision == LB_FX64 ? upload_single_desc<long long>(c) : upload_single_desc<float>(c));
-    if (e != cudaSuccess) return e;
     c->tb_k = K;
     c->tb_tile = tile;
     c->tb_threads = threads;
-    c->tb_ntiles = (int)tv.size();
-    c->tb_maxw = maxw;
-    c->tb_maxh = maxh;
+    c->tb_ntiles = (int)ntiles;
+    c->tb_tx = tx;
+    c->tb_ty = ty;
     return cudaSuccess;
 }
 
 cudaError_t blocked_launch(lb_ctx *c, const void *src, void *dst, int K, cudaStream_t s)
 {
-    int *range = c->precision == LB_FX64 ? c->dflag + kFlagRange : nullptr;
-    void *args[] = {&c->tb_desc, &c->tb_tiles, (void *)&src, &dst, &K, &range};
-    const size_t smem = tb_smem_bytes(9, (int)c->elem, c->tb_maxw + 2 * K, c->tb_maxh + 2 * K);
-    return cudaLaunchKernel(tb_kernel_prec(c->precision, c->tb_threads), dim3((unsigned)c->tb_ntiles),
-                            dim3((unsigned)c->tb_threads), args, smem, s);
+    switch (c->precision) {
+    case LB_FP64: return blocked_launch_t<double>(c, src, dst, K, s);
+    case LB_FX64: return blocked_launch_t<long long>(c, src, dst, K, s);
+    default: return blocked_launch_t<float>(c, src, dst, K, s);
+    }
 }
 
 }  // namespace lbk

@@ -203,6 +203,23 @@ struct InitK {
     int fx_bits;  // F
 };
 
+// How sweeps of several steps per launch cut a grid (lb_march.cu): windows of
+// bx (x by) output columns, chunks of rows along the slowest axis.
+struct MarchPlan {
+    int steps;          // per launch; 0: this grid takes one sweep per launch
+    int bx, by, chunk;  // output columns per window along x (and y in 3D), output rows per chunk
+    int nx, ny, nc;     // windows along x (and y), chunks
+    int threads;        // per block
+};
+
+// How lb_step runs its sweeps.
+enum Sched {
+    kSchedAuto = 0,    // the library's own rule (choose_schedule)
+    kSchedSweeps = 1,  // one sweep per launch
+    kSchedTiles = 2,   // tb_k steps per launch on square tiles (lb_batch.cu)
+    kSchedMarch = 3    // march.steps steps per launch along the slowest axis (lb_march.cu)
+};
+
 }  // namespace lbk
 
 // ---------------------------------------------------------------------------
@@ -233,11 +250,13 @@ struct lb_ctx {
     int64_t step = 0;
     int device = 0;
     uint64_t gen = 0;  // bumped whenever the walls or the viscosity change (recorded launches go stale)
-    // temporally blocked sweeps (lb_set_blocking, 2D periodic): tb_k steps per launch, 0 = one sweep per launch
-    int tb_k = 0, tb_tile = 0, tb_threads = 0, tb_ntiles = 0, tb_maxw = 0, tb_maxh = 0;
-    void *tb_desc = nullptr;   // instance descriptor of the grid (device)
-    void *tb_tiles = nullptr;  // tile table (device)
-    cudaGraphExec_t tb_graph[2] = {nullptr, nullptr};  // recorded blocked launches, by starting buffer
+    int sms = 148;     // multiprocessors of the device
+    // sweeps of several steps per launch: sched as the caller set it, run as what it resolves to
+    int sched = lbk::kSchedAuto, run = lbk::kSchedSweeps;
+    // square tiles (2D periodic): tb_k steps per launch
+    int tb_k = 0, tb_tile = 0, tb_threads = 0, tb_ntiles = 0, tb_tx = 0, tb_ty = 0;
+    cudaGraphExec_t tb_graph[2] = {nullptr, nullptr};  // recorded tiled launches, by starting buffer
+    lbk::MarchPlan march{};
     std::string err;
 };
 
@@ -297,13 +316,17 @@ cudaError_t launch_maxabs(lb_ctx *c, const double *x, int64_t n, double *out_dev
 cudaError_t launch_sweep_fx(lb_ctx *c, const void *src, void *dst);
 cudaError_t launch_norms(lb_ctx *c, const double *theta, const double *u, const double *ex_theta,
                          const double *ex_u, double *out_dev);
-// Temporally blocked sweeps of one 2D periodic grid (lb_batch.cu, the batched
-// blocked kernel on a batch of one): set up the tile table and descriptor for
-// K steps per launch (K = 0 releases them), and launch K steps from src to dst.
-// The fixed-point path checks the values it stores (|f| < 2^61) into
-// ctx->dflag[kFlagRange].
+// Square-tile sweeps of one 2D periodic grid (lb_batch.cu, the batched blocked
+// kernel on one grid): set up K steps per launch (K = 0 releases them), and
+// launch K steps from src to dst.  The fixed-point path checks the values of
+// every step (|f| < 2^61) into ctx->dflag[kFlagRange].
 cudaError_t blocked_setup(lb_ctx *c, int K, int tile, int threads, bool *fits);
 cudaError_t blocked_launch(lb_ctx *c, const void *src, void *dst, int K, cudaStream_t s);
 void blocked_release(lb_ctx *c);
+// Marching sweeps of a periodic 2D or 3D grid (lb_march.cu): the cut of the
+// grid (steps = 0 where they are not built), whether the rule takes them over
+// one sweep per launch, and one launch of plan.steps steps.
+cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth);
+cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s);
 
 }  // namespace lbk

@@ -1,0 +1,381 @@
+// Marching sweeps: several time steps per launch on large periodic 2D and 3D
+// grids, with the intermediate states on chip.
+//
+// A block owns a window of columns (2D: x positions; 3D: an x-y patch), one
+// column per thread, and marches along the slowest axis (the rows of 2D, the
+// planes of 3D).  KS steps run as a pipeline of KS stages: in iteration t,
+// stage 1 pulls row t of the stored state from global memory and collides it;
+// stage s + 1 collides, two rows behind stage s, the state that stage s made;
+// stage KS stores.  HBM is read and written once per KS steps, rows are never
+// recomputed inside a block's march (only at its two ends), and columns only
+// over the KS - 1 outermost columns of each window edge.  The square tiles of
+// batch_tb_kernel recompute a halo on four sides (23 % more updates at 4
+// steps, 28^2), move every value through shared memory once per step and
+// separate their load, step and store phases by barriers; here the loads of
+// the next row are in flight while all stages of this one compute, the KS
+// collisions of an iteration are independent of each other, and one barrier
+// per iteration orders them.
+//
+// Between two stages, a population that moves within the row goes through
+// shared memory (another thread's column reads it) and one that keeps its
+// column stays in the thread's registers.  A population with velocity component
+// em along the march, made for row r in iteration t, is read in iteration
+// t + 2 + em, so rings of 3 + em rows (2, 3, 4) let every iteration write one
+// slot while the slots still to be read stay untouched: the slot read is always
+// the next one to be overwritten.
+//
+// The arithmetic per node is the sweep's own collision on the same inputs, so
+// the results are bit for bit those of one sweep per launch.  Threads whose
+// stage lies outside its valid columns or rows compute on whatever the slots
+// hold (fixed point, float) or skip the collision (FP64, whose integer form
+// would leave its fast path on such values); nothing of theirs is stored,
+// checked or read by a valid node.
+#include <algorithm>
+
+#include "lb_device.cuh"
+
+namespace lbk {
+// Collision constants as the sweeps take them.
+template <typename T> struct MarchK {
+    using type = Coll<T>;
+    static type make(lb_ctx *c) { return make_coll<T>(*c); }
+};
+template <> struct MarchK<double> {
+    using type = CollF64;
+    static type make(lb_ctx *c) { return make_coll_f64(*c); }
+};
+template <> struct MarchK<long long> {
+    using type = CollFxR;
+    static type make(lb_ctx *c)
+    {
+        CollFxR k;
+        static_cast<CollFx &>(k) = make_coll_fx(c);
+        k.range = c->dflag + kFlagRange;
+        return k;
+    }
+};
+
+template <class L> struct MarchL {
+    static constexpr int A = L::D - 1;  // the march axis
+    // zero velocity within the row: held in registers
+    __host__ __device__ static constexpr bool own(int i)
+    {
+        for (int a = 0; a < A; ++a)
+            if (L::E[i][a] != 0) return false;
+        return true;
+    }
+    // ring slots of the shared populations before i
+    __host__ __device__ static constexpr int slot0(int i)
+    {
+        int s = 0;
+        for (int j = 0; j < i; ++j)
+            if (!own(j)) s += 3 + L::E[j][A];
+        return s;
+    }
+    static constexpr int kSlots = slot0(L::Q);
+    __host__ __device__ static constexpr int pick(int em)  // the register population with march component em
+    {
+        for (int i = 0; i < L::Q; ++i)
+            if (own(i) && L::E[i][A] == em) return i;
+        return -1;
+    }
+};
+
+// 3D windows are 32 columns along x, one warp per row of the patch: a warp's
+// loads then cover 8-9 sectors per 8-byte population (16 columns: 5-6 sectors
+// for half the columns; 256^3 fixed point 27.4 -> 30.6 GLUPS, FP32 51 -> 62),
+// and wider windows leave fewer rows in a block, so more recomputed ones.
+constexpr int kMarchW = 32;
+// Pad columns before and after the rings: the reads of the outermost columns stay inside the allocation.
+template <class L> __host__ __device__ constexpr int march_pad() { return L::D == 3 ? kMarchW + 1 : 2; }
+template <class L, int KS, int TH> constexpr size_t march_smem(int elem)
+{
+    return ((size_t)(KS - 1) * MarchL<L>::kSlots * TH + 2 * (size_t)march_pad<L>()) * elem;
+}
+
+// SKIP: a stage outside its rows (the pipeline's fill and drain) does nothing.
+// The branch is block-uniform, but ends a scheduling region; where the
+// collisions are short (3D float) that costs more than the idle work (256^3:
+// 78 against 66 GLUPS), elsewhere less (1024^2 fixed point 76 against 66).
+template <class L, typename T, class K, int KS, int TH, int MINB, bool SKIP>
+__global__ void __launch_bounds__(TH, MINB) march_kernel(const T *__restrict__ src, T *__restrict__ dst, Geom g, K k,
+                                                         MarchPlan p)
+{
+    constexpr int D = L::D, Q = L::Q, A = D - 1, S = MarchL<L>::kSlots, E = (int)sizeof(T);
+    constexpr int IM = MarchL<L>::pick(-1), IC = MarchL<L>::pick(0), IP = MarchL<L>::pick(1);
+    extern __shared__ __align__(16) unsigned char march_raw[];
+    T *const sm = reinterpret_cast<T *>(march_raw);
+    const int tid = threadIdx.x;
+
+    // the window and chunk of this block
+    unsigned b = blockIdx.x;
+    const int wx = (int)(b % (unsigned)p.nx);
+    b /= (unsigned)p.nx;
+    const int wy = D == 3 ? (int)(b % (unsigned)p.ny) : 0;
+    const int ch = D == 3 ? (int)(b / (unsigned)p.ny) : (int)b;
+    const int NR = D == 3 ? g.N2 : g.N1;  // rows of the march
+    constexpr int bw = D == 3 ? kMarchW : TH;
+    const int cx = D == 3 ? tid % bw : tid, cy = D == 3 ? tid / bw : 0;
+    const int x0 = wx * p.bx, y0 = wy * p.by, r0 = ch * p.chunk;
+    const int nx = min(p.bx, g.N0 - x0), nr = min(p.chunk, NR - r0);
+    const int ny = D == 3 ? min(p.by, g.N1 - y0) : 1;
+    // stage s is valid on columns s - 1 <= cx < nx + 2 KS - 1 - s (cy likewise): its distance to the window's edge
+    int edge = min(cx, nx + 2 * (KS - 1) - 1 - cx);
+    if (D == 3) edge = min(edge, min(cy, ny + 2 * (KS - 1) - 1 - cy));
+
+    // offsets of this column's sources within a population: x - ex (and y - ey) wrapped
+    auto wrapn = [](int v, int n) {
+        v %= n;
+        return v < 0 ? v + n : v;
+    };
+    const int gx = wrapn(x0 - (KS - 1) + cx, g.N0);
+    const int gxs[3] = {gx + 1 == g.N0 ? 0 : gx + 1, gx, gx == 0 ? g.N0 - 1 : gx - 1};  // by ex + 1
+    int gys[3] = {0, 0, 0};
+    if (D == 3) {
+        const int gy = wrapn(y0 - (KS - 1) + cy, g.N1);
+        gys[0] = (gy + 1 == g.N1 ? 0 : gy + 1) * g.pitch;
+        gys[1] = gy * g.pitch;
+        gys[2] = (gy == 0 ? g.N1 - 1 : gy - 1) * g.pitch;
+    }
+    const int64_t rstride = D == 3 ? (int64_t)g.N1 * g.pitch : (int64_t)g.pitch;
+
+    // rows r - 1, r, r + 1 of stage 1, wrapped
+    int rc = wrapn(r0 - (KS - 1), NR);
+    auto load_row = [&](T(&f)[Q], int r) {
+        const T *rows[3] = {src + (r + 1 == NR ? 0 : r + 1) * rstride, src + r * rstride,
+                            src + (r == 0 ? NR - 1 : r - 1) * rstride};  // by em + 1
+        static_for<0, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int ex = L::E[i][0], ey = D == 3 ? L::E[i][1] : 0, em = L::E[i][A];
+            const int col = gxs[ex + 1] + (D == 3 ? gys[ey + 1] : 0);
+            f[i] = __ldcg(rows[em + 1] + (int64_t)i * g.slab + col);
+        });
+    };
+
+    // shared rings: [gap][slot of the population][column]
+    T *const mine = sm + march_pad<L>() + tid;
+    int w2 = 0, w3 = 0, w4 = 0;  // slot written in this iteration, per ring, in elements
+
+    // register populations between stages: made in the last one (m, c, p), two (c, p) and three (p) iterations
+    T hm[KS - 1 > 0 ? KS - 1 : 1], hc[KS - 1 > 0 ? KS - 1 : 1][2], hp[KS - 1 > 0 ? KS - 1 : 1][3];
+#pragma unroll
+    for (int s = 0; s < KS - 1; ++s) {
+        hm[s] = T(0);
+        hc[s][0] = hc[s][1] = T(0);
+        hp[s][0] = hp[s][1] = hp[s][2] = T(0);
+    }
+
+    unsigned acc = 0u;  // fixed point: OR of the high words + 2^29 (|v| < 2^61 check of every stage)
+    const int last = nr + 3 * (KS - 1);  // iterations
+    T f[Q];
+    load_row(f, rc);
+    for (int t = 0; t < last; ++t) {
+        const int r2 = w2 ? 0 : TH, r3 = w3 == 2 * TH ? 0 : w3 + TH, r4 = w4 == 3 * TH ? 0 : w4 + TH;  // slots read
+        T nm, nc, np;  // stage s's register populations, entering the history after stage s + 1 has read it
+        static_for<1, KS + 1>([&](auto Si) {
+            constexpr int s = decltype(Si)::value;
+            // stage s's row of this iteration, counted from the chunk's first row, and where it is valid
+            const int row = t - (KS - 1) - 2 * (s - 1);
+            const bool rok = row >= s - KS && row < nr + KS - s;  // block-uniform
+            const bool ok = rok && edge >= s - 1;
+            T n[Q];
+            if (!SKIP || rok) {
+                if constexpr (s == 1) {
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) n[i] = f[i];
+                } else {
+                    constexpr int gp = s - 2;
+                    const T *const at = mine + gp * S * TH;
+                    static_for<0, Q>([&](auto I) {
+                        constexpr int i = decltype(I)::value;
+                        constexpr int ex = L::E[i][0], ey = D == 3 ? L::E[i][1] : 0, em = L::E[i][A];
+                        if constexpr (i == IM)
+                            n[i] = hm[gp];
+                        else if constexpr (i == IC)
+                            n[i] = hc[gp][1];
+                        else if constexpr (i == IP)
+                            n[i] = hp[gp][2];
+                        else
+                            n[i] = at[MarchL<L>::slot0(i) * TH - ex - ey * bw + (em < 0 ? r2 : (em > 0 ? r4 : r3))];
+                    });
+                }
+                if constexpr (std::is_same<T, double>::value) {
+                    if (ok) collide(L{}, n, k);
+                } else {
+                    collide(L{}, n, k);
+                }
+                if constexpr (std::is_same<K, CollFxR>::value) {
+                    unsigned a = 0u;
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) {
+                        if (i < 1 + 2 * D || ((i - 1 - 2 * D) & 3) < 2)  // a diagonal pair's two values are equal
+                            a |= (unsigned)((unsigned long long)n[i] >> 32) + 0x20000000u;
+                    }
+                    if (ok) acc |= a;
+                }
+                if constexpr (s < KS) {
+                    T *const at = mine + (s - 1) * S * TH;
+                    static_for<0, Q>([&](auto I) {
+                        constexpr int i = decltype(I)::value;
+                        constexpr int em = L::E[i][A];
+                        if constexpr (!MarchL<L>::own(i))
+                            at[MarchL<L>::slot0(i) * TH + (em < 0 ? w2 : (em > 0 ? w4 : w3))] = n[i];
+                    });
+                } else if (ok) {
+                    T *dp = dst + (r0 + row) * rstride + gxs[1] + gys[1];
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) dp[(int64_t)i * g.slab] = n[i];
+                }
+            }
+            if constexpr (s > 1) {  // stage s - 1's register populations of this iteration
+                constexpr int gp = s - 2;
+                hm[gp] = nm;
+                hc[gp][1] = hc[gp][0];
+                hc[gp][0] = nc;
+                hp[gp][2] = hp[gp][1];
+                hp[gp][1] = hp[gp][0];
+                hp[gp][0] = np;
+            }
+            if constexpr (s < KS) {
+                nm = n[IM];
+                nc = n[IC];
+                np = n[IP];
+            }
+            if constexpr (s == 1) {  // the next row's loads fly while the other stages compute
+                rc = rc + 1 == NR ? 0 : rc + 1;
+                if (t + 1 < nr + 2 * (KS - 1)) load_row(f, rc);
+            }
+        });
+        __syncthreads();
+        w2 = r2;
+        w3 = r3;
+        w4 = r4;
+    }
+    if constexpr (std::is_same<K, CollFxR>::value) {
+        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && (tid & 31) == 0) atomicOr(k.range, 1);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Host side.
+// ---------------------------------------------------------------------------
+// Cut `n` into the fewest near-equal parts of at most `most`.
+static void cut(int n, int most, int &parts, int &size)
+{
+    parts = (n + most - 1) / most;
+    size = (n + parts - 1) / parts;
+    parts = (n + size - 1) / size;
+}
+
+template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March {
+    using KT = typename MarchK<T>::type;
+    static constexpr int kRing = KS - 1;
+
+    // The cheapest cut by a model of the launch: full waves of the resident
+    // blocks, each as long as its iterations (its rows, the pipeline's fill and
+    // about 4 rows of latency), an iteration taking the time of the resident
+    // blocks' work, or of 0.7 MINB blocks where fewer no longer hide latency.
+    // `worth`: enough nodes to fill the chip, and the share of a launch's
+    // thread-iterations that end in stored nodes not below least_use.
+    static void plan(const lb_ctx *c, int64_t least_nodes, double least_use, MarchPlan *out, bool *worth)
+    {
+        const Geom &g = c->geom;
+        MarchPlan p{};
+        *out = p;
+        *worth = false;
+        if (g.slab >= (1ll << 30)) return;  // offsets within a population are int
+        const int NR = L::D == 3 ? g.N2 : g.N1;
+        p.steps = KS;
+        p.threads = TH;
+        cut(g.N0, (L::D == 3 ? kMarchW : TH) - 2 * kRing, p.nx, p.bx);
+        p.ny = p.by = 1;
+        if (L::D == 3) cut(g.N1, TH / kMarchW - 2 * kRing, p.ny, p.by);
+        const int64_t win = (int64_t)p.nx * p.ny, slots = (int64_t)c->sms * MINB;
+        double least = 1e300;
+        for (int nc = 1; nc <= NR; ++nc) {
+            const int chunk = (NR + nc - 1) / nc;
+            if (nc > 1 && chunk < 4 * kRing) break;
+            const int64_t blocks = win * ((NR + chunk - 1) / chunk);
+            const int64_t waves = (blocks + slots - 1) / slots;
+            if (blocks > 0x7fffffff || (p.chunk && waves > 64)) break;
+            const double resident = (double)((blocks + waves * c->sms - 1) / (waves * c->sms));
+            const double t = (double)waves * (chunk + 3 * kRing + 4) * std::max(resident, 0.7 * MINB);
+            if (t < least) {
+                least = t;
+                p.chunk = chunk;
+                p.nc = (NR + chunk - 1) / chunk;
+            }
+        }
+        if (p.chunk == 0) return;  // more windows than a launch has blocks
+        const double use = (double)c->nodes / ((double)win * p.nc * TH * (p.chunk + 3 * kRing));
+        *out = p;
+        *worth = c->nodes >= least_nodes && use >= least_use;
+    }
+    static const void *kernel() { return (const void *)march_kernel<L, T, KT, KS, TH, MINB, SKIP>; }
+    static cudaError_t setup(lb_ctx *c, int64_t least_nodes, double least_use, MarchPlan *out, bool *worth)
+    {
+        plan(c, least_nodes, least_use, out, worth);
+        return cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)march_smem<L, KS, TH>(sizeof(T)));
+    }
+    static cudaError_t launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s)
+    {
+        const MarchPlan &p = c->march;
+        march_kernel<L, T, KT, KS, TH, MINB, SKIP>
+            <<<(unsigned)((int64_t)p.nx * p.ny * p.nc), TH, march_smem<L, KS, TH>(sizeof(T)), s>>>(
+                (const T *)src, (T *)dst, c->geom, MarchK<T>::make(c), p);
+        return cudaGetLastError();
+    }
+};
+
+// Steps per launch, threads and blocks per SM, as measured at 4096^2 and 256^3
+// (GLUPS).  More steps than these need rings that leave too little L1 for the
+// rows in flight, or registers that leave too few warps.
+//   2D fixed point: 3 steps, 64 threads x 10: 108.5 (2 steps: 88; 4: 96; 256 x 2: 104)
+//   2D FP32:        5 steps, 128 x 5: 315 (4 steps: 276; 6: 297; 128 x 7 at 4 steps: 227)
+//   2D FP64:        2 steps, 128 x 6: 52 (3 steps: 50.6; 256 x 3: 47)
+//   3D fixed point: 2 steps, 416 x 1: 35.5 (512: 32; 384: 33.5)
+//   3D FP32:        3 steps, 512 x 1: 78 (2 steps: 62; 448: 71)
+// 3D FP64 (19 integer-form collisions' worth of registers) was slower than one
+// sweep per launch, and 4D has no room for a window.
+using March2Fx = March<D2Q9, long long, 3, 64, 10, true>;
+using March2F = March<D2Q9, float, 5, 128, 5, true>;
+using March2D = March<D2Q9, double, 2, 128, 6, true>;
+using March3Fx = March<D3Q19, long long, 2, 416, 1, true>;
+using March3F = March<D3Q19, float, 3, 512, 1, false>;
+
+// Where marching beats one sweep per launch (GLUPS, march / sweep):
+//   2D fixed point 256^2 16 / 20, 384^2 29 / 31, 512^2 52 / 41, 1024^2 76 / 43, 1999x1501 94 / 44, 4096^2 108 / 47
+//   2D FP32        256^2 22 / 23, 384^2 50 / 46, 512^2 77 / 60, 1024^2 194 / 124, 1999x1501 258 / 85, 4096^2 315 / 97
+//   2D FP64        768^2 34 / 40, 1024^2 37 / 39, 1999x1501 48 / 42, 4096^2 52 / 47
+//   3D fixed point 48^3 15 / 13, 64^3 21 / 21, 101x90x77 25 / 19, 128^3 32 / 22, 256^3 36 / 23
+//   3D FP32        48^3 14 / 17, 64^3 32 / 31, 101x90x77 42 / 46, 128^3 61 / 42, 256^3 78 / 46
+cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth)
+{
+    *plan = MarchPlan{};
+    *worth = false;
+    if (c->geom.mirror) return cudaSuccess;
+    if (c->d == 2) {
+        if (c->precision == LB_FX64) return March2Fx::setup(c, 200000, 0.45, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March2F::setup(c, 180000, 0.45, plan, worth);
+        return March2D::setup(c, 1800000, 0.8, plan, worth);
+    }
+    if (c->d == 3) {
+        if (c->precision == LB_FX64) return March3Fx::setup(c, 300000, 0.4, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, 1200000, 0.4, plan, worth);
+    }
+    return cudaSuccess;
+}
+
+cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s)
+{
+    if (c->d == 2) {
+        if (c->precision == LB_FX64) return March2Fx::launch(c, src, dst, s);
+        if (c->precision == LB_FP32_SHIFTED) return March2F::launch(c, src, dst, s);
+        return March2D::launch(c, src, dst, s);
+    }
+    if (c->precision == LB_FX64) return March3Fx::launch(c, src, dst, s);
+    return March3F::launch(c, src, dst, s);
+}
+
+}  // namespace lbk

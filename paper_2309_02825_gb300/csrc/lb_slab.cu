@@ -79,6 +79,7 @@ lb_status lb_slab_create(int d, const int64_t *N, int part, int nparts, double n
         delete s;
         return st;
     }
+    s->ctx->sched = s->ctx->run = lbk::kSchedSweeps;  // the ghost layers serve one sweep
     const lbk::Geom &g = s->ctx->geom;
     s->layer_rows = g.rows / (s->nz + 2);
     s->layer_elems = s->layer_rows * g.pitch;
