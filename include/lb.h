@@ -200,7 +200,9 @@ lb_status lb_step(lb_ctx *ctx, int64_t nsteps);
  * whole state every step, so it is bound by HBM bandwidth.  A new context runs
  * the library's own choice: on periodic 2D and 3D grids large enough to fill
  * the device, launches of two to five steps that march windows of the grid
- * along its slowest axis; one sweep per launch elsewhere.  This call selects
+ * along its slowest axis; on small periodic 2D grids, launches of eight steps on
+ * square tiles; on 1D grids of up to 4096 nodes (2048 for LB_FP64), all the
+ * steps of a call in one launch; one sweep per launch elsewhere.  This call selects
  * one sweep per launch or, on periodic 2D grids, launches of K steps on square
  * tiles: a block loads one tile of
  * the grid with a K-node periodic halo into shared memory, runs the same

@@ -144,14 +144,19 @@ cudaError_t record_blocked(lb_ctx *c, int from)
 // The schedule lb_step runs when the caller has set none (kSchedAuto).  On
 // periodic 2D and 3D grids large enough to fill the chip, marching sweeps
 // (lb_march.cu); on small 2D grids, whose single sweeps last about as long as
-// their launch, several steps per launch on square tiles; else one sweep per
-// launch.  Every choice gives the same bits.
+// their launch, several steps per launch on square tiles; on short 1D grids
+// all steps in one launch; else one sweep per launch.  Every choice gives the
+// same bits.
 cudaError_t choose_schedule(lb_ctx *c)
 {
     if (c->sched != lbk::kSchedAuto) return cudaSuccess;
     c->run = lbk::kSchedSweeps;
     lbk::blocked_release(c);
     c->march = lbk::MarchPlan{};
+    if (lbk::line_fits(c)) {
+        c->run = lbk::kSchedLine;
+        return cudaSuccess;
+    }
     if (c->geom.mirror) return cudaSuccess;
     bool worth = false;
     cudaError_t e = lbk::march_setup(c, &c->march, &worth);
@@ -159,6 +164,23 @@ cudaError_t choose_schedule(lb_ctx *c)
     if (worth) {
         c->run = lbk::kSchedMarch;
         return cudaSuccess;
+    }
+    if (c->d == 2) {
+        // The smallest square tile, from 8 nodes in steps of 4, that leaves at
+        // most one tile per SM; 8 steps per launch.  us per step (fixed point,
+        // FP32, FP64) against one sweep per launch replayed from a graph:
+        // 64^2 1.35, 1.08, 1.9 / 2.9, 2.7, 3.9; 128^2 1.6, 1.1, 2.4 / 2.9, 2.8,
+        // 4.0; 192^2 1.6, 1.3, 2.9 / 3.0, 2.7, 4.2; 256^2 2.4, 1.6, 4.4 / 3.4,
+        // 2.8, 4.6; 384^2 3.2, 1.9 / 4.7, 3.1.  FP64 tiles above 24 nodes (SMs
+        // busy with the recomputed halo) lose: 320^2 5.7 / 5.1.
+        const int most = c->precision == LB_FP64 ? 24 : (c->precision == LB_FX64 ? 40 : 48);
+        for (int tile = 8; tile <= most; tile += 4) {
+            if (((c->N[0] + tile - 1) / tile) * ((c->N[1] + tile - 1) / tile) > c->sms) continue;
+            bool fits = true;
+            if ((e = lbk::blocked_setup(c, 8, tile, tile <= 32 ? 512 : 1024, &fits)) != cudaSuccess) return e;
+            if (fits) c->run = lbk::kSchedTiles;
+            break;
+        }
     }
     return cudaSuccess;
 }
@@ -600,6 +622,18 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     // directly so that they land in the caller's graph.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+    if (c->run == lbk::kSchedLine && nsteps > 0) {
+        constexpr int64_t kMost = 1 << 20;  // steps per launch
+        while (nsteps > 0) {
+            const int64_t n = nsteps < kMost ? nsteps : kMost;
+            cudaError_t e = lbk::line_launch(c, c->f[c->cur], c->f[c->cur ^ 1], n);
+            if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: resident launch");
+            c->cur ^= 1;
+            c->step += n;
+            nsteps -= n;
+        }
+        return LB_OK;
+    }
     if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps) {
         // marching launches; the remainder below, one sweep per launch
         while (nsteps >= c->march.steps) {

@@ -860,9 +860,6 @@ template <class L> __device__ __forceinline__ void collide(L, double *f, const C
     }
     collide(L{}, f, k.k);
 }
-// One axis: three populations, nine FP64 operations; the direct form.
-__device__ __forceinline__ void collide(D1Q3, double *f, const CollF64 &k) { collide(D1Q3{}, f, k.k); }
-
 // Threads per block of the sweep: more, smaller blocks balance the SMs better.
 template <typename T> __host__ __device__ constexpr int sweep_threads() { return 128; }
 

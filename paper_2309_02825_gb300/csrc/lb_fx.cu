@@ -48,7 +48,8 @@ CollF64 make_coll_f64(const lb_ctx &c)
 {
     CollF64 r;
     r.k = make_coll<double>(c);
-    r.ints = fx_constants_ok(c) && fabs(r.k.c0) + 4.0 * fabs(r.k.k2) < 1.9;
+    r.ints = fx_constants_ok(c) && fabs(r.k.c0) + (c.d == 1 ? 2.0 : 4.0) * fabs(r.k.k2) < 1.9 &&
+             !(c.d == 1 && c.N[0] <= 160);
     r.x = r.ints ? make_coll_fx(&c) : CollFx{};
     return r;
 }

@@ -217,6 +217,7 @@ enum Sched {
     kSchedAuto = 0,    // the library's own rule (choose_schedule)
     kSchedSweeps = 1,  // one sweep per launch
     kSchedTiles = 2,   // tb_k steps per launch on square tiles (lb_batch.cu)
+    kSchedLine = 4,    // any number of steps, a short 1D grid resident in one block (lb_line.cu)
     kSchedMarch = 3    // march.steps steps per launch along the slowest axis (lb_march.cu)
 };
 
@@ -287,7 +288,11 @@ bool fx_constants_ok(const lb_ctx &c);
 // The FP64 collision's constants.  Its integer form is taken (ints = 1) for
 // constants that fx_constants_ok admits and whose rest population
 // c0 theta - 2 k2 sum P_aa stays below 2^63 for magnitudes that sum below 2^62
-// (|c0| + 4 |k2| < 1.9: the paper's set at every eps of its examples).
+// (|c0| + 4 |k2| < 1.9, or |c0| + 2 |k2| on one axis: the paper's set at every
+// eps of its examples).  Short 1D grids keep the direct form: their few warps
+// wait on latency, and three populations make a shorter chain there (us per
+// step resident in one block: 81 nodes 0.34 against 0.54, 129 nodes 0.49 / 0.60,
+// 256 nodes 0.72 / 0.44, 1024 nodes 2.7 / 1.4).
 CollF64 make_coll_f64(const lb_ctx &c);
 // Device flags of a context (ctx->dflag): 0 initialisation, 1 recovery
 // (bit 0: theta <= 0 or non-finite, bit 2: a staging wait timed out),
@@ -328,5 +333,9 @@ void blocked_release(lb_ctx *c);
 // one sweep per launch, and one launch of plan.steps steps.
 cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth);
 cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s);
+// Resident sweeps of a short 1D grid (lb_line.cu): whether it is one, and one
+// launch of any number of steps.
+bool line_fits(const lb_ctx *c);
+cudaError_t line_launch(lb_ctx *c, const void *src, void *dst, int64_t steps);
 
 }  // namespace lbk
