@@ -819,47 +819,72 @@ template <int PB> __device__ __forceinline__ double f64_from_aligned(long long s
     return s == 0 ? 0.0 : __hiloint2double(__double2hiint(r) + (int)((emax - 1075u - (unsigned)PB) << 20), __double2loint(r));
 }
 
+// The doubles f aligned to their largest exponent (emax) as int64, every bit
+// kept; false where they are not alignable or their magnitudes sum to 2^62.
+template <int Q, int PB>
+__device__ __forceinline__ bool f64_align(const double (&f)[Q], long long (&v)[Q], unsigned &emax)
+{
+    unsigned e[Q], mx = 0u, mn = 0x7ff00000u;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        e[i] = (unsigned)__double2hiint(f[i]) & 0x7ff00000u;
+        mx = max(mx, e[i]);
+        mn = min(mn, e[i]);
+    }
+    emax = mx >> 20;
+    if (!(mx - mn <= ((unsigned)PB << 20) && mx - (100u << 20) <= (1900u << 20))) return false;
+    unsigned sum = 0u;  // of the magnitudes' high words (each below 2^(21 + PB))
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
+        const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+        const unsigned sh = (unsigned)PB - ((mx - e[i]) >> 20);  // 0 .. PB
+        const unsigned vh = __funnelshift_l(lo, mh, sh), vl = lo << sh;
+        sum += vh;
+        const unsigned s = (unsigned)((int)hi >> 31);
+        v[i] = (long long)((((unsigned long long)(vh ^ s) << 32) | (vl ^ s)) - (((unsigned long long)s << 32) | s));
+    }
+    return sum < 0x3fffffc0u;
+}
+
 template <class L> __device__ __forceinline__ void collide(L, double *f, const CollF64 &k)
 {
     constexpr int Q = L::Q, PB = f64_align_bit<L>(), B0 = 1 + 2 * L::D;
     if (k.ints) {
-        unsigned e[Q], mx = 0u, mn = 0x7ff00000u;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            e[i] = (unsigned)__double2hiint(f[i]) & 0x7ff00000u;
-            mx = max(mx, e[i]);
-            mn = min(mn, e[i]);
-        }
-        if (mx - mn <= ((unsigned)PB << 20) && mx - (100u << 20) <= (1900u << 20)) {
-            long long v[Q];
-            unsigned sum = 0u;  // of the magnitudes' high words (each below 2^(21 + PB))
+        long long v[Q];
+        unsigned emax;
+        if (f64_align<Q, PB>(*reinterpret_cast<const double(*)[Q]>(f), v, emax)) {
+            collide(L{}, v, k.x);
+            // the two velocities of a diagonal pair hold equal values
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
-                const unsigned mh = (hi & 0xfffffu) | 0x100000u;
-                const unsigned sh = (unsigned)PB - ((mx - e[i]) >> 20);  // 0 .. PB
-                const unsigned vh = __funnelshift_l(lo, mh, sh), vl = lo << sh;
-                sum += vh;
-                const unsigned s = (unsigned)((int)hi >> 31);
-                v[i] = (long long)((((unsigned long long)(vh ^ s) << 32) | (vl ^ s)) - (((unsigned long long)s << 32) | s));
+                if (i >= B0 && ((i - B0) & 3) >= 2)
+                    f[i] = f[i - 2];
+                else
+                    f[i] = f64_from_aligned<PB>(v[i], emax);
             }
-            if (sum < 0x3fffffc0u) {  // magnitudes sum below 2^62
-                const unsigned emax = mx >> 20;
-                collide(L{}, v, k.x);
-                // the two velocities of a diagonal pair hold equal values
-#pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    if (i >= B0 && ((i - B0) & 3) >= 2)
-                        f[i] = f[i - 2];
-                    else
-                        f[i] = f64_from_aligned<PB>(v[i], emax);
-                }
-                return;
-            }
+            return;
         }
     }
     collide(L{}, f, k.k);
 }
+
+// A double rounded to float (to nearest, ties to even) on the integer pipes;
+// results outside the normal floats by the hardware conversion.
+__device__ __forceinline__ float f64_to_f32_rn(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u > 253u) {  // below 2^-126, or 2^127 and more (volatile: not computed beside the usual path)
+        float r;
+        asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(v));
+        return r;
+    }
+    const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29), rem = lo << 3;
+    const unsigned up = (rem > 0x80000000u || (rem == 0x80000000u && (m & 1u))) ? 1u : 0u;
+    return __uint_as_float(((hi & 0x80000000u) | m) + up);
+}
+
 // Threads per block of the sweep: more, smaller blocks balance the SMs better.
 template <typename T> __host__ __device__ constexpr int sweep_threads() { return 128; }
 
