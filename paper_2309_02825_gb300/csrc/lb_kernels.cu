@@ -33,8 +33,20 @@ namespace lbk {
 //
 // FXI (64-bit fixed point formed in integers): theta and dx * grad theta are
 // converted to fixed point once per node, every product with a constant is
-// a rounded 64x62-bit product, and the rest population is theta minus the
-// others, so sum_i f_i(x) = round(theta0(x) 2^F) exactly.
+// rounded once, and the rest population is theta minus the others, so
+// sum_i f_i(x) = round(theta0(x) 2^F) exactly.  FXI = 2 takes the collision's
+// split product (mulfx_c, constants of 64 fraction bits), for constants in
+// (-1/2, 1/2); FXI = 1 the 128-bit product with 62 fraction bits, about three
+// times the instructions, for the rest (1D eps above 0.83).
+//
+// Otherwise the values are formed in FP64, which issues at 1/64 of the FP32 and
+// integer rates and binds the kernel there: each shared term is formed once (a
+// plane's four velocities have e . grad = +-(g_a + g_b), +-(g_a - g_b)) and FP32
+// values are rounded to float on the integer pipes: 13 (FP64) and 16 (FP32)
+// FP64 operations per D2Q9 node instead of 35 and 31.
+//
+// Each value is stored as soon as it is formed, so that few registers hold a
+// node and enough warps are resident to keep the scattered stores in flight.
 // ---------------------------------------------------------------------------
 // round(v 2^F) to nearest, ties to even, from the fields of the IEEE double
 // v in integer arithmetic (v 2^F is exact; only its rounding to an integer is
@@ -62,13 +74,16 @@ __device__ __forceinline__ long long fx_round(double v, int F, bool &range)
     return bits < 0 ? -r : r;
 }
 
-template <class L, typename T, bool FXI>
-__global__ void init_kernel(T *__restrict__ dst, Geom g, InitK K, const double *__restrict__ theta0,
-                            const double *__restrict__ grad, int *__restrict__ flag)
+constexpr int kInitThreads = 128;
+
+template <class L, typename T, int FXI, bool MIR>
+__global__ void __launch_bounds__(kInitThreads) init_kernel(T *__restrict__ dst, Geom g, InitK K,
+                                                            const double *__restrict__ theta0,
+                                                            const double *__restrict__ grad, int *__restrict__ flag)
 {
-    constexpr int D = L::D, Q = L::Q;
+    constexpr int D = L::D, Q = L::Q, B0 = 1 + 2 * D;
     const int64_t nodes = (int64_t)g.N0 * g.rows;
-    const int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t node = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
     if (node >= nodes) return;
     // coordinates in 32-bit arithmetic (nodes <= 2^31)
     const unsigned nd = (unsigned)node;
@@ -92,189 +107,166 @@ __global__ void init_kernel(T *__restrict__ dst, Geom g, InitK K, const double *
     for (int a = 0; a < D; ++a) {
         gr[a] = grad[a * nodes + node];
         bad |= ((__double_as_longlong(gr[a]) >> 52) & 0x7ff) == 0x7ff;
-        if (((g.mirror >> a) & 1u) && (c[a] == 0 || c[a] == n[a] - 1)) gr[a] = 0.0;
+        if (MIR && ((g.mirror >> a) & 1u) && (c[a] == 0 || c[a] == n[a] - 1)) gr[a] = 0.0;
     }
     if (bad) atomicOr(flag, 1);
 
-    T val[Q];
-    bool range = false;
-    if constexpr (FXI) {
-        const long long t = fx_round(th, K.fx_bits, range);
-        long long G[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) G[a] = fx_round(gr[a] * K.gscale, 0, range);
-        const long long W1 = mulfx(t, K.w1k), WD = mulfx(t, K.wdk);
-        long long rest = 0;
-        static_for<1, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int nz = (L::E[i][0] != 0) + (L::E[i][1] != 0) + (L::E[i][2] != 0) + (L::E[i][3] != 0);
-            long long v;
-            if constexpr (nz == 1) {
-                constexpr int a = (L::E[i][0] != 0) ? 0 : ((L::E[i][1] != 0) ? 1 : ((L::E[i][2] != 0) ? 2 : 3));
-                constexpr int ea = L::E[i][a];
-                const long long A = mulfx(G[a], K.iak);
-                v = (ea > 0) ? W1 - A : W1 + A;
-            } else {
-                constexpr int a = (L::E[i][0] != 0) ? 0 : ((L::E[i][1] != 0) ? 1 : 2);
-                constexpr int b = (L::E[i][3] != 0) ? 3 : ((L::E[i][2] != 0 && a < 2) ? 2 : 1);
-                constexpr int ea = L::E[i][a], eb = L::E[i][b];
-                // e . (dx grad) = +-(G_a + G_b) or +-(G_a - G_b); one rounded product per pair and sign
-                const long long P = mulfx(ea == eb ? G[a] + G[b] : G[a] - G[b], K.wdk);
-                v = (ea > 0) ? WD - P : WD + P;
-            }
-            if (!(v < (1ll << 61) && v > -(1ll << 61))) range = true;
-            val[i] = v;
-            rest += v;
-        });
-        val[0] = t - rest;
-    } else if constexpr (std::is_same<T, float>::value) {
-        // FP32 shifted storage: f_i - w_i theta_ref formed from theta0 - theta_ref
-        // and the gradient terms, each shared term computed once (the float
-        // rounding of the stored value dominates; FP64 issues at 1/64 of the
-        // FP32 rate on this part, so the FP64 operations per node are kept few)
-        const double dth = th - K.theta_ref;
-        const double b0 = K.w0 * dth, b1 = K.w1 * dth, bd = K.wd * dth;
-        double ga[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) ga[a] = K.iax * gr[a];
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int ex = L::E[i][0], ey = L::E[i][1], ez = L::E[i][2], ew = L::E[i][3];
-            constexpr int nz = (ex != 0) + (ey != 0) + (ez != 0) + (ew != 0);
-            double v;
-            if constexpr (nz == 0) {
-                v = b0;
-            } else if constexpr (nz == 1) {
-                constexpr int a = (ex != 0) ? 0 : ((ey != 0) ? 1 : ((ez != 0) ? 2 : 3));
-                constexpr int sgn = (ex != 0) ? ex : ((ey != 0) ? ey : ((ez != 0) ? ez : ew));
-                v = sgn > 0 ? b1 - ga[a] : b1 + ga[a];
-            } else {
-                double edg = 0.0;
-                if constexpr (ex != 0) edg += (double)ex * gr[0];
-                if constexpr (ey != 0) edg += (double)ey * gr[1];
-                if constexpr (ez != 0) edg += (double)ez * gr[2];
-                if constexpr (ew != 0) edg += (double)ew * gr[3];
-                v = fma(-K.idg, edg, bd);
-            }
-            val[i] = (T)v;
-        });
-    } else {
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int ex = L::E[i][0], ey = L::E[i][1], ez = L::E[i][2], ew = L::E[i][3];
-            constexpr int nz = (ex != 0) + (ey != 0) + (ez != 0) + (ew != 0);
-            double v;
-            if constexpr (nz == 0) {
-                v = K.w0 * th;
-                v -= K.w0 * K.theta_ref;
-            } else if constexpr (nz == 1) {
-                constexpr int a = (ex != 0) ? 0 : ((ey != 0) ? 1 : ((ez != 0) ? 2 : 3));
-                constexpr int sgn = (ex != 0) ? ex : ((ey != 0) ? ey : ((ez != 0) ? ez : ew));
-                v = K.w1 * th - (double)sgn * K.iax * gr[a];
-                v -= K.w1 * K.theta_ref;
-            } else {
-                double edg = 0.0;
-                if constexpr (ex != 0) edg += (double)ex * gr[0];
-                if constexpr (ey != 0) edg += (double)ey * gr[1];
-                if constexpr (ez != 0) edg += (double)ez * gr[2];
-                if constexpr (ew != 0) edg += (double)ew * gr[3];
-                v = K.wd * th - K.idg * edg;
-                v -= K.wd * K.theta_ref;
-            }
-            val[i] = to_store<T>(v, K.fxscale, range);
-        });
-    }
-    if (range) atomicOr(flag, 2);
-
-    if (!g.mirror) {
-        // periodic: destination offset = sum over axes of one of three wrapped
-        // offsets (shift -1, 0, +1), formed once per node
-        int64_t off[4][3];
-        int64_t stride = 1;
+    // periodic: destination offset = sum over axes of one of three wrapped
+    // offsets (shift -1, 0, +1), formed once per node (a population has at most
+    // 2^31 nodes and a row's padding each: below 2^32)
+    unsigned off[4][3];
+    {
+        unsigned stride = 1;
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int dn = c[a] == 0 ? n[a] - 1 : c[a] - 1;  // x_a - 1
             const int up = c[a] == n[a] - 1 ? 0 : c[a] + 1;  // x_a + 1
-            off[a][0] = (int64_t)up * stride;                // e = -1 stores at x_a + 1
-            off[a][1] = (int64_t)c[a] * stride;
-            off[a][2] = (int64_t)dn * stride;                // e = +1 stores at x_a - 1
-            stride *= (a == 0) ? (int64_t)g.pitch : (int64_t)n[a];
+            off[a][0] = (unsigned)up * stride;               // e = -1 stores at x_a + 1
+            off[a][1] = (unsigned)c[a] * stride;
+            off[a][2] = (unsigned)dn * stride;               // e = +1 stores at x_a - 1
+            stride *= (a == 0) ? (unsigned)g.pitch : (unsigned)n[a];
         }
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            const int64_t at = off[0][L::E[i][0] + 1] + off[1][L::E[i][1] + 1] + off[2][L::E[i][2] + 1] +
-                               off[3][L::E[i][3] + 1];
-            dst[(int64_t)i * g.slab + at] = val[i];
-        });
-        return;
     }
-    static_for<0, Q>([&](auto I) {
+    const auto put = [&](auto I, T v) {
         constexpr int i = decltype(I)::value;
         constexpr int E0 = L::E[i][0], E1 = L::E[i][1], E2 = L::E[i][2], E3 = L::E[i][3];
-        const int ev[4] = {E0, E1, E2, E3};
-        int y[4];
-        bool ghost = false;
-        unsigned near = 0;  // axes where x is next to a wall it streams onto
+        if constexpr (!MIR) {
+            const unsigned at = off[0][E0 + 1] + off[1][E1 + 1] + off[2][E2 + 1] + off[3][E3 + 1];
+            dst[(int64_t)i * g.slab + at] = v;
+        } else {
+            const int ev[4] = {E0, E1, E2, E3};
+            int y[4];
+            bool ghost = false;
+            unsigned near = 0;  // axes where x is next to a wall it streams onto
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int e = ev[a];
-            int v = c[a] - e;
-            if (e != 0 && ((g.mirror >> a) & 1u)) {
-                if (v < 0 || v >= n[a]) ghost = true;
-                if ((e > 0 && c[a] == 1) || (e < 0 && c[a] == n[a] - 2)) near |= 1u << a;
-            } else if (v < 0) {
-                v += n[a];
-            } else if (v >= n[a]) {
-                v -= n[a];
-            }
-            y[a] = v;
-        }
-        if (ghost) return;
-        const int64_t at = (((int64_t)y[3] * g.N2 + y[2]) * g.N1 + y[1]) * g.pitch + y[0];
-        dst[(int64_t)i * g.slab + at] = val[i];
-        if (near) {
-            constexpr int nzm = (E0 != 0 ? 1 : 0) | (E1 != 0 ? 2 : 0) | (E2 != 0 ? 4 : 0) | (E3 != 0 ? 8 : 0);
-            static_for<1, 16>([&](auto Mi) {
-                constexpr int M = decltype(Mi)::value;
-                if constexpr ((M & ~nzm) == 0) {
-                    if ((M & ~near) == 0) dst[(int64_t)reflect_pop<L>(i, M) * g.slab + at] = val[i];
+            for (int a = 0; a < 4; ++a) {
+                const int e = ev[a];
+                int w = c[a] - e;
+                if (e != 0 && ((g.mirror >> a) & 1u)) {
+                    if (w < 0 || w >= n[a]) ghost = true;
+                    if ((e > 0 && c[a] == 1) || (e < 0 && c[a] == n[a] - 2)) near |= 1u << a;
+                } else if (w < 0) {
+                    w += n[a];
+                } else if (w >= n[a]) {
+                    w -= n[a];
                 }
-            });
+                y[a] = w;
+            }
+            if (ghost) return;
+            const int64_t at = (((int64_t)y[3] * g.N2 + y[2]) * g.N1 + y[1]) * g.pitch + y[0];
+            dst[(int64_t)i * g.slab + at] = v;
+            if (near) {
+                constexpr int nzm = (E0 != 0 ? 1 : 0) | (E1 != 0 ? 2 : 0) | (E2 != 0 ? 4 : 0) | (E3 != 0 ? 8 : 0);
+                static_for<1, 16>([&](auto Mi) {
+                    constexpr int M = decltype(Mi)::value;
+                    if constexpr ((M & ~nzm) == 0) {
+                        if ((M & ~near) == 0) dst[(int64_t)reflect_pop<L>(i, M) * g.slab + at] = v;
+                    }
+                });
+            }
         }
-    });
+    };
+
+    bool range = false;
+    if constexpr (FXI != 0) {
+        const auto mul = [](long long a, long long k) { return FXI == 2 ? mulfx_c(a, k) : mulfx(a, k); };
+        unsigned acc = 0u;  // OR of the values' high words + 2^29: |v| < 2^61 exactly when it stays below 2^30
+        const auto put_fx = [&](auto I, long long v) {
+            acc |= (unsigned)((unsigned long long)v >> 32) + 0x20000000u;
+            put(I, v);
+        };
+        const long long t = fx_round(th, K.fx_bits, range);
+        long long G[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) G[a] = fx_round(gr[a] * K.gscale, 0, range);
+        // the velocities of an axis sum to 2 W1, those of a plane to 4 WD
+        const long long W1 = mul(t, K.w1k), WD = D > 1 ? mul(t, K.wdk) : 0;
+        put(std::integral_constant<int, 0>{}, t - (2 * D * W1 + 2 * D * (D - 1) * WD));
+        static_for<0, D>([&](auto Ai) {
+            constexpr int a = decltype(Ai)::value;
+            const long long A = mul(G[a], K.iak);
+            put_fx(std::integral_constant<int, 1 + a>{}, W1 - A);
+            put_fx(std::integral_constant<int, 1 + D + a>{}, W1 + A);
+        });
+        static_for<0, D *(D - 1) / 2>([&](auto Pi) {
+            constexpr int p = decltype(Pi)::value;
+            constexpr int a = pair_a<D>(p), b = pair_b<D>(p);
+            // e . (dx grad) = +-(G_a + G_b) or +-(G_a - G_b); one rounded product per pair and sign
+            const long long P = mul(G[a] + G[b], K.wdk), M = mul(G[a] - G[b], K.wdk);
+            put_fx(std::integral_constant<int, B0 + 4 * p>{}, WD - P);      // (+1, +1)
+            put_fx(std::integral_constant<int, B0 + 4 * p + 1>{}, WD + M);  // (-1, +1)
+            put_fx(std::integral_constant<int, B0 + 4 * p + 2>{}, WD + P);  // (-1, -1)
+            put_fx(std::integral_constant<int, B0 + 4 * p + 3>{}, WD - M);  // (+1, -1)
+        });
+        if (acc >= 0x40000000u) range = true;
+    } else {
+        constexpr bool kF32 = std::is_same<T, float>::value;
+        const auto put_d = [&](auto I, double v) {
+            if constexpr (kF32)
+                put(I, f64_to_f32_rn(v));
+            else
+                put(I, to_store<T>(v, K.fxscale, range));
+        };
+        const double dth = kF32 ? th - K.theta_ref : th;  // FP32 stores f_i - w_i theta_ref
+        const double b1 = K.w1 * dth, bd = K.wd * dth;
+        put_d(std::integral_constant<int, 0>{}, K.w0 * dth);
+        static_for<0, D>([&](auto Ai) {
+            constexpr int a = decltype(Ai)::value;
+            const double ga = K.iax * gr[a];
+            put_d(std::integral_constant<int, 1 + a>{}, kF32 ? b1 - ga : fma(-K.iax, gr[a], b1));
+            put_d(std::integral_constant<int, 1 + D + a>{}, kF32 ? b1 + ga : fma(K.iax, gr[a], b1));
+        });
+        static_for<0, D *(D - 1) / 2>([&](auto Pi) {
+            constexpr int p = decltype(Pi)::value;
+            constexpr int a = pair_a<D>(p), b = pair_b<D>(p);
+            const double sp = gr[a] + gr[b], sm = gr[a] - gr[b];
+            put_d(std::integral_constant<int, B0 + 4 * p>{}, fma(-K.idg, sp, bd));
+            put_d(std::integral_constant<int, B0 + 4 * p + 1>{}, fma(K.idg, sm, bd));
+            put_d(std::integral_constant<int, B0 + 4 * p + 2>{}, fma(K.idg, sp, bd));
+            put_d(std::integral_constant<int, B0 + 4 * p + 3>{}, fma(-K.idg, sm, bd));
+        });
+    }
+    if (range) atomicOr(flag, 2);
 }
 
 // Fourth-order central difference of theta along each axis: periodic, or,
 // on an axis with mirror walls (bit a of mirror), the even reflection of
-// theta across the wall nodes (theta(-k) = theta(k)).
-__global__ void fd4_kernel(const double *__restrict__ th, double *__restrict__ grad, int d, int N0, int N1,
-                           int N2, int N3, unsigned mirror, double inv12dx)
+// theta across the wall nodes (theta(-k) = theta(k)).  An axis of fewer than
+// four nodes wraps more than once.
+__device__ __forceinline__ int fd4_at(int t, int n, bool mir)
 {
-    const int64_t nodes = (int64_t)N0 * N1 * N2 * N3;
+    if (mir) return t < 0 ? -t : (t >= n ? 2 * (n - 1) - t : t);
+    while (t < 0) t += n;
+    while (t >= n) t -= n;
+    return t;
+}
+__global__ void __launch_bounds__(256) fd4_kernel(const double *__restrict__ th, double *__restrict__ grad, int d,
+                                                  int N0, int N1, int N2, int N3, unsigned mirror, double inv12dx)
+{
+    const int64_t nodes = (int64_t)N0 * N1 * N2 * N3;  // <= 2^31
     const int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (node >= nodes) return;
-    int64_t rest = node;
-    const int x = (int)(rest % N0);
-    rest /= N0;
-    const int y = (int)(rest % N1);
-    rest /= N1;
-    const int z = (int)(rest % N2);
-    const int w = (int)(rest / N2);
+    const unsigned nd = (unsigned)node;
+    const unsigned r1 = nd / (unsigned)N0, r2 = r1 / (unsigned)N1, r3 = r2 / (unsigned)N2;
+    const int c[4] = {(int)(nd - r1 * (unsigned)N0), (int)(r1 - r2 * (unsigned)N1), (int)(r2 - r3 * (unsigned)N2),
+                      (int)r3};
     const int n[4] = {N0, N1, N2, N3};
-    for (int a = 0; a < d; ++a) {
-        double acc = 0.0;
-        const int off[4] = {2, 1, -1, -2};
-        const double cof[4] = {-1.0, 8.0, -8.0, 1.0};
-        for (int k = 0; k < 4; ++k) {
-            int c[4] = {x, y, z, w};
-            const int t = c[a] + off[k];
-            if ((mirror >> a) & 1u)
-                c[a] = t < 0 ? -t : (t >= n[a] ? 2 * (n[a] - 1) - t : t);
-            else
-                c[a] = (t % n[a] + n[a]) % n[a];
-            acc += cof[k] * th[(((int64_t)c[3] * N2 + c[2]) * N1 + c[1]) * N0 + c[0]];
+    unsigned stride = 1;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        if (a < d) {
+            const unsigned base = nd - (unsigned)c[a] * stride;
+            const bool mir = (mirror >> a) & 1u;
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = th[base + (unsigned)fd4_at(c[a] + (k < 2 ? 2 - k : 1 - k), n[a], mir) * stride];
+            double acc = -v[0];
+            acc += 8.0 * v[1];
+            acc += -8.0 * v[2];
+            acc += v[3];
+            grad[a * nodes + node] = acc * inv12dx;
         }
-        grad[a * nodes + node] = acc * inv12dx;
+        stride *= (unsigned)n[a];
     }
 }
 
@@ -286,29 +278,36 @@ template <int NS> struct Acc {
     double v[NS];
 };
 
-// op[k]: 0 = sum, 1 = max
+// op[k]: 0 = sum, 1 = max.  The block's values go through shared memory, 16
+// threads to a slot: the FP64 pipe takes a whole warp instruction's time for
+// every step of a shuffle tree (5 per slot and warp: 16 of the 47 us of a 3D
+// norms pass at 7e5 nodes), while each of these adds serves 32 lanes.
 template <int NS>
 __device__ __forceinline__ void block_reduce_store(Acc<NS> &a, const int (&op)[NS], double *dst)
 {
-    __shared__ double sh[kRedThreads / 32][NS];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int P = 16;  // partial sums per slot
+    __shared__ double sh[NS][kRedThreads + 1];
+    __shared__ double part[NS][P];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
+    for (int k = 0; k < NS; ++k) sh[k][threadIdx.x] = a.v[k];
+    __syncthreads();
+    for (int j = threadIdx.x; j < NS * P; j += kRedThreads) {
+        const int k = j / P, p = j - k * P;
+        bool mx = false;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double t = __shfl_xor_sync(0xffffffffu, a.v[k], o);
-            a.v[k] = op[k] ? fmax(a.v[k], t) : a.v[k] + t;
-        }
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < NS; ++k) sh[wid][k] = a.v[k];
+        for (int q = 0; q < NS; ++q) mx = q == k ? op[q] != 0 : mx;
+        double s = sh[k][p];
+        for (int w = p + P; w < kRedThreads; w += P) s = mx ? fmax(s, sh[k][w]) : s + sh[k][w];
+        part[k][p] = s;
     }
     __syncthreads();
     if (threadIdx.x < NS) {
         const int k = threadIdx.x;
-        double s = sh[0][k];
-        for (int w = 1; w < kRedThreads / 32; ++w) s = op[k] ? fmax(s, sh[w][k]) : s + sh[w][k];
+        bool mx = false;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) mx = q == k ? op[q] != 0 : mx;
+        double s = part[k][0];
+        for (int w = 1; w < P; ++w) s = mx ? fmax(s, part[k][w]) : s + part[k][w];
         dst[k] = s;
     }
 }
@@ -344,15 +343,14 @@ __device__ __forceinline__ double to_double(__int128 v)
     return (double)hi * 0x1p64 + (double)lo;
 }
 
-// Sum of the stored state over populations and valid nodes (weighted by
-// the wall weights when the grid has mirror walls): one warp per row of
-// one population, aligned 16-byte vector loads along the row.
+// Sum of the stored state over populations and nodes of a grid with mirror
+// walls, weighted by the wall weights: one warp per row of one population,
+// aligned 16-byte vector loads along the row.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) sum_state_kernel(const T *__restrict__ src, Geom g, int q,
                                                                 double scale, double *__restrict__ partial)
 {
     constexpr int V = Vec<T>::V;
-    typename SumAcc<T>::type acc = 0;
     double accw = 0.0;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -364,7 +362,7 @@ __global__ void __launch_bounds__(kRedThreads) sum_state_kernel(const T *__restr
     for (int64_t r = warp; r < nrows; r += nwarps) {
         const int64_t pop = r / g.rows, row = r - pop * g.rows;
         const T *rowp = src + pop * g.slab + row * g.pitch;
-        const double rw = g.mirror ? row_wall_weight(g, row) : 1.0;
+        const double rw = row_wall_weight(g, row);
         for (int x0 = lane * V; x0 < g.N0; x0 += U * 32 * V) {
             T a[U][V];
 #pragma unroll
@@ -372,30 +370,80 @@ __global__ void __launch_bounds__(kRedThreads) sum_state_kernel(const T *__restr
                 if (x0 + j * 32 * V < g.N0) ld_vec(rowp + x0 + j * 32 * V, a[j]);
 #pragma unroll
             for (int j = 0; j < U; ++j) {
-                if constexpr (std::is_same<T, float>::value) {
-                    // a whole vector of floats: one integer-pipe sum and one FP64 addition
-                    if (!g.mirror && x0 + j * 32 * V + V <= g.N0) {
-                        acc += sum_f32_int(a[j]);
-                        continue;
-                    }
-                }
 #pragma unroll
                 for (int k = 0; k < V; ++k) {
                     const int x = x0 + j * 32 * V + k;
                     if (x >= g.N0) continue;
-                    if (!g.mirror) {
-                        acc += a[j][k];
-                    } else {
-                        const double xw = ((g.mirror & 1u) && (x == 0 || x == g.N0 - 1)) ? 0.5 : 1.0;
-                        accw += (double)a[j][k] * (rw * xw);
-                    }
+                    const double xw = ((g.mirror & 1u) && (x == 0 || x == g.N0 - 1)) ? 0.5 : 1.0;
+                    accw += (double)a[j][k] * (rw * xw);
                 }
             }
         }
     }
-    Acc<1> a{{(to_double(acc) + accw) * scale}};
+    Acc<1> a{{accw * scale}};
     const int op[1] = {0};
     block_reduce_store<1>(a, op, partial + (int64_t)blockIdx.x * kRedSlots);
+}
+
+// The same without walls: the rows of a population lie one after the other, so
+// a thread takes 16-byte vectors at a grid-wide stride, whatever the row
+// length, U of them in flight; padding is masked to zero.  Fixed point: exact
+// 128-bit sums.  FP32: the U vectors' floats in one integer-pipe sum
+// (sum_f32_int) and one FP64 addition.  The walled kernel above gives each row
+// to a warp: rows of 101 floats kept 26 of 32 lanes busy once per row (101 x 90
+// x 77: 274 us for 53 MB).
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) sum_flat_kernel(const T *__restrict__ src, Geom g, int q, double scale,
+                                                               double *__restrict__ partial)
+{
+    constexpr int V = Vec<T>::V, U = 4;
+    typename SumAcc<T>::type acc = 0;
+    const int vr = g.pitch / V;                      // vectors per row
+    const int64_t nv = g.rows * vr;                  // per population (populations g.slab values apart)
+    const int64_t stride = (int64_t)gridDim.x * kRedThreads;
+    int64_t i = (int64_t)blockIdx.x * kRedThreads + threadIdx.x;
+    const int dx = (int)(stride % vr);
+    int xv = (int)(i % vr), pop = 0;
+    const bool pad = g.pitch != g.N0;
+    while (i >= nv && pop < q) {
+        i -= nv;
+        ++pop;
+    }
+    while (pop < q) {
+        T a[U][V];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            if (pop < q)
+                ld_vec(src + pop * g.slab + i * V, a[j]);
+            else
+#pragma unroll
+                for (int k = 0; k < V; ++k) a[j][k] = T(0);
+            if (pad) {
+#pragma unroll
+                for (int k = 0; k < V; ++k)
+                    if (xv * V + k >= g.N0) a[j][k] = T(0);
+                xv += dx;
+                if (xv >= vr) xv -= vr;
+            }
+            i += stride;
+            while (i >= nv && pop < q) {
+                i -= nv;
+                ++pop;
+            }
+        }
+        if constexpr (std::is_same<T, float>::value) {
+            float f[U * V];
+#pragma unroll
+            for (int j = 0; j < U * V; ++j) f[j] = a[j / V][j % V];
+            acc += sum_f32_int(f);
+        } else {
+#pragma unroll
+            for (int j = 0; j < U * V; ++j) acc += a[j / V][j % V];
+        }
+    }
+    Acc<1> s{{to_double(acc) * scale}};
+    const int op[1] = {0};
+    block_reduce_store<1>(s, op, partial + (int64_t)blockIdx.x * kRedSlots);
 }
 
 // Error norms: slots 3v+0 sum err^2, 3v+1 max |err|, 3v+2 sum exact^2 for
@@ -417,6 +465,7 @@ __global__ void __launch_bounds__(kRedThreads) norms_kernel(const double *__rest
 #pragma unroll
     for (int c = 0; c <= D; ++c) mx[c] = 0;
     constexpr long long kAbs = 0x7fffffffffffffffll;
+#pragma unroll 2
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < nodes;
          n += (int64_t)gridDim.x * blockDim.x) {
         const double t = th[n], te = eth[n];
@@ -455,28 +504,28 @@ __global__ void __launch_bounds__(kRedThreads) maxabs_kernel(const double *__res
     block_reduce_store<1>(a, op, partial + (int64_t)blockIdx.x * kRedSlots);
 }
 
-// Fold nb partial rows of kRedSlots in a fixed order.  opmask bit k = max.
-__global__ void __launch_bounds__(kRedThreads) fold_kernel(const double *__restrict__ partial, int nb, int ns,
-                                                           unsigned opmask, double *__restrict__ out)
+// Fold nb partial rows of kRedSlots in a fixed order.  opmask bit k = max.  A
+// warp per slot, so all slots wait for their loads together.
+__global__ void __launch_bounds__(32 * kRedSlots) fold_kernel(const double *__restrict__ partial, int nb, int ns,
+                                                              unsigned opmask, double *__restrict__ out)
 {
-    __shared__ double sh[kRedThreads];
-    for (int k = 0; k < ns; ++k) {
-        const bool mx = (opmask >> k) & 1u;
-        double s = mx ? 0.0 : 0.0;
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-            const double v = partial[(int64_t)b * kRedSlots + k];
-            s = mx ? fmax(s, v) : s + v;
-        }
-        sh[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sh[threadIdx.x] = mx ? fmax(sh[threadIdx.x], sh[threadIdx.x + w])
-                                                       : sh[threadIdx.x] + sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[k] = sh[0];
-        __syncthreads();
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k >= ns) return;
+    const bool mx = (opmask >> k) & 1u;
+    double s = 0.0;
+    for (int b0 = lane; b0 < nb; b0 += 32 * 8) {
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = b0 + 32 * j < nb ? partial[(int64_t)(b0 + 32 * j) * kRedSlots + k] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s = mx ? fmax(s, v[j]) : s + v[j];
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(0xffffffffu, s, o);
+        s = mx ? fmax(s, t) : s + t;
+    }
+    if (lane == 0) out[k] = s;
 }
 
 // ---------------------------------------------------------------------------
@@ -553,6 +602,17 @@ cudaError_t launch_fd4_grad(const lb_ctx *c, const double *theta0, double *grad)
     return cudaGetLastError();
 }
 
+template <class L, typename T, int FXI>
+static cudaError_t init_go(lb_ctx *c, const InitK &K, const double *theta0, const double *grad, int *flag)
+{
+    const unsigned nb = (unsigned)((c->nodes + kInitThreads - 1) / kInitThreads);
+    if (c->geom.mirror)
+        init_kernel<L, T, FXI, true><<<nb, kInitThreads, 0, c->stream>>>((T *)c->f[c->cur], c->geom, K, theta0, grad, flag);
+    else
+        init_kernel<L, T, FXI, false><<<nb, kInitThreads, 0, c->stream>>>((T *)c->f[c->cur], c->geom, K, theta0, grad, flag);
+    return cudaGetLastError();
+}
+
 template <class L, typename T>
 static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, int *flag)
 {
@@ -568,23 +628,23 @@ static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, i
     K.fxscale = ldexp(1.0, c->fx_bits);
     K.gscale = c->dx * K.fxscale;
     K.fx_bits = c->fx_bits;
-    const unsigned nb = (unsigned)((c->nodes + 255) / 256);
+    K.w1k = K.wdk = K.iak = 0;
     if constexpr (std::is_same<T, long long>::value) {
-        // integer formation needs every constant inside the 62-bit range and
+        // integer formation needs every constant inside the product's range and
         // a total weight that keeps the rest population's sum below 2^61
         const double ia = K.iax / c->dx;
         const double wmass = fabs(c->w0) + 2.0 * d * fabs(c->w1) + 2.0 * d * (d - 1.0) * fabs(wd);
         if (fabs(ia) < 1.5 && fabs(c->w1) < 1.0 && fabs(wd) < 1.0 && wmass <= 4.0) {
-            K.w1k = llrint(ldexp(c->w1, kFxCoefBits));
-            K.wdk = llrint(ldexp(wd, kFxCoefBits));
-            K.iak = llrint(ldexp(ia, kFxCoefBits));
-            init_kernel<L, T, true><<<nb, 256, 0, c->stream>>>((T *)c->f[c->cur], c->geom, K, theta0, grad, flag);
-            return cudaGetLastError();
+            const double most = 0.5 - 0x1p-30;  // mulfx_c's range
+            const bool split = fabs(ia) < most && fabs(c->w1) < most && fabs(wd) < most;
+            const int bits = split ? kFxCollBits : kFxCoefBits;
+            K.w1k = llrint(ldexp(c->w1, bits));
+            K.wdk = llrint(ldexp(wd, bits));
+            K.iak = llrint(ldexp(ia, bits));
+            return split ? init_go<L, T, 2>(c, K, theta0, grad, flag) : init_go<L, T, 1>(c, K, theta0, grad, flag);
         }
     }
-    K.w1k = K.wdk = K.iak = 0;
-    init_kernel<L, T, false><<<nb, 256, 0, c->stream>>>((T *)c->f[c->cur], c->geom, K, theta0, grad, flag);
-    return cudaGetLastError();
+    return init_go<L, T, 0>(c, K, theta0, grad, flag);
 }
 
 cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, int *flag)
@@ -613,18 +673,23 @@ cudaError_t launch_sum_state_rows(lb_ctx *c, const void *src, double *out_dev, i
     g.rows = nrow;
     if (row0 != 0 || nrow != c->geom.rows) g.mirror = 0;
     const int64_t off = row0 * g.pitch;
+    const double scale = c->precision == LB_FX64 ? ldexp(1.0, -c->fx_bits) : 1.0;
+    const auto launch = [&](auto *p) {
+        using T = std::remove_pointer_t<decltype(p)>;
+        if (g.mirror)
+            sum_state_kernel<T><<<nb, kRedThreads, 0, c->stream>>>((const T *)src + off, g, c->q, scale, c->scratch);
+        else
+            sum_flat_kernel<T><<<nb, kRedThreads, 0, c->stream>>>((const T *)src + off, g, c->q, scale, c->scratch);
+    };
     if (c->precision == LB_FP64)
-        sum_state_kernel<double><<<nb, kRedThreads, 0, c->stream>>>((const double *)src + off, g, c->q, 1.0,
-                                                                     c->scratch);
+        launch((double *)nullptr);
     else if (c->precision == LB_FX64)
-        sum_state_kernel<long long><<<nb, kRedThreads, 0, c->stream>>>(
-            (const long long *)src + off, g, c->q, ldexp(1.0, -c->fx_bits), c->scratch);
+        launch((long long *)nullptr);
     else
-        sum_state_kernel<float><<<nb, kRedThreads, 0, c->stream>>>((const float *)src + off, g, c->q, 1.0,
-                                                                    c->scratch);
+        launch((float *)nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    fold_kernel<<<1, kRedThreads, 0, c->stream>>>(c->scratch, nb, 1, 0u, out_dev);
+    fold_kernel<<<1, 32 * kRedSlots, 0, c->stream>>>(c->scratch, nb, 1, 0u, out_dev);
     return cudaGetLastError();
 }
 
@@ -639,7 +704,7 @@ cudaError_t launch_maxabs(lb_ctx *c, const double *x, int64_t n, double *out_dev
     maxabs_kernel<<<nb, kRedThreads, 0, c->stream>>>(x, n, c->scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    fold_kernel<<<1, kRedThreads, 0, c->stream>>>(c->scratch, nb, 1, 1u, out_dev);
+    fold_kernel<<<1, 32 * kRedSlots, 0, c->stream>>>(c->scratch, nb, 1, 1u, out_dev);
     return cudaGetLastError();
 }
 
@@ -659,7 +724,7 @@ cudaError_t launch_norms(lb_ctx *c, const double *th, const double *u, const dou
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    fold_kernel<<<1, kRedThreads, 0, c->stream>>>(c->scratch, nb, ns, mask, out_dev);
+    fold_kernel<<<1, 32 * kRedSlots, 0, c->stream>>>(c->scratch, nb, ns, mask, out_dev);
     return cudaGetLastError();
 }
 
@@ -679,7 +744,7 @@ cudaError_t launch_norms_into(int d, int64_t nodes, const double *th, const doub
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    fold_kernel<<<1, kRedThreads, 0, s>>>(partials, nb, ns, mask, raw_out);
+    fold_kernel<<<1, 32 * kRedSlots, 0, s>>>(partials, nb, ns, mask, raw_out);
     return cudaGetLastError();
 }
 
