@@ -38,7 +38,7 @@ typedef struct lb_adj lb_adj;
  * (whose forward map is FP32-accurate), and for LB_FX64 contexts in 64-bit
  * fixed point: the adjoint field is held as round(phi 2^G), G chosen from
  * the seed so that max|phi_T| 2^G < 2^56, K^T is formed from exact integer
- * sums and rounded 62-bit products, and the dL/dnu term from exact 128-bit
+ * sums and rounded products, and the dL/dnu term from exact 128-bit
  * dot products (FP64 instead when the collision constants are too large for
  * that range: see lb_adjoint.cu).
  * The seed, the initialisation adjoint and the dL/dnu accumulation are FP64
@@ -93,8 +93,9 @@ lb_status lb_adjoint_step(lb_adj *a, int64_t nsteps);
  * After T reverse steps: dL/dtheta0 (device, nodes) and, if requested at
  * creation, dL/dnu (host, 1 value; NULL to skip).  Synchronises the stream.
  * Errors: LB_ESTATE if the reverse pass is incomplete; LB_EINVAL if a
- * fixed-point adjoint field left |value| < 2^59 (not seen in practice: the
- * field grows by less than 1.3x over a reverse pass, against 8x of headroom).
+ * fixed-point adjoint field left |value| < 2^59, or 2^58 for d = 3 (not seen in
+ * practice: the field grows by less than 1.3x over a reverse pass, against 4x of
+ * headroom).
  */
 lb_status lb_adjoint_result(lb_adj *a, double *dL_dtheta0, double *dL_dnu);
 

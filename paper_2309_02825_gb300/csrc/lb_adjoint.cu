@@ -37,10 +37,11 @@ struct AdjK {
     double mshift_th, mshift_paa;  // the shift's moments: theta_ref and sigma theta_ref
     float mshift_th_f, mshift_paa_f;
     // Fixed-point reverse pass (64-bit fixed-point states): the adjoint fields
-    // hold round(phi 2^G); aunit = 2^-G.  K^T uses the collision constants with
-    // kFxCoefBits fraction bits (c0k .. wdk); the eps-term uses the FP64
-    // eps-derivatives scaled by 2^-(F+G) (kdx), F the state's fraction bits.
-    long long c0k, cAk, wdk, k1k, k2k, k3k;
+    // hold round(phi 2^G); aunit = 2^-G.  K^T uses the forward collision's
+    // constants (x); the eps-term uses the FP64 eps-derivatives scaled by
+    // 2^-(F+G) (kdx), F the state's fraction bits.
+    CollFx x;
+    int ints;  // FP64 fields: the node update may take the integer form (adj_node_f64)
     double aunit;
     Coll<double> kdx;
     double ucoef, ducoef;                      // (2 - s1) c and d/deps
@@ -325,44 +326,52 @@ __device__ __forceinline__ A adj_node(A *l, const T *fv, const AdjK &K)
     return eterm;
 }
 
-// The eps-term of fixed-point nodes, before its last conversions: the FP64
-// part theta * (c0' l0 + cA' sum_a + wd' sum_diag), and the exact 128-bit
-// dot products S2 = sum P_aa s2_a, S1 = sum J_a dd_a, S3 = sum P_ab P_p of
-// the state's integer moments with the integer lambda channels.  A lane sums
-// its nodes' S (each below 6 * 2^122 in magnitude for channels below 2^59 and
-// moments below 2^63, so two nodes' sum stays far inside 2^127) and converts
-// each sum once: eps-term = d + k2' S2 + k1' S1 + k3' S3.
+// The eps-term of fixed-point nodes, before its conversions: the exact 128-bit
+// dot products of the state's integer moments with the integer lambda channels,
+//   S2 = sum P_aa s2_a, S1 = sum J_a dd_a, S3 = sum P_ab P_p, SA = theta xa, SD = theta xd,
+// eps-term = k2' S2 + k1' S1 + k3' S3 + cA' SA + wd' SD (the rest channel's
+// constant is c0 = 1 - 2d cA - 2d(d-1) wd, so its derivative goes into SA and
+// SD).  A thread sums its nodes' S (at most two; each below 2^125.6 for channels
+// inside the range check and moments below 2^63) and converts each sum once.
 struct EpsFx {
-    double d = 0.0;
-    __int128 S2 = 0, S1 = 0, S3 = 0;
+    __int128 S2 = 0, S1 = 0, S3 = 0, SA = 0, SD = 0;
+    __device__ __forceinline__ double value(const Coll<double> &kd) const
+    {
+        return fma(kd.k2, i128_to_f64_rn(S2),
+                   fma(kd.k1, i128_to_f64_rn(S1),
+                       fma(kd.k3, i128_to_f64_rn(S3), fma(kd.cA, i128_to_f64_rn(SA), kd.wd * i128_to_f64_rn(SD)))));
+    }
 };
 
+// Range of the fixed-point adjoint fields: |v| < 2^kAdjBits (they start below
+// 2^56 and grow by less than 1.3x), so that the next step's channels fit 63
+// bits: 2d + 2d and 2d(d-1) + 2d(d-1) terms at most, 8 for d = 2, 24 for d = 3.
+template <class L> __host__ __device__ constexpr int adj_bits() { return L::D <= 2 ? 59 : 58; }
+
 // The node update of the fixed-point reverse pass (64-bit fixed-point states):
-// K^T from exact integer channel sums and rounded 64x62-bit products; with
-// NU, the eps-term lambda . (dK/deps) f as EpsFx (the int64 channel and
-// moment values of its FP64 part by the hardware conversion, which keeps the
-// FP64 and integer pipes in balance).  ORs into `rng` the high words of the
-// outputs plus 2^27: an output is inside |v| < 2^59 (the fields start below
-// 2^56) exactly when that sum stays below 2^28.
+// K^T from exact integer channel sums and the collision's own rounded products
+// (mulfx_c, the forward step's constants); with NU, adds the eps-term's dot
+// products to ep.  ORs into `rng` the high words of the outputs plus
+// 2^(kAdjBits - 32): an output is inside the range exactly when that sum stays
+// below 2^(kAdjBits - 31).
 template <class L, bool NU>
 __device__ __forceinline__ void adj_node_fx(long long *l, const long long *fv, const AdjK &K, unsigned &rng, EpsFx &ep)
 {
     constexpr int D = L::D, NP = D * (D - 1) / 2, B0 = 1 + 2 * D;
     const long long l0 = l[0];
     long long s2[D], dd[D], P[NP > 0 ? NP : 1];  // s2 = l_{+a} + l_{-a} - 2 l0
-    long long sax = 0, sdg = 0;
+    long long xa = 0, xd = 0;                    // sums over the axes and the planes, less as many l0
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const long long sa = l[1 + a] + l[1 + D + a];
-        sax += sa;
-        s2[a] = sa - 2 * l0;
+        s2[a] = l[1 + a] + l[1 + D + a] - 2 * l0;
+        xa += s2[a];
         dd[a] = l[1 + a] - l[1 + D + a];
     }
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         const Plane<long long> pl = plane(l[B0 + 4 * p], l[B0 + 4 * p + 1], l[B0 + 4 * p + 2], l[B0 + 4 * p + 3]);
         P[p] = pl.P;
-        sdg += pl.F;
+        xd += pl.F - 4 * l0;
     }
     if constexpr (NU) {
         const NodeMoments<L, long long> m = node_moments<L, long long>(fv);
@@ -373,18 +382,16 @@ __device__ __forceinline__ void adj_node_fx(long long *l, const long long *fv, c
         }
 #pragma unroll
         for (int p = 0; p < NP; ++p) ep.S3 += (__int128)m.Pab[p] * P[p];
-        const Coll<double> &kd = K.kdx;
-        const double lt = fma(kd.c0, (double)l0, fma(kd.cA, (double)sax, kd.wd * (double)sdg));
-        ep.d = fma((double)m.th, lt, ep.d);
+        ep.SA += (__int128)m.th * xa;
+        if constexpr (NP > 0) ep.SD += (__int128)m.th * xd;
     }
-    // the rest channel: one rounding of the exact sum of its three products
-    const __int128 lts = (__int128)l0 * K.c0k + (__int128)sax * K.cAk + (__int128)sdg * K.wdk;
-    const long long Lt = (long long)((lts + ((__int128)1 << (kFxCoefBits - 1))) >> kFxCoefBits);
+    long long Lt = l0 + mulfx_c(xa, K.x.cA);
+    if constexpr (NP > 0) Lt += mulfx_c(xd, K.x.wd);
     long long LP[D], LJ[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        LP[a] = mulfx(s2[a], K.k2k);
-        LJ[a] = mulfx(dd[a], K.k1k);
+        LP[a] = mulfx_c(s2[a], K.x.k2);
+        LJ[a] = mulfx_c(dd[a], K.x.k1);
     }
     l[0] = Lt;
 #pragma unroll
@@ -398,16 +405,44 @@ __device__ __forceinline__ void adj_node_fx(long long *l, const long long *fv, c
         constexpr int a = pair_a<D>(p), b = pair_b<D>(p);
         const long long X = Lt + (LP[a] + LP[b]);
         const long long U = LJ[a] + LJ[b], W = LJ[a] - LJ[b];
-        const long long lab = mulfx(P[p], K.k3k);
+        const long long lab = mulfx_c(P[p], K.x.k3);
         const long long Xp = X + lab, Xm = X - lab;
         l[B0 + 4 * p] = Xp + U;      // (+1, +1)
         l[B0 + 4 * p + 1] = Xm - W;  // (-1, +1)
         l[B0 + 4 * p + 2] = Xp - U;  // (-1, -1)
         l[B0 + 4 * p + 3] = Xm + W;  // (+1, -1)
     });
-    // next step's channel sums (<= 12 terms below 2^59) stay below 2^63
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) rng |= (unsigned)((unsigned long long)l[i] >> 32) + (1u << 27);
+    for (int i = 0; i < L::Q; ++i) rng |= (unsigned)((unsigned long long)l[i] >> 32) + (1u << (adj_bits<L>() - 32));
+}
+
+// The node update of FP64 fields on the integer pipes (FP64 operations, 71 per
+// D2Q9 node, bind the direct form): lambda aligned to its largest exponent, the
+// bits below 2^-59 of it rounded off (the direct form rounds every step at 2^-53
+// of values that large), the state's doubles aligned without loss as in the
+// forward collision, then adj_node_fx, and each result rounded once.  Nodes
+// where either does not align take the direct form.
+template <class L, bool NU> __device__ __forceinline__ double adj_node_f64(double (&l)[L::Q], const double (&f)[L::Q], const AdjK &K)
+{
+    constexpr int PL = 6, PF = f64_align_bit<L>();
+    if (K.ints) {
+        long long lv[L::Q], fv[L::Q];
+        unsigned el, ef = 0u;
+        bool ok = f64_align_round<L::Q, PL>(l, lv, el);
+        if constexpr (NU) ok = ok && f64_align<L::Q, PF>(f, fv, ef);
+        if (ok) {
+            unsigned rng = 0u;
+            EpsFx ep;
+            adj_node_fx<L, NU>(lv, fv, K, rng, ep);
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i) l[i] = f64_from_aligned<PL>(lv[i], el);
+            if constexpr (!NU) return 0.0;
+            const double ul = __hiloint2double((int)((el - 52u - PL) << 20), 0);  // the units as powers of two
+            const double uf = __hiloint2double((int)((ef - 52u - PF) << 20), 0);
+            return ep.value(K.kd) * ul * uf;
+        }
+    }
+    return adj_node<L, double, NU, double>(l, f, K);
 }
 
 // The integer -> FP64 conversions of the fixed-point eps-term, for their self-test.
@@ -473,15 +508,17 @@ __global__ void __launch_bounds__(kSweepThreads) adj_seed_kernel(const T *__rest
                 if constexpr (e != 0) J[a] += e * fv;
             });
         });
-        double gu[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0}, gt = 0.0;
+        // dL/df_i = sum_a (g_a / theta) (e_ia ucoef - u_a) + dL/dtheta: FP64 divisions
+        // bind this kernel, so theta divides once per component of g and u
+        double gu[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0}, gt = 0.0;  // gu: g / theta
         if (x < g.N0) {
             const int64_t node = row * g.N0 + x;
             if (dLdu) {
 #pragma unroll
                 for (int a = 0; a < L::D; ++a) {
-                    gu[a] = dLdu[a * nodes + node];
+                    gu[a] = dLdu[a * nodes + node] / th;
                     u[a] = K.ucoef * J[a] / th;
-                    acc += gu[a] * K.ducoef * J[a] / th;
+                    acc += gu[a] * K.ducoef * J[a];
                 }
             }
             if (dLdth) gt = dLdth[node];
@@ -494,7 +531,7 @@ __global__ void __launch_bounds__(kSweepThreads) adj_seed_kernel(const T *__rest
                 constexpr int e = L::E[i][a];
                 s += gu[a] * ((double)e * K.ucoef - u[a]);
             });
-            out[i][v] = (x < g.N0) ? s / th + gt : 0.0;
+            out[i][v] = (x < g.N0) ? s + gt : 0.0;
         });
     }
     if (x0 + V * lane < g.pitch) {  // lanes beyond the row only loaded
@@ -521,7 +558,9 @@ template <typename A> __host__ __device__ constexpr int adj_threads()
     return 128;
 }
 
-// One reverse step: phi_out = K^T lambda(phi_in); eps-term if NU.
+// One reverse step: phi_out = K^T lambda(phi_in); eps-term if NU.  Two nodes per
+// lane: FP32, and grids with walls; periodic grids in 8-byte arithmetic take
+// adj_flat_kernel.
 template <class L, typename T, bool NU, typename A, bool MIR = false>
 __global__ void __launch_bounds__(adj_threads<A>()) adj_step_kernel(const A *__restrict__ phi_in,
                                                                  const T *__restrict__ Pn, A *__restrict__ phi_out,
@@ -549,7 +588,7 @@ __global__ void __launch_bounds__(adj_threads<A>()) adj_step_kernel(const A *__r
         if constexpr (MIR)
             gather_rev_walls<L, A>(phi_in, g, row, x0, lane, lam);
         else
-            gather_rev<L, A>(phi_in, g, row, x0, lane, lam);
+            gather_rev<L, A>(phi_in, g, row, x0, lane, lam);  // FP32 without the eps-term
         if constexpr (NU) gather<L, T, V, MIR>(Pn, g, row, x0, lane, f);
     }
     EpsAcc<A> acc = 0;  // this lane's dL/deps terms
@@ -572,11 +611,12 @@ __global__ void __launch_bounds__(adj_threads<A>()) adj_step_kernel(const A *__r
             EpsFx e;
             adj_node_fx<L, NU>(l, fv, K, rng, e);
             if (own) {
-                range |= rng >= (1u << 28);
-                ep.d += e.d;
+                range |= rng >= (1u << (adj_bits<L>() - 31));
                 ep.S2 += e.S2;
                 ep.S1 += e.S1;
                 ep.S3 += e.S3;
+                ep.SA += e.SA;
+                ep.SD += e.SD;
             }
         } else {
             const EpsAcc<A> e = adj_node<L, T, NU, A>(l, fv, K);
@@ -586,8 +626,7 @@ __global__ void __launch_bounds__(adj_threads<A>()) adj_step_kernel(const A *__r
         for (int i = 0; i < L::Q; ++i) lam[i][v] = l[i];
     }
     if constexpr (std::is_same<A, long long>::value && NU) {
-        const Coll<double> &kd = K.kdx;
-        acc = ep.d + fma(kd.k2, i128_to_f64_rn(ep.S2), fma(kd.k1, i128_to_f64_rn(ep.S1), kd.k3 * i128_to_f64_rn(ep.S3)));
+        acc = ep.value(K.kdx);
     }
     if (x0 + V * lane < g.pitch) {  // lanes beyond the row only loaded
         A *dp = phi_out + row * g.pitch + x0 + V * lane;
@@ -602,6 +641,97 @@ __global__ void __launch_bounds__(adj_threads<A>()) adj_step_kernel(const A *__r
         // reduction (no return value, so the warp does not wait) is deterministic
         acc = warp_sum(acc);
         if (lane == 0) atomicAdd(slot + seg, (double)acc);
+    }
+}
+
+// The reverse step of periodic grids in 8-byte arithmetic: one node at a time
+// per thread, in row-major order across row ends.  Each value is one load at
+// its wrapped source, all 2 q of a node in flight at once, with no shuffles, and
+// a node's values fit in about half the registers of the two-node lanes of
+// adj_step_kernel, so more warps wait on the gathers.  A thread takes NPT nodes
+// one after the other (two for 2D fixed point where that still leaves two blocks
+// per SM): the eps-term's sums are converted and reduced once for both, 15.7
+// against 16.6 us per step; in 3D and FP64 one, 14.8 against 16.4 and 43.6
+// against 48.  The block's eps-terms are added through shared memory, a quarter
+// of the FP64 steps of a shuffle tree per warp.  Bound by L2: 57 MB per 512^2
+// step and 38 MB of the recompute sweep beside it.  Per step with the recompute
+// sweeps, before -> now: 512^2 fixed point 17.9 -> 15.7 us, FP64 (with
+// adj_node_f64) 52.3 -> 23.9; 48^3 21.7 -> 14.8, 64.2 -> 27.1.
+template <class L, typename T, bool NU, typename A, int NPT>
+__global__ void __launch_bounds__(adj_threads<A>()) adj_flat_kernel(const A *__restrict__ phi_in, const T *__restrict__ Pn,
+                                                                   A *__restrict__ phi_out, Geom g, AdjK K,
+                                                                   double *__restrict__ slot, int *__restrict__ flag)
+{
+    constexpr int TH = adj_threads<A>();
+    const unsigned nodes = (unsigned)(g.N0 * g.rows);  // <= 2^31
+    EpsAcc<A> acc = 0;
+    EpsFx ep;
+    bool range = false;
+#pragma unroll 1
+    for (int v = 0; v < NPT; ++v) {
+        const unsigned nd = (blockIdx.x * NPT + v) * TH + threadIdx.x;
+        if (nd >= nodes) break;
+        const unsigned row = nd / (unsigned)g.N0;
+        const int x = (int)(nd - row * (unsigned)g.N0);
+        const RowPos rpos = row_pos<L::D>(g, row);
+        const int xs[3] = {x == g.N0 - 1 ? 0 : x + 1, x, x == 0 ? g.N0 - 1 : x - 1};  // x - e by e + 1
+        // The source x - e_i within a population; the reverse pull reads x + e_i =
+        // x - e_opp(i).  In 3D the 19 offsets are formed once, in 32 bits (at most
+        // 2^31 nodes and their rows' padding), for both fields (48^3 fixed point 15.7
+        // -> 14.8 us); in 2D addresses formed at each load keep more loads in flight
+        // (512^2 15.7 against 16.3 us).
+        using O = typename std::conditional<(L::D > 2), unsigned, int64_t>::type;
+        const auto source = [&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int ex = L::E[i][0], ey = L::E[i][1], ez = L::E[i][2], ew = L::E[i][3];
+            return (O)src_row<L::D, ey, ez, ew>(g, rpos) * (O)g.pitch + (O)xs[1 + ex];
+        };
+        O o[L::Q];
+        if constexpr (L::D > 2) static_for<0, L::Q>([&](auto I) { o[decltype(I)::value] = source(I); });
+        A l[L::Q];
+        T f[L::Q];
+        static_for<0, L::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value, j = reflect_pop<L>(i, 7);
+            if constexpr (L::D > 2)
+                l[i] = __ldg(phi_in + (int64_t)i * g.slab + o[j]);
+            else
+                l[i] = __ldg(phi_in + (int64_t)i * g.slab + source(std::integral_constant<int, j>{}));
+        });
+        if constexpr (NU) {
+            static_for<0, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                if constexpr (L::D > 2)
+                    f[i] = __ldg(Pn + (int64_t)i * g.slab + o[i]);
+                else
+                    f[i] = __ldg(Pn + (int64_t)i * g.slab + source(I));
+            });
+        }
+        if constexpr (std::is_same<A, long long>::value) {
+            unsigned rng = 0u;
+            adj_node_fx<L, NU>(l, f, K, rng, ep);
+            range |= rng >= (1u << (adj_bits<L>() - 31));
+        } else if constexpr (std::is_same<T, double>::value && L::D > 1) {
+            acc += adj_node_f64<L, NU>(l, f, K);
+        } else {
+            acc += adj_node<L, T, NU, A>(l, f, K);
+        }
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) phi_out[(int64_t)i * g.slab + (int64_t)row * g.pitch + x] = l[i];
+    }
+    if (range) atomicOr(flag, 1);
+    if constexpr (NU) {
+        if constexpr (std::is_same<A, long long>::value) acc = ep.value(K.kdx);
+        __shared__ double sh[TH];
+        sh[threadIdx.x] = acc;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double s = sh[threadIdx.x];
+#pragma unroll
+            for (int w = 32; w < TH; w += 32) s += sh[threadIdx.x + w];
+            s = warp_sum(s);
+            // one writer per slot per launch, launches in stream order: deterministic
+            if (threadIdx.x == 0) atomicAdd(slot + blockIdx.x, s);
+        }
     }
 }
 
@@ -632,28 +762,36 @@ __global__ void adj_init_kernel(const A *__restrict__ phi, Geom g, AdjK K, const
             onwall[a] = ((g.mirror >> a) & 1u) && (cc[a] == 0 || cc[a] == nn[a] - 1);
             gr[a] = onwall[a] ? 0.0 : grad[a * nodes + n];
         }
-        double s = 0.0, hh[3] = {0.0, 0.0, 0.0};
-        static_for<0, L::Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int ex = L::E[i][0], ey = L::E[i][1], ez = L::E[i][2];
-            constexpr int nz = (ex != 0) + (ey != 0) + (ez != 0);
-            const double ph = std::is_same<A, long long>::value ? (double)p[(int64_t)i * g.slab] * K.aunit
-                                                               : (double)p[(int64_t)i * g.slab];
-            s = fma(K.w[i], ph, s);
-            double dfi = K.dw[i] * t0;
-            if constexpr (nz == 1) {
-                constexpr int a = (ex != 0) ? 0 : ((ey != 0) ? 1 : 2);
-                constexpr int sg = (ex != 0) ? ex : ((ey != 0) ? ey : ez);
-                hh[a] -= sg * K.iax * ph;
-                dfi -= sg * K.diax * gr[a];
-            } else if constexpr (nz == 2) {
-                if constexpr (ex != 0) hh[0] -= ex * K.idg * ph;
-                if constexpr (ey != 0) hh[1] -= ey * K.idg * ph;
-                if constexpr (ez != 0) hh[2] -= ez * K.idg * ph;
-                dfi -= K.didg * (ex * gr[0] + ey * gr[1] + ez * gr[2]);
-            }
-            acc = fma(ph, dfi, acc);
+        // phi enters through a few sums per node (rest, axes, planes), exact
+        // integers for fixed point: FP64 operations bind this kernel
+        using C = typename std::conditional<std::is_same<A, long long>::value, long long, double>::type;
+        constexpr int D = L::D, B0 = 1 + 2 * D;
+        C v[L::Q], sax = 0, sdg = 0, da[3] = {0, 0, 0}, ja[3] = {0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) v[i] = (C)p[(int64_t)i * g.slab];
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            sax += v[1 + a] + v[1 + D + a];
+            da[a] = v[1 + a] - v[1 + D + a];
+        }
+        static_for<0, D *(D - 1) / 2>([&](auto Pi) {
+            constexpr int q = decltype(Pi)::value;
+            const Plane<C> pl = plane(v[B0 + 4 * q], v[B0 + 4 * q + 1], v[B0 + 4 * q + 2], v[B0 + 4 * q + 3]);
+            sdg += pl.F;
+            ja[pair_a<D>(q)] += pl.Ja;
+            ja[pair_b<D>(q)] += pl.Jb;
         });
+        const double un = std::is_same<A, long long>::value ? K.aunit : 1.0;
+        const double f0 = (double)v[0] * un, fa = (double)sax * un, fd = (double)sdg * un;
+        const double s = fma(K.w[0], f0, fma(K.w[1], fa, D > 1 ? K.w[B0] * fd : 0.0));
+        double hh[3] = {0.0, 0.0, 0.0};
+        acc = t0 * fma(K.dw[0], f0, fma(K.dw[1], fa, D > 1 ? K.dw[B0] * fd : 0.0));
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const double xa = (double)da[a] * un, ya = (double)ja[a] * un;
+            hh[a] = -fma(K.iax, xa, K.idg * ya);
+            acc = fma(-gr[a], fma(K.diax, xa, K.didg * ya), acc);
+        }
         dth0[n] = s;
 #pragma unroll
         for (int a = 0; a < L::D; ++a) h[a * nodes + n] = onwall[a] ? 0.0 : hh[a];
@@ -744,19 +882,16 @@ struct lb_adj {
     int pcur = 0;
     double *th0 = nullptr, *grad = nullptr, *h = nullptr;
     double *slot_step = nullptr, *slot_init = nullptr, *dsum = nullptr;
-    int64_t nslot_init = 0;
+    int64_t nslot_init = 0, nslot_step = 0;
     int64_t done = 0;  // reverse steps completed
     bool forward_done = false, seeded = false;
     lbk::AdjK K{};
     size_t bytes = 0;
-    // Recorded graphs.  fgraph[p]: C forward sweeps from buffer p (valid for
-    // the walls they were recorded with).  rgraph[p][b][pre]: one whole
+    // Recorded graphs.  rgraph[p][b][pre]: one whole
     // reverse segment, C reverse steps from adjoint buffer p over the segment
     // held in seg[b], and with pre = 1 beside them, on a second branch, the
     // C - 1 recompute sweeps of the previous segment into seg[b ^ 1] (valid
     // for the constants K and walls they were recorded with).
-    cudaGraphExec_t fgraph[2] = {nullptr, nullptr};
-    uint64_t fgen[2] = {0, 0};  // the context's generation (walls, viscosity) each was recorded in
     uint64_t fwd_gen = 0;       // the context's generation at the last forward pass
     cudaGraphExec_t rgraph[2][2][2] = {};
     lbk::AdjK rK[2][2][2]{};
@@ -793,7 +928,6 @@ void free_adj(lb_adj *a)
     cudaFree(a->dsum);
     cudaFree(a->dflag);
     for (int p = 0; p < 2; ++p) {
-        if (a->fgraph[p]) cudaGraphExecDestroy(a->fgraph[p]);
         for (auto &gb : a->rgraph[p])
             for (cudaGraphExec_t g : gb)
                 if (g) cudaGraphExecDestroy(g);
@@ -835,6 +969,19 @@ bool stream_capturing(cudaStream_t s)
     return cap != cudaStreamCaptureStatusNone;
 }
 
+// Whether the integer node update (adj_node_fx) serves a context's constants:
+// inside the split product's range (every fixed-point context), and outputs of
+// K^T, bounded by (|c0| + 2d|cA| + 4P|wd| + 8|k2| + 4|k1| + 4|k3|) 2^59 with P =
+// d(d-1)/2 planes for fields below 2^59 (d = 3: 2^58), below 2^63.
+bool adj_ints_ok(const lb_ctx &c)
+{
+    const lbk::Coll<double> kc = lbk::make_coll<double>(c);
+    const double d = c.d, planes = d * (d - 1) / 2;
+    const double bound = fabs(kc.c0) + 2 * d * fabs(kc.cA) + 4 * planes * fabs(kc.wd) + 8 * fabs(kc.k2) +
+                         4 * fabs(kc.k1) + 4 * fabs(kc.k3);
+    return bound < 15.0 && lbk::fx_constants_ok(c);
+}
+
 // Collision, recovery and initialisation constants and their eps-derivatives
 // (Theorem 2, Eq. (Bur-Sol), differentiated in eps).
 void make_adjk(lb_adj *a)
@@ -863,13 +1010,8 @@ void make_adjk(lb_adj *a)
     K.kd.cA = (ds2x * sigma + c.s2x * dsigma) / 2.0 - 2.0 * (d - 1) * dwd;
     K.kd.wd = dwd;
     K.kf = lbk::make_coll<float>(c);
-    const auto fxk = [](double v) { return llrint(ldexp(v, lbk::kFxCoefBits)); };
-    K.c0k = fxk(K.k.c0);
-    K.cAk = fxk(K.k.cA);
-    K.wdk = fxk(K.k.wd);
-    K.k1k = fxk(K.k.k1);
-    K.k2k = fxk(K.k.k2);
-    K.k3k = fxk(K.k.k3);
+    K.ints = adj_ints_ok(c);
+    K.x = K.ints ? lbk::make_coll_fx(&c) : lbk::CollFx{};
     K.aunit = 1.0;
     K.kdx = K.kd;
     K.kdf = {(float)K.kd.k1, (float)K.kd.k2, (float)K.kd.k3, (float)K.kd.c0, (float)K.kd.cA, (float)K.kd.wd};
@@ -966,15 +1108,27 @@ template <class L, typename T, typename A, bool MIR> cudaError_t step_m(lb_adj *
 {
     lb_ctx *c = a->ctx;
     constexpr int TH = lbk::adj_threads<A>();
-    const unsigned nb = (unsigned)((a->ag.nseg + TH / 32 - 1) / (TH / 32));
     const A *in = (const A *)a->phi[a->pcur];
     A *out = (A *)a->phi[a->pcur ^ 1];
-    if (a->want_nu)
-        lbk::adj_step_kernel<L, T, true, A, MIR><<<nb, TH, 0, c->stream>>>(
-            in, (const T *)Pn, out, a->ag, a->K, a->slot_step, a->dflag);
-    else
-        lbk::adj_step_kernel<L, T, false, A, MIR><<<nb, TH, 0, c->stream>>>(
-            in, (const T *)Pn, out, a->ag, a->K, a->slot_step, a->dflag);
+    const T *P = (const T *)Pn;
+    if constexpr (!MIR && sizeof(A) == 8) {
+        const int64_t n1 = (c->nodes + TH - 1) / TH;
+        const unsigned n2 = (unsigned)((n1 + 1) / 2);
+        if (!a->want_nu)
+            lbk::adj_flat_kernel<L, T, false, A, 1><<<(unsigned)n1, TH, 0, c->stream>>>(in, P, out, a->ag, a->K,
+                                                                                       a->slot_step, a->dflag);
+        else if (std::is_same<A, long long>::value && L::D <= 2 && n1 >= 4 * c->sms)
+            lbk::adj_flat_kernel<L, T, true, A, 2><<<n2, TH, 0, c->stream>>>(in, P, out, a->ag, a->K, a->slot_step, a->dflag);
+        else
+            lbk::adj_flat_kernel<L, T, true, A, 1><<<(unsigned)n1, TH, 0, c->stream>>>(in, P, out, a->ag, a->K,
+                                                                                      a->slot_step, a->dflag);
+    } else {
+        const unsigned nb = (unsigned)((a->ag.nseg + TH / 32 - 1) / (TH / 32));
+        if (a->want_nu)
+            lbk::adj_step_kernel<L, T, true, A, MIR><<<nb, TH, 0, c->stream>>>(in, P, out, a->ag, a->K, a->slot_step, a->dflag);
+        else
+            lbk::adj_step_kernel<L, T, false, A, MIR><<<nb, TH, 0, c->stream>>>(in, P, out, a->ag, a->K, a->slot_step, a->dflag);
+    }
     return cudaGetLastError();
 }
 
@@ -1125,20 +1279,7 @@ lb_status lb_adjoint_create(lb_ctx *ctx, int64_t T, int64_t C, int want_nu, lb_a
     a->T = T;
     a->C = C;
     a->want_nu = want_nu != 0;
-    {
-        // The integer reverse pass holds the constants with 62 fraction bits
-        // (each inside (-2, 2)) and keeps every field below 2^59 (checked per
-        // store).  An output of K^T is then bounded by
-        // (|c0| + 2d|cA| + 4P|wd| + 8|k2| + 4|k1| + 4|k3|) 2^59, P = d(d-1)/2
-        // planes, which must stay below 2^63; otherwise the pass runs in FP64.
-        const lbk::Coll<double> kc = lbk::make_coll<double>(*ctx);
-        const double d = ctx->d, planes = d * (d - 1) / 2;
-        const double bound = fabs(kc.c0) + 2 * d * fabs(kc.cA) + 4 * planes * fabs(kc.wd) + 8 * fabs(kc.k2) +
-                             4 * fabs(kc.k1) + 4 * fabs(kc.k3);
-        const double lim = 1.999;
-        a->fx = ctx->precision == LB_FX64 && bound < 15.0 && fabs(kc.c0) < lim && fabs(kc.cA) < lim &&
-                fabs(kc.wd) < lim && fabs(kc.k1) < lim && fabs(kc.k2) < lim && fabs(kc.k3) < lim;
-    }
+    a->fx = ctx->precision == LB_FX64 && adj_ints_ok(*ctx);
     a->state_bytes = (size_t)ctx->q * ctx->geom.slab * ctx->elem;
     cudaError_t e = cudaSuccess;
     const size_t aelem = (ctx->precision == LB_FP32_SHIFTED) ? sizeof(float) : sizeof(double);
@@ -1161,7 +1302,8 @@ lb_status lb_adjoint_create(lb_ctx *ctx, int64_t T, int64_t C, int want_nu, lb_a
     if (e == cudaSuccess) e = cudaMalloc(&a->th0, sizeof(double) * ctx->nodes);
     if (e == cudaSuccess) e = cudaMalloc(&a->grad, sizeof(double) * ctx->d * ctx->nodes);
     if (e == cudaSuccess) e = cudaMalloc(&a->h, sizeof(double) * ctx->d * ctx->nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&a->slot_step, sizeof(double) * a->ag.nseg);
+    a->nslot_step = std::max<int64_t>(a->ag.nseg, (ctx->nodes + 127) / 128);  // a warp or a block of the reverse step each
+    if (e == cudaSuccess) e = cudaMalloc(&a->slot_step, sizeof(double) * a->nslot_step);
     if (e == cudaSuccess) e = cudaMalloc(&a->slot_init, sizeof(double) * a->nslot_init);
     if (e == cudaSuccess) e = cudaMalloc(&a->dsum, sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&a->dflag, sizeof(int));
@@ -1220,32 +1362,15 @@ lb_status lb_adjoint_forward(lb_adj *a, const double *theta0, double *theta, dou
         (e = cudaMemcpyAsync(a->grad, c->gradtmp, sizeof(double) * c->d * c->nodes, cudaMemcpyDeviceToDevice,
                              c->stream)) != cudaSuccess)
         return acuda(a, e, "lb_adjoint_forward");
-    const bool cap = stream_capturing(c->stream);
-    for (int64_t k = 0; k * a->C < a->T; ++k) {
-        if (a->want_nu &&
-            (e = cudaMemcpyAsync(a->ck[k], c->f[c->cur], a->state_bytes, cudaMemcpyDeviceToDevice, c->stream)) !=
+    if (!a->want_nu) {  // no state is needed on the way
+        if ((st = lb_step(c, a->T)) != LB_OK) return st;
+    } else {
+        for (int64_t k = 0; k * a->C < a->T; ++k) {
+            if ((e = cudaMemcpyAsync(a->ck[k], c->f[c->cur], a->state_bytes, cudaMemcpyDeviceToDevice, c->stream)) !=
                 cudaSuccess)
-            return acuda(a, e, "lb_adjoint_forward: checkpoint");
-        const int64_t n = std::min<int64_t>(a->C, a->T - k * a->C);
-        if (n < a->C || cap) {  // a short last segment, or inside the caller's capture: plain launches
-            if ((st = lb_step(c, n)) != LB_OK) return st;
-            continue;
+                return acuda(a, e, "lb_adjoint_forward: checkpoint");
+            if ((st = lb_step(c, std::min<int64_t>(a->C, a->T - k * a->C))) != LB_OK) return st;
         }
-        const int p = c->cur;
-        if (!a->fgraph[p] || a->fgen[p] != c->gen) {
-            e = record_graph(c, &a->fgraph[p], [&]() {
-                cudaError_t r = cudaSuccess;
-                for (int64_t m = 0, q = p; m < n && r == cudaSuccess; ++m, q ^= 1)
-                    r = lbk::launch_sweep(c, c->f[q], c->f[q ^ 1]);
-                return r;
-            });
-            if (e != cudaSuccess) return acuda(a, e, "lb_adjoint_forward: record");
-            a->fgen[p] = c->gen;
-        }
-        if ((e = cudaGraphLaunch(a->fgraph[p], c->stream)) != cudaSuccess)
-            return acuda(a, e, "lb_adjoint_forward: graph");
-        c->cur ^= (int)(n & 1);
-        c->step += n;
     }
     if ((theta || u) && (st = lb_macros(c, theta, nullptr, u)) != LB_OK) return st;
     a->forward_done = true;
@@ -1261,7 +1386,7 @@ lb_status lb_adjoint_seed(lb_adj *a, const double *dLdu, const double *dLdth)
         return afail(a, LB_ESTATE, "lb_adjoint_seed: run lb_adjoint_forward first (and do not step the context)");
     lb_ctx *c = a->ctx;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(a->slot_step, 0, sizeof(double) * a->ag.nseg, c->stream)) != cudaSuccess ||
+    if ((e = cudaMemsetAsync(a->slot_step, 0, sizeof(double) * a->nslot_step, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(a->slot_init, 0, sizeof(double) * a->nslot_init, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(a->dflag, 0, sizeof(int), c->stream)) != cudaSuccess)
         return acuda(a, e, "lb_adjoint_seed");
@@ -1370,7 +1495,7 @@ lb_status lb_adjoint_result(lb_adj *a, double *dL_dtheta0, double *dL_dnu)
     }
     if (dL_dnu) {
         if (!a->want_nu) return afail(a, LB_EINVAL, "lb_adjoint_result: dL/dnu was not requested");
-        lbk::sum_slots_kernel<<<1, 256, 0, c->stream>>>(a->slot_step, a->ag.nseg, a->slot_init, a->nslot_init,
+        lbk::sum_slots_kernel<<<1, 256, 0, c->stream>>>(a->slot_step, a->nslot_step, a->slot_init, a->nslot_init,
                                                         a->dsum);
         double deps = 0.0;
         if ((e = cudaGetLastError()) != cudaSuccess ||

@@ -871,6 +871,28 @@ template <class L> __device__ __forceinline__ void collide(L, double *f, const C
 
 // A double rounded to float (to nearest, ties to even) on the integer pipes;
 // results outside the normal floats by the hardware conversion.
+// The same for values of any spread: bits below 2^-(53 + PB) of the largest are
+// rounded to nearest.  False where the largest is zero, subnormal, not finite or
+// at the ends of the range.
+template <int Q, int PB>
+__device__ __forceinline__ bool f64_align_round(const double (&f)[Q], long long (&v)[Q], unsigned &emax)
+{
+    unsigned mx = 0u;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) mx = max(mx, (unsigned)__double2hiint(f[i]) & 0x7ff00000u);
+    emax = mx >> 20;
+    if (mx - (100u << 20) > (1900u << 20)) return false;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
+        const unsigned e = (hi >> 20) & 0x7ffu, sh = min(emax - e, 62u);
+        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32 | lo) << PB;
+        const long long r = (long long)((m + ((1ull << sh) >> 1)) >> sh);
+        v[i] = (int)hi < 0 ? -r : r;
+    }
+    return true;
+}
+
 __device__ __forceinline__ float f64_to_f32_rn(double v)
 {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);

@@ -302,3 +302,38 @@ def test_autograd_theta_output_matches_oracle():
     g = theta0.grad.cpu().numpy()
     assert np.max(np.abs(g - go)) <= TOL * np.max(np.abs(go))
     assert float(nu_t.grad) == pytest.approx(dnuo, rel=TOL)
+
+
+@pytest.mark.parametrize("d,N", [(2, (33, 21)), (3, (11, 9, 7))])
+def test_fp64_reverse_step_on_seeds_of_wide_spread(d, N):
+    """FP64 fields whose node values spread over many binades, change sign and
+    vanish (the reverse step's integer form rounds such values to 2^-59 of the
+    node's largest, or leaves the node to the direct form): dL/dtheta0 and
+    dL/dnu for a linear loss against the oracle's, at the bound of the other
+    parity tests."""
+    T = 6
+    rng = np.random.default_rng(5)
+    nu, eps = 0.02, {2: 0.2048, 3: 0.0512}[d]
+    dx = 1.0 / N[0]
+    dt = eps * dx * dx / nu
+    prob = W.FourierProblem.random(d, nu, 6, 3, 0.05, 1.5, 4)
+    th0 = prob.theta(N, dx)
+    shape = (d,) + tuple(reversed(N))
+    g = rng.standard_normal(shape) * 2.0 ** rng.integers(-40, 1, size=shape)
+    g[rng.random(shape) < 0.2] = 0.0
+    m = O.Model(d, N, nu, dx, dt)
+    # the oracle's loss is 1/2 |u - target|^2: its gradient seed is u(T) - target
+    u = m.recover(m.run(m.initialize(th0), T))[2]
+    _, go, dnuo = m.adjoint(th0, u - g, T)
+    s = lb.Solver(d, N, nu, dx, dt)
+    a = lb.Adjoint(s, T, want_nu=True)
+    a.forward(torch.from_numpy(th0).cuda())
+    a.seed(torch.from_numpy(np.ascontiguousarray(g)).cuda())
+    a.step(T)
+    g0, dnu = a.result()
+    scale = np.max(np.abs(go))
+    # u - (u - g) in the oracle's own seed rounds g at 2^-53 of u
+    assert np.max(np.abs(g0.cpu().numpy() - go)) <= 1e-12 * scale + 1e-12 * np.max(np.abs(u)) * scale / np.max(np.abs(g))
+    assert abs(dnu - dnuo) <= 1e-11 * max(abs(dnuo), 1e-30) + 1e-12 * np.sum(np.abs(g * u)) / nu
+    a.close()
+    s.close()
