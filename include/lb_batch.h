@@ -10,7 +10,7 @@
  * array and 2*N0_j*N1_j (x component first) to a vector array; offsets are
  * the prefix sums of N0_j*N1_j.
  *
- * Scheduling, two kinds:
+ * Scheduling, three kinds:
  *  - one launch per step: instances are bin-packed (largest first) into
  *    groups whose two state buffers fit a byte budget chosen to stay
  *    resident in L2; a group runs all requested steps back to back (each
@@ -20,9 +20,13 @@
  *    halo into shared memory, runs K steps there (the halo shrinking by one
  *    node per step) and stores the tile, so HBM is read and written once per
  *    K steps instead of every step.  Blocks never wait on one another.
- * Either way the launches are recorded once into CUDA graphs and replayed,
- * and every instance evolves bit for bit as the same grid would alone.
- * lb_batch_autotune times both kinds (budgets, block sizes, steps per
+ *  - marching: each launch advances every instance two to five steps; a block
+ *    marches a window of columns of one instance along its rows with the steps
+ *    as pipeline stages.  A new batch takes these launches by itself where the
+ *    batch is large enough for them to pay.
+ * The launches of the first two kinds are recorded once into CUDA graphs and
+ * replayed; every instance evolves bit for bit as the same grid would alone.
+ * lb_batch_autotune times all kinds (budgets, block sizes, steps per
  * launch, tile sizes) on the caller's batch and keeps the fastest.
  */
 #ifndef LB_BATCH_H
@@ -122,8 +126,9 @@ lb_status lb_batch_set_blocking(lb_batch *b, int steps_per_launch, int tile, int
  */
 lb_status lb_batch_set_schedule(lb_batch *b, double budget_bytes, int threads, int use_graph);
 
-/* Current schedule (host, 7 values): {budget_bytes, threads_per_block, groups, total nodes, steps per launch
- * (0: one launch per step), tile edge, tiles}. */
+/* Current schedule as set or tuned (host, 7 values): {budget_bytes, threads_per_block, groups, total nodes, steps per
+ * launch (0: one launch per step, or marching launches the batch took by itself), tile edge (marching: columns per
+ * window), tiles (marching: blocks)}. */
 lb_status lb_batch_schedule(const lb_batch *b, double *info);
 
 const char *lb_batch_last_error(const lb_batch *b);

@@ -493,8 +493,15 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
                 for (int th : {256, 512, 1024}) cands.push_back({lbk::kSchedTiles, K, tile, th});
             }
         }
+    if (c->precision == LB_FP64) {
+        // the trials step whatever the buffers hold: one normal double everywhere
+        // (0x3f3f...), whose collisions take the integer form as a run's do
+        const size_t bytes = (size_t)c->q * c->geom.slab * c->elem;
+        for (void *p : c->f)
+            if ((e = cudaMemsetAsync(p, 0x3f, bytes, c->stream)) != cudaSuccess) return cuda_fail(c, e, "lb_autotune: fill");
+    }
     const bool was_init = c->initialized;
-    c->initialized = true;  // the trials step whatever the buffers hold
+    c->initialized = true;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(c, LB_ECUDA, "lb_autotune: events");

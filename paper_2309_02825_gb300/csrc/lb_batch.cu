@@ -22,23 +22,6 @@
 
 namespace lbk {
 
-// Collision constants of a storage type: floating point, or 64-bit fixed point.
-template <typename T> struct CollOf {
-    using type = Coll<T>;
-};
-template <> struct CollOf<double> {
-    using type = CollF64;
-};
-template <> struct CollOf<long long> {
-    using type = CollFx;
-};
-
-template <typename T> struct InstDesc {
-    Geom g;
-    typename CollOf<T>::type k;
-    int64_t off;  // element offset of the instance's state in each buffer
-};
-
 constexpr int kBatchMaxThreads = 512;
 
 template <class L, typename T>
@@ -408,6 +391,15 @@ struct lb_batch {
     int ntiles = 0, tb_maxw = 0, tb_maxh = 0;  // tile count, largest tile (without halo)
     lbk::TileDesc *d_tiles = nullptr;
     cudaGraphExec_t tb_graph[2] = {nullptr, nullptr};  // kTbGraphLaunches blocked launches, by starting buffer
+    // marching launches (lb_march.cu): mv the variant, m_steps steps per launch, 0 = none; m_auto: the
+    // library's own choice rather than the autotuner's
+    int mv = 0, m_steps = 0, m_threads = 0, m_cols = 0, m_blocks = 0;
+    bool m_auto = false;
+    lbk::MarchBlock *d_march = nullptr;
+    // one launch for all instances' initialisation and recovery: the table, whether the constants have
+    // changed since it was uploaded, and whether they all admit the batched initialisation
+    lbk::BatchInst *d_inst = nullptr;
+    bool inst_stale = true, inst_ok = false;
     bool initialized = false;
     std::string err;
 };
@@ -450,15 +442,65 @@ void free_tiles(lb_batch *b)
     b->tb_k = 0;
 }
 
+void free_march(lb_batch *b)
+{
+    cudaFree(b->d_march);
+    b->d_march = nullptr;
+    b->m_steps = b->m_blocks = 0;
+    b->m_auto = false;
+}
+
+// Bring the table of initialisation and recovery constants up to date (stream order).
+cudaError_t upload_inst(lb_batch *b)
+{
+    if (!b->inst_stale) return cudaSuccess;
+    std::vector<lbk::BatchInst> h(b->count);
+    bool ok = true;
+    for (int j = 0; j < b->count; ++j) ok = lbk::make_batch_inst(&b->inst[j], b->off[j], &h[j]) && ok;
+    // (from pageable memory: the source has been read when the call returns)
+    const cudaError_t e = cudaMemcpyAsync(b->d_inst, h.data(), sizeof(lbk::BatchInst) * b->count, cudaMemcpyHostToDevice,
+                                          b->stream);
+    if (e != cudaSuccess) return e;
+    b->inst_ok = ok;
+    b->inst_stale = false;
+    return cudaSuccess;
+}
+
+// Take marching launches of variant `v` (tables of the blocks).
+cudaError_t build_march(lb_batch *b, int v, bool own)
+{
+    free_march(b);
+    int sms = 148;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
+    if (e != cudaSuccess) return e;
+    std::vector<lbk::MarchBlock> blocks;
+    int steps, threads, cols;
+    lbk::march_batch_plan(b->inst.data(), b->count, b->precision, v, sms, &blocks, &steps, &threads, &cols);
+    if (blocks.empty() || blocks.size() > 0x7fffffff) return cudaSuccess;
+    if ((e = cudaMalloc(&b->d_march, sizeof(lbk::MarchBlock) * blocks.size())) != cudaSuccess ||
+        (e = cudaMemcpy(b->d_march, blocks.data(), sizeof(lbk::MarchBlock) * blocks.size(), cudaMemcpyHostToDevice)) !=
+            cudaSuccess)
+        return e;
+    b->mv = v;
+    b->m_steps = steps;
+    b->m_threads = threads;
+    b->m_cols = cols;
+    b->m_blocks = (int)blocks.size();
+    b->m_auto = own;
+    return cudaSuccess;
+}
+
 void free_batch(lb_batch *b)
 {
     if (!b) return;
     free_groups(b);
     free_tiles(b);
+    free_march(b);
     cudaFree(b->buf[0]);
     cudaFree(b->buf[1]);
     cudaFree(b->d_desc);
     cudaFree(b->d_node_off);
+    cudaFree(b->d_inst);
     cudaFree(b->d_err);
     cudaFree(b->d_flag);
     cudaFree(b->gradtmp);
@@ -585,6 +627,16 @@ lb_status build_tiles(lb_batch *b, int K, int tile, int threads)
     return LB_OK;
 }
 
+// Whether a new batch takes marching launches over one launch per step.
+// Measured GLUPS, march / one launch per step in 96 MB groups, by total nodes:
+//   FP32: 21.4M 230 / 90, 3.8M 178 / 93, 0.65M 129 / 73, 0.41M 89 / 63, 0.05M 12.6 / 10.4
+//   fixed point: 21.4M 108 / 43, 3.8M 92 / 44, 0.65M 55 / 42, 0.41M 54 / 41, 0.05M 8.6 / 10.2
+//   FP64: 21.4M 45 / 20, 3.8M 41 / 21, 0.65M 26 / 15, 0.41M 20 / 15, 0.05M 2.9 / 6.3
+bool march_worth(const lb_batch *b)
+{
+    return b->total_nodes >= (b->precision == LB_FP32_SHIFTED ? 40000 : (b->precision == LB_FX64 ? 200000 : 350000));
+}
+
 // Record kTbGraphLaunches blocked launches of tb_k steps starting from buffer `from`.
 cudaError_t record_tb_graph(lb_batch *b, int from)
 {
@@ -686,6 +738,14 @@ cudaError_t record_graph(lb_batch *b, Group &g, int from)
 cudaError_t run_steps(lb_batch *b, int64_t n)
 {
     cudaError_t e = cudaSuccess;
+    if (b->m_steps > 0) {  // marching launches; the remainder below, one launch per step
+        for (; n >= b->m_steps; n -= b->m_steps) {
+            e = lbk::march_batch_launch(b->precision, b->mv, b->d_desc, b->d_march, b->m_blocks, b->buf[b->cur],
+                                        b->buf[b->cur ^ 1], b->stream);
+            if (e != cudaSuccess) return e;
+            b->cur ^= 1;
+        }
+    }
     if (b->tb_k > 0) {
         // blocked: launches of tb_k steps (recorded in graphs), then one launch for the remainder
         int64_t launches = n / b->tb_k;
@@ -885,6 +945,7 @@ lb_status lb_batch_create(int count, const int64_t *N, const double *nu, const d
     if (e == cudaSuccess) e = cudaMalloc(&b->d_node_off, sizeof(int64_t) * (count + 1));
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_node_off, b->node_off.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_inst, sizeof(lbk::BatchInst) * count);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(double) * 4 * count);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_flag, sizeof(int) * 2);
     if (e != cudaSuccess) {
@@ -900,6 +961,10 @@ lb_status lb_batch_create(int count, const int64_t *N, const double *nu, const d
     if (st != LB_OK) {
         free_batch(b);
         return st;
+    }
+    if (march_worth(b) && (e = build_march(b, 0, true)) != cudaSuccess) {
+        free_batch(b);
+        return e == cudaErrorMemoryAllocation ? LB_ENOMEM : LB_ECUDA;
     }
     *out = b;
     return LB_OK;
@@ -920,6 +985,7 @@ lb_status lb_batch_set_theta_ref(lb_batch *b, const double *tr)
         if (!isfinite(tr[j])) return bfail(b, LB_EINVAL, "lb_batch_set_theta_ref: non-finite value");
         b->inst[j].theta_ref = tr[j];
     }
+    b->inst_stale = true;
     return LB_OK;
 }
 
@@ -954,8 +1020,11 @@ lb_status lb_batch_set_theta0(lb_batch *b, const double *theta0, const double *g
             if (b->inst[j].fx_bits > 1000 || b->inst[j].fx_bits < -1000)
                 return bfail(b, LB_EINVAL, "lb_batch_set_theta0: theta0 magnitude outside the fixed-point range");
         }
+        b->inst_stale = true;
     }
     b->cur = 0;
+    if ((e = upload_inst(b)) != cudaSuccess) return bcuda(b, e, "lb_batch_set_theta0: constants");
+    const bool all = b->inst_ok;  // one launch for all instances
     for (int j = 0; j < b->count; ++j) {
         lb_ctx &c = b->inst[j];
         c.cur = 0;
@@ -963,9 +1032,12 @@ lb_status lb_batch_set_theta0(lb_batch *b, const double *theta0, const double *g
         const double *gr = grad0 ? grad0 + 2 * b->node_off[j] : b->gradtmp + 2 * b->node_off[j];
         if (!grad0 && (e = lbk::launch_fd4_grad(&c, th, const_cast<double *>(gr))) != cudaSuccess)
             return bcuda(b, e, "lb_batch_set_theta0: fd4");
-        if ((e = lbk::launch_init(&c, th, gr, b->d_flag)) != cudaSuccess)
+        if (!all && (e = lbk::launch_init(&c, th, gr, b->d_flag)) != cudaSuccess)
             return bcuda(b, e, "lb_batch_set_theta0: init");
     }
+    if (all && (e = lbk::launch_batch_init(b->precision, b->d_node_off, b->count, b->total_nodes, b->d_inst, b->buf[0], theta0,
+                                           grad0 ? grad0 : b->gradtmp, b->d_flag, b->stream)) != cudaSuccess)
+        return bcuda(b, e, "lb_batch_set_theta0: init");
     int flag = 0;
     if ((e = cudaMemcpyAsync(&flag, b->d_flag, sizeof(int), cudaMemcpyDeviceToHost, b->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(b->stream)) != cudaSuccess)
@@ -993,6 +1065,19 @@ lb_status lb_batch_macros(lb_batch *b, double *theta, double *u)
     lbk::NvtxRange nvtx_range("lb_batch_macros");
     if (!b) return LB_EINVAL;
     if (!b->initialized) return bfail(b, LB_ESTATE, "lb_batch_macros: call lb_batch_set_theta0 first");
+    if (b->inst_stale) {  // lb_batch_set_theta_ref since: not inside the caller's capture, which would keep the copy
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(b->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+            const cudaError_t e = upload_inst(b);
+            if (e != cudaSuccess) return bcuda(b, e, "lb_batch_macros: constants");
+        }
+    }
+    if (!b->inst_stale) {
+        const cudaError_t e = lbk::launch_batch_recover(b->precision, b->d_node_off, b->count, b->total_nodes, b->d_inst,
+                                                        b->buf[b->cur], theta, u, b->d_flag + 1, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "lb_batch_macros");
+        return LB_OK;
+    }
     for (int j = 0; j < b->count; ++j) {
         lb_ctx &c = b->inst[j];
         c.cur = b->cur;
@@ -1035,13 +1120,16 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, double *choice)
     // (b) blocked launches: K steps per launch x tile edge (the largest that
     // fits one, two, three or four blocks per SM with a K-node halo, and that
     // edge less 4) x block size.
+    // (c) marching windows, each variant of the storage type.
     struct Cand {
         double budget;
-        int threads, K, tile;
+        int threads, K, tile, march;  // march: variant + 1, 0 none
     };
     std::vector<Cand> cands;
+    free_march(b);
+    for (int v = 0; v < lbk::march_batch_variants(b->precision); ++v) cands.push_back({b->budget, b->threads, 0, 0, v + 1});
     for (double bud : {48e6, 96e6, 128e6, 1e18})
-        for (int th : {64, 128, 256, 512}) cands.push_back({bud, th, 0, 0});
+        for (int th : {64, 128, 256, 512}) cands.push_back({bud, th, 0, 0, 0});
     int optin = 0;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device) != cudaSuccess)
         return bfail(b, LB_ECUDA, "lb_batch_autotune: device attribute");
@@ -1053,24 +1141,40 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, double *choice)
             // that tile, and one 4 nodes smaller (less work per block)
             for (int tile : {edge - 2 * K, edge - 2 * K - 4}) {
                 if (tile < 8) continue;
-                for (int th : {256, 512, 1024}) cands.push_back({b->budget, th, K, tile});
+                for (int th : {256, 512, 1024}) cands.push_back({b->budget, th, K, tile, 0});
             }
         }
+    if (b->precision == LB_FP64) {
+        // the trials step whatever the buffers hold: one normal double everywhere
+        // (0x3f3f...), whose collisions take the integer form as a run's do
+        const size_t bytes = b->elem * (size_t)b->total_elems;
+        for (void *p : b->buf)
+            if (cudaMemsetAsync(p, 0x3f, bytes, b->stream) != cudaSuccess) return bfail(b, LB_ECUDA, "lb_batch_autotune: fill");
+    }
     double best = 1e300;
-    Cand win = {b->budget, b->threads, b->tb_k, b->tb_tile};
+    Cand win = {b->budget, b->threads, b->tb_k, b->tb_tile, 0};
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return bfail(b, LB_ECUDA, "lb_batch_autotune: events");
     lb_status st = LB_OK;
     for (const Cand &cd : cands) {
-        if (cd.K == 0) {
+        free_march(b);  // (the stream is idle here)
+        if (cd.march) {
+            const cudaError_t em = build_march(b, cd.march - 1, false);
+            if (em != cudaSuccess) {
+                st = bcuda(b, em, "lb_batch_autotune");
+                break;
+            }
+            if (b->m_steps == 0) continue;
+        } else if (cd.K == 0) {
             if ((st = build_tiles(b, 0, 0, 0)) != LB_OK || (st = build_schedule(b, cd.budget, cd.threads, true)) != LB_OK)
                 break;
         } else if ((st = build_tiles(b, cd.K, cd.tile, cd.threads)) != LB_OK) {
             st = LB_OK;  // a tile that does not fit this device is skipped
             continue;
         }
-        const int64_t n = cd.K ? (trial_steps + cd.K - 1) / cd.K * cd.K : trial_steps;
+        const int64_t per = cd.march ? b->m_steps : (cd.K ? cd.K : 1);
+        const int64_t n = (trial_steps + per - 1) / per * per;
         cudaError_t e = run_steps(b, n);  // warm-up: records the graphs, fills L2
         if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
         if (e == cudaSuccess) e = run_steps(b, n);
@@ -1090,10 +1194,15 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, double *choice)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    free_march(b);
     if (st != LB_OK) return st;
     b->initialized = false;  // the trials overwrote the state
     if (cudaStreamSynchronize(b->stream) != cudaSuccess) return bfail(b, LB_ECUDA, "lb_batch_autotune: sync");
-    if (win.K == 0) {
+    if (win.march) {
+        if ((st = build_tiles(b, 0, 0, 0)) != LB_OK) return st;
+        const cudaError_t em = build_march(b, win.march - 1, false);
+        if (em != cudaSuccess) return bcuda(b, em, "lb_batch_autotune");
+    } else if (win.K == 0) {
         if ((st = build_tiles(b, 0, 0, 0)) != LB_OK) return st;
         if ((st = build_schedule(b, win.budget, win.threads, true)) != LB_OK) return st;
     } else if ((st = build_tiles(b, win.K, win.tile, win.threads)) != LB_OK) {
@@ -1101,11 +1210,11 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, double *choice)
     }
     if (choice) {
         choice[0] = b->budget;
-        choice[1] = win.K ? win.threads : b->threads;
+        choice[1] = win.march ? b->m_threads : (win.K ? win.threads : b->threads);
         choice[2] = (double)b->groups.size();
         choice[3] = 1e3 * best;
-        choice[4] = win.K;
-        choice[5] = win.tile;
+        choice[4] = win.march ? b->m_steps : win.K;
+        choice[5] = win.march ? b->m_cols : win.tile;
     }
     return LB_OK;
 }
@@ -1117,6 +1226,7 @@ lb_status lb_batch_set_schedule(lb_batch *b, double budget, int threads, int use
     cudaError_t e = cudaStreamSynchronize(b->stream);  // tables in use by queued launches
     if (e != cudaSuccess) return bcuda(b, e, "lb_batch_set_schedule");
     free_tiles(b);
+    free_march(b);
     return build_schedule(b, budget, threads, use_graph != 0);
 }
 
@@ -1126,7 +1236,8 @@ lb_status lb_batch_set_blocking(lb_batch *b, int steps_per_launch, int tile, int
     if (steps_per_launch < 0 || steps_per_launch > 64 || (steps_per_launch > 0 && (tile < 1 || tile > 4096)) ||
         (steps_per_launch > 0 && !(threads == 256 || threads == 512 || threads == 1024)))
         return bfail(b, LB_EINVAL, "lb_batch_set_blocking: steps per launch in 0..64, tile >= 1, threads 256, 512 or 1024");
-    lb_status st = build_tiles(b, steps_per_launch, tile, threads);
+    lb_status st = build_tiles(b, steps_per_launch, tile, threads);  // (synchronises the stream)
+    free_march(b);
     if (st == LB_OK) b->use_graph = use_graph != 0;
     return st;
 }
@@ -1135,12 +1246,13 @@ lb_status lb_batch_schedule(const lb_batch *b, double *info)
 {
     if (!b || !info) return LB_EINVAL;
     info[0] = b->budget;
-    info[1] = b->tb_k ? b->tb_threads : b->threads;
+    const bool march = b->m_steps > 0 && !b->m_auto;
+    info[1] = march ? b->m_threads : (b->tb_k ? b->tb_threads : b->threads);
     info[2] = (double)b->groups.size();
     info[3] = (double)b->total_nodes;
-    info[4] = b->tb_k;
-    info[5] = b->tb_k ? b->tb_tile : 0;
-    info[6] = b->ntiles;
+    info[4] = march ? b->m_steps : b->tb_k;
+    info[5] = march ? b->m_cols : (b->tb_k ? b->tb_tile : 0);
+    info[6] = march ? b->m_blocks : b->ntiles;
     return LB_OK;
 }
 

@@ -22,6 +22,30 @@ __device__ __forceinline__ void static_for(F &&f)
 
 __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
+// The instance of node n in the concatenated numbering of a batch (node_off:
+// count + 1 prefix sums), -1 past the last node.  One thread searches for the
+// block's first node; the others step on from there.  Called by whole blocks.
+__device__ __forceinline__ int batch_instance(const int64_t *__restrict__ node_off, int count, int64_t n)
+{
+    __shared__ int first;
+    if (threadIdx.x == 0) {
+        int lo = 0, hi = count - 1;  // the last instance that starts at or before n
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (node_off[mid] <= n)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        first = lo;
+    }
+    __syncthreads();
+    if (n >= node_off[count]) return -1;
+    int j = first;
+    while (n >= node_off[j + 1]) ++j;
+    return j;
+}
+
 __device__ __forceinline__ void ld_vec(const double *p, double (&a)[2])
 {
     double2 v = __ldg(reinterpret_cast<const double2 *>(p));
@@ -847,6 +871,28 @@ __device__ __forceinline__ bool f64_align(const double (&f)[Q], long long (&v)[Q
     return sum < 0x3fffffc0u;
 }
 
+// The same for values of any spread: bits below 2^-(53 + PB) of the largest are
+// rounded to nearest.  False where the largest is zero, subnormal, not finite or
+// at the ends of the range.
+template <int Q, int PB>
+__device__ __forceinline__ bool f64_align_round(const double (&f)[Q], long long (&v)[Q], unsigned &emax)
+{
+    unsigned mx = 0u;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) mx = max(mx, (unsigned)__double2hiint(f[i]) & 0x7ff00000u);
+    emax = mx >> 20;
+    if (mx - (100u << 20) > (1900u << 20)) return false;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
+        const unsigned e = (hi >> 20) & 0x7ffu, sh = min(emax - e, 62u);
+        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32 | lo) << PB;
+        const long long r = (long long)((m + ((1ull << sh) >> 1)) >> sh);
+        v[i] = (int)hi < 0 ? -r : r;
+    }
+    return true;
+}
+
 template <class L> __device__ __forceinline__ void collide(L, double *f, const CollF64 &k)
 {
     constexpr int Q = L::Q, PB = f64_align_bit<L>(), B0 = 1 + 2 * L::D;
@@ -871,28 +917,6 @@ template <class L> __device__ __forceinline__ void collide(L, double *f, const C
 
 // A double rounded to float (to nearest, ties to even) on the integer pipes;
 // results outside the normal floats by the hardware conversion.
-// The same for values of any spread: bits below 2^-(53 + PB) of the largest are
-// rounded to nearest.  False where the largest is zero, subnormal, not finite or
-// at the ends of the range.
-template <int Q, int PB>
-__device__ __forceinline__ bool f64_align_round(const double (&f)[Q], long long (&v)[Q], unsigned &emax)
-{
-    unsigned mx = 0u;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) mx = max(mx, (unsigned)__double2hiint(f[i]) & 0x7ff00000u);
-    emax = mx >> 20;
-    if (mx - (100u << 20) > (1900u << 20)) return false;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const unsigned hi = (unsigned)__double2hiint(f[i]), lo = (unsigned)__double2loint(f[i]);
-        const unsigned e = (hi >> 20) & 0x7ffu, sh = min(emax - e, 62u);
-        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32 | lo) << PB;
-        const long long r = (long long)((m + ((1ull << sh) >> 1)) >> sh);
-        v[i] = (int)hi < 0 ? -r : r;
-    }
-    return true;
-}
-
 __device__ __forceinline__ float f64_to_f32_rn(double v)
 {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);

@@ -15,6 +15,7 @@
 
 #include <string>
 #include <type_traits>
+#include <vector>
 
 #include "../../include/lb.h"
 
@@ -212,6 +213,39 @@ struct MarchPlan {
     int threads;        // per block
 };
 
+// Collision constants of a batched instance by storage type.
+template <typename T> struct CollOf {
+    using type = Coll<T>;
+};
+template <> struct CollOf<double> {
+    using type = CollF64;
+};
+template <> struct CollOf<long long> {
+    using type = CollFx;
+};
+
+// One instance of a batch, or one grid launched as such.
+template <typename T> struct InstDesc {
+    Geom g;
+    typename CollOf<T>::type k;
+    int64_t off;  // element offset of the instance's state in each buffer
+};
+
+// What a batched instance's initialisation and recovery need.
+struct BatchInst {
+    Geom g;
+    InitK init;
+    Recov rec;
+    double scale;
+    int64_t off;  // element offset of the instance's state in each buffer
+};
+
+// One block of a batched marching launch: a window of nx columns from x0 and a
+// chunk of nr rows from r0 of an instance.
+struct MarchBlock {
+    int inst, x0, nx, r0, nr;
+};
+
 // How lb_step runs its sweeps.
 enum Sched {
     kSchedAuto = 0,    // the library's own rule (choose_schedule)
@@ -333,6 +367,23 @@ void blocked_release(lb_ctx *c);
 // one sweep per launch, and one launch of plan.steps steps.
 cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth);
 cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s);
+// The same for batched 2D instances: variants of a storage type (the first is
+// the default), the blocks of a launch over `count` instances with the steps,
+// threads and columns per window of the variant, and one launch.
+int march_batch_variants(int precision);
+void march_batch_plan(const lb_ctx *inst, int count, int precision, int variant, int sms, std::vector<MarchBlock> *blocks,
+                      int *steps, int *threads, int *cols);
+cudaError_t march_batch_launch(int precision, int variant, const void *desc, const MarchBlock *blocks, int n,
+                               const void *src, void *dst, cudaStream_t s);
+// All instances of a batch in one launch each (node_off: count + 1 prefix sums
+// of the nodes, device).  make_batch_inst is false for constants that the
+// batched fixed-point initialisation does not serve (then one launch each).
+Recov make_recov(const lb_ctx *c, double *scale);
+bool make_batch_inst(const lb_ctx *c, int64_t off, BatchInst *out);
+cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
+                              void *dst, const double *theta0, const double *grad, int *flag, cudaStream_t s);
+cudaError_t launch_batch_recover(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
+                                 const void *src, double *theta, double *u, int *flag, cudaStream_t s);
 // Resident sweeps of a short 1D grid (lb_line.cu): whether it is one, and one
 // launch of any number of steps.
 bool line_fits(const lb_ctx *c);

@@ -77,14 +77,11 @@ __device__ __forceinline__ long long fx_round(double v, int F, bool &range)
 constexpr int kInitThreads = 128;
 
 template <class L, typename T, int FXI, bool MIR>
-__global__ void __launch_bounds__(kInitThreads) init_kernel(T *__restrict__ dst, Geom g, InitK K,
-                                                            const double *__restrict__ theta0,
-                                                            const double *__restrict__ grad, int *__restrict__ flag)
+__device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, const InitK &K, int64_t node, int64_t nodes,
+                                          const double *__restrict__ theta0, const double *__restrict__ grad,
+                                          int *__restrict__ flag)
 {
-    constexpr int D = L::D, Q = L::Q, B0 = 1 + 2 * D;
-    const int64_t nodes = (int64_t)g.N0 * g.rows;
-    const int64_t node = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
-    if (node >= nodes) return;
+    constexpr int D = L::D, B0 = 1 + 2 * D;
     // coordinates in 32-bit arithmetic (nodes <= 2^31)
     const unsigned nd = (unsigned)node;
     int c[4];
@@ -227,6 +224,31 @@ __global__ void __launch_bounds__(kInitThreads) init_kernel(T *__restrict__ dst,
         });
     }
     if (range) atomicOr(flag, 2);
+}
+
+template <class L, typename T, int FXI, bool MIR>
+__global__ void __launch_bounds__(kInitThreads) init_kernel(T *__restrict__ dst, Geom g, InitK K,
+                                                            const double *__restrict__ theta0,
+                                                            const double *__restrict__ grad, int *__restrict__ flag)
+{
+    const int64_t nodes = (int64_t)g.N0 * g.rows;
+    const int64_t node = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
+    if (node < nodes) init_node<L, T, FXI, MIR>(dst, g, K, node, nodes, theta0, grad, flag);
+}
+
+// All instances of a batch in one launch (batch_instance finds a node's own).
+template <typename T, int FXI>
+__global__ void __launch_bounds__(kInitThreads) batch_init_kernel(const int64_t *__restrict__ node_off, int count,
+                                                                  const BatchInst *__restrict__ inst, T *__restrict__ dst,
+                                                                  const double *__restrict__ theta0,
+                                                                  const double *__restrict__ grad, int *__restrict__ flag)
+{
+    const int64_t n = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
+    const int j = batch_instance(node_off, count, n);
+    if (j < 0) return;
+    const int64_t n0 = node_off[j];
+    const BatchInst &d = inst[j];
+    init_node<D2Q9, T, FXI, false>(dst + d.off, d.g, d.init, n - n0, node_off[j + 1] - n0, theta0 + n0, grad + 2 * n0, flag);
 }
 
 // Fourth-order central difference of theta along each axis: periodic, or,
@@ -613,10 +635,10 @@ static cudaError_t init_go(lb_ctx *c, const InitK &K, const double *theta0, cons
     return cudaGetLastError();
 }
 
-template <class L, typename T>
-static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, int *flag)
+// The constants of a context's initialisation and the formation they admit
+// (FXI of init_node; 0 but for fixed point).
+static int make_initk(const lb_ctx *c, InitK &K)
 {
-    InitK K;
     const double d = c->d;
     const double wd = (c->d > 1) ? c->wd : 0.0;
     K.w0 = c->w0;
@@ -629,22 +651,53 @@ static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, i
     K.gscale = c->dx * K.fxscale;
     K.fx_bits = c->fx_bits;
     K.w1k = K.wdk = K.iak = 0;
+    if (c->precision != LB_FX64) return 0;
+    // integer formation needs every constant inside the product's range and a
+    // total weight that keeps the rest population's sum below 2^61
+    const double ia = K.iax / c->dx;
+    const double wmass = fabs(c->w0) + 2.0 * d * fabs(c->w1) + 2.0 * d * (d - 1.0) * fabs(wd);
+    if (!(fabs(ia) < 1.5 && fabs(c->w1) < 1.0 && fabs(wd) < 1.0 && wmass <= 4.0)) return 0;
+    const double most = 0.5 - 0x1p-30;  // mulfx_c's range
+    const bool split = fabs(ia) < most && fabs(c->w1) < most && fabs(wd) < most;
+    const int bits = split ? kFxCollBits : kFxCoefBits;
+    K.w1k = llrint(ldexp(c->w1, bits));
+    K.wdk = llrint(ldexp(wd, bits));
+    K.iak = llrint(ldexp(ia, bits));
+    return split ? 2 : 1;
+}
+
+template <class L, typename T>
+static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, int *flag)
+{
+    InitK K;
+    const int fxi = make_initk(c, K);
     if constexpr (std::is_same<T, long long>::value) {
-        // integer formation needs every constant inside the product's range and
-        // a total weight that keeps the rest population's sum below 2^61
-        const double ia = K.iax / c->dx;
-        const double wmass = fabs(c->w0) + 2.0 * d * fabs(c->w1) + 2.0 * d * (d - 1.0) * fabs(wd);
-        if (fabs(ia) < 1.5 && fabs(c->w1) < 1.0 && fabs(wd) < 1.0 && wmass <= 4.0) {
-            const double most = 0.5 - 0x1p-30;  // mulfx_c's range
-            const bool split = fabs(ia) < most && fabs(c->w1) < most && fabs(wd) < most;
-            const int bits = split ? kFxCollBits : kFxCoefBits;
-            K.w1k = llrint(ldexp(c->w1, bits));
-            K.wdk = llrint(ldexp(wd, bits));
-            K.iak = llrint(ldexp(ia, bits));
-            return split ? init_go<L, T, 2>(c, K, theta0, grad, flag) : init_go<L, T, 1>(c, K, theta0, grad, flag);
-        }
+        if (fxi == 2) return init_go<L, T, 2>(c, K, theta0, grad, flag);
+        if (fxi == 1) return init_go<L, T, 1>(c, K, theta0, grad, flag);
     }
     return init_go<L, T, 0>(c, K, theta0, grad, flag);
+}
+
+bool make_batch_inst(const lb_ctx *c, int64_t off, BatchInst *out)
+{
+    out->g = c->geom;
+    out->off = off;
+    const int fxi = make_initk(c, out->init);
+    out->rec = make_recov(c, &out->scale);
+    return c->precision != LB_FX64 || fxi == 2;
+}
+
+cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
+                              void *dst, const double *theta0, const double *grad, int *flag, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((nodes + kInitThreads - 1) / kInitThreads);
+    if (precision == LB_FX64)
+        batch_init_kernel<long long, 2><<<nb, kInitThreads, 0, s>>>(node_off, count, inst, (long long *)dst, theta0, grad, flag);
+    else if (precision == LB_FP32_SHIFTED)
+        batch_init_kernel<float, 0><<<nb, kInitThreads, 0, s>>>(node_off, count, inst, (float *)dst, theta0, grad, flag);
+    else
+        batch_init_kernel<double, 0><<<nb, kInitThreads, 0, s>>>(node_off, count, inst, (double *)dst, theta0, grad, flag);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, int *flag)

@@ -97,28 +97,18 @@ template <class L, int KS, int TH> constexpr size_t march_smem(int elem)
 // The branch is block-uniform, but ends a scheduling region; where the
 // collisions are short (3D float) that costs more than the idle work (256^3:
 // 78 against 66 GLUPS), elsewhere less (1024^2 fixed point 76 against 66).
-template <class L, typename T, class K, int KS, int TH, int MINB, bool SKIP>
-__global__ void __launch_bounds__(TH, MINB) march_kernel(const T *__restrict__ src, T *__restrict__ dst, Geom g, K k,
-                                                         MarchPlan p)
+template <class L, typename T, class K, int KS, int TH, bool SKIP>
+__device__ __forceinline__ void march_body(const T *__restrict__ src, T *__restrict__ dst, const Geom &g, const K &k,
+                                           int x0, int nx, int y0, int ny, int r0, int nr)
 {
-    constexpr int D = L::D, Q = L::Q, A = D - 1, S = MarchL<L>::kSlots, E = (int)sizeof(T);
+    constexpr int D = L::D, Q = L::Q, A = D - 1, S = MarchL<L>::kSlots;
     constexpr int IM = MarchL<L>::pick(-1), IC = MarchL<L>::pick(0), IP = MarchL<L>::pick(1);
     extern __shared__ __align__(16) unsigned char march_raw[];
     T *const sm = reinterpret_cast<T *>(march_raw);
     const int tid = threadIdx.x;
-
-    // the window and chunk of this block
-    unsigned b = blockIdx.x;
-    const int wx = (int)(b % (unsigned)p.nx);
-    b /= (unsigned)p.nx;
-    const int wy = D == 3 ? (int)(b % (unsigned)p.ny) : 0;
-    const int ch = D == 3 ? (int)(b / (unsigned)p.ny) : (int)b;
     const int NR = D == 3 ? g.N2 : g.N1;  // rows of the march
     constexpr int bw = D == 3 ? kMarchW : TH;
     const int cx = D == 3 ? tid % bw : tid, cy = D == 3 ? tid / bw : 0;
-    const int x0 = wx * p.bx, y0 = wy * p.by, r0 = ch * p.chunk;
-    const int nx = min(p.bx, g.N0 - x0), nr = min(p.chunk, NR - r0);
-    const int ny = D == 3 ? min(p.by, g.N1 - y0) : 1;
     // stage s is valid on columns s - 1 <= cx < nx + 2 KS - 1 - s (cy likewise): its distance to the window's edge
     int edge = min(cx, nx + 2 * (KS - 1) - 1 - cx);
     if (D == 3) edge = min(edge, min(cy, ny + 2 * (KS - 1) - 1 - cy));
@@ -256,6 +246,32 @@ __global__ void __launch_bounds__(TH, MINB) march_kernel(const T *__restrict__ s
     }
 }
 
+template <class L, typename T, class K, int KS, int TH, int MINB, bool SKIP>
+__global__ void __launch_bounds__(TH, MINB) march_kernel(const T *__restrict__ src, T *__restrict__ dst, Geom g, K k,
+                                                         MarchPlan p)
+{
+    unsigned b = blockIdx.x;
+    const int x0 = (int)(b % (unsigned)p.nx) * p.bx;
+    b /= (unsigned)p.nx;
+    const int y0 = L::D == 3 ? (int)(b % (unsigned)p.ny) * p.by : 0;
+    const int r0 = (L::D == 3 ? (int)(b / (unsigned)p.ny) : (int)b) * p.chunk;
+    const int NR = L::D == 3 ? g.N2 : g.N1;
+    march_body<L, T, K, KS, TH, SKIP>(src, dst, g, k, x0, min(p.bx, g.N0 - x0), y0,
+                                      L::D == 3 ? min(p.by, g.N1 - y0) : 1, r0, min(p.chunk, NR - r0));
+}
+
+// Batched 2D instances: the block's window, chunk and instance from tables.
+template <typename T, int KS, int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) march_batch_kernel(const InstDesc<T> *__restrict__ inst,
+                                                               const MarchBlock *__restrict__ blocks,
+                                                               const T *__restrict__ src, T *__restrict__ dst)
+{
+    const MarchBlock b = blocks[blockIdx.x];
+    const InstDesc<T> d = inst[b.inst];
+    march_body<D2Q9, T, typename CollOf<T>::type, KS, TH, true>(src + d.off, dst + d.off, d.g, d.k, b.x0, b.nx, 0, 1, b.r0,
+                                                                b.nr);
+}
+
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
@@ -376,6 +392,95 @@ cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s)
     }
     if (c->precision == LB_FX64) return March3Fx::launch(c, src, dst, s);
     return March3F::launch(c, src, dst, s);
+}
+
+// ---------------------------------------------------------------------------
+// Batched 2D instances.
+// ---------------------------------------------------------------------------
+template <typename T, int KS, int TH, int MINB> struct MarchB {
+    // Chunks of about `c` rows, c the cheapest by the work of all blocks over the
+    // resident ones plus half a block's own length for the last wave; the
+    // longest blocks first.
+    static void plan(const lb_ctx *inst, int count, int sms, std::vector<MarchBlock> *out, int *steps, int *threads, int *cols)
+    {
+        constexpr int ring = KS - 1;
+        *steps = KS;
+        *threads = TH;
+        *cols = TH - 2 * ring;
+        const double slots = (double)sms * MINB;
+        double least = 1e300;
+        int best = 16;
+        for (int c = 16; c <= 4096; c += c / 2) {
+            double work = 0.0;
+            int longest = 0;
+            for (int j = 0; j < count; ++j) {
+                int nx, bx, nc, ch;
+                cut((int)inst[j].N[0], TH - 2 * ring, nx, bx);
+                cut((int)inst[j].N[1], c, nc, ch);
+                work += (double)nx * nc * (ch + 3 * ring + 4);
+                longest = std::max(longest, ch + 3 * ring + 4);
+            }
+            const double t = std::max(work / slots, 0.7 * longest) + 0.5 * longest;
+            if (t < least) {
+                least = t;
+                best = c;
+            }
+        }
+        out->clear();
+        for (int j = 0; j < count; ++j) {
+            const int n0 = (int)inst[j].N[0], n1 = (int)inst[j].N[1];
+            int nx, bx, nc, ch;
+            cut(n0, TH - 2 * ring, nx, bx);
+            cut(n1, best, nc, ch);
+            for (int r = 0; r < n1; r += ch)
+                for (int x = 0; x < n0; x += bx) out->push_back({j, x, std::min(bx, n0 - x), r, std::min(ch, n1 - r)});
+        }
+        std::stable_sort(out->begin(), out->end(), [](const MarchBlock &a, const MarchBlock &b) { return a.nr > b.nr; });
+    }
+    static cudaError_t launch(const void *desc, const MarchBlock *blocks, int n, const void *src, void *dst, cudaStream_t s)
+    {
+        constexpr size_t smem = march_smem<D2Q9, KS, TH>(sizeof(T));
+        static_assert(smem <= 48 * 1024, "no opt-in needed");
+        march_batch_kernel<T, KS, TH, MINB><<<(unsigned)n, TH, smem, s>>>((const InstDesc<T> *)desc, blocks, (const T *)src,
+                                                                          (T *)dst);
+        return cudaGetLastError();
+    }
+};
+
+// Variant 0 is a new batch's own choice.  Instances of 32 to 512 columns leave
+// fewer of a 64-thread window's columns idle: FP32 21.4M nodes 230 GLUPS
+// against 215 with 128 threads, 0.65M 129 against 112; fixed point about equal.
+template <class F> static void march_batch_pick(int precision, int variant, F &&f)
+{
+    if (precision == LB_FX64) {
+        if (variant == 0)
+            f(MarchB<long long, 3, 64, 10>{});
+        else
+            f(MarchB<long long, 3, 128, 5>{});
+    } else if (precision == LB_FP32_SHIFTED) {
+        if (variant == 0)
+            f(MarchB<float, 5, 64, 10>{});
+        else
+            f(MarchB<float, 5, 128, 5>{});
+    } else {
+        f(MarchB<double, 2, 128, 6>{});
+    }
+}
+
+int march_batch_variants(int precision) { return precision == LB_FP64 ? 1 : 2; }
+
+void march_batch_plan(const lb_ctx *inst, int count, int precision, int variant, int sms, std::vector<MarchBlock> *blocks,
+                      int *steps, int *threads, int *cols)
+{
+    march_batch_pick(precision, variant, [&](auto m) { decltype(m)::plan(inst, count, sms, blocks, steps, threads, cols); });
+}
+
+cudaError_t march_batch_launch(int precision, int variant, const void *desc, const MarchBlock *blocks, int n,
+                               const void *src, void *dst, cudaStream_t s)
+{
+    cudaError_t e = cudaSuccess;
+    march_batch_pick(precision, variant, [&](auto m) { e = decltype(m)::launch(desc, blocks, n, src, dst, s); });
+    return e;
 }
 
 }  // namespace lbk

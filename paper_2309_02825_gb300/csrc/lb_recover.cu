@@ -281,6 +281,60 @@ __global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__
     recover_node<L, T>(vals, r, scale, nodes, n, theta, grad, u, flag);
 }
 
+// All 2D instances of a batch in one launch: the flat recovery of each node's
+// own instance.
+template <typename T>
+__global__ void __launch_bounds__(128) batch_recover_kernel(const int64_t *__restrict__ node_off, int count,
+                                                            const BatchInst *__restrict__ inst, const T *__restrict__ src,
+                                                            double *__restrict__ theta, double *__restrict__ u,
+                                                            int *__restrict__ flag)
+{
+    const int64_t n = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int j = batch_instance(node_off, count, n);
+    if (j < 0) return;
+    const BatchInst &d = inst[j];
+    const Geom &g = d.g;
+    const int64_t n0 = node_off[j];
+    const unsigned nd = (unsigned)(n - n0), row = nd / (unsigned)g.N0;
+    const int x = (int)(nd - row * (unsigned)g.N0);
+    const RowPos rpos = row_pos<2>(g, row);
+    const T *s = src + d.off;
+    const int xs[3] = {x == g.N0 - 1 ? 0 : x + 1, x, x == 0 ? g.N0 - 1 : x - 1};  // x - e by e + 1
+    T vals[D2Q9::Q];
+    static_for<0, D2Q9::Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        constexpr int ex = D2Q9::E[i][0], ey = D2Q9::E[i][1];
+        vals[i] = __ldg(s + (int64_t)i * g.slab + src_row<2, ey, 0, 0>(g, rpos) * g.pitch + xs[1 + ex]);
+    });
+    recover_node<D2Q9, T>(vals, d.rec, d.scale, node_off[j + 1] - n0, nd, theta ? theta + n0 : nullptr, nullptr,
+                          u ? u + 2 * n0 : nullptr, flag);
+}
+
+cudaError_t launch_batch_recover(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
+                                 const void *src, double *theta, double *u, int *flag, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((nodes + 127) / 128);
+    if (precision == LB_FX64)
+        batch_recover_kernel<long long><<<nb, 128, 0, s>>>(node_off, count, inst, (const long long *)src, theta, u, flag);
+    else if (precision == LB_FP32_SHIFTED)
+        batch_recover_kernel<float><<<nb, 128, 0, s>>>(node_off, count, inst, (const float *)src, theta, u, flag);
+    else
+        batch_recover_kernel<double><<<nb, 128, 0, s>>>(node_off, count, inst, (const double *)src, theta, u, flag);
+    return cudaGetLastError();
+}
+
+// Recovery constants of a context; *scale: the storage unit.
+Recov make_recov(const lb_ctx *c, double *scale)
+{
+    Recov r;
+    *scale = (c->precision == LB_FX64) ? ldexp(1.0, -c->fx_bits) : 1.0;
+    // J is summed in storage units: the scale (a power of two, exact) goes into the constants
+    r.ucoef = (2.0 - c->s1) * c->c * *scale;
+    r.gcoef = -c->s1 / (c->sigma * c->dx) * *scale;
+    r.theta_ref = (c->precision == LB_FP32_SHIFTED) ? c->theta_ref : 0.0;
+    return r;
+}
+
 template <class L, typename T, bool MIR>
 static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag, int64_t row0,
                              int64_t nrow)
@@ -291,12 +345,8 @@ static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr,
     cudaError_t e = cudaFuncSetAttribute(recover_kernel<L, T, MIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    Recov r;
-    const double scale = (c->precision == LB_FX64) ? ldexp(1.0, -c->fx_bits) : 1.0;
-    // J is summed in storage units: the scale (a power of two, exact) goes into the constants
-    r.ucoef = (2.0 - c->s1) * c->c * scale;
-    r.gcoef = -c->s1 / (c->sigma * c->dx) * scale;
-    r.theta_ref = (c->precision == LB_FP32_SHIFTED) ? c->theta_ref : 0.0;
+    double scale;
+    const Recov r = make_recov(c, &scale);
     const int64_t tiles = (c->geom.N0 + kTile - 1) / kTile, blocks = nrow * tiles;
     if (blocks == 0) return cudaSuccess;
     if (c->geom.N0 * 4 < tiles * kTile * 3) {  // under three quarters of the tiles' nodes
