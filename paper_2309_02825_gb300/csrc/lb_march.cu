@@ -96,7 +96,7 @@ template <class L, int KS, int TH> constexpr size_t march_smem(int elem)
 // SKIP: a stage outside its rows (the pipeline's fill and drain) does nothing.
 // The branch is block-uniform, but ends a scheduling region; where the
 // collisions are short (3D float) that costs more than the idle work (256^3:
-// 78 against 66 GLUPS), elsewhere less (1024^2 fixed point 76 against 66).
+// 75 against 66 GLUPS), elsewhere less (1024^2 fixed point 76 against 66).
 template <class L, typename T, class K, int KS, int TH, bool SKIP>
 __device__ __forceinline__ void march_body(const T *__restrict__ src, T *__restrict__ dst, const Geom &g, const K &k,
                                            int x0, int nx, int y0, int ny, int r0, int nr)
@@ -289,42 +289,57 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
 
     // The cheapest cut by a model of the launch: full waves of the resident
     // blocks, each as long as its iterations (its rows, the pipeline's fill and
-    // about 4 rows of latency), an iteration taking the time of the resident
-    // blocks' work, or of 0.7 MINB blocks where fewer no longer hide latency.
+    // about 4 rows of latency), an iteration taking the time of the warps at
+    // work, or of 0.7 of a full SM's where fewer no longer hide latency (0.85 of the
+    // one block per SM in 3D).  In 3D also more, lower windows than the rings have
+    // room for, in blocks of fewer warps, where they fill the SMs better
+    // (101 x 90 x 77 FP32: 36 windows of 10 rows by 4 chunks on 152 SMs instead of
+    // 32 of 12, 50 GLUPS against 44).
     // `worth`: enough nodes to fill the chip, and the share of a launch's
     // thread-iterations that end in stored nodes not below least_use.
     static void plan(const lb_ctx *c, int64_t least_nodes, double least_use, MarchPlan *out, bool *worth)
     {
         const Geom &g = c->geom;
-        MarchPlan p{};
-        *out = p;
+        *out = MarchPlan{};
         *worth = false;
         if (g.slab >= (1ll << 30)) return;  // offsets within a population are int
-        const int NR = L::D == 3 ? g.N2 : g.N1;
+        const int NR = L::D == 3 ? g.N2 : g.N1, high = TH / kMarchW;
+        MarchPlan p{};
         p.steps = KS;
-        p.threads = TH;
         cut(g.N0, (L::D == 3 ? kMarchW : TH) - 2 * kRing, p.nx, p.bx);
-        p.ny = p.by = 1;
-        if (L::D == 3) cut(g.N1, TH / kMarchW - 2 * kRing, p.ny, p.by);
-        const int64_t win = (int64_t)p.nx * p.ny, slots = (int64_t)c->sms * MINB;
+        const int64_t slots = (int64_t)c->sms * MINB;
         double least = 1e300;
-        for (int nc = 1; nc <= NR; ++nc) {
-            const int chunk = (NR + nc - 1) / nc;
-            if (nc > 1 && chunk < 4 * kRing) break;
-            const int64_t blocks = win * ((NR + chunk - 1) / chunk);
-            const int64_t waves = (blocks + slots - 1) / slots;
-            if (blocks > 0x7fffffff || (p.chunk && waves > 64)) break;
-            const double resident = (double)((blocks + waves * c->sms - 1) / (waves * c->sms));
-            const double t = (double)waves * (chunk + 3 * kRing + 4) * std::max(resident, 0.7 * MINB);
-            if (t < least) {
-                least = t;
-                p.chunk = chunk;
-                p.nc = (NR + chunk - 1) / chunk;
+        for (int extra = 0; extra <= (L::D == 3 ? 8 : 0); ++extra) {
+            p.ny = p.by = 1;
+            if (L::D == 3) {
+                cut(g.N1, high - 2 * kRing, p.ny, p.by);
+                cut(g.N1, (g.N1 + p.ny + extra - 1) / (p.ny + extra), p.ny, p.by);
+            }
+            p.threads = L::D == 3 ? kMarchW * (p.by + 2 * kRing) : TH;  // 3D: a warp is a row of the window
+            const double rows = L::D == 3 ? (double)(p.by + 2 * kRing) / high : 1.0;  // of the most warps that a block has
+            const int64_t win = (int64_t)p.nx * p.ny;
+            for (int nc = 1; nc <= NR; ++nc) {
+                const int chunk = (NR + nc - 1) / nc;
+                if (nc > 1 && chunk < 4 * kRing) break;
+                const int64_t blocks = win * ((NR + chunk - 1) / chunk);
+                const int64_t waves = (blocks + slots - 1) / slots;
+                if (blocks > 0x7fffffff || (out->chunk && waves > 64)) break;
+                const double resident = (double)((blocks + waves * c->sms - 1) / (waves * c->sms));
+                const double t = (double)waves * (chunk + 3 * kRing + 4) * std::max(resident * rows, (L::D == 3 ? 0.85 : 0.7) * MINB);
+                if (t < least) {
+                    least = t;
+                    p.chunk = chunk;
+                    p.nc = (NR + chunk - 1) / chunk;
+                    *out = p;
+                }
             }
         }
-        if (p.chunk == 0) return;  // more windows than a launch has blocks
-        const double use = (double)c->nodes / ((double)win * p.nc * TH * (p.chunk + 3 * kRing));
-        *out = p;
+        if (out->chunk == 0) {  // more windows than a launch has blocks
+            *out = MarchPlan{};
+            return;
+        }
+        const double use =
+            (double)c->nodes / ((double)out->nx * out->ny * out->nc * out->threads * (out->chunk + 3 * kRing));
         *worth = c->nodes >= least_nodes && use >= least_use;
     }
     static const void *kernel() { return (const void *)march_kernel<L, T, KT, KS, TH, MINB, SKIP>; }
@@ -338,7 +353,7 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
     {
         const MarchPlan &p = c->march;
         march_kernel<L, T, KT, KS, TH, MINB, SKIP>
-            <<<(unsigned)((int64_t)p.nx * p.ny * p.nc), TH, march_smem<L, KS, TH>(sizeof(T)), s>>>(
+            <<<(unsigned)((int64_t)p.nx * p.ny * p.nc), p.threads, march_smem<L, KS, TH>(sizeof(T)), s>>>(
                 (const T *)src, (T *)dst, c->geom, MarchK<T>::make(c), p);
         return cudaGetLastError();
     }
@@ -351,7 +366,7 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
 //   2D FP32:        5 steps, 128 x 5: 315 (4 steps: 276; 6: 297; 128 x 7 at 4 steps: 227)
 //   2D FP64:        2 steps, 128 x 6: 52 (3 steps: 50.6; 256 x 3: 47)
 //   3D fixed point: 2 steps, 416 x 1: 35.5 (512: 32; 384: 33.5)
-//   3D FP32:        3 steps, 512 x 1: 78 (2 steps: 62; 448: 71)
+//   3D FP32:        3 steps, 512 x 1: 75 (2 steps: 62; 448: 71)
 // 3D FP64 (19 integer-form collisions' worth of registers) was slower than one
 // sweep per launch, and 4D has no room for a window.
 using March2Fx = March<D2Q9, long long, 3, 64, 10, true>;
@@ -364,8 +379,8 @@ using March3F = March<D3Q19, float, 3, 512, 1, false>;
 //   2D fixed point 256^2 16 / 20, 384^2 29 / 31, 512^2 52 / 41, 1024^2 76 / 43, 1999x1501 94 / 44, 4096^2 108 / 47
 //   2D FP32        256^2 22 / 23, 384^2 50 / 46, 512^2 77 / 60, 1024^2 194 / 124, 1999x1501 258 / 85, 4096^2 315 / 97
 //   2D FP64        768^2 34 / 40, 1024^2 37 / 39, 1999x1501 48 / 42, 4096^2 52 / 47
-//   3D fixed point 48^3 15 / 13, 64^3 21 / 21, 101x90x77 25 / 19, 128^3 32 / 22, 256^3 36 / 23
-//   3D FP32        48^3 14 / 17, 64^3 32 / 31, 101x90x77 42 / 46, 128^3 61 / 42, 256^3 78 / 46
+//   3D fixed point 48^3 16 / 13, 64^3 20 / 21, 101x90x77 26 / 19, 128^3 32 / 22, 256^3 36 / 23
+//   3D FP32        64^3 31 / 31, 72^3 41 / 36, 80^3 49 / 41, 101x90x77 50 / 42, 128^3 61 / 42, 256^3 75 / 46
 cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth)
 {
     *plan = MarchPlan{};
@@ -378,7 +393,7 @@ cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth)
     }
     if (c->d == 3) {
         if (c->precision == LB_FX64) return March3Fx::setup(c, 300000, 0.4, plan, worth);
-        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, 1200000, 0.4, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, 350000, 0.3, plan, worth);
     }
     return cudaSuccess;
 }
@@ -398,9 +413,13 @@ cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s)
 // Batched 2D instances.
 // ---------------------------------------------------------------------------
 template <typename T, int KS, int TH, int MINB> struct MarchB {
-    // Chunks of about `c` rows, c the cheapest by the work of all blocks over the
-    // resident ones plus half a block's own length for the last wave; the
-    // longest blocks first.
+    // Chunks of at most c rows, c the cheapest by a model of the launch: the
+    // longest block's iterations (latency), and twice the mean block's work per
+    // wave of resident blocks (its rows, the recomputed ones and about 6 rows of
+    // fill).  Against chunks of 8 to 512 rows measured one by one on 7 batches
+    // (8 to 512 instances of 32^2 to 512^2) in each precision, its choice was
+    // 1.4 % above the fastest in the mean and 8 % at the most.  The longest blocks
+    // start first.
     static void plan(const lb_ctx *inst, int count, int sms, std::vector<MarchBlock> *out, int *steps, int *threads, int *cols)
     {
         constexpr int ring = KS - 1;
@@ -410,21 +429,24 @@ template <typename T, int KS, int TH, int MINB> struct MarchB {
         const double slots = (double)sms * MINB;
         double least = 1e300;
         int best = 16;
-        for (int c = 16; c <= 4096; c += c / 2) {
-            double work = 0.0;
-            int longest = 0;
+        for (int c = 8; c <= 65536; c += std::max(1, c / 8)) {
+            double work = 0.0, blocks = 0.0;
+            int longest = 0, highest = 0;
             for (int j = 0; j < count; ++j) {
                 int nx, bx, nc, ch;
                 cut((int)inst[j].N[0], TH - 2 * ring, nx, bx);
                 cut((int)inst[j].N[1], c, nc, ch);
-                work += (double)nx * nc * (ch + 3 * ring + 4);
-                longest = std::max(longest, ch + 3 * ring + 4);
+                blocks += (double)nx * nc;
+                work += (double)nx * nc * (ch + ring + 6);
+                longest = std::max(longest, ch + 3 * ring);
+                highest = std::max(highest, (int)inst[j].N[1]);
             }
-            const double t = std::max(work / slots, 0.7 * longest) + 0.5 * longest;
+            const double t = longest + 2.0 * ceil(blocks / slots) * work / blocks;
             if (t < least) {
                 least = t;
                 best = c;
             }
+            if (c >= highest) break;
         }
         out->clear();
         for (int j = 0; j < count; ++j) {
