@@ -843,18 +843,21 @@ __global__ void adj_fd4t_kernel(const double *__restrict__ h, double *__restrict
     dth0[n] += s * inv12dx;
 }
 
-// Fixed-order sum of n doubles into out[0] (one block).
-__global__ void __launch_bounds__(256) sum_slots_kernel(const double *__restrict__ a, int64_t n,
-                                                        const double *__restrict__ b, int64_t nb,
-                                                        double *__restrict__ out)
+// Fixed-order sum of n + nb doubles into out[0] (one block; four loads in flight
+// per thread).
+__global__ void __launch_bounds__(1024) sum_slots_kernel(const double *__restrict__ a, int64_t n,
+                                                         const double *__restrict__ b, int64_t nb,
+                                                         double *__restrict__ out)
 {
-    __shared__ double sh[256];
+    __shared__ double sh[1024];
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += 256) s += a[i];
-    for (int64_t i = threadIdx.x; i < nb; i += 256) s += b[i];
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < n; i += 1024) s += a[i];
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < nb; i += 1024) s += b[i];
     sh[threadIdx.x] = s;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
+    for (int w = 512; w > 0; w >>= 1) {
         if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
@@ -881,7 +884,7 @@ struct lb_adj {
     int *dflag = nullptr;                // fixed-point range flag
     int pcur = 0;
     double *th0 = nullptr, *grad = nullptr, *h = nullptr;
-    double *slot_step = nullptr, *slot_init = nullptr, *dsum = nullptr;
+    double *slot_step = nullptr, *slot_init = nullptr;
     int64_t nslot_init = 0, nslot_step = 0;
     int64_t done = 0;  // reverse steps completed
     bool forward_done = false, seeded = false;
@@ -925,7 +928,6 @@ void free_adj(lb_adj *a)
     cudaFree(a->h);
     cudaFree(a->slot_step);
     cudaFree(a->slot_init);
-    cudaFree(a->dsum);
     cudaFree(a->dflag);
     for (int p = 0; p < 2; ++p) {
         for (auto &gb : a->rgraph[p])
@@ -1080,11 +1082,10 @@ template <class L, typename T> cudaError_t seed_t(lb_adj *a, const double *dLdu,
                     (const T *)c->f[c->cur], a->ag, a->K, dLdu, dLdth, tmp, a->slot_step);
             cudaError_t e = cudaGetLastError();
             const int64_t n = (int64_t)c->q * a->ag.slab;
-            double mx = 0.0;
             if (e == cudaSuccess) e = lbk::launch_maxabs(c, tmp, n, c->dout);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&mx, c->dout, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             if (e != cudaSuccess) return e;
+            const double mx = c->hout[0];
             int ex = 0;
             if (mx > 0.0) frexp(mx, &ex);
             const int G = 56 - ex;
@@ -1305,7 +1306,6 @@ lb_status lb_adjoint_create(lb_ctx *ctx, int64_t T, int64_t C, int want_nu, lb_a
     a->nslot_step = std::max<int64_t>(a->ag.nseg, (ctx->nodes + 127) / 128);  // a warp or a block of the reverse step each
     if (e == cudaSuccess) e = cudaMalloc(&a->slot_step, sizeof(double) * a->nslot_step);
     if (e == cudaSuccess) e = cudaMalloc(&a->slot_init, sizeof(double) * a->nslot_init);
-    if (e == cudaSuccess) e = cudaMalloc(&a->dsum, sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&a->dflag, sizeof(int));
     a->bytes += 2 * pbytes + sizeof(double) * ctx->nodes * (1 + 2 * ctx->d);
     if (e != cudaSuccess) {
@@ -1485,27 +1485,20 @@ lb_status lb_adjoint_result(lb_adj *a, double *dL_dtheta0, double *dL_dnu)
     lb_ctx *c = a->ctx;
     cudaError_t e = do_init(a, dL_dtheta0);
     if (e != cudaSuccess) return acuda(a, e, "lb_adjoint_result: init adjoint");
-    if (a->fx) {
-        int flag = 0;
-        if ((e = cudaMemcpyAsync(&flag, a->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
-            return acuda(a, e, "lb_adjoint_result");
-        if (flag)
-            return afail(a, LB_EINVAL, "lb_adjoint_result: the fixed-point adjoint field left its range");
+    if (dL_dnu && a->want_nu) {
+        lbk::sum_slots_kernel<<<1, 1024, 0, c->stream>>>(a->slot_step, a->nslot_step, a->slot_init, a->nslot_init, c->dout);
+        if ((e = cudaGetLastError()) != cudaSuccess) return acuda(a, e, "lb_adjoint_result: eps sum");
     }
+    int flag = 0;
+    if (a->fx && (e = cudaMemcpyAsync(&flag, a->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
+        return acuda(a, e, "lb_adjoint_result");
+    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return acuda(a, e, "lb_adjoint_result");
+    if (flag) return afail(a, LB_EINVAL, "lb_adjoint_result: the fixed-point adjoint field left its range");
     if (dL_dnu) {
         if (!a->want_nu) return afail(a, LB_EINVAL, "lb_adjoint_result: dL/dnu was not requested");
-        lbk::sum_slots_kernel<<<1, 256, 0, c->stream>>>(a->slot_step, a->nslot_step, a->slot_init, a->nslot_init,
-                                                        a->dsum);
-        double deps = 0.0;
-        if ((e = cudaGetLastError()) != cudaSuccess ||
-            (e = cudaMemcpyAsync(&deps, a->dsum, sizeof(double), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
-            return acuda(a, e, "lb_adjoint_result: eps sum");
-        if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return acuda(a, e, "lb_adjoint_result");
-        *dL_dnu = deps * c->dt / (c->dx * c->dx);  // d eps / d nu
+        *dL_dnu = c->hout[0] * c->dt / (c->dx * c->dx);  // d eps / d nu
         return LB_OK;
     }
-    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return acuda(a, e, "lb_adjoint_result");
     return LB_OK;
 }
 

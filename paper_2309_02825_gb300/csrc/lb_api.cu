@@ -1,10 +1,12 @@
 // C-ABI of the solver (declared in include/lb.h): argument checks, device
 // memory, parameters, and the order of kernel launches.  No arithmetic of
 // the method runs on the host beyond the scalar relaxation set.
+#include <cuda.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -33,6 +35,61 @@ lb_status cuda_fail(lb_ctx *c, cudaError_t e, const char *where)
 
 bool finite_pos(double v) { return isfinite(v) && v > 0.0; }
 
+constexpr size_t kHostArea = 64 * sizeof(double) + 4 * sizeof(int);  // results, then flags
+
+// The unique number of the calling thread's CUDA context; false where the driver has none.
+bool context_id(unsigned long long *id)
+{
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found{};
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess || !fn) {
+        cudaGetLastError();
+        return false;
+    }
+    return ((CUresult(CUDAAPI *)(CUcontext, unsigned long long *))fn)(nullptr, id) == CUDA_SUCCESS;
+}
+
+// Page-locked areas of destroyed solvers, kept for the next ones (page-locking
+// takes about 300 us): a bounded number for the process, from any thread, and
+// only within the CUDA context that made them, so that what a cudaDeviceReset
+// has released is not handed out again.
+constexpr int kAreasKept = 32;
+struct Area {
+    void *p;
+    unsigned long long context;
+};
+std::mutex g_areas_mutex;
+Area g_areas[kAreasKept];
+int g_nareas = 0;
+
+cudaError_t take_area(lb_ctx *c)
+{
+    c->host_context = 0;
+    if (context_id(&c->host_context)) {
+        std::lock_guard<std::mutex> lock(g_areas_mutex);
+        for (int k = g_nareas; k-- > 0;) {
+            if (g_areas[k].context != c->host_context) continue;
+            c->host_area = g_areas[k].p;
+            g_areas[k] = g_areas[--g_nareas];
+            return cudaSuccess;
+        }
+    }
+    return cudaHostAlloc(&c->host_area, kHostArea, cudaHostAllocMapped);
+}
+
+void give_area(lb_ctx *c)  // its stream has been waited for
+{
+    if (!c->host_area) return;
+    if (c->host_context != 0) {
+        std::lock_guard<std::mutex> lock(g_areas_mutex);
+        if (g_nareas < kAreasKept) {
+            g_areas[g_nareas++] = {c->host_area, c->host_context};
+            return;
+        }
+    }
+    cudaFreeHost(c->host_area);
+}
+
 void free_ctx(lb_ctx *c)
 {
     if (!c) return;
@@ -42,8 +99,7 @@ void free_ctx(lb_ctx *c)
     cudaFree(c->f[0]);
     cudaFree(c->f[1]);
     cudaFree(c->scratch);
-    cudaFree(c->dout);
-    cudaFree(c->dflag);
+    give_area(c);
     cudaFree(c->gradtmp);
     delete c;
 }
@@ -89,6 +145,14 @@ cudaError_t record_sweeps(lb_ctx *c, int from)
     return e;
 }
 
+// A status flag, cleared; the stream has been waited for, so nothing is setting it.
+int take_flag(lb_ctx *c, int k)
+{
+    const int f = c->hflag[k];
+    if (f) c->hflag[k] = 0;
+    return f;
+}
+
 // Read back and clear the recovery and range flags (ctx->dflag[1..2]) after
 // the work enqueued so far; synchronises the stream.  A staging timeout or a
 // fixed-point range overflow leaves the context uninitialised: the state (or
@@ -96,11 +160,9 @@ cudaError_t record_sweeps(lb_ctx *c, int from)
 // until lb_set_theta0 or lb_load_state sets a state again.
 lb_status read_flags(lb_ctx *c, const char *who)
 {
-    int fl[2] = {0, 0};
-    cudaError_t e = cudaMemcpyAsync(fl, c->dflag + lbk::kFlagRecover, sizeof fl, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag + lbk::kFlagRecover, 0, sizeof fl, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    const cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, who);
+    const int fl[2] = {take_flag(c, lbk::kFlagRecover), take_flag(c, lbk::kFlagRange)};
     const std::string w(who);
     if (fl[0] & 4) {
         c->initialized = false;
@@ -305,12 +367,15 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     if (sms > 0) c->sms = sms;
     c->scratch_blocks = c->sms * 4;
     if ((e = cudaMalloc(&c->scratch, sizeof(double) * lbk::kRedSlots * c->scratch_blocks)) != cudaSuccess ||
-        (e = cudaMalloc(&c->dout, sizeof(double) * 64)) != cudaSuccess ||
-        (e = cudaMalloc(&c->dflag, sizeof(int) * 4)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 4, c->stream)) != cudaSuccess) {
+        (e = take_area(c)) != cudaSuccess ||
+        (e = cudaHostGetDevicePointer((void **)&c->dout, c->host_area, 0)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: scratch allocation");
     }
+    memset(c->host_area, 0, kHostArea);
+    c->dflag = (int *)(c->dout + 64);
+    c->hout = (volatile double *)c->host_area;
+    c->hflag = (volatile int *)(c->hout + 64);
     if ((e = choose_schedule(c)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: schedule");
@@ -579,18 +644,18 @@ lb_status lb_set_theta0(lb_ctx *c, const double *theta0, const double *grad)
             return cuda_fail(c, e, "lb_set_theta0: fd4 launch");
         grad = c->gradtmp;
     }
-    if ((e = cudaMemsetAsync(c->dflag, 0, sizeof(int) * 3, c->stream)) != cudaSuccess)
+    // in stream order: sweeps enqueued before may still set them
+    if ((e = lbk::launch_clear_flags(c->dflag, 3, c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "lb_set_theta0: flag reset");
     if (c->precision == LB_FX64) {
         // Fixed-point scale: max|theta0| * 2^F < 2^59.  Every moment sum is
         // bounded by sum_k |f_k|, which stays near theta for a stable run, so
         // 4 bits of headroom (16 max|theta0|) cover the sums and transients;
         // the initialisation flags any value beyond 4 max|theta0|.
-        double mx = 0.0;
         if ((e = lbk::launch_maxabs(c, theta0, c->nodes, c->dout)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(&mx, c->dout, sizeof(double), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
             (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
             return cuda_fail(c, e, "lb_set_theta0: max|theta0|");
+        double mx = c->hout[0];
         if (c->fx_max > 0.0) {  // a slab: the scale of the whole grid (at least this part's maximum)
             if (!isfinite(mx) || mx > c->fx_max)
                 return fail(c, LB_EINVAL, "lb_set_theta0: max|theta0| of this part exceeds the grid's maximum");
@@ -606,10 +671,8 @@ lb_status lb_set_theta0(lb_ctx *c, const double *theta0, const double *grad)
     c->cur = 0;
     if ((e = lbk::launch_init(c, theta0, grad, c->dflag)) != cudaSuccess)
         return cuda_fail(c, e, "lb_set_theta0: init launch");
-    int flag = 0;
-    if ((e = cudaMemcpyAsync(&flag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
-        return cuda_fail(c, e, "lb_set_theta0");
+    if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "lb_set_theta0");
+    const int flag = c->hflag[lbk::kFlagInit];
     if (flag & 2) return fail(c, LB_EINVAL, "lb_set_theta0: initial distributions exceed the fixed-point range");
     if (flag) return fail(c, LB_ENONPOS, "lb_set_theta0: theta0 must be finite and > 0 (and grad finite)");
     c->initialized = true;
@@ -731,15 +794,10 @@ lb_status lb_sum_theta(lb_ctx *c, double *out)
     if (!c->initialized) return fail(c, LB_ESTATE, "lb_sum_theta: call lb_set_theta0 first");
     DeviceGuard dg(c);
     cudaError_t e = lbk::launch_sum_state(c, c->f[c->cur], c->dout);
-    double v = 0.0;
-    int range = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&v, c->dout, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&range, c->dflag + lbk::kFlagRange, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag + lbk::kFlagRange, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_sum_theta");
-    if (range) {
+    double v = c->hout[0];
+    if (take_flag(c, lbk::kFlagRange)) {
         c->initialized = false;
         return fail(c, LB_EINVAL, "lb_sum_theta: a fixed-point distribution reached |f| >= 2^61 (the run is "
                                   "unstable: an FP64 run would overflow); set the state again");
@@ -764,15 +822,11 @@ lb_status lb_reduce(lb_ctx *c, const double *theta, const double *u, const doubl
     DeviceGuard dg(c);
     const int ns = 3 * (c->d + 1) + 1;
     cudaError_t e = lbk::launch_norms(c, theta, u, ex_theta, ex_u, c->dout);
-    double raw[lbk::kRedSlots];
-    int flag = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(raw, c->dout, sizeof(double) * ns, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&flag, c->dflag + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag + 1, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_reduce");
+    double raw[lbk::kRedSlots];
+    for (int k = 0; k < ns; ++k) raw[k] = c->hout[k];
+    const int flag = take_flag(c, lbk::kFlagRecover);
     const double n = (double)c->nodes;
     for (int v = 0; v <= c->d; ++v) {
         const double se = raw[3 * v], mx = raw[3 * v + 1], sx = raw[3 * v + 2];
@@ -818,7 +872,7 @@ lb_status lb_load_state(lb_ctx *c, const void *buf, int64_t step)
     DeviceGuard dg(c);
     cudaError_t e = cudaMemcpyAsync(c->f[c->cur], buf, (size_t)c->q * c->geom.slab * c->elem,
                                     cudaMemcpyDeviceToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dflag + lbk::kFlagRecover, 0, sizeof(int) * 2, c->stream);
+    if (e == cudaSuccess) e = lbk::launch_clear_flags(c->dflag + lbk::kFlagRecover, 2, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_load_state");
     c->initialized = true;
     c->step = step;

@@ -277,8 +277,16 @@ struct lb_ctx {
     int cur = 0;
     double *scratch = nullptr;     // reduction partials
     int scratch_blocks = 0;
-    double *dout = nullptr;        // small device result area
-    int *dflag = nullptr;          // device status flags
+    // Results and status flags in page-locked host memory that kernels write
+    // directly (one block, host_area): a call that returns a number then waits for
+    // its kernels once and reads it, where it copied each value back and cleared
+    // the flags with operations of their own.
+    void *host_area = nullptr;
+    unsigned long long host_context = 0;  // number of the CUDA context that page-locked it, 0 unknown
+    double *dout = nullptr;        // 64 results: device address
+    int *dflag = nullptr;          // status flags: device address
+    volatile double *hout = nullptr;  // the same, host addresses (read when the stream has been waited for)
+    volatile int *hflag = nullptr;
     double *gradtmp = nullptr;     // FD gradient when none is supplied
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // recorded sweeps, by starting buffer
     bool initialized = false;
@@ -350,6 +358,7 @@ cudaError_t launch_sum_state(lb_ctx *c, const void *src, double *out_dev);
 cudaError_t launch_sum_state_rows(lb_ctx *c, const void *src, double *out_dev, int64_t row0, int64_t nrow);
 cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *theta, double *grad, double *u, int *flag,
                                int64_t row0, int64_t nrow);
+cudaError_t launch_clear_flags(int *flag, int n, cudaStream_t s);
 cudaError_t launch_maxabs(lb_ctx *c, const double *x, int64_t n, double *out_dev);
 // 64-bit fixed-point path (lb_fx.cu).
 cudaError_t launch_sweep_fx(lb_ctx *c, const void *src, void *dst);

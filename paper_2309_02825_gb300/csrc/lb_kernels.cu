@@ -515,6 +515,17 @@ __global__ void __launch_bounds__(kRedThreads) norms_kernel(const double *__rest
     block_reduce_store<NS>(a, op, partial + (int64_t)blockIdx.x * kRedSlots);
 }
 
+// Clears n status flags in stream order.
+__global__ void clear_flags_kernel(int *flag, int n)
+{
+    if ((int)threadIdx.x < n) flag[threadIdx.x] = 0;
+}
+cudaError_t launch_clear_flags(int *flag, int n, cudaStream_t s)
+{
+    clear_flags_kernel<<<1, 32, 0, s>>>(flag, n);
+    return cudaGetLastError();
+}
+
 // max |x| over n values.
 __global__ void __launch_bounds__(kRedThreads) maxabs_kernel(const double *__restrict__ x, int64_t n,
                                                              double *__restrict__ partial)

@@ -256,10 +256,9 @@ lb_status lb_slab_sum_theta(lb_slab *s, double *out)
     lb_ctx *c = s->ctx;
     if (!c->initialized) return sfail(s, LB_ESTATE, "lb_slab_sum_theta: no state");
     cudaError_t e = lbk::launch_sum_state_rows(c, c->f[c->cur], c->dout, s->layer_rows, s->nz * s->layer_rows);
-    double v = 0.0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&v, c->dout, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return scuda(s, e, "lb_slab_sum_theta");
+    double v = c->hout[0];
     if (c->precision == LB_FP32_SHIFTED) v += c->theta_ref * (double)(s->nz * s->layer_rows * c->geom.N0);
     *out = v;
     return LB_OK;
