@@ -692,10 +692,16 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     // directly so that they land in the caller's graph.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+    // Every launch below swaps the two buffers once, whatever its number of
+    // steps.  A captured call is replayed from the buffer that it read, so there
+    // the launches are cut such that an even number of steps ends in that buffer
+    // again, as one sweep per launch does, and replays go on from one another.
+    const bool held = cap != cudaStreamCaptureStatusNone;
     if (c->run == lbk::kSchedLine && nsteps > 0) {
         constexpr int64_t kMost = 1 << 20;  // steps per launch
         while (nsteps > 0) {
-            const int64_t n = nsteps < kMost ? nsteps : kMost;
+            int64_t n = nsteps < kMost ? nsteps : kMost;
+            if (held && n % 2 == 0) --n;
             cudaError_t e = lbk::line_launch(c, c->f[c->cur], c->f[c->cur ^ 1], n);
             if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: resident launch");
             c->cur ^= 1;
@@ -706,7 +712,9 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     }
     if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps) {
         // marching launches; the remainder below, one sweep per launch
-        while (nsteps >= c->march.steps) {
+        int64_t launches = nsteps / c->march.steps;
+        if (held && c->march.steps % 2 == 0) launches -= launches % 2;
+        for (; launches > 0; --launches) {
             cudaError_t e = lbk::march_launch(c, c->f[c->cur], c->f[c->cur ^ 1], c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: marching launch");
             c->cur ^= 1;
@@ -716,9 +724,16 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     }
     if (c->run == lbk::kSchedTiles && c->tb_k > 0) {
         // blocked: launches of tb_k steps (recorded in graphs), then one launch for the remainder
+        cudaError_t e = cudaSuccess;
+        while (held && ((nsteps + c->tb_k - 1) / c->tb_k - nsteps) % 2 != 0) {  // at most two steps on their own
+            if ((e = lbk::blocked_launch(c, c->f[c->cur], c->f[c->cur ^ 1], 1, c->stream)) != cudaSuccess)
+                return cuda_fail(c, e, "lb_step: blocked launch");
+            c->cur ^= 1;
+            ++c->step;
+            --nsteps;
+        }
         int64_t launches = nsteps / c->tb_k;
         const int rem = (int)(nsteps % c->tb_k);
-        cudaError_t e = cudaSuccess;
         while (cap == cudaStreamCaptureStatusNone && launches >= kTbGraphLaunches) {
             if (!c->tb_graph[c->cur]) e = record_blocked(c, c->cur);
             if (e == cudaSuccess) e = cudaGraphLaunch(c->tb_graph[c->cur], c->stream);

@@ -739,7 +739,14 @@ cudaError_t run_steps(lb_batch *b, int64_t n)
 {
     cudaError_t e = cudaSuccess;
     if (b->m_steps > 0) {  // marching launches; the remainder below, one launch per step
-        for (; n >= b->m_steps; n -= b->m_steps) {
+        // inside the caller's capture an even number of steps ends in the buffer it
+        // began in, as one launch per step does: replays go on from one another
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(b->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+        int64_t launches = n / b->m_steps;
+        if (cap != cudaStreamCaptureStatusNone && b->m_steps % 2 == 0) launches -= launches % 2;
+        n -= launches * b->m_steps;
+        for (; launches > 0; --launches) {
             e = lbk::march_batch_launch(b->precision, b->mv, b->d_desc, b->d_march, b->m_blocks, b->buf[b->cur],
                                         b->buf[b->cur ^ 1], b->stream);
             if (e != cudaSuccess) return e;

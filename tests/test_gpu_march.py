@@ -105,6 +105,67 @@ def test_marching_inside_a_captured_graph():
         x.close()
 
 
+@pytest.mark.parametrize("d,N,prec", [(1, (81,), "fx64"), (2, (64, 50), "fx64"), (2, (700, 613), "fx64"),
+                                      (2, (1201, 1000), "fp32s"), (3, (101, 90, 77), "fp32s")])
+@pytest.mark.parametrize("n", [1, 8, 14, 17])
+def test_captured_steps_replay_one_after_another(d, N, prec, n):
+    """An even captured call, or an odd one captured twice, ends in the buffer it
+    began in, whatever the number of steps of a launch: replays continue."""
+    th, gr = _inputs(d, N)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    dx = 1.0 / N[0]
+    eps = 0.0512 if d == 3 else 0.2048
+    s = lb.Solver(d, N, 0.02, dx, eps * dx * dx / 0.02, precision=prec, theta_ref=1.5, stream=stream)
+    calls = 1 + n % 2
+    with torch.cuda.stream(stream):
+        s.set_theta0(th, gr)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            for _ in range(calls):
+                s.step(n)
+        for _ in range(3):
+            g.replay()
+        got = s.macros()
+        s.set_theta0(th, gr)
+        for _ in range(3 * calls * n):
+            s.step(1)
+        want = s.macros()
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    s.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32s", "fx64"])
+def test_captured_batch_steps_replay_one_after_another(prec):
+    sizes = [(130, 96), (257, 201)]
+    dx = [1.0 / n[0] for n in sizes]
+    stream = torch.cuda.Stream()
+    ins = [_inputs(2, n) for n in sizes]
+    th = torch.cat([t.reshape(-1) for t, _ in ins])
+    gr = torch.cat([g.reshape(-1) for _, g in ins])
+    torch.cuda.synchronize()
+    kw = {"theta_ref": [1.5, 1.5]} if prec == "fp32s" else {}
+    b = lb.Batch(sizes, [0.02] * 2, dx, [0.2048 * x * x / 0.02 for x in dx], precision=prec, stream=stream, **kw)
+    with torch.cuda.stream(stream):
+        b.set_theta0(th, gr)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            b.step(14)
+        for _ in range(3):
+            g.replay()
+        got = b.macros()
+        b.set_schedule(1e18, 128, False)
+        b.set_theta0(th, gr)
+        b.step(42)
+        want = b.macros()
+    torch.cuda.synchronize()
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
+    b.close()
+
+
 def test_blocking_call_still_selects_single_sweeps():
     s = lb.Solver(2, (600, 500), 0.02, 1.0 / 600, 0.2048 / 600**2 / 0.02, precision="fx64")
     assert s.blocking()["steps_per_launch"] == 0
