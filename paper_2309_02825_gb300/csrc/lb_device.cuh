@@ -148,7 +148,9 @@ __device__ __forceinline__ long long mulfx_c(long long a, long long k)
 // (above half, or exactly half with an odd significand, round up; a carry out
 // of the significand moves into the exponent field by the same addition), and
 // the biased exponent is e + 1023.
-__device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned long long sign)
+//
+// k: a power of two 2^k folded into the exponent; the result must be a normal number.
+__device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned long long sign, int k = 0)
 {
     if (a == 0ull) return 0.0;
     const int e = 63 - __clzll((long long)a);
@@ -162,13 +164,46 @@ __device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned
         up = (rem > half || (rem == half && (mant & 1ull))) ? 1ull : 0ull;
     }
     // (e + 1022) << 52 plus the significand's implicit 2^52 gives the biased exponent e + 1023
-    return __longlong_as_double((long long)((((unsigned long long)(e + 1022) << 52) + mant + up) | sign));
+    return __longlong_as_double((long long)((((unsigned long long)(e + k + 1022) << 52) + mant + up) | sign));
 }
 
-__device__ __forceinline__ double i64_to_f64_rn(long long v)
+__device__ __forceinline__ double i64_to_f64_rn(long long v, int k = 0)
 {
     const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    return u64_bits_to_f64(a, v < 0 ? 0x8000000000000000ull : 0ull);
+    return u64_bits_to_f64(a, v < 0 ? 0x8000000000000000ull : 0ull, k);
+}
+
+// num / den for a normal den > 0, rounded to nearest like the operator.  An
+// FP64 division is a chain of about nine FP64 instructions, which bound the
+// recovery (82 % of that pipe); here the significands, as 64-bit fractions d and
+// c in [1/2, 1), are divided on the integer pipes: 1/d from a 32-bit estimate by
+// two Newton steps r <- r + r (1 - d r) in 62 fraction bits (errors 2^-22, 2^-44,
+// then a few units of the last bit), c times it rounded to 53 bits, and the exact
+// remainder of that decides between it and its neighbours (no quotient of two
+// 53-bit significands is a tie).  Recovery of 1999 x 1501 FP32: 98 -> 75 us.
+__device__ __forceinline__ double quot_int(double num, double den)
+{
+    const unsigned long long nb = (unsigned long long)__double_as_longlong(num), db = (unsigned long long)__double_as_longlong(den);
+    const int en = (int)(nb >> 52) & 0x7ff, ed = (int)(db >> 52);  // den negative: ed above 0x7ff
+    const int e = en - ed;
+    if (en == 0 || en == 0x7ff || ed == 0 || ed >= 0x7ff || e < -1000 || e > 1000) return num / den;
+    const unsigned long long d = (db << 11) | (1ull << 63), c = (nb << 11) | (1ull << 63);
+    const unsigned dh = (unsigned)(d >> 32);
+    const unsigned r0 = __float2uint_rz(__frcp_rn(__uint2float_rz(dh)) * 0x1p63f);  // 31 fraction bits, in (1, 2]; 2 saturates
+    // 1 - d r0 in units of 2^-63: below 2^42 in magnitude
+    const unsigned long long p0 = (unsigned long long)dh * r0 + __umulhi((unsigned)d, r0);
+    const int s0 = (int)((long long)((1ull << 63) - p0) >> 12);
+    const unsigned long long r1 = ((unsigned long long)r0 << 31) + (unsigned long long)(((long long)s0 * (int)(r0 >> 1)) >> 19);
+    // 1 - d r1 in units of 2^-62: below 2^22
+    const int s1 = (int)((1ull << 62) - __umul64hi(d, r1));
+    const unsigned long long r2 = r1 + (unsigned long long)(((long long)s1 * (int)(r1 >> 33)) >> 29);
+    const unsigned long long q = __umul64hi(c, r2);
+    const int sh = q >> 62 ? 10 : 9;  // c / d in [1, 2), or below 1
+    const long long dm = (long long)(d >> 11);
+    long long m = (long long)((q + (1ull << (sh - 1))) >> sh);
+    const long long rem2 = (long long)(((c >> 11) << (62 - sh)) - (unsigned long long)m * (unsigned long long)dm) * 2;
+    m += rem2 > dm ? 1 : (rem2 < -dm ? -1 : 0);
+    return __longlong_as_double((long long)((((unsigned long long)(e + sh + 1012) << 52) + (unsigned long long)m) | (nb & (1ull << 63))));
 }
 
 // Exact sums of floats on the integer pipes (GB300 issues FP64 at 1/64 of its
@@ -197,6 +232,7 @@ template <int PB> __device__ __forceinline__ long long f32_align(float v, unsign
     const long long mag = (long long)(sh < 64u ? (m >> sh) : 0ull);
     return (b >> 31) ? -mag : mag;
 }
+template <int PB> __device__ __forceinline__ int f32_unit(unsigned emax) { return (int)emax - 150 - PB; }  // 2^this
 template <int PB> __device__ __forceinline__ double f32_scale(unsigned emax)
 {
     return __longlong_as_double((long long)(emax + 1023u - 150u - PB) << 52);  // normal for every emax <= 254

@@ -79,7 +79,7 @@ __device__ __forceinline__ void recover_store(double thm, const double (&Jd)[4],
         const long long tb = __double_as_longlong(thd);
         if (!(tb > 0) || ((tb >> 52) & 0x7ff) == 0x7ff) atomicOr(flag, 1);
     }
-    const double cu = r.ucoef / thd;  // the storage scale is folded into ucoef and gcoef
+    const double cu = quot_int(r.ucoef, thd);  // the storage scale is folded into ucoef and gcoef
 #pragma unroll
     for (int a = 0; a < L::D; ++a) {
         const double Ja = Jd[a];
@@ -114,10 +114,10 @@ __device__ __forceinline__ void recover_node(const T (&vals)[L::Q], const Recov 
                 if constexpr (ev == -1) Ji[a] -= fv;
             });
         });
-        const double sc = f32_scale<PB>(emax);
-        thm = emax == 0xffu ? __longlong_as_double(0x7ff8000000000000ll) : i64_to_f64_rn(thi) * sc;
+        const int k = f32_unit<PB>(emax);
+        thm = emax == 0xffu ? __longlong_as_double(0x7ff8000000000000ll) : i64_to_f64_rn(thi, k);
 #pragma unroll
-        for (int a = 0; a < L::D; ++a) Jd[a] = i64_to_f64_rn(Ji[a]) * sc;
+        for (int a = 0; a < L::D; ++a) Jd[a] = i64_to_f64_rn(Ji[a], k);
     } else {
         if constexpr (std::is_same<T, double>::value) {
             // FP64 states: the sums formed exactly on the integer pipes where the
