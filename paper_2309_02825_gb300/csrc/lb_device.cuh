@@ -173,6 +173,20 @@ __device__ __forceinline__ double i64_to_f64_rn(long long v, int k = 0)
     return u64_bits_to_f64(a, v < 0 ? 0x8000000000000000ull : 0ull, k);
 }
 
+// v 2^k rounded to FP32, nearest, ties to even: the 32 bits from the leading
+// one down, the last of them also set where a lower bit is, through the 32-bit
+// conversion (the 64-bit one issues at the FP64 rate).  Zero, or a result that
+// is a normal number.
+__device__ __forceinline__ float i64_to_f32_rn(long long v, int k)
+{
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    if (a == 0ull) return 0.0f;
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz;
+    const float r = __uint2float_rn((unsigned)(n >> 32) | ((unsigned)n != 0u ? 1u : 0u));
+    return __uint_as_float((__float_as_uint(r) + ((unsigned)(k + 32 - lz) << 23)) | (v < 0 ? 0x80000000u : 0u));
+}
+
 // num / den for a normal den > 0, rounded to nearest like the operator.  An
 // FP64 division is a chain of about nine FP64 instructions, which bound the
 // recovery (82 % of that pipe); here the significands, as 64-bit fractions d and

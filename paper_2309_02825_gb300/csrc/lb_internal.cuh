@@ -200,7 +200,11 @@ struct InitK {
     // gradient component -> round(dx grad 2^F) (gscale = dx 2^F), and the
     // constants w1, wd, iax/dx with kFxCoefBits fraction bits.
     double gscale;
+    // FP32 storage forms its values the same way in a unit of the node's own
+    // where the constants allow it (ints).
     long long w1k, wdk, iak;
+    double dx;
+    int ints;
     int fx_bits;  // F
 };
 

@@ -1,4 +1,5 @@
-"""The recovery's quotient, formed on the integer pipes, against IEEE division."""
+"""Single-precision initialisation and the recovery's quotient, both formed on
+the integer pipes, against FP64 and IEEE division."""
 
 import numpy as np
 import pytest
@@ -7,6 +8,78 @@ import torch
 from paper_2309_02825_gb300 import lb
 
 pytestmark = pytest.mark.gpu
+
+SHAPES = {1: (301,), 2: (67, 41), 3: (13, 11, 9), 4: (7, 6, 5, 5)}
+EPS = {1: 0.16, 2: 0.2048, 3: 0.0512, 4: 0.08}
+
+
+def _velocities(d):
+    e = [[0] * d]
+    for s in (1, -1):
+        for a in range(d):
+            e.append([s if b == a else 0 for b in range(d)])
+    for a in range(d):
+        for b in range(a + 1, d):
+            for sa, sb in ((1, 1), (-1, 1), (-1, -1), (1, -1)):
+                v = [0] * d
+                v[a], v[b] = sa, sb
+                e.append(v)
+    return e
+
+
+@pytest.mark.parametrize("d", [1, 2, 3, 4])
+@pytest.mark.parametrize("case", ["run", "near the reference", "flat", "large gradient", "outside the range"])
+def test_fp32_initialisation_is_rounded_once(d, case):
+    """Each stored value is the exact population rounded to FP32, up to the
+    formation's own rounding: constants at 2^-53 of themselves, theta and the
+    gradient aligned at 2^-60 of the larger, so below 2^-48 of the terms' sum;
+    beyond the aligned range of magnitudes the FP64 form, within the same."""
+    N = SHAPES[d]
+    shape = tuple(reversed(N))
+    rng = np.random.default_rng(11 * d)
+    th = 1.5 + 0.4 * rng.standard_normal(shape).clip(-3, 3)
+    g = rng.standard_normal((d,) + shape)
+    dx = 1.0 / N[0]
+    if case == "near the reference":
+        th = 1.5 + 1e-9 * rng.standard_normal(shape)
+        th.flat[::5] = 1.5
+    elif case == "flat":
+        th.flat[::3] = 1.5
+        g[:] = 0.0
+    elif case == "large gradient":
+        g *= 1e7
+    elif case == "outside the range":  # theta - theta_ref below 2^-40, no gradient
+        th = 1.5 + 2.0 ** -45 * rng.integers(-9, 9, shape)
+        g *= 1e-14
+    s = lb.Solver(d, N, 0.02, dx, EPS[d] * dx * dx / 0.02, precision="fp32s", theta_ref=1.5)
+    s.set_theta0(torch.from_numpy(th).cuda(), torch.from_numpy(g).cuda())
+    pitch, slab, eb = s.state_layout()
+    p = s.params
+    buf = s.save_state().cpu().numpy().view(np.float32)
+    s.close()
+    e = _velocities(d)
+    q = len(e)
+    rows = int(np.prod(N[1:]))
+    got = [buf[i * slab:i * slab + rows * pitch].reshape(rows, pitch)[:, :N[0]].reshape(shape) for i in range(q)]
+    sigma = p["cs2"] / p["c"] ** 2
+    wd = p["wd"] if d > 1 else 0.0
+    iax = 0.5 * dx * (sigma / p["s1"] - 4.0 * (d - 1.0) * wd)
+    idg = wd * dx
+    L = np.longdouble
+    dth, gl = (th - 1.5).astype(L), g.astype(L)
+    scale = np.abs(dth) + dx * np.abs(gl).sum(0)
+    for i in range(q):
+        ax = [a for a in range(d) if e[i][a]]
+        if not ax:
+            f = L(p["w0"]) * dth
+        elif len(ax) == 1:
+            f = L(p["w1"]) * dth - e[i][ax[0]] * L(iax) * gl[ax[0]]
+        else:
+            f = L(wd) * dth - L(idg) * sum(e[i][a] * gl[a] for a in ax)
+        f = np.roll(f, [-v for v in reversed(e[i])], tuple(range(d)))  # stored at x - e_i
+        sz = np.roll(scale, [-v for v in reversed(e[i])], tuple(range(d)))
+        tol = np.abs(f) * L(2.0) ** -24 + sz * L(2.0) ** -48
+        assert np.all(np.abs(got[i].astype(L) - f) <= tol), (i, float(np.max(np.abs(got[i] - f) / tol)))
 
 
 def test_recovered_velocity_is_the_ieee_quotient():
