@@ -293,32 +293,45 @@ __device__ __forceinline__ int fd4_at(int t, int n, bool mir)
     while (t >= n) t -= n;
     return t;
 }
-__global__ void __launch_bounds__(256) fd4_kernel(const double *__restrict__ th, double *__restrict__ grad, int d,
-                                                  int N0, int N1, int N2, int N3, unsigned mirror, double inv12dx)
+// -th(2) + 8 th(1) - 8 th(-1) + th(-2) of an axis: exactly in integers, rounded
+// once, where the four values' exponents lie within 4 of each other (57 bits, 2 +
+// 16 of them below 2^62), which saves three of five FP64 instructions.
+// 1999 x 1501: 51 -> 38 us.
+template <int D>
+__global__ void __launch_bounds__(256) fd4_kernel(const double *__restrict__ th, double *__restrict__ grad, int N0, int N1,
+                                                  int N2, int N3, unsigned mirror, double inv12dx)
 {
     const int64_t nodes = (int64_t)N0 * N1 * N2 * N3;  // <= 2^31
     const int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (node >= nodes) return;
-    const unsigned nd = (unsigned)node;
-    const unsigned r1 = nd / (unsigned)N0, r2 = r1 / (unsigned)N1, r3 = r2 / (unsigned)N2;
-    const int c[4] = {(int)(nd - r1 * (unsigned)N0), (int)(r1 - r2 * (unsigned)N1), (int)(r2 - r3 * (unsigned)N2),
-                      (int)r3};
     const int n[4] = {N0, N1, N2, N3};
-    unsigned stride = 1;
+    unsigned left = (unsigned)node, stride = 1;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        if (a < d) {
-            const unsigned base = nd - (unsigned)c[a] * stride;
-            const bool mir = (mirror >> a) & 1u;
-            double v[4];
+    for (int a = 0; a < D; ++a) {
+        const unsigned q = a + 1 < D ? left / (unsigned)n[a] : 0u;
+        const int c = (int)(left - q * (unsigned)n[a]);
+        left = q;
+        const bool mir = (mirror >> a) & 1u;
+        const bool inner = c >= 2 && c < n[a] - 2;
+        double v[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = th[base + (unsigned)fd4_at(c[a] + (k < 2 ? 2 - k : 1 - k), n[a], mir) * stride];
-            double acc = -v[0];
+        for (int k = 0; k < 4; ++k) {
+            const int m = k < 2 ? 2 - k : 1 - k;  // 2, 1, -1, -2
+            const int to = inner ? m : fd4_at(c + m, n[a], mir) - c;
+            v[k] = __ldg(th + (node + (int64_t)to * stride));
+        }
+        long long x[4];
+        unsigned emax;
+        double acc;
+        if (f64_align<4, 4>(v, x, emax)) {
+            acc = f64_from_aligned<4>((x[3] - x[0]) + 8 * (x[1] - x[2]), emax);
+        } else {
+            acc = -v[0];
             acc += 8.0 * v[1];
             acc += -8.0 * v[2];
             acc += v[3];
-            grad[a * nodes + node] = acc * inv12dx;
         }
+        grad[a * nodes + node] = acc * inv12dx;
         stride *= (unsigned)n[a];
     }
 }
@@ -660,9 +673,16 @@ cudaError_t launch_sweep(lb_ctx *c, const void *src, void *dst)
 cudaError_t launch_fd4_grad(const lb_ctx *c, const double *theta0, double *grad)
 {
     const int64_t nodes = c->nodes;
-    fd4_kernel<<<(unsigned)((nodes + 255) / 256), 256, 0, c->stream>>>(
-        theta0, grad, c->d, (int)c->N[0], (int)c->N[1], (int)c->N[2], (int)c->N[3], c->geom.mirror,
-        1.0 / (12.0 * c->dx));
+    const auto go = [&](auto kernel) {
+        kernel<<<(unsigned)((nodes + 255) / 256), 256, 0, c->stream>>>(theta0, grad, (int)c->N[0], (int)c->N[1], (int)c->N[2],
+                                                                       (int)c->N[3], c->geom.mirror, 1.0 / (12.0 * c->dx));
+    };
+    switch (c->d) {
+    case 1: go(fd4_kernel<1>); break;
+    case 2: go(fd4_kernel<2>); break;
+    case 3: go(fd4_kernel<3>); break;
+    default: go(fd4_kernel<4>);
+    }
     return cudaGetLastError();
 }
 

@@ -105,3 +105,46 @@ def test_recovered_velocity_is_the_ieee_quotient():
     assert ok.sum() > 0.99 * n
     want = ((2.0 - p["s1"]) * p["c"]) / got_th
     assert np.array_equal(u[ok], want[ok])
+
+
+@pytest.mark.parametrize("N", [(1,), (3,), (37,), (5, 4), (67, 41), (9, 2, 7), (6, 5, 4, 3)])
+@pytest.mark.parametrize("walls", [False, True])
+def test_central_difference_in_integers(N, walls):
+    """The gradient that lb_set_theta0 forms is the fourth-order difference rounded
+    once and multiplied by 1 / (12 dx): within 2 ulp of itself where the exponents
+    of theta allow the integers, else within 8 roundings of the largest term.  Read
+    off the fixed-point state's J = -(sigma dx / s1) grad, whose own rounding is
+    2^-57 of max|theta| per population."""
+    if walls and min(N) < 5:
+        pytest.skip("walls need five nodes")
+    d = len(N)
+    shape = tuple(reversed(N))
+    rng = np.random.default_rng(sum(N))
+    th = rng.uniform(0.9, 3.0, shape)
+    th.flat[::7] *= 2.0 ** rng.integers(-9, 9, th.flat[::7].shape)
+    dx = 1.0 / 16
+    kw = {"boundary": ["mirror"] * d} if walls else {}
+    grads = []
+    for given in (False, True):
+        s = lb.Solver(d, N, 0.02, dx, EPS[d] * dx * dx / 0.02, precision="fx64", **kw)
+        g = None
+        if given:
+            L = np.longdouble
+            g = np.empty((d,) + shape)
+            for a in range(d):
+                ax, n = d - 1 - a, N[a]
+                idx = np.arange(n)
+                def at(m):
+                    j = idx + m
+                    if walls:
+                        j = np.where(j < 0, -j, j)
+                        j = np.where(j >= n, 2 * (n - 1) - j, j)
+                    return np.take(th, j % n if not walls else j, axis=ax).astype(L)
+                g[a] = ((at(-2) - at(2) + 8 * (at(1) - at(-1))) / (12 * L(dx))).astype(np.float64)
+            g = torch.from_numpy(g).cuda()
+        s.set_theta0(torch.from_numpy(th).cuda(), g)
+        grads.append(s.macros()[1].cpu().numpy())
+        s.close()
+    big = np.abs(th).max()
+    tol = 18 * big / (12 * dx) * 2.0 ** -49
+    assert np.abs(grads[0] - grads[1]).max() <= tol
