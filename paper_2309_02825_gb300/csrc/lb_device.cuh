@@ -148,9 +148,7 @@ __device__ __forceinline__ long long mulfx_c(long long a, long long k)
 // (above half, or exactly half with an odd significand, round up; a carry out
 // of the significand moves into the exponent field by the same addition), and
 // the biased exponent is e + 1023.
-//
-// k: a power of two 2^k folded into the exponent; the result must be a normal number.
-__device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned long long sign, int k = 0)
+__device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned long long sign)
 {
     if (a == 0ull) return 0.0;
     const int e = 63 - __clzll((long long)a);
@@ -164,13 +162,21 @@ __device__ __forceinline__ double u64_bits_to_f64(unsigned long long a, unsigned
         up = (rem > half || (rem == half && (mant & 1ull))) ? 1ull : 0ull;
     }
     // (e + 1022) << 52 plus the significand's implicit 2^52 gives the biased exponent e + 1023
-    return __longlong_as_double((long long)((((unsigned long long)(e + k + 1022) << 52) + mant + up) | sign));
+    return __longlong_as_double((long long)((((unsigned long long)(e + 1022) << 52) + mant + up) | sign));
 }
 
-__device__ __forceinline__ double i64_to_f64_rn(long long v, int k = 0)
+__device__ __forceinline__ double i64_to_f64_rn(long long v)
 {
     const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    return u64_bits_to_f64(a, v < 0 ? 0x8000000000000000ull : 0ull, k);
+    return u64_bits_to_f64(a, v < 0 ? 0x8000000000000000ull : 0ull);
+}
+
+// v 2^k by the conversion instruction, for kernels that leave the FP64 pipe room;
+// zero, or a result that is a normal number.
+__device__ __forceinline__ double i64_to_f64_hw(long long v, int k)
+{
+    const double r = (double)v;
+    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(r) + (int)((unsigned)k << 20), __double2loint(r));
 }
 
 // v 2^k rounded to FP32, nearest, ties to even: the 32 bits from the leading
@@ -194,7 +200,8 @@ __device__ __forceinline__ float i64_to_f32_rn(long long v, int k)
 // two Newton steps r <- r + r (1 - d r) in 62 fraction bits (errors 2^-22, 2^-44,
 // then a few units of the last bit), c times it rounded to 53 bits, and the exact
 // remainder of that decides between it and its neighbours (no quotient of two
-// 53-bit significands is a tie).  Recovery of 1999 x 1501 FP32: 98 -> 75 us.
+// 53-bit significands is a tie).  Recovery of 1999 x 1501 FP32: 98 -> 75 us
+// (62 with the sums' conversions on the FP64 pipe that this left idle).
 __device__ __forceinline__ double quot_int(double num, double den)
 {
     const unsigned long long nb = (unsigned long long)__double_as_longlong(num), db = (unsigned long long)__double_as_longlong(den);
@@ -343,18 +350,53 @@ struct RowPos {
 };
 template <int D> __device__ __forceinline__ RowPos row_pos(const Geom &g, int64_t row)
 {
-    RowPos r;
-    r.y = (int)(row % g.N1);
-    if constexpr (D <= 3) {
-        r.z = (int)(row / g.N1);
-        r.w = 0;
+    RowPos r;  // (a grid has at most 2^31 nodes: 32-bit divisions)
+    if constexpr (D <= 2) {
+        r.y = (int)row;
+        r.z = r.w = 0;
     } else {
-        const int64_t r2 = row / g.N1;
-        r.z = (int)(r2 % g.N2);
-        r.w = (int)(r2 / g.N2);
+        const unsigned rw = (unsigned)row, r2 = rw / (unsigned)g.N1;
+        r.y = (int)(rw - r2 * (unsigned)g.N1);
+        if constexpr (D == 3) {
+            r.z = (int)r2;
+            r.w = 0;
+        } else {
+            const unsigned r3 = r2 / (unsigned)g.N2;
+            r.z = (int)(r2 - r3 * (unsigned)g.N2);
+            r.w = (int)r3;
+        }
     }
     return r;
 }
+
+// Offsets within a population of a periodic node's sources, by axis and
+// velocity component e + 1: the pull from x - e reads the sum of one per axis.
+// Below 2^32 each: at most 2^31 nodes, and with padding two states of nine
+// populations of 2^32 values would not fit the device.
+template <int D> struct PullOffsets {
+    unsigned off[D][3];
+    __device__ __forceinline__ PullOffsets(const Geom &g, int x, const RowPos &r)
+    {
+        const int c[4] = {x, r.y, r.z, r.w}, n[4] = {g.N0, g.N1, g.N2, g.N3};
+        unsigned stride = 1;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            off[a][0] = (unsigned)(c[a] == n[a] - 1 ? 0 : c[a] + 1) * stride;
+            off[a][1] = (unsigned)c[a] * stride;
+            off[a][2] = (unsigned)(c[a] == 0 ? n[a] - 1 : c[a] - 1) * stride;
+            stride *= a == 0 ? (unsigned)g.pitch : (unsigned)n[a];
+        }
+    }
+    template <class L, int I> __device__ __forceinline__ unsigned at() const
+    {
+        unsigned o = 0;
+        static_for<0, D>([&](auto Ai) {
+            constexpr int a = decltype(Ai)::value, e = L::E[I][a] + 1;
+            o += off[a][e];
+        });
+        return o;
+    }
+};
 template <int D, int EY, int EZ, int EW>
 __device__ __forceinline__ int64_t src_row(const Geom &g, const RowPos &r)
 {

@@ -111,16 +111,15 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
 {
     constexpr int D = L::D, B0 = 1 + 2 * D;
     // coordinates in 32-bit arithmetic (nodes <= 2^31)
-    const unsigned nd = (unsigned)node;
-    int c[4];
-    const unsigned rw = nd / (unsigned)g.N0;
-    c[0] = (int)(nd - rw * (unsigned)g.N0);
-    const unsigned r2 = rw / (unsigned)g.N1;
-    c[1] = (int)(rw - r2 * (unsigned)g.N1);
-    const unsigned r3 = r2 / (unsigned)g.N2;
-    c[2] = (int)(r2 - r3 * (unsigned)g.N2);
-    c[3] = (int)r3;
     const int n[4] = {g.N0, g.N1, g.N2, g.N3};
+    int c[4] = {0, 0, 0, 0};
+    unsigned left = (unsigned)node;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const unsigned q = a + 1 < D ? left / (unsigned)n[a] : 0u;
+        c[a] = (int)(left - q * (unsigned)n[a]);
+        left = q;
+    }
 
     // checks on the bit patterns (integer pipes): theta > 0 and finite, a
     // finite gradient (exponent field not all ones)
@@ -139,11 +138,11 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
     // periodic: destination offset = sum over axes of one of three wrapped
     // offsets (shift -1, 0, +1), formed once per node (a population has at most
     // 2^31 nodes and a row's padding each: below 2^32)
-    unsigned off[4][3];
+    unsigned off[4][3] = {};
     {
         unsigned stride = 1;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < D; ++a) {
             const int dn = c[a] == 0 ? n[a] - 1 : c[a] - 1;  // x_a - 1
             const int up = c[a] == n[a] - 1 ? 0 : c[a] + 1;  // x_a + 1
             off[a][0] = (unsigned)up * stride;               // e = -1 stores at x_a + 1
@@ -220,8 +219,8 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
             // The fixed-point formation below, on theta - theta_ref and dx grad
             // aligned to the larger exponent (f64_align_round: 60 bits), each
             // population rounded once to FP32: 1 + D FP64 instructions in place of
-            // 16 (2D; 85 % of that pipe).  1999 x 1501: 145 -> 68 us, 101 x 90 x 77:
-            // 70 -> 32 us.
+            // 16 (2D; 85 % of that pipe).  1999 x 1501: 145 -> 66 us, 101 x 90 x 77:
+            // 70 -> 33 us.
             double x[1 + D];
             x[0] = dth;
 #pragma unroll
