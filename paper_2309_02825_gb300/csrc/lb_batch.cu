@@ -7,7 +7,10 @@
 // instance descriptor once and then runs the same pull + collide as the
 // single-grid sweep.  Groups are sized so that their two buffers stay in
 // L2 while the group runs all its steps back to back; the launches are
-// replayed from CUDA graphs.
+// replayed from CUDA graphs.  Batches large enough to fill the device take
+// several steps per launch instead: marching windows over all instances
+// (lb_march.cu; march_worth says from which size), or, where asked for or found
+// faster by lb_batch_autotune, square tiles in shared memory (batch_tb_kernel).
 #include <math.h>
 #include <string.h>
 
@@ -629,9 +632,9 @@ lb_status build_tiles(lb_batch *b, int K, int tile, int threads)
 
 // Whether a new batch takes marching launches over one launch per step.
 // Measured GLUPS, march / one launch per step in 96 MB groups, by total nodes:
-//   FP32: 21.4M 230 / 90, 3.8M 178 / 93, 0.65M 129 / 73, 0.41M 89 / 63, 0.05M 12.6 / 10.4
-//   fixed point: 21.4M 108 / 43, 3.8M 92 / 44, 0.65M 55 / 42, 0.41M 54 / 41, 0.05M 8.6 / 10.2
-//   FP64: 21.4M 45 / 20, 3.8M 41 / 21, 0.65M 26 / 15, 0.41M 20 / 15, 0.05M 2.9 / 6.3
+//   FP32: 21.4M 236 / 90, 3.8M 197 / 94, 0.65M 129 / 73, 0.41M 108 / 65, 0.05M 17.6 / 11.6
+//   fixed point: 21.4M 105 / 43, 3.8M 88 / 44, 0.65M 59 / 42, 0.41M 54 / 41, 0.05M 8.6 / 10.2
+//   FP64: 21.4M 45 / 20, 3.8M 42 / 21, 0.65M 24 / 15, 0.41M 26 / 15, 0.05M 2.9 / 6.3
 bool march_worth(const lb_batch *b)
 {
     return b->total_nodes >= (b->precision == LB_FP32_SHIFTED ? 40000 : (b->precision == LB_FX64 ? 200000 : 350000));

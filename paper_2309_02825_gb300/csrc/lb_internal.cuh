@@ -179,8 +179,8 @@ struct CollF64 {
     CollFx x;
     int ints;
 };
-constexpr int kFxCoefBits = 62;  // initialisation and adjoint constants
-constexpr int kFxCollBits = 64;  // collision constants (CollFx)
+constexpr int kFxCoefBits = 62;  // constants outside (-1/2, 1/2) (mulfx)
+constexpr int kFxCollBits = 64;  // constants of mulfx_c: collision, initialisation, adjoint
 
 // Recovery constants (Sec. III.C): u_a = ucoef * J_a / theta with
 // ucoef = (2 - s1) c; grad_a = gcoef * J_a with gcoef = -s1 / (sigma dx);
@@ -198,7 +198,8 @@ struct InitK {
     double fxscale;  // 2^F for 64-bit fixed-point storage, unused otherwise
     // 64-bit fixed point formed in integers: theta -> round(theta 2^F), a
     // gradient component -> round(dx grad 2^F) (gscale = dx 2^F), and the
-    // constants w1, wd, iax/dx with kFxCoefBits fraction bits.
+    // constants w1, wd, iax/dx with kFxCollBits fraction bits (mulfx_c), or
+    // kFxCoefBits where one leaves its range.
     double gscale;
     // FP32 storage forms its values the same way in a unit of the node's own
     // where the constants allow it (ints).
