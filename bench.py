@@ -64,7 +64,7 @@ def parse():
                    help="one N^2 FX64 grid cut into one slab per rank (ghost-layer exchange every step) instead of "
                         "independent replicas: strong scaling")
     p.add_argument("--no-blocking", action="store_true",
-                   help="one sweep per launch only (skip the autotuner's blocked candidates)")
+                   help="one sweep per launch only (no autotuned choice of several steps per launch)")
     p.add_argument("--no-variant", action="store_true", help="skip the other precisions' sub-results")
     p.add_argument("--no-batched", action="store_true", help="skip the batched 512-instance measurement")
     p.add_argument("--no-adjoint", action="store_true", help="skip the 512^2 adjoint measurement")
@@ -82,7 +82,7 @@ def parse():
                    help="run STEPS sweeps of one D-dimensional N^D grid at PREC and exit (for ncu captures)")
     p.add_argument("--blocking", default=None, metavar="K,TILE,THREADS",
                    help="blocked sweeps of K steps per launch for the headline step (instead of the autotuner's "
-                        "pick) or for --profile-sweep")
+                        "pick) or for --profile-sweep; there 'auto' takes the library's own choice")
     return p.parse_args()
 
 
@@ -112,13 +112,13 @@ def kernel_source_sha():
 
 
 def blocked_source_sha():
-    """sha256 (16 hex digits) of the blocked kernel's sources (comments and
-    whitespace removed)."""
+    """sha256 (16 hex digits) of the sources of the kernels that take several
+    steps per launch (comments and whitespace removed)."""
     import hashlib
     import re
     csrc = os.path.join(ROOT, "paper_2309_02825_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("lb_internal.cuh", "lb_device.cuh", "lb_batch.cu"):
+    for name in ("lb_internal.cuh", "lb_device.cuh", "lb_batch.cu", "lb_march.cu"):
         text = open(os.path.join(csrc, name)).read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)
         text = re.sub(r"//[^\n]*", " ", text)
@@ -147,20 +147,10 @@ def blocked_launch_bytes(N0, N1, K, tile, elem, q=9):
     return blocked_bytes_per_lu([(N0, N1)], K, tile, elem, q) * N0 * N1 * K
 
 
-def profile_fp64_inst(kernel_key):
-    """FP64 instructions per lattice update (thread-level, i.e. 32 x the warp
-    instructions ncu counts in sm__inst_executed_pipe_fp64.sum, per node) of a
-    sweep, from a committed ncu summary; valid only while the kernel source is
-    unchanged (same sha)."""
-    try:
-        sha = kernel_source_sha()
-        for line in open(os.path.join(ROOT, "profiles", "fp64_inst.txt")):
-            parts = line.split()
-            if len(parts) >= 3 and parts[0] == kernel_key and parts[1] == sha:
-                return float(parts[2])
-    except OSError:
-        pass
-    return None
+def is_march(choice):
+    """Whether an autotuned choice is marching windows (blocks of two or four
+    warps) and not square tiles (blocks of 256 threads and more)."""
+    return choice["steps_per_launch"] > 0 and 0 < choice["threads"] < 256
 
 
 def profile_traffic(kernel_key):
@@ -300,8 +290,10 @@ def run_ours(args, precision, world, rank, local, peaks, with_e2e, label_main, b
         elif blocking and not args.no_blocking:
             tune = s.autotune(24)
         else:
+            s.set_blocking(0)  # a fresh solver takes several steps per launch by itself
             tune = {"steps_per_launch": 0}
     K = tune["steps_per_launch"]
+    march = is_march(tune)
     th = torch.empty(tuple(reversed(N)), dtype=torch.float64, device="cuda")
     gr = torch.empty((d,) + tuple(reversed(N)), dtype=torch.float64, device="cuda")
     u = torch.empty_like(gr)
@@ -367,21 +359,24 @@ def run_ours(args, precision, world, rank, local, peaks, with_e2e, label_main, b
             "peak_source": peaks["source"],
         }
     else:
-        # blocked: K sweeps per launch in shared memory, bound by instruction
-        # issue (4 warp instructions per SM per clock); its HBM traffic is the
-        # tiles with their halos
+        # K sweeps per launch in shared memory, bound by instruction issue (4
+        # warp instructions per SM per clock).  Its HBM traffic is the tiles with
+        # their halos, or for marching windows each population read once and
+        # written once (the windows' overlaps hit in L2)
         launch_s = sweep_ms / 1e3 * K
-        key = "blocked_d2q9_%s_%d_K%d_T%d_TH%d" % (precision, args.N, K, tune["tile"], tune["threads"])
+        key = "%s_d2q9_%s_%d_K%d_T%d_TH%d" % ("march" if march else "blocked", precision, args.N, K, tune["tile"],
+                                              tune["threads"])
         inst, dram = profile_blocked(key)
         peak_issue = 4 * sms * sm_mhz * 1e6 / 1e9
         ach_issue = None if inst is None else inst / launch_s / 1e9
-        blk_bytes = blocked_launch_bytes(N[0], N[1], K, tune["tile"], elem)
+        blk_bytes = bytes_lu * nodes if march else blocked_launch_bytes(N[0], N[1], K, tune["tile"], elem)
         roofline = {
             "bound": "alu", "achieved": ach_issue, "peak": peak_issue, "unit": "G warp-inst/s",
             "frac": None if ach_issue is None else ach_issue / peak_issue,
             "traffic": dram,
-            "kernel": "batch_tb_kernel<D2Q9,%s,%d> (%d sweeps per launch, tiles of %d)" % (
-                ctype, tune["threads"], K, tune["tile"]),
+            "kernel": "%s<D2Q9,%s,%d> (%d sweeps per launch, %s of %d)" % (
+                "march_kernel" if march else "batch_tb_kernel", ctype, tune["threads"], K,
+                "windows" if march else "tiles", tune["tile"]),
             "warp_inst_per_launch": inst, "sms": sms, "sm_mhz": sm_mhz,
             "peak_source": "4 warp instructions per SM per clock x SMs x sampled SM clock",
             "algorithmic_bytes_per_launch": blk_bytes,
@@ -403,22 +398,11 @@ def run_ours(args, precision, world, rank, local, peaks, with_e2e, label_main, b
                   "u_rel_l2": math.sqrt(sum(norms["u%d" % a]["rel_l2"] ** 2 for a in range(d)) / d),
                   "sum_theta_drift": abs(out["total"] - float(th0_h.sum())) / float(th0_h.sum())},
         "clocks": clk,
-        "gpu_launches": args.steps * ((S // K + (1 if S % K else 0) if K else S) + 6 + (2 if precision == "fx64" else 0)),
+        # sweeps (a marching schedule's remainder is single sweeps, a tiled one's a launch), then flags, initialisation,
+        # recovery, and two launches each for the total, the norms and (fixed point) max|theta0|
+        "gpu_launches": args.steps * ((S // K + (S % K if march else min(1, S % K)) if K else S) + 7
+                                      + (2 if precision == "fx64" else 0)),
     }
-    if precision == "fp64" and K == 0:
-        # The FP64 sweep is bound by the FP64 pipe: GB300 issues 2 FP64 lane
-        # operations per SM per clock (1/64 of FP32).  The instructions per
-        # update come from an ncu capture of this kernel source (null when the
-        # kernel changed since), the SM count from the device.
-        peak_inst = sms * 2 * sm_mhz * 1e6 / 1e9
-        ipl = profile_fp64_inst("sweep_d2q9_fp64")
-        ach_inst = None if ipl is None else ipl * nodes / (sweep_ms / 1e3) / 1e9
-        res["roofline_fp64_pipe"] = {"bound": "alu", "achieved": ach_inst, "peak": peak_inst,
-                                     "unit": "G FP64 lane-ops/s",
-                                     "frac": None if ach_inst is None else ach_inst / peak_inst,
-                                     "fp64_inst_per_lu": ipl, "sms": sms, "sm_mhz": sm_mhz,
-                                     "fp64_inst_source": "profiles/fp64_inst.txt (ncu sm__inst_executed_pipe_fp64)"}
-
     if with_e2e:
         res["e2e"] = run_e2e(args, s, case, th0_h, g0_h, ex_t_h, ex_u_h, stream, world)
     s.close()
@@ -517,7 +501,7 @@ def blocked_bytes_per_lu(sizes, K, tile, elem, q=9):
 def run_batched(local):
     """512 independent 2D instances (N log-uniform in [32, 512], nu log-uniform
     in [0.005, 0.1], dt = 4 dx^2), FP32 shifted, 2000 steps: the autotuned
-    schedule (blocked launches of K steps in shared memory, or one launch per
+    schedule (marching windows or tiles of K steps per launch, or one launch per
     step) vs one launch per instance per step vs one flat launch per step."""
     import torch
     from paper_2309_02825_gb300 import lb
@@ -582,11 +566,14 @@ def run_batched(local):
 
     def roof(choice, t, elem):
         """Per-step-equivalent fraction (2 q elem bytes per update, what one
-        launch per step must move) and, for blocked launches, the fraction of
-        the bytes they do move."""
+        launch per step must move) and, for launches of several steps, the
+        fraction of the bytes they do move."""
         out = {"per_step_equivalent_hbm_frac": 2 * 9 * elem * lu / t / 1e9 / peak}
         if choice["steps_per_launch"]:
-            bpl = blocked_bytes_per_lu(sizes, choice["steps_per_launch"], choice["tile"], elem)
+            if is_march(choice):  # each population read and written once per launch
+                bpl = 2 * 9 * elem / choice["steps_per_launch"]
+            else:
+                bpl = blocked_bytes_per_lu(sizes, choice["steps_per_launch"], choice["tile"], elem)
             out.update({"blocked_bytes_per_lu": bpl, "blocked_hbm_gbs": bpl * lu / t / 1e9,
                         "blocked_hbm_frac": bpl * lu / t / 1e9 / peak})
         return out
@@ -776,8 +763,9 @@ def _run_case(case, precision, theta_ref, stream, th0=None, g0=None, nsteps=None
 
 
 def run_3d(local, peaks):
-    """3D D3Q19 periodic 256^3 (the 3D Fourier family): sweep throughput and
-    %HBM for each precision, and the error against the exact solution at
+    """3D D3Q19 periodic 256^3 (the 3D Fourier family): sweep throughput for
+    each precision, its rate of the bytes that one sweep per launch moves (a
+    marching launch of several steps moves fewer), and the error against the exact solution at
     t_end = 0.02 (256 steps)."""
     import torch
     from paper_2309_02825_gb300 import lb
@@ -805,8 +793,8 @@ def run_3d(local, peaks):
         gbs = 2 * 19 * elem * case.nodes / (ms / 1e3) / 1e9
         err = _run_case(case, prec, 1.5, stream, th0, g0, exact=exact)
         out[prec] = {"sweep_ms": ms, "mlups": case.nodes / (ms / 1e3) / 1e6, "bytes_per_lu": 2 * 19 * elem,
-                     "hbm_frac": gbs / peaks["hbm_gbs"], "achieved_gbs": gbs, "error_t_end": err,
-                     "traffic": profile_traffic("sweep_d3q19_%s_256" % prec)}
+                     "per_step_equivalent_hbm_frac": gbs / peaks["hbm_gbs"], "error_t_end": err,
+                     "traffic_one_sweep_per_launch": profile_traffic("sweep_d3q19_%s_256" % prec)}
     return out
 
 
@@ -846,7 +834,7 @@ def run_walls(local, peaks):
         s.close()
         gbs = 2 * 9 * 8 * n * n / (ms / 1e3) / 1e9
         out["sweep_2d_4096_fx64_" + kind] = {"sweep_ms": ms, "mlups": n * n / (ms / 1e3) / 1e6,
-                                              "hbm_frac": gbs / peaks["hbm_gbs"]}
+                                              "per_step_equivalent_hbm_frac": gbs / peaks["hbm_gbs"]}
     c3 = W.fourier_3d(256)
     th3 = torch.from_numpy(c3.problem.theta(c3.N, c3.dx)).cuda()
     g3 = torch.from_numpy(np.ascontiguousarray(c3.problem.grad(c3.N, c3.dx))).cuda()
@@ -864,7 +852,7 @@ def run_walls(local, peaks):
         s.close()
         gbs = 2 * 19 * 8 * c3.nodes / (ms / 1e3) / 1e9
         out["sweep_3d_256_fx64_" + kind] = {"sweep_ms": ms, "mlups": c3.nodes / (ms / 1e3) / 1e6,
-                                             "hbm_frac": gbs / peaks["hbm_gbs"]}
+                                             "per_step_equivalent_hbm_frac": gbs / peaks["hbm_gbs"]}
     ex1 = {}
     for eps in (0.5, 1.0, 1.5, 2.0):
         rows = {"theta": [], "u": []}
@@ -1009,13 +997,16 @@ def run_profile_sweep(local, spec, blocking=None):
     else:
         prob, N, nu, dx, dt = case.problem, case.N, case.nu, case.dx, case.dt
     s = lb.Solver(d, N, nu, dx, dt, precision=prec, theta_ref=1.5)
-    blk = [int(v) for v in blocking.split(",")] if blocking else None
-    if blk:
-        s.set_blocking(*blk)
+    blk = [int(v) for v in blocking.split(",")] if blocking and blocking != "auto" else None
+    if d == 2 and blocking != "auto":
+        s.set_blocking(*(blk or (0,)))
     s.set_theta0(torch.from_numpy(prob.theta(N, dx)).cuda(),
                  torch.from_numpy(np.ascontiguousarray(prob.grad(N, dx))).cuda())
-    for _ in range(steps // blk[0] if blk else steps):
-        s.step(blk[0] if blk else 1)
+    if blocking == "auto":
+        s.step(steps)
+    else:
+        for _ in range(steps // blk[0] if blk else steps):
+            s.step(blk[0] if blk else 1)
     th, _, u = s.macros(want=("theta", "u"))
     s.sum_theta()
     T = steps * dt
@@ -1180,11 +1171,9 @@ def main():
             v = run_ours(args, other, world, rank, local, peaks, False, False)
             entry = {"precision": other, "value": v["value"], "unit": UNIT, "roofline": v["roofline"],
                      "error": v["error"], "sweep_ms": v["sweep_ms"], "blocking": v["blocking"]}
-            if "roofline_fp64_pipe" in v:
-                entry["roofline_fp64_pipe"] = v["roofline_fp64_pipe"]
             if other == "fp64":
-                entry["note"] = ("native FP64 arithmetic, bound by the FP64 pipe (1/64 of the FP32 rate on this part); "
-                                 "the FP64-accurate result at the HBM rate and beyond is the 64-bit fixed-point line")
+                entry["note"] = ("FP64 storage; each collision on the node's 64-bit integers aligned to its largest "
+                                 "exponent, since the FP64 pipe has 1/64 of the FP32 rate on this part")
             variants.append(entry)
     batched = None
     if not args.no_batched:
@@ -1239,8 +1228,6 @@ def main():
         line["blocking"] = main_res["blocking"]
         if per_step:
             line["one_sweep_per_launch"] = per_step
-        if "roofline_fp64_pipe" in main_res:
-            line["roofline_fp64_pipe"] = main_res["roofline_fp64_pipe"]
         if variants:
             line["variants"] = variants
         if batched:
