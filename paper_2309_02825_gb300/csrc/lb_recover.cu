@@ -251,12 +251,13 @@ __global__ void __launch_bounds__(kTile) recover_kernel(const T *__restrict__ sr
 // that leave much of the staged kernel's 256-node tiles idle (a 50-node row: 80
 // %).  Each population is one load at its wrapped or reflected source;
 // neighbouring threads read neighbouring elements, so the loads stay coalesced
-// across row ends.  50^4 fixed point: 1274 -> 300 us (2.1 GB of state and fields).
+// across row ends.  50^4 fixed point: 1274 -> 300 us (2.1 GB of state and fields),
+// with all 33 loads in flight: without a count of resident blocks the compiler takes
+// 68 registers instead of 92 there and adds between the loads, 346 us.
 template <class L, typename T, bool MIR>
-__global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
-                                                           double *__restrict__ theta, double *__restrict__ grad,
-                                                           double *__restrict__ u, int *__restrict__ flag, int64_t row0,
-                                                           int64_t nrow)
+__device__ __forceinline__ void recover_flat(const T *__restrict__ src, const Geom &g, const Recov &r, double scale,
+                                             double *__restrict__ theta, double *__restrict__ grad,
+                                             double *__restrict__ u, int *__restrict__ flag, int64_t row0, int64_t nrow)
 {
     const int64_t nodes = (int64_t)g.N0 * nrow;
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -291,6 +292,24 @@ __global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__
         vals[i] = __ldg(src + (int64_t)pop * g.slab + ps.row * g.pitch + sx);
     });
     recover_node<L, T>(vals, r, scale, nodes, n, theta, grad, u, flag);
+}
+
+template <class L, typename T, bool MIR>
+__global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
+                                                           double *__restrict__ theta, double *__restrict__ grad,
+                                                           double *__restrict__ u, int *__restrict__ flag, int64_t row0,
+                                                           int64_t nrow)
+{
+    recover_flat<L, T, MIR>(src, g, r, scale, theta, grad, u, flag, row0, nrow);
+}
+// The same with a register budget for five blocks per SM (4D fixed point).
+template <class L, typename T, bool MIR>
+__global__ void __launch_bounds__(128, 5) recover_flat5_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
+                                                               double *__restrict__ theta, double *__restrict__ grad,
+                                                               double *__restrict__ u, int *__restrict__ flag, int64_t row0,
+                                                               int64_t nrow)
+{
+    recover_flat<L, T, MIR>(src, g, r, scale, theta, grad, u, flag, row0, nrow);
 }
 
 // All 2D instances of a batch in one launch: the flat recovery of each node's
@@ -362,8 +381,13 @@ static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr,
     if (blocks == 0) return cudaSuccess;
     if (c->geom.N0 * 4 < tiles * kTile * 3) {  // under three quarters of the tiles' nodes
         const int64_t nodes = nrow * c->geom.N0;
-        recover_flat_kernel<L, T, MIR><<<(unsigned)((nodes + 127) / 128), 128, 0, c->stream>>>(
-            (const T *)src, c->geom, r, scale, th, gr, u, flag, row0, nrow);
+        const unsigned nb = (unsigned)((nodes + 127) / 128);
+        if constexpr (L::D == 4 && std::is_same<T, long long>::value)
+            recover_flat5_kernel<L, T, MIR><<<nb, 128, 0, c->stream>>>((const T *)src, c->geom, r, scale, th, gr, u, flag,
+                                                                        row0, nrow);
+        else
+            recover_flat_kernel<L, T, MIR><<<nb, 128, 0, c->stream>>>((const T *)src, c->geom, r, scale, th, gr, u, flag,
+                                                                       row0, nrow);
         return cudaGetLastError();
     }
     recover_kernel<L, T, MIR><<<(unsigned)blocks, kTile, smem, c->stream>>>((const T *)src, c->geom, r, scale, th,
