@@ -49,45 +49,77 @@ bool context_id(unsigned long long *id)
     return ((CUresult(CUDAAPI *)(CUcontext, unsigned long long *))fn)(nullptr, id) == CUDA_SUCCESS;
 }
 
-// Page-locked areas of destroyed solvers, kept for the next ones (page-locking
-// takes about 300 us): a bounded number for the process, from any thread, and
-// only within the CUDA context that made them, so that what a cudaDeviceReset
-// has released is not handed out again.
-constexpr int kAreasKept = 32;
-struct Area {
-    void *p;
-    unsigned long long context;
+// Page-locked areas, cut from slabs of 64 (page-locking takes about 300 us
+// whatever the size).  From any thread, and only within the CUDA context that
+// made a slab, so that what a cudaDeviceReset has released is not handed out
+// again.  A slab without solvers is released unless it is its context's only one
+// with room.
+constexpr size_t kAreaPitch = (kHostArea + 127) / 128 * 128;
+constexpr int kSlabAreas = 64;
+struct AreaSlab {
+    char *host, *dev;
+    unsigned long long context, used;  // a bit per area
 };
-std::mutex g_areas_mutex;
-Area g_areas[kAreasKept];
-int g_nareas = 0;
+std::mutex g_slabs_mutex;
+std::vector<AreaSlab> g_slabs;
 
 cudaError_t take_area(lb_ctx *c)
 {
-    c->host_context = 0;
-    if (context_id(&c->host_context)) {
-        std::lock_guard<std::mutex> lock(g_areas_mutex);
-        for (int k = g_nareas; k-- > 0;) {
-            if (g_areas[k].context != c->host_context) continue;
-            c->host_area = g_areas[k].p;
-            g_areas[k] = g_areas[--g_nareas];
-            return cudaSuccess;
+    unsigned long long id = 0;
+    const bool shared = context_id(&id);
+    std::lock_guard<std::mutex> lock(g_slabs_mutex);
+    AreaSlab *slab = nullptr;
+    for (AreaSlab &s : g_slabs)
+        if (shared && s.context == id && s.used != ~0ull) slab = &s;
+    AreaSlab own{};
+    if (!slab) {
+        cudaError_t e = cudaHostAlloc((void **)&own.host, kAreaPitch * (shared ? kSlabAreas : 1), cudaHostAllocMapped);
+        if (e != cudaSuccess) return e;
+        if ((e = cudaHostGetDevicePointer((void **)&own.dev, own.host, 0)) != cudaSuccess) {
+            cudaFreeHost(own.host);
+            return e;
+        }
+        own.context = id;
+        slab = &own;
+        if (shared) {
+            g_slabs.push_back(own);
+            slab = &g_slabs.back();
         }
     }
-    return cudaHostAlloc(&c->host_area, kHostArea, cudaHostAllocMapped);
+    int k = 0;
+    while ((slab->used >> k) & 1u) ++k;
+    slab->used |= 1ull << k;
+    c->host_context = id;
+    c->host_area = slab->host + k * kAreaPitch;
+    c->dout = (double *)(slab->dev + k * kAreaPitch);
+    return cudaSuccess;
 }
 
 void give_area(lb_ctx *c)  // its stream has been waited for
 {
     if (!c->host_area) return;
-    if (c->host_context != 0) {
-        std::lock_guard<std::mutex> lock(g_areas_mutex);
-        if (g_nareas < kAreasKept) {
-            g_areas[g_nareas++] = {c->host_area, c->host_context};
-            return;
-        }
+    char *const p = (char *)c->host_area;
+    std::lock_guard<std::mutex> lock(g_slabs_mutex);
+    bool room = false;  // in another slab of the same context
+    size_t mine = g_slabs.size();
+    for (size_t k = 0; k < g_slabs.size(); ++k) {
+        const AreaSlab &s = g_slabs[k];
+        if (s.context != c->host_context) continue;
+        if (p >= s.host && p < s.host + kAreaPitch * kSlabAreas)
+            mine = k;
+        else
+            room = room || s.used != ~0ull;
     }
-    cudaFreeHost(c->host_area);
+    if (mine == g_slabs.size()) {  // an area of its own
+        cudaFreeHost(p);
+        return;
+    }
+    AreaSlab &s = g_slabs[mine];
+    s.used &= ~(1ull << ((p - s.host) / kAreaPitch));
+    if (s.used == 0 && room) {
+        cudaFreeHost(s.host);
+        g_slabs.erase(g_slabs.begin() + (long)mine);
+    }
 }
 
 void free_ctx(lb_ctx *c)
@@ -367,8 +399,7 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     if (sms > 0) c->sms = sms;
     c->scratch_blocks = c->sms * 4;
     if ((e = cudaMalloc(&c->scratch, sizeof(double) * lbk::kRedSlots * c->scratch_blocks)) != cudaSuccess ||
-        (e = take_area(c)) != cudaSuccess ||
-        (e = cudaHostGetDevicePointer((void **)&c->dout, c->host_area, 0)) != cudaSuccess) {
+        (e = take_area(c)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: scratch allocation");
     }
