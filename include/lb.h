@@ -190,6 +190,8 @@ lb_status lb_set_theta0(lb_ctx *ctx, const double *theta0, const double *grad_th
  * moment space (m* = m - S (m - m^eq), m^eq = M w theta) and stored.
  * Asynchronous.  For LB_FX64 every stored value is checked against
  * |f| < 2^61 (reported by lb_macros, lb_sum_theta or lb_check).
+ * Captured into the caller's graph, an even nsteps ends in the buffer it
+ * began in, so replays of the graph continue from one another.
  * Errors: LB_EINVAL (nsteps < 0), LB_ESTATE (no
  * lb_set_theta0 yet, or a reported timeout or range overflow since), LB_ECUDA.
  */
