@@ -61,7 +61,7 @@ struct AreaSlab {
     unsigned long long context, used;  // a bit per area
 };
 std::mutex g_slabs_mutex;
-std::vector<AreaSlab> g_slabs;
+std::vector<AreaSlab> &g_slabs = *new std::vector<AreaSlab>;  // never destroyed: solvers may be closed at exit
 
 cudaError_t take_area(lb_ctx *c)
 {
