@@ -343,17 +343,26 @@ struct EpsFx {
     }
 };
 
-// Range of the fixed-point adjoint fields: |v| < 2^kAdjBits (they start below
-// 2^56 and grow by less than 1.3x), so that the next step's channels fit 63
-// bits: 2d + 2d and 2d(d-1) + 2d(d-1) terms at most, 8 for d = 2, 24 for d = 3.
+// Range of the integers that adj_node_fx takes: |v| < 2^adj_bits, so that its
+// channel sums fit 63 bits: 2d + 2d and 2d(d-1) + 2d(d-1) terms, 8 at most for
+// d = 2, 24 for d = 3 (and stay inside mulfx_c's range).  Fixed-point fields
+// start below 2^56, grow by less than 1.3x and are checked; FP64 fields are
+// aligned below it (adj_node_f64).
 template <class L> __host__ __device__ constexpr int adj_bits() { return L::D <= 2 ? 59 : 58; }
+template <class L> __host__ __device__ constexpr int adj_terms()
+{
+    return L::D == 1 ? 4 : 4 * L::D * (L::D - 1);
+}
+static_assert(adj_terms<D1Q3>() < 1 << (63 - adj_bits<D1Q3>()) && adj_terms<D2Q9>() < 1 << (63 - adj_bits<D2Q9>()) &&
+                  adj_terms<D3Q19>() < 1 << (63 - adj_bits<D3Q19>()),
+              "channel sums of the reverse step");
 
 // The node update of the fixed-point reverse pass (64-bit fixed-point states):
 // K^T from exact integer channel sums and the collision's own rounded products
 // (mulfx_c, the forward step's constants); with NU, adds the eps-term's dot
 // products to ep.  ORs into `rng` the high words of the outputs plus
-// 2^(kAdjBits - 32): an output is inside the range exactly when that sum stays
-// below 2^(kAdjBits - 31).
+// 2^(adj_bits - 32): an output is inside the range exactly when that sum stays
+// below 2^(adj_bits - 31).
 template <class L, bool NU>
 __device__ __forceinline__ void adj_node_fx(long long *l, const long long *fv, const AdjK &K, unsigned &rng, EpsFx &ep)
 {
@@ -417,14 +426,15 @@ __device__ __forceinline__ void adj_node_fx(long long *l, const long long *fv, c
 }
 
 // The node update of FP64 fields on the integer pipes (FP64 operations, 71 per
-// D2Q9 node, bind the direct form): lambda aligned to its largest exponent, the
-// bits below 2^-59 of it rounded off (the direct form rounds every step at 2^-53
-// of values that large), the state's doubles aligned without loss as in the
+// D2Q9 node, bind the direct form): lambda aligned to its largest exponent with
+// as many bits as adj_node_fx has room for, the bits below 2^-59 of the largest
+// (2^-58 for d = 3) rounded off (the direct form rounds every step at 2^-53 of
+// values that large), the state's doubles aligned without loss as in the
 // forward collision, then adj_node_fx, and each result rounded once.  Nodes
 // where either does not align take the direct form.
 template <class L, bool NU> __device__ __forceinline__ double adj_node_f64(double (&l)[L::Q], const double (&f)[L::Q], const AdjK &K)
 {
-    constexpr int PL = 6, PF = f64_align_bit<L>();
+    constexpr int PL = adj_bits<L>() - 53, PF = f64_align_bit<L>();  // a double has 53 bits
     if (K.ints) {
         long long lv[L::Q], fv[L::Q];
         unsigned el, ef = 0u;
