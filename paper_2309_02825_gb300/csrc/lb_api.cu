@@ -35,7 +35,8 @@ lb_status cuda_fail(lb_ctx *c, cudaError_t e, const char *where)
 
 bool finite_pos(double v) { return isfinite(v) && v > 0.0; }
 
-constexpr size_t kHostArea = 64 * sizeof(double) + 4 * sizeof(int);  // results, then flags
+constexpr int kFlags = 4;
+constexpr size_t kHostArea = 64 * sizeof(double) + kFlags * sizeof(int);  // results, then the flags' mirrors
 
 // The unique number of the calling thread's CUDA context; false where the driver has none.
 bool context_id(unsigned long long *id)
@@ -181,11 +182,14 @@ cudaError_t record_sweeps(lb_ctx *c, int from)
 int take_flag(lb_ctx *c, int k)
 {
     const int f = c->hflag[k];
-    if (f) c->hflag[k] = 0;
+    if (f) {
+        c->hflag[k] = 0;
+        cudaMemsetAsync(&c->dflag[k].bits, 0, sizeof(int), c->stream);
+    }
     return f;
 }
 
-// Read back and clear the recovery and range flags (ctx->dflag[1..2]) after
+// Read and clear the recovery and range flags (ctx->dflag[1..2]) after
 // the work enqueued so far; synchronises the stream.  A staging timeout or a
 // fixed-point range overflow leaves the context uninitialised: the state (or
 // a staging tile) may be corrupt, so lb_step and lb_macros refuse to run
@@ -398,15 +402,23 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (sms > 0) c->sms = sms;
     c->scratch_blocks = c->sms * 4;
-    if ((e = cudaMalloc(&c->scratch, sizeof(double) * lbk::kRedSlots * c->scratch_blocks)) != cudaSuccess ||
+    const size_t partials = (size_t)lbk::kRedSlots * c->scratch_blocks;
+    if ((e = cudaMalloc(&c->scratch, sizeof(double) * partials + sizeof(lbk::StatusFlag) * kFlags)) != cudaSuccess ||
         (e = take_area(c)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: scratch allocation");
     }
     memset(c->host_area, 0, kHostArea);
-    c->dflag = (int *)(c->dout + 64);
     c->hout = (volatile double *)c->host_area;
     c->hflag = (volatile int *)(c->hout + 64);
+    c->dflag = (lbk::StatusFlag *)(c->scratch + partials);
+    lbk::StatusFlag flags[kFlags] = {};
+    for (int k = 0; k < kFlags; ++k) flags[k].host = (int *)(c->dout + 64) + k;
+    // (from pageable memory: the source has been read when the call returns)
+    if ((e = cudaMemcpyAsync(c->dflag, flags, sizeof flags, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess) {
+        free_ctx(c);
+        return cuda_fail(nullptr, e, "lb_create: status flags");
+    }
     if ((e = choose_schedule(c)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: schedule");

@@ -160,7 +160,7 @@ template <class L, typename T, int TH, bool ONE>
 __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const InstDesc<T> *__restrict__ inst,
                                                                      const TileDesc *__restrict__ tiles,
                                                                      const T *__restrict__ src, T *__restrict__ dst,
-                                                                     int K, int *__restrict__ range, OneGrid<T> one)
+                                                                     int K, StatusFlag *__restrict__ range, OneGrid<T> one)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int Q = L::Q, NW = TH / 32;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
         }
     }
     if constexpr (std::is_same<T, long long>::value) {
-        if (range && __any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) atomicOr(range, 1);
+        if (range && __any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) raise_flag(range, 1);
     }
 }
 
@@ -383,7 +383,7 @@ struct lb_batch {
     void *d_desc = nullptr;
     int64_t *d_node_off = nullptr;
     double *d_err = nullptr;
-    int *d_flag = nullptr;
+    lbk::StatusFlag *d_flag = nullptr;  // initialisation, recovery (no mirrors)
     double *gradtmp = nullptr;
     double budget = 0;
     int threads = 256;
@@ -585,7 +585,7 @@ size_t tb_smem(const lb_batch *b, int K)
 // One blocked launch of K steps over every tile, from buffer `from`.
 cudaError_t launch_tb(lb_batch *b, int from, int K, cudaStream_t s)
 {
-    int *range = nullptr;
+    lbk::StatusFlag *range = nullptr;
     lbk::OneGrid<double> unused{};  // at least as large as the other types' (the kernel does not read it)
     static_assert(sizeof(lbk::OneGrid<double>) >= sizeof(lbk::OneGrid<long long>) &&
                       sizeof(lbk::OneGrid<double>) >= sizeof(lbk::OneGrid<float>),
@@ -823,7 +823,7 @@ template <typename T> static cudaError_t blocked_launch_t(lb_ctx *c, const void 
     one.ty = c->tb_ty;
     one.ntx = ((int)c->N[0] + c->tb_tx - 1) / c->tb_tx;
     const void *none = nullptr;
-    int *range = c->precision == LB_FX64 ? c->dflag + kFlagRange : nullptr;
+    StatusFlag *range = c->precision == LB_FX64 ? c->dflag + kFlagRange : nullptr;
     void *args[] = {&none, &none, (void *)&src, &dst, &K, &range, &one};
     const size_t smem = tb_smem_bytes(9, (int)c->elem, c->tb_tx + 2 * K, c->tb_ty + 2 * K);
     return cudaLaunchKernel(tb_kernel_for<T, true>(c->tb_threads), dim3((unsigned)c->tb_ntiles),
@@ -957,7 +957,7 @@ lb_status lb_batch_create(int count, const int64_t *N, const double *nu, const d
         e = cudaMemcpy(b->d_node_off, b->node_off.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_inst, sizeof(lbk::BatchInst) * count);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(double) * 4 * count);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_flag, sizeof(int) * 2);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_flag, sizeof(lbk::StatusFlag) * 2);
     if (e != cudaSuccess) {
         free_batch(b);
         return e == cudaErrorMemoryAllocation ? LB_ENOMEM : LB_ECUDA;
@@ -1010,7 +1010,7 @@ lb_status lb_batch_set_theta0(lb_batch *b, const double *theta0, const double *g
         if (!b->gradtmp && (e = cudaMalloc(&b->gradtmp, sizeof(double) * 2 * b->total_nodes)) != cudaSuccess)
             return bcuda(b, e, "lb_batch_set_theta0: gradient buffer");
     }
-    if ((e = cudaMemsetAsync(b->d_flag, 0, sizeof(int) * 2, b->stream)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(b->d_flag, 0, sizeof(lbk::StatusFlag) * 2, b->stream)) != cudaSuccess)
         return bcuda(b, e, "lb_batch_set_theta0");
     if (b->precision == LB_FX64) {
         // each instance's scale as for one grid: max|theta0_j| 2^F_j < 2^59
@@ -1049,7 +1049,7 @@ lb_status lb_batch_set_theta0(lb_batch *b, const double *theta0, const double *g
                                            grad0 ? grad0 : b->gradtmp, b->d_flag, b->stream)) != cudaSuccess)
         return bcuda(b, e, "lb_batch_set_theta0: init");
     int flag = 0;
-    if ((e = cudaMemcpyAsync(&flag, b->d_flag, sizeof(int), cudaMemcpyDeviceToHost, b->stream)) != cudaSuccess ||
+    if ((e = cudaMemcpyAsync(&flag, &b->d_flag[0].bits, sizeof(int), cudaMemcpyDeviceToHost, b->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(b->stream)) != cudaSuccess)
         return bcuda(b, e, "lb_batch_set_theta0");
     if (flag & 1) return bfail(b, LB_ENONPOS, "lb_batch_set_theta0: theta0 must be finite and > 0");
@@ -1111,7 +1111,7 @@ lb_status lb_batch_errors(lb_batch *b, const double *theta, const double *u, con
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(out, b->d_err, sizeof(double) * 4 * b->count, cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&flag, b->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+        e = cudaMemcpyAsync(&flag, &b->d_flag[1].bits, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "lb_batch_errors");
     if (flag & 4) return bfail(b, LB_ETIMEOUT, "lb_batch_macros: a shared-memory staging wait timed out");

@@ -20,6 +20,14 @@ __device__ __forceinline__ void static_for(F &&f)
     }
 }
 
+// Sets bits of a status flag; the same bits for all threads of a call.
+__device__ __forceinline__ void raise_flag(StatusFlag *f, int bits)
+{
+    if ((*(volatile int *)&f->bits & bits) == bits) return;
+    if ((int)(threadIdx.x & 31) != __ffs((int)__activemask()) - 1) return;  // one thread of the warp
+    if ((atomicOr(&f->bits, bits) & bits) != bits && f->host) atomicOr(f->host, bits);
+}
+
 __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // The instance of node n in the concatenated numbering of a batch (node_off:
@@ -1065,7 +1073,7 @@ __global__ void __launch_bounds__(sweep_threads<T>()) sweep_kernel(const T *__re
                 for (int i = 0; i < L::Q; ++i) acc |= (unsigned)((unsigned long long)f[i][v] >> 32) + 0x20000000u;
             }
         }
-        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) atomicOr(k.range, 1);
+        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) raise_flag(k.range, 1);
     }
 
     if (x0 + V * lane >= g.pitch) return;  // beyond the row: loads only
@@ -1113,7 +1121,7 @@ __global__ void __launch_bounds__(sweep_threads<T>()) sweep_flat_kernel(const T 
 #pragma unroll
             for (int i = 0; i < L::Q; ++i) acc |= (unsigned)((unsigned long long)f[i] >> 32) + 0x20000000u;
         }
-        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) atomicOr(k.range, 1);
+        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) raise_flag(k.range, 1);
     }
     if (q >= g.rows * g.N0) return;  // past the last node: loads only
     T *dp = dst + row * g.pitch + x;

@@ -163,6 +163,16 @@ template <typename T> struct Coll {
 struct CollFx {
     long long k1, k2, k3, cA, wd;
 };
+// A status flag in device memory.  A kernel sets bits through raise_flag: the
+// first setting of a bit goes on to the mirror in page-locked host memory, so
+// that the host can read it without a copy; the rest stay in L2 (every warp of a
+// field gone bad would send an atomic over the host link otherwise: recovery of
+// 4096^2 non-positive nodes 5.7-6.1 ms).
+struct StatusFlag {
+    int bits, unused;
+    int *host;  // mirror, or nullptr
+};
+
 // The single-grid fixed-point sweep also checks every value it stores
 // against |v| < 2^61 and sets *range when one is not (an unstable custom
 // relaxation set grows the state until int64 would wrap; FP64 would reach
@@ -170,7 +180,7 @@ struct CollFx {
 // are exact, so a run whose values cross 2^61 is caught at the step it does,
 // unless that one step grows them from below 2^61 past 2^63 / q.
 struct CollFxR : CollFx {
-    int *range;
+    StatusFlag *range;
 };
 // FP64 storage: the constants as doubles, and with 64 fraction bits for the
 // collision formed on the integer pipes (used where ints != 0).
@@ -282,15 +292,15 @@ struct lb_ctx {
     int cur = 0;
     double *scratch = nullptr;     // reduction partials
     int scratch_blocks = 0;
-    // Results and status flags in page-locked host memory that kernels write
-    // directly (one block, host_area): a call that returns a number then waits for
-    // its kernels once and reads it, where it copied each value back and cleared
+    // Results and the status flags' mirrors in page-locked host memory that kernels
+    // write directly (one block, host_area): a call that returns a number then waits
+    // for its kernels once and reads it, where it copied each value back and cleared
     // the flags with operations of their own.
     void *host_area = nullptr;
     unsigned long long host_context = 0;  // number of the CUDA context that page-locked it, 0 unknown
     double *dout = nullptr;        // 64 results: device address
-    int *dflag = nullptr;          // status flags: device address
-    volatile double *hout = nullptr;  // the same, host addresses (read when the stream has been waited for)
+    lbk::StatusFlag *dflag = nullptr;  // status flags (device, behind scratch)
+    volatile double *hout = nullptr;   // results and the flags' mirrors: host addresses (read when the stream has been waited for)
     volatile int *hflag = nullptr;
     double *gradtmp = nullptr;     // FD gradient when none is supplied
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // recorded sweeps, by starting buffer
@@ -343,7 +353,7 @@ bool fx_constants_ok(const lb_ctx &c);
 CollF64 make_coll_f64(const lb_ctx &c);
 // Device flags of a context (ctx->dflag): 0 initialisation, 1 recovery
 // (bit 0: theta <= 0 or non-finite, bit 2: a staging wait timed out),
-// 2 fixed-point sweep range (CollFxR).
+// 2 fixed-point sweep range (CollFxR).  hflag holds their mirrors.
 constexpr int kFlagInit = 0, kFlagRecover = 1, kFlagRange = 2;
 
 constexpr int kRedThreads = 256;
@@ -352,18 +362,18 @@ constexpr int kRedSlots = 16;  // doubles per block partial (>= 3*(d+1)+1)
 // Launchers (lb_kernels.cu).  All enqueue on ctx->stream and return the
 // launch error.
 cudaError_t launch_fd4_grad(const lb_ctx *c, const double *theta0, double *grad);
-cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, int *flag);
+cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, StatusFlag *flag);
 cudaError_t launch_sweep(lb_ctx *c, const void *src, void *dst);
 // Recovery (lb_recover.cu); flag bit 0: theta <= 0 seen, bit 2: a staging wait timed out.
-cudaError_t launch_macros(lb_ctx *c, const void *src, double *theta, double *grad, double *u, int *flag);
+cudaError_t launch_macros(lb_ctx *c, const void *src, double *theta, double *grad, double *u, StatusFlag *flag);
 cudaError_t launch_sum_state(lb_ctx *c, const void *src, double *out_dev);
 // The same on rows row0 .. row0 + nrow - 1 of the grid only (rows = the
 // products of all axes but x, slowest last); the recovery's outputs then hold
 // those rows only.
 cudaError_t launch_sum_state_rows(lb_ctx *c, const void *src, double *out_dev, int64_t row0, int64_t nrow);
-cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *theta, double *grad, double *u, int *flag,
+cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *theta, double *grad, double *u, StatusFlag *flag,
                                int64_t row0, int64_t nrow);
-cudaError_t launch_clear_flags(int *flag, int n, cudaStream_t s);
+cudaError_t launch_clear_flags(StatusFlag *flag, int n, cudaStream_t s);
 cudaError_t launch_maxabs(lb_ctx *c, const double *x, int64_t n, double *out_dev);
 // 64-bit fixed-point path (lb_fx.cu).
 cudaError_t launch_sweep_fx(lb_ctx *c, const void *src, void *dst);
@@ -395,9 +405,9 @@ cudaError_t march_batch_launch(int precision, int variant, const void *desc, con
 Recov make_recov(const lb_ctx *c, double *scale);
 bool make_batch_inst(const lb_ctx *c, int64_t off, BatchInst *out);
 cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
-                              void *dst, const double *theta0, const double *grad, int *flag, cudaStream_t s);
+                              void *dst, const double *theta0, const double *grad, StatusFlag *flag, cudaStream_t s);
 cudaError_t launch_batch_recover(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
-                                 const void *src, double *theta, double *u, int *flag, cudaStream_t s);
+                                 const void *src, double *theta, double *u, StatusFlag *flag, cudaStream_t s);
 // Resident sweeps of a short 1D grid (lb_line.cu): whether it is one, and one
 // launch of any number of steps.
 bool line_fits(const lb_ctx *c);

@@ -107,7 +107,7 @@ __device__ __forceinline__ void init_fx(const long long (&v)[1 + L::D], const In
 template <class L, typename T, int FXI, bool MIR>
 __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, const InitK &K, int64_t node, int64_t nodes,
                                           const double *__restrict__ theta0, const double *__restrict__ grad,
-                                          int *__restrict__ flag)
+                                          StatusFlag *__restrict__ flag)
 {
     constexpr int D = L::D, B0 = 1 + 2 * D;
     // coordinates in 32-bit arithmetic (nodes <= 2^31)
@@ -133,7 +133,7 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
         bad |= ((__double_as_longlong(gr[a]) >> 52) & 0x7ff) == 0x7ff;
         if (MIR && ((g.mirror >> a) & 1u) && (c[a] == 0 || c[a] == n[a] - 1)) gr[a] = 0.0;
     }
-    if (bad) atomicOr(flag, 1);
+    if (bad) raise_flag(flag, 1);
 
     // periodic: destination offset = sum over axes of one of three wrapped
     // offsets (shift -1, 0, +1), formed once per node (a population has at most
@@ -253,13 +253,13 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
             put_d(std::integral_constant<int, B0 + 4 * p + 3>{}, fma(-K.idg, sm, bd));
         });
     }
-    if (range) atomicOr(flag, 2);
+    if (range) raise_flag(flag, 2);
 }
 
 template <class L, typename T, int FXI, bool MIR>
 __global__ void __launch_bounds__(kInitThreads) init_kernel(T *__restrict__ dst, Geom g, InitK K,
                                                             const double *__restrict__ theta0,
-                                                            const double *__restrict__ grad, int *__restrict__ flag)
+                                                            const double *__restrict__ grad, StatusFlag *__restrict__ flag)
 {
     const int64_t nodes = (int64_t)g.N0 * g.rows;
     const int64_t node = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
@@ -271,7 +271,7 @@ template <typename T, int FXI>
 __global__ void __launch_bounds__(kInitThreads) batch_init_kernel(const int64_t *__restrict__ node_off, int count,
                                                                   const BatchInst *__restrict__ inst, T *__restrict__ dst,
                                                                   const double *__restrict__ theta0,
-                                                                  const double *__restrict__ grad, int *__restrict__ flag)
+                                                                  const double *__restrict__ grad, StatusFlag *__restrict__ flag)
 {
     const int64_t n = (int64_t)blockIdx.x * kInitThreads + threadIdx.x;
     const int j = batch_instance(node_off, count, n);
@@ -558,12 +558,14 @@ __global__ void __launch_bounds__(kRedThreads) norms_kernel(const double *__rest
     block_reduce_store<NS>(a, op, partial + (int64_t)blockIdx.x * kRedSlots);
 }
 
-// Clears n status flags in stream order.
-__global__ void clear_flags_kernel(int *flag, int n)
+// Clears n status flags and their mirrors in stream order.
+__global__ void clear_flags_kernel(StatusFlag *flag, int n)
 {
-    if ((int)threadIdx.x < n) flag[threadIdx.x] = 0;
+    if ((int)threadIdx.x >= n) return;
+    flag[threadIdx.x].bits = 0;
+    *flag[threadIdx.x].host = 0;
 }
-cudaError_t launch_clear_flags(int *flag, int n, cudaStream_t s)
+cudaError_t launch_clear_flags(StatusFlag *flag, int n, cudaStream_t s)
 {
     clear_flags_kernel<<<1, 32, 0, s>>>(flag, n);
     return cudaGetLastError();
@@ -686,7 +688,7 @@ cudaError_t launch_fd4_grad(const lb_ctx *c, const double *theta0, double *grad)
 }
 
 template <class L, typename T, int FXI>
-static cudaError_t init_go(lb_ctx *c, const InitK &K, const double *theta0, const double *grad, int *flag)
+static cudaError_t init_go(lb_ctx *c, const InitK &K, const double *theta0, const double *grad, StatusFlag *flag)
 {
     const unsigned nb = (unsigned)((c->nodes + kInitThreads - 1) / kInitThreads);
     if (c->geom.mirror)
@@ -732,7 +734,7 @@ static int make_initk(const lb_ctx *c, InitK &K)
 }
 
 template <class L, typename T>
-static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, int *flag)
+static cudaError_t init_t(lb_ctx *c, const double *theta0, const double *grad, StatusFlag *flag)
 {
     InitK K;
     const int fxi = make_initk(c, K);
@@ -753,7 +755,7 @@ bool make_batch_inst(const lb_ctx *c, int64_t off, BatchInst *out)
 }
 
 cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
-                              void *dst, const double *theta0, const double *grad, int *flag, cudaStream_t s)
+                              void *dst, const double *theta0, const double *grad, StatusFlag *flag, cudaStream_t s)
 {
     const unsigned nb = (unsigned)((nodes + kInitThreads - 1) / kInitThreads);
     if (precision == LB_FX64)
@@ -765,7 +767,7 @@ cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count,
     return cudaGetLastError();
 }
 
-cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, int *flag)
+cudaError_t launch_init(lb_ctx *c, const double *theta0, const double *grad, StatusFlag *flag)
 {
     if (c->precision == LB_FX64) {
         switch (c->d) {

@@ -73,13 +73,13 @@ template <> struct RecAcc<long long> {
 template <class L, typename T>
 __device__ __forceinline__ void recover_store(double thm, const double (&Jd)[4], const Recov &r, int64_t nodes,
                                               int64_t node, double *__restrict__ theta, double *__restrict__ grad,
-                                              double *__restrict__ u, int *__restrict__ flag)
+                                              double *__restrict__ u, StatusFlag *__restrict__ flag)
 {
     const double thd = std::is_same<T, float>::value ? thm + r.theta_ref : thm;
     if (theta) theta[node] = thd;
     {  // theta > 0 and finite, as bit tests on the integer pipes
         const long long tb = __double_as_longlong(thd);
-        if (!(tb > 0) || ((tb >> 52) & 0x7ff) == 0x7ff) atomicOr(flag, 1);
+        if (!(tb > 0) || ((tb >> 52) & 0x7ff) == 0x7ff) raise_flag(flag, 1);
     }
     const double cu = quot_int(r.ucoef, thd);  // the storage scale is folded into ucoef and gcoef
 #pragma unroll
@@ -94,7 +94,7 @@ __device__ __forceinline__ void recover_store(double thm, const double (&Jd)[4],
 template <class L, typename T>
 __device__ __forceinline__ void recover_node(const T (&vals)[L::Q], const Recov &r, double scale, int64_t nodes,
                                              int64_t node, double *__restrict__ theta, double *__restrict__ grad,
-                                             double *__restrict__ u, int *__restrict__ flag)
+                                             double *__restrict__ u, StatusFlag *__restrict__ flag)
 {
     double thm, Jd[4];  // theta - theta_ref and J in storage units
     if constexpr (std::is_same<T, float>::value) {
@@ -177,7 +177,7 @@ __device__ __forceinline__ void recover_node(const T (&vals)[L::Q], const Recov 
 template <class L, typename T, bool MIR>
 __global__ void __launch_bounds__(kTile) recover_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
                                                        double *__restrict__ theta, double *__restrict__ grad,
-                                                       double *__restrict__ u, int *__restrict__ flag, int64_t row0,
+                                                       double *__restrict__ u, StatusFlag *__restrict__ flag, int64_t row0,
                                                        int64_t nrow)
 {
     constexpr int H = 16 / (int)sizeof(T);  // halo = one 16-byte vector
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kTile) recover_kernel(const T *__restrict__ sr
         });
     }
     if (!mbar_wait_bounded(barp, 0)) {
-        if (threadIdx.x == 0) atomicOr(flag, 4);
+        if (threadIdx.x == 0) raise_flag(flag, 4);
         // Give this block's copies a second bounded interval to land before its
         // shared memory goes away.  If that also runs out the block returns with
         // copies possibly still in flight; the host treats flag bit 2 as fatal
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kTile) recover_kernel(const T *__restrict__ sr
 template <class L, typename T, bool MIR>
 __device__ __forceinline__ void recover_flat(const T *__restrict__ src, const Geom &g, const Recov &r, double scale,
                                              double *__restrict__ theta, double *__restrict__ grad,
-                                             double *__restrict__ u, int *__restrict__ flag, int64_t row0, int64_t nrow)
+                                             double *__restrict__ u, StatusFlag *__restrict__ flag, int64_t row0, int64_t nrow)
 {
     const int64_t nodes = (int64_t)g.N0 * nrow;
     const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -297,7 +297,7 @@ __device__ __forceinline__ void recover_flat(const T *__restrict__ src, const Ge
 template <class L, typename T, bool MIR>
 __global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
                                                            double *__restrict__ theta, double *__restrict__ grad,
-                                                           double *__restrict__ u, int *__restrict__ flag, int64_t row0,
+                                                           double *__restrict__ u, StatusFlag *__restrict__ flag, int64_t row0,
                                                            int64_t nrow)
 {
     recover_flat<L, T, MIR>(src, g, r, scale, theta, grad, u, flag, row0, nrow);
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(128) recover_flat_kernel(const T *__restrict__
 template <class L, typename T, bool MIR>
 __global__ void __launch_bounds__(128, 5) recover_flat5_kernel(const T *__restrict__ src, Geom g, Recov r, double scale,
                                                                double *__restrict__ theta, double *__restrict__ grad,
-                                                               double *__restrict__ u, int *__restrict__ flag, int64_t row0,
+                                                               double *__restrict__ u, StatusFlag *__restrict__ flag, int64_t row0,
                                                                int64_t nrow)
 {
     recover_flat<L, T, MIR>(src, g, r, scale, theta, grad, u, flag, row0, nrow);
@@ -318,7 +318,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) batch_recover_kernel(const int64_t *__restrict__ node_off, int count,
                                                             const BatchInst *__restrict__ inst, const T *__restrict__ src,
                                                             double *__restrict__ theta, double *__restrict__ u,
-                                                            int *__restrict__ flag)
+                                                            StatusFlag *__restrict__ flag)
 {
     const int64_t n = (int64_t)blockIdx.x * 128 + threadIdx.x;
     const int j = batch_instance(node_off, count, n);
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(128) batch_recover_kernel(const int64_t *__res
 }
 
 cudaError_t launch_batch_recover(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
-                                 const void *src, double *theta, double *u, int *flag, cudaStream_t s)
+                                 const void *src, double *theta, double *u, StatusFlag *flag, cudaStream_t s)
 {
     const unsigned nb = (unsigned)((nodes + 127) / 128);
     if (precision == LB_FX64)
@@ -366,7 +366,7 @@ Recov make_recov(const lb_ctx *c, double *scale)
 }
 
 template <class L, typename T, bool MIR>
-static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag, int64_t row0,
+static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr, double *u, StatusFlag *flag, int64_t row0,
                              int64_t nrow)
 {
     constexpr int H = 16 / (int)sizeof(T);
@@ -396,7 +396,7 @@ static cudaError_t recover_t(lb_ctx *c, const void *src, double *th, double *gr,
 }
 
 template <class L, bool MIR>
-static cudaError_t recover_m(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag, int64_t row0,
+static cudaError_t recover_m(lb_ctx *c, const void *src, double *th, double *gr, double *u, StatusFlag *flag, int64_t row0,
                              int64_t nrow)
 {
     switch (c->precision) {
@@ -407,7 +407,7 @@ static cudaError_t recover_m(lb_ctx *c, const void *src, double *th, double *gr,
 }
 
 template <class L>
-static cudaError_t recover_l(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag, int64_t row0,
+static cudaError_t recover_l(lb_ctx *c, const void *src, double *th, double *gr, double *u, StatusFlag *flag, int64_t row0,
                              int64_t nrow)
 {
     return c->geom.mirror ? recover_m<L, true>(c, src, th, gr, u, flag, row0, nrow)
@@ -427,7 +427,7 @@ __global__ void staging_timeout_selftest_kernel(int *flag, unsigned long long li
     if (!mbar_wait_bounded(barp, 0, limit_ns) && threadIdx.x == 0) atomicOr(flag, 4);
 }
 
-cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag, int64_t row0,
+cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *th, double *gr, double *u, StatusFlag *flag, int64_t row0,
                                int64_t nrow)
 {
     switch (c->d) {
@@ -438,7 +438,7 @@ cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *th, double *g
     }
 }
 
-cudaError_t launch_macros(lb_ctx *c, const void *src, double *th, double *gr, double *u, int *flag)
+cudaError_t launch_macros(lb_ctx *c, const void *src, double *th, double *gr, double *u, StatusFlag *flag)
 {
     return launch_macros_rows(c, src, th, gr, u, flag, 0, c->geom.rows);
 }
