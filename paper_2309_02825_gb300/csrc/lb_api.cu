@@ -256,10 +256,14 @@ cudaError_t choose_schedule(lb_ctx *c)
         return cudaSuccess;
     }
     if (c->geom.mirror) return cudaSuccess;
+    // FP64 whose collisions take the direct form is bound by the FP64 pipe, which
+    // recomputed nodes only load further: us per step, marching / one sweep per
+    // launch at eps = 0.01, 1400^2 139 / 122, 2048^2 285 / 254, 4096^2 1062 / 1005.
+    const bool direct = c->precision == LB_FP64 && !lbk::coll_f64_aligns(*c);
     bool worth = false;
     cudaError_t e = lbk::march_setup(c, &c->march, &worth);
     if (e != cudaSuccess) return e;
-    if (worth) {
+    if (worth && !direct) {
         c->run = lbk::kSchedMarch;
         return cudaSuccess;
     }
@@ -270,8 +274,9 @@ cudaError_t choose_schedule(lb_ctx *c)
         // 64^2 1.35, 1.08, 1.9 / 2.9, 2.7, 3.9; 128^2 1.6, 1.1, 2.4 / 2.9, 2.8,
         // 4.0; 192^2 1.6, 1.3, 2.9 / 3.0, 2.7, 4.2; 256^2 2.4, 1.6, 4.4 / 3.4,
         // 2.8, 4.6; 384^2 3.2, 1.9 / 4.7, 3.1.  FP64 tiles above 24 nodes (SMs
-        // busy with the recomputed halo) lose: 320^2 5.7 / 5.1.
-        const int most = c->precision == LB_FP64 ? 24 : (c->precision == LB_FX64 ? 40 : 48);
+        // busy with the recomputed halo) lose: 320^2 5.7 / 5.1; in the direct form
+        // those above 8 nodes: 96^2 3.3 / 4.0, 128^2 4.6 / 4.1, 256^2 10.5 / 6.7.
+        const int most = c->precision == LB_FP64 ? (direct ? 8 : 24) : (c->precision == LB_FX64 ? 40 : 48);
         for (int tile = 8; tile <= most; tile += 4) {
             if (((c->N[0] + tile - 1) / tile) * ((c->N[1] + tile - 1) / tile) > c->sms) continue;
             bool fits = true;
@@ -498,6 +503,7 @@ lb_status lb_set_viscosity(lb_ctx *c, double nu)
     if (c->precision == LB_FX64 && !lbk::fx_constants_ok(trial))
         return fail(c, LB_EINVAL, "lb_set_viscosity: a fixed-point collision constant leaves (-1, 1) at this nu");
     DeviceGuard dg(c);
+    const bool aligned = lbk::coll_f64_aligns(*c);
     // recorded sweeps carry the old collision constants; drain the stream before dropping them
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_set_viscosity");
@@ -522,6 +528,8 @@ lb_status lb_set_viscosity(lb_ctx *c, double nu)
             cudaGraphExecDestroy(g);
             g = nullptr;
         }
+    if (c->precision == LB_FP64 && aligned != lbk::coll_f64_aligns(*c) && (e = choose_schedule(c)) != cudaSuccess)
+        return cuda_fail(c, e, "lb_set_viscosity: schedule");
     return LB_OK;
 }
 

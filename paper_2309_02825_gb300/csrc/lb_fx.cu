@@ -54,6 +54,14 @@ CollF64 make_coll_f64(const lb_ctx &c)
     return r;
 }
 
+bool coll_f64_aligns(const lb_ctx &c)
+{
+    if (!make_coll_f64(c).ints) return false;
+    const double w[3] = {fabs(c.w0), fabs(c.w1), c.d > 1 ? fabs(c.wd) : fabs(c.w1)};
+    const double most = fmax(w[0], fmax(w[1], w[2])), least = fmin(w[0], fmin(w[1], w[2]));
+    return most < ldexp(least, c.d <= 2 ? f64_align_bit<D2Q9>() : f64_align_bit<D3Q19>());
+}
+
 // The constants with the context's range flag, for the single-grid sweeps.
 static CollFxR make_coll_fxr(lb_ctx *c)
 {

@@ -351,6 +351,12 @@ bool fx_constants_ok(const lb_ctx &c);
 // step resident in one block: 81 nodes 0.34 against 0.54, 129 nodes 0.49 / 0.60,
 // 256 nodes 0.72 / 0.44, 1024 nodes 2.7 / 1.4).
 CollF64 make_coll_f64(const lb_ctx &c);
+// Whether the populations near equilibrium, w_i theta, align there (f64_align): the
+// weights within its exponent range.  The paper's set does for eps from 0.0033 in
+// 1D, 0.022 to 0.74 in 2D, 0.028 to 0.54 in 3D and 0.036 to 0.41 in 4D but near
+// where a weight vanishes (within 3 % of 1/2 in 2D, 10 % of 1/4 in 3D, 1 % of 1/12
+// and 6 % of 1/6 in 4D); elsewhere every node takes the direct form.
+bool coll_f64_aligns(const lb_ctx &c);
 // Device flags of a context (ctx->dflag): 0 initialisation, 1 recovery
 // (bit 0: theta <= 0 or non-finite, bit 2: a staging wait timed out),
 // 2 fixed-point sweep range (CollFxR).  hflag holds their mirrors.

@@ -1,0 +1,74 @@
+"""Which launches lb_step and lb_batch_step take by themselves: read from the
+kernels of a captured call, and the same bits as one sweep per launch."""
+
+import re
+
+import pytest
+import torch
+
+from paper_2309_02825_gb300 import lb
+
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore:DEBUG")]
+
+EPS = {1: 0.16, 2: 0.2048, 3: 0.0512}
+NU = 0.02
+
+
+def _solver(N, precision, eps=None, stream=None, boundary=None):
+    d = len(N)
+    dx = 1.0 / N[0]
+    return lb.Solver(d, N, NU, dx, (eps or EPS[d]) * dx * dx / NU, precision=precision,
+                     theta_ref=1.5 if precision == "fp32s" else 0.0, stream=stream, boundary=boundary)
+
+
+def _inputs(N, seed=3):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    shape = tuple(reversed(N))
+    th = 1.0 + torch.rand(shape, dtype=torch.float64, device="cuda", generator=g)
+    return th, torch.zeros((len(N),) + shape, dtype=torch.float64, device="cuda")
+
+
+def _kernels(stream, call, tmp_path):
+    """Names of the kernels that a call launches, from its captured graph."""
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g, stream=stream):
+        call()
+    path = str(tmp_path / "graph.dot")
+    g.debug_dump(path)
+    with open(path) as f:
+        return re.findall(r"_ZN3lbk\d+(\w+?)_kernelI", f.read())
+
+
+def _steps(s, stream, n, tmp_path):
+    torch.cuda.synchronize()  # the inputs were made on another stream
+    with torch.cuda.stream(stream):
+        names = _kernels(stream, lambda: s.step(n), tmp_path)
+    torch.cuda.synchronize()
+    return names
+
+
+@pytest.mark.parametrize("N,several", [((96, 96), "batch_tb"), ((256, 256), "batch_tb"), ((1408, 1408), "march")])
+def test_fp64_takes_several_steps_per_launch_where_its_collisions_align(N, several, tmp_path):
+    """Populations near w_i theta align at eps = 0.2048, not at 0.01 (weights a
+    factor 200 apart) nor at 1/2 (a weight vanishes): there one sweep per launch,
+    but for the smallest grids, also after a change of the viscosity."""
+    stream = torch.cuda.Stream()
+    th, gr = _inputs(N)
+    s = _solver(N, "fp64", stream=stream)
+    one = _solver(N, "fp64", stream=stream)
+    one.set_blocking(0)
+    for eps in (0.2048, 0.01, 0.5, 0.2048):
+        for x in (s, one):
+            x.set_viscosity(NU * eps / 0.2048)
+            x.set_theta0(th, gr)
+        direct = "batch_tb" if N == (96, 96) else "sweep"
+        assert set(_steps(s, stream, 8, tmp_path)) == {several if eps == 0.2048 else direct}
+        assert set(_steps(one, stream, 8, tmp_path)) == {"sweep"}
+        for x in (s, one):
+            x.set_theta0(th, gr)
+            x.step(21)
+        for a, b in zip(s.macros(), one.macros()):
+            assert torch.equal(a, b)
+    s.close()
+    one.close()
