@@ -748,18 +748,18 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
     // the launches are cut such that an even number of steps ends in that buffer
     // again, as one sweep per launch does, and replays go on from one another.
     const bool held = cap != cudaStreamCaptureStatusNone;
-    if (c->run == lbk::kSchedLine && nsteps > 0) {
+    if (c->run == lbk::kSchedLine) {
         constexpr int64_t kMost = 1 << 20;  // steps per launch
-        while (nsteps > 0) {
+        const int64_t least = lbk::line_least(c);
+        while (nsteps >= least) {  // fewer below, one sweep per launch
             int64_t n = nsteps < kMost ? nsteps : kMost;
-            if (held && n % 2 == 0) --n;
+            if (held && n % 2 == 0 && --n < least) break;
             cudaError_t e = lbk::line_launch(c, c->f[c->cur], c->f[c->cur ^ 1], n);
             if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: resident launch");
             c->cur ^= 1;
             c->step += n;
             nsteps -= n;
         }
-        return LB_OK;
     }
     if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps) {
         // marching launches; the remainder below, one sweep per launch
@@ -774,15 +774,28 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
         }
     }
     if (c->run == lbk::kSchedTiles && c->tb_k > 0) {
-        // blocked: launches of tb_k steps (recorded in graphs), then one launch for the remainder
+        // blocked: launches of tb_k steps (recorded in graphs), then one launch for
+        // the remainder.  The library's own choice runs a remainder of one step, or
+        // two with tiles above 32 nodes, one sweep per launch: us per call, tiles /
+        // sweeps, one step FP32 416^2 8.9 / 4.2, 256^2 6.2 / 4.2, fixed point 416^2
+        // 10.3 / 6.2, 256^2 6.2 / 4.2; two steps FP32 416^2 10.3 / 8.3, 320^2 6.2 / 8.3.
+        const int least = c->sched == lbk::kSchedAuto ? (c->tb_tile > 32 ? 3 : 2) : 1;
         cudaError_t e = cudaSuccess;
-        while (held && ((nsteps + c->tb_k - 1) / c->tb_k - nsteps) % 2 != 0) {  // at most two steps on their own
-            if ((e = lbk::blocked_launch(c, c->f[c->cur], c->f[c->cur ^ 1], 1, c->stream)) != cudaSuccess)
-                return cuda_fail(c, e, "lb_step: blocked launch");
+        const auto one = [&]() {
+            e = least > 1 ? lbk::launch_sweep(c, c->f[c->cur], c->f[c->cur ^ 1])
+                          : lbk::blocked_launch(c, c->f[c->cur], c->f[c->cur ^ 1], 1, c->stream);
+            if (e != cudaSuccess) return false;
             c->cur ^= 1;
             ++c->step;
             --nsteps;
-        }
+            return true;
+        };
+        const auto swaps = [&](int64_t n) {  // of the buffers, in n steps
+            const int64_t rem = n % c->tb_k;
+            return n / c->tb_k + (rem < least ? rem : 1);
+        };
+        while (held && (swaps(nsteps) - nsteps) % 2 != 0)  // a few steps on their own
+            if (!one()) return cuda_fail(c, e, "lb_step: sweep launch");
         int64_t launches = nsteps / c->tb_k;
         const int rem = (int)(nsteps % c->tb_k);
         while (cap == cudaStreamCaptureStatusNone && launches >= kTbGraphLaunches) {
@@ -798,12 +811,16 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
             c->cur ^= 1;
             c->step += c->tb_k;
         }
-        if (rem > 0) {
+        nsteps = rem;
+        if (rem >= least) {
             if ((e = lbk::blocked_launch(c, c->f[c->cur], c->f[c->cur ^ 1], rem, c->stream)) != cudaSuccess)
                 return cuda_fail(c, e, "lb_step: blocked launch");
             c->cur ^= 1;
             c->step += rem;
+            nsteps = 0;
         }
+        while (nsteps > 0)
+            if (!one()) return cuda_fail(c, e, "lb_step: sweep launch");
         return LB_OK;
     }
     while (cap == cudaStreamCaptureStatusNone && nsteps >= kGraphSteps) {

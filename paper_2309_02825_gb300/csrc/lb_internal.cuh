@@ -414,9 +414,10 @@ cudaError_t launch_batch_init(int precision, const int64_t *node_off, int count,
                               void *dst, const double *theta0, const double *grad, StatusFlag *flag, cudaStream_t s);
 cudaError_t launch_batch_recover(int precision, const int64_t *node_off, int count, int64_t nodes, const BatchInst *inst,
                                  const void *src, double *theta, double *u, StatusFlag *flag, cudaStream_t s);
-// Resident sweeps of a short 1D grid (lb_line.cu): whether it is one, and one
-// launch of any number of steps.
+// Resident sweeps of a short 1D grid (lb_line.cu): whether it is one, the fewest
+// steps that a launch pays for, and one launch of any number of steps.
 bool line_fits(const lb_ctx *c);
+int line_least(const lb_ctx *c);
 cudaError_t line_launch(lb_ctx *c, const void *src, void *dst, int64_t steps);
 
 }  // namespace lbk

@@ -97,6 +97,13 @@ bool line_fits(const lb_ctx *c)
     return c->d == 1 && c->N[0] <= (c->precision == LB_FP64 ? 2 : 4) * kLineThreads;
 }
 
+// A call of few steps: the one block's loads and stores are spread over no more
+// steps than that.  us per call, resident / one sweep per launch: one step FP64 2048 nodes
+// 6.2 / 4.1, FP32 4096 8.2 / 4.1, fixed point 2048 6.2 / 4.1; fixed point 4096 one
+// to five steps 12.4, 14.4, 15.5, 16.5, 18.5 / 4.1, 8.2, 12.3, 16.4, 20.5; two
+// steps elsewhere no more than two sweeps.
+int line_least(const lb_ctx *c) { return c->precision == LB_FX64 && c->N[0] > 2 * kLineThreads ? 5 : 2; }
+
 cudaError_t line_launch(lb_ctx *c, const void *src, void *dst, int64_t steps)
 {
     if (c->precision == LB_FP64) return line_t<double>(c, src, dst, steps, make_coll_f64(*c));
