@@ -900,11 +900,14 @@ struct lb_adj {
     bool forward_done = false, seeded = false;
     lbk::AdjK K{};
     size_t bytes = 0;
-    // Recorded graphs.  rgraph[p][b][pre]: one whole
-    // reverse segment, C reverse steps from adjoint buffer p over the segment
+    // Recorded graphs.  fgraph[p]: C forward sweeps from buffer p, for contexts that
+    // run one sweep per launch (valid for the context's generation fgen[p]: its walls
+    // and viscosity).  rgraph[p][b][pre]: one whole reverse segment, C reverse steps from adjoint buffer p over the segment
     // held in seg[b], and with pre = 1 beside them, on a second branch, the
     // C - 1 recompute sweeps of the previous segment into seg[b ^ 1] (valid
     // for the constants K and walls they were recorded with).
+    cudaGraphExec_t fgraph[2] = {nullptr, nullptr};
+    uint64_t fgen[2] = {0, 0};
     uint64_t fwd_gen = 0;       // the context's generation at the last forward pass
     cudaGraphExec_t rgraph[2][2][2] = {};
     lbk::AdjK rK[2][2][2]{};
@@ -940,6 +943,7 @@ void free_adj(lb_adj *a)
     cudaFree(a->slot_init);
     cudaFree(a->dflag);
     for (int p = 0; p < 2; ++p) {
+        if (a->fgraph[p]) cudaGraphExecDestroy(a->fgraph[p]);
         for (auto &gb : a->rgraph[p])
             for (cudaGraphExec_t g : gb)
                 if (g) cudaGraphExecDestroy(g);
@@ -1379,7 +1383,28 @@ lb_status lb_adjoint_forward(lb_adj *a, const double *theta0, double *theta, dou
             if ((e = cudaMemcpyAsync(a->ck[k], c->f[c->cur], a->state_bytes, cudaMemcpyDeviceToDevice, c->stream)) !=
                 cudaSuccess)
                 return acuda(a, e, "lb_adjoint_forward: checkpoint");
-            if ((st = lb_step(c, std::min<int64_t>(a->C, a->T - k * a->C))) != LB_OK) return st;
+            const int64_t n = std::min<int64_t>(a->C, a->T - k * a->C);
+            if (n < a->C || c->run != lbk::kSchedSweeps || stream_capturing(c->stream)) {
+                if ((st = lb_step(c, n)) != LB_OK) return st;
+                continue;
+            }
+            // One sweep per launch: segments are shorter than the graphs of lb_step,
+            // and launched one by one a sweep of a small grid takes 4.1 us, not 2.3.
+            const int p = c->cur;
+            if (!a->fgraph[p] || a->fgen[p] != c->gen) {
+                e = record_graph(c, &a->fgraph[p], [&]() {
+                    cudaError_t r = cudaSuccess;
+                    for (int64_t m = 0, q = p; m < n && r == cudaSuccess; ++m, q ^= 1)
+                        r = lbk::launch_sweep(c, c->f[q], c->f[q ^ 1]);
+                    return r;
+                });
+                if (e != cudaSuccess) return acuda(a, e, "lb_adjoint_forward: record");
+                a->fgen[p] = c->gen;
+            }
+            if ((e = cudaGraphLaunch(a->fgraph[p], c->stream)) != cudaSuccess)
+                return acuda(a, e, "lb_adjoint_forward: graph");
+            c->cur ^= (int)(n & 1);
+            c->step += n;
         }
     }
     if ((theta || u) && (st = lb_macros(c, theta, nullptr, u)) != LB_OK) return st;
