@@ -469,7 +469,46 @@ cudaError_t upload_inst(lb_batch *b)
     return cudaSuccess;
 }
 
-// Take marching launches of variant `v` (tables of the blocks).
+// Whether a new batch takes marching launches (these blocks, of `steps` steps) over
+// one launch per step: enough nodes to fill the device, and a shorter step by the
+// two schedules' costs in ns.  One launch per step: the launch, its blocks of 8
+// warps, its warps' row segments and its nodes.  Marching: the rows that a block's stages
+// process, each a fixed cost and one per warp with columns, as if the blocks filled
+// a wave.  The costs are fitted to 46 batches of equal instances (2 to 2000 columns,
+// 1 to 1024 rows, 0.24M to 4.2M nodes; FP32 from 0.04M) per precision; the schedule that they pick was
+// within 7 % of the faster one.  Windows of few rows or mostly idle columns do not pay: us
+// per step, marching / one launch per step, 976 x (512 x 2) FP32 12.8 / 8.8, 1953 x (512
+// x 1) fixed point 30.8 / 22.1, 200 x 64^2 FP64 34.9 / 25.6; 122 x (512 x 16) FP32 6.5 /
+// 8.8, 31 x (2000 x 16) fixed point 13.1 / 21.5, 4 x 1024^2 FP64 96.6 / 121.  FP64
+// instances whose collisions take the direct form load the FP64 pipe with
+// the recomputed nodes too (eps = 0.01: 10 x 512^2 221 / 180, 200 x 64^2 96 / 59).
+bool march_worth(const lb_batch *b, const std::vector<lbk::MarchBlock> &blocks, int steps, int resident)
+{
+    struct Cost {
+        int64_t least;
+        double launch, block, segment, node, row, warp_row;
+    };
+    const Cost k = b->precision == LB_FP32_SHIFTED ? Cost{40000, 3180.0, 1.06, 0.35, 0.0017, 0.0355, 0.0033}
+                   : b->precision == LB_FX64       ? Cost{200000, 0.0, 1.36, 0.48, 0.0118, 0.149, 0.0206}
+                                                   : Cost{350000, 0.0, 3.65, 1.64, 0.0, 0.426, 0.212};
+    if (b->total_nodes < k.least) return false;
+    const int ring = steps - 1;
+    std::vector<char> direct(b->count, 0);
+    double one = k.launch, march = 0.0;
+    for (int j = 0; j < b->count; ++j) {
+        const lb_ctx &c = b->inst[j];
+        direct[j] = b->precision == LB_FP64 && !lbk::coll_f64_aligns(c);
+        one += (direct[j] ? 2.3 : 1.0) *
+               (k.block * (double)((c.geom.nseg + 7) / 8) + k.segment * (double)c.geom.nseg + k.node * (double)c.nodes);
+    }
+    for (const lbk::MarchBlock &m : blocks)
+        march += (direct[m.inst] ? 4.0 : 1.0) * steps * (m.nr + ring) *
+                 (k.row + k.warp_row * ((m.nx + 2 * ring + 31) / 32));
+    return march * std::max(1.0, (double)resident / (double)blocks.size()) < one;
+}
+
+// Take marching launches of variant `v` (tables of the blocks); own: the library's
+// own choice, where they are worth it.
 cudaError_t build_march(lb_batch *b, int v, bool own)
 {
     free_march(b);
@@ -477,9 +516,10 @@ cudaError_t build_march(lb_batch *b, int v, bool own)
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     if (e != cudaSuccess) return e;
     std::vector<lbk::MarchBlock> blocks;
-    int steps, threads, cols;
-    lbk::march_batch_plan(b->inst.data(), b->count, b->precision, v, sms, &blocks, &steps, &threads, &cols);
+    int steps, threads, cols, resident;
+    lbk::march_batch_plan(b->inst.data(), b->count, b->precision, v, sms, &blocks, &steps, &threads, &cols, &resident);
     if (blocks.empty() || blocks.size() > 0x7fffffff) return cudaSuccess;
+    if (own && !march_worth(b, blocks, steps, resident)) return cudaSuccess;
     if ((e = cudaMalloc(&b->d_march, sizeof(lbk::MarchBlock) * blocks.size())) != cudaSuccess ||
         (e = cudaMemcpy(b->d_march, blocks.data(), sizeof(lbk::MarchBlock) * blocks.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
@@ -628,16 +668,6 @@ lb_status build_tiles(lb_batch *b, int K, int tile, int threads)
     b->tb_tile = tile;
     b->tb_threads = threads;
     return LB_OK;
-}
-
-// Whether a new batch takes marching launches over one launch per step.
-// Measured GLUPS, march / one launch per step in 96 MB groups, by total nodes:
-//   FP32: 21.4M 236 / 90, 3.8M 197 / 94, 0.65M 129 / 73, 0.41M 108 / 65, 0.05M 17.6 / 11.6
-//   fixed point: 21.4M 105 / 43, 3.8M 88 / 44, 0.65M 59 / 42, 0.41M 54 / 41, 0.05M 8.6 / 10.2
-//   FP64: 21.4M 45 / 20, 3.8M 42 / 21, 0.65M 24 / 15, 0.41M 26 / 15, 0.05M 2.9 / 6.3
-bool march_worth(const lb_batch *b)
-{
-    return b->total_nodes >= (b->precision == LB_FP32_SHIFTED ? 40000 : (b->precision == LB_FX64 ? 200000 : 350000));
 }
 
 // Record kTbGraphLaunches blocked launches of tb_k steps starting from buffer `from`.
@@ -972,7 +1002,7 @@ lb_status lb_batch_create(int count, const int64_t *N, const double *nu, const d
         free_batch(b);
         return st;
     }
-    if (march_worth(b) && (e = build_march(b, 0, true)) != cudaSuccess) {
+    if ((e = build_march(b, 0, true)) != cudaSuccess) {
         free_batch(b);
         return e == cudaErrorMemoryAllocation ? LB_ENOMEM : LB_ECUDA;
     }

@@ -399,10 +399,10 @@ cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth);
 cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s);
 // The same for batched 2D instances: variants of a storage type (the first is
 // the default), the blocks of a launch over `count` instances with the steps,
-// threads and columns per window of the variant, and one launch.
+// threads, columns per window and blocks in a wave of the variant, and one launch.
 int march_batch_variants(int precision);
 void march_batch_plan(const lb_ctx *inst, int count, int precision, int variant, int sms, std::vector<MarchBlock> *blocks,
-                      int *steps, int *threads, int *cols);
+                      int *steps, int *threads, int *cols, int *resident);
 cudaError_t march_batch_launch(int precision, int variant, const void *desc, const MarchBlock *blocks, int n,
                                const void *src, void *dst, cudaStream_t s);
 // All instances of a batch in one launch each (node_off: count + 1 prefix sums

@@ -420,10 +420,12 @@ template <typename T, int KS, int TH, int MINB> struct MarchB {
     // (8 to 512 instances of 32^2 to 512^2) in each precision, its choice was
     // 1.4 % above the fastest in the mean and 8 % at the most.  The longest blocks
     // start first.
-    static void plan(const lb_ctx *inst, int count, int sms, std::vector<MarchBlock> *out, int *steps, int *threads, int *cols)
+    static void plan(const lb_ctx *inst, int count, int sms, std::vector<MarchBlock> *out, int *steps, int *threads, int *cols,
+                     int *resident)
     {
         constexpr int ring = KS - 1;
         *steps = KS;
+        *resident = sms * MINB;
         *threads = TH;
         *cols = TH - 2 * ring;
         const double slots = (double)sms * MINB;
@@ -492,9 +494,10 @@ template <class F> static void march_batch_pick(int precision, int variant, F &&
 int march_batch_variants(int precision) { return precision == LB_FP64 ? 1 : 2; }
 
 void march_batch_plan(const lb_ctx *inst, int count, int precision, int variant, int sms, std::vector<MarchBlock> *blocks,
-                      int *steps, int *threads, int *cols)
+                      int *steps, int *threads, int *cols, int *resident)
 {
-    march_batch_pick(precision, variant, [&](auto m) { decltype(m)::plan(inst, count, sms, blocks, steps, threads, cols); });
+    march_batch_pick(precision, variant,
+                     [&](auto m) { decltype(m)::plan(inst, count, sms, blocks, steps, threads, cols, resident); });
 }
 
 cudaError_t march_batch_launch(int precision, int variant, const void *desc, const MarchBlock *blocks, int n,

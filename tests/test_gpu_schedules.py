@@ -117,3 +117,20 @@ def test_replays_of_mixed_launches_go_on_from_one_another(N, precision, n):
     for a, b in zip(got, want):
         assert torch.equal(a, b)
     s.close()
+
+
+@pytest.mark.parametrize("count,N,precision,eps,march", [
+    (976, (512, 2), "fp32s", None, False), (122, (512, 16), "fp32s", None, True), (1953, (512, 1), "fx64", None, False),
+    (31, (2000, 16), "fx64", None, True), (200, (64, 64), "fp64", None, False), (4, (1024, 1024), "fp64", None, True),
+    (4, (1024, 1024), "fp64", 0.01, False)])
+def test_batches_march_where_the_windows_pay(count, N, precision, eps, march, tmp_path):
+    dx = 1.0 / N[0]
+    stream = torch.cuda.Stream()
+    kw = {"theta_ref": [1.5] * count} if precision == "fp32s" else {}
+    b = lb.Batch([N] * count, [NU] * count, [dx] * count, [(eps or EPS[2]) * dx * dx / NU] * count, precision=precision,
+                 stream=stream, **kw)
+    nodes = count * N[0] * N[1]
+    b.set_theta0(torch.full((nodes,), 1.25, dtype=torch.float64, device="cuda"),
+                 torch.zeros(2 * nodes, dtype=torch.float64, device="cuda"))
+    assert ("march_batch" in _steps(b, stream, 10, tmp_path)) == march
+    b.close()
