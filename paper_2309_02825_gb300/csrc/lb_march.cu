@@ -283,6 +283,16 @@ static void cut(int n, int most, int &parts, int &size)
     parts = (n + size - 1) / size;
 }
 
+// What marching has to offer against one sweep per launch (march_setup).
+struct MarchRule {
+    int64_t nodes;  // at least so many nodes
+    double use;     // of a launch's thread-iterations at least this share ends in stored nodes
+    double full;    // 2D, below 450000 nodes: the same with as many blocks on every SM as on the fullest
+    // 3D: us per step and unit of the plan's model, less than the sweeps' us per 1000
+    // nodes, lanes of the rows' warps, and nodes beyond 650000 (no longer in L2)
+    double unit, node, lane, far;
+};
+
 template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March {
     using KT = typename MarchK<T>::type;
     static constexpr int kRing = KS - 1;
@@ -295,9 +305,7 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
     // room for, in blocks of fewer warps, where they fill the SMs better
     // (101 x 90 x 77 FP32: 36 windows of 10 rows by 4 chunks on 152 SMs instead of
     // 32 of 12, 50 GLUPS against 44).
-    // `worth`: enough nodes to fill the chip, and the share of a launch's
-    // thread-iterations that end in stored nodes not below least_use.
-    static void plan(const lb_ctx *c, int64_t least_nodes, double least_use, MarchPlan *out, bool *worth)
+    static void plan(const lb_ctx *c, const MarchRule &rule, MarchPlan *out, bool *worth)
     {
         const Geom &g = c->geom;
         *out = MarchPlan{};
@@ -338,14 +346,21 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
             *out = MarchPlan{};
             return;
         }
-        const double use =
-            (double)c->nodes / ((double)out->nx * out->ny * out->nc * out->threads * (out->chunk + 3 * kRing));
-        *worth = c->nodes >= least_nodes && use >= least_use;
+        const int64_t blocks = (int64_t)out->nx * out->ny * out->nc, waves = (blocks + slots - 1) / slots;
+        const int64_t filled = (blocks + waves * c->sms - 1) / (waves * c->sms) * waves * c->sms;
+        const double each = (double)out->threads * (out->chunk + 3 * kRing), nodes = (double)c->nodes;
+        *worth = c->nodes >= rule.nodes && nodes / (blocks * each) >= rule.use;
+        if (L::D == 2 && c->nodes < 450000) *worth = *worth && nodes / (filled * each) >= rule.full;
+        if (L::D == 3) {
+            const double lanes = (double)g.nseg * 32 * lane_width<L, T>();
+            *worth = *worth && rule.unit * least / KS < 1e-3 * (rule.node * nodes + rule.lane * lanes +
+                                                               rule.far * std::max(0.0, nodes - 650000));
+        }
     }
     static const void *kernel() { return (const void *)march_kernel<L, T, KT, KS, TH, MINB, SKIP>; }
-    static cudaError_t setup(lb_ctx *c, int64_t least_nodes, double least_use, MarchPlan *out, bool *worth)
+    static cudaError_t setup(lb_ctx *c, const MarchRule &rule, MarchPlan *out, bool *worth)
     {
-        plan(c, least_nodes, least_use, out, worth);
+        plan(c, rule, out, worth);
         return cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)march_smem<L, KS, TH>(sizeof(T)));
     }
@@ -375,25 +390,33 @@ using March2D = March<D2Q9, double, 2, 128, 6, true>;
 using March3Fx = March<D3Q19, long long, 2, 416, 1, true>;
 using March3F = March<D3Q19, float, 3, 512, 1, false>;
 
-// Where marching beats one sweep per launch (GLUPS, march / sweep):
-//   2D fixed point 256^2 16 / 20, 384^2 29 / 31, 512^2 52 / 41, 1024^2 76 / 43, 1999x1501 94 / 44, 4096^2 108 / 47
-//   2D FP32        256^2 22 / 23, 384^2 50 / 46, 512^2 77 / 60, 1024^2 194 / 124, 1999x1501 258 / 85, 4096^2 315 / 97
+// Where marching beats one sweep per launch, replayed from graphs (GLUPS, march / sweep):
+//   2D fixed point 256^2 16 / 20, 384^2 29 / 31, 526^2 58 / 49, 1024^2 76 / 43, 1999x1501 94 / 44, 4096^2 108 / 47
+//   2D FP32        256^2 22 / 23, 384^2 50 / 46, 526^2 84 / 79, 1024^2 194 / 124, 1999x1501 258 / 85, 4096^2 315 / 97
 //   2D FP64        768^2 34 / 40, 1024^2 37 / 39, 1999x1501 48 / 42, 4096^2 52 / 47
-//   3D fixed point 48^3 16 / 13, 64^3 20 / 21, 101x90x77 26 / 19, 128^3 32 / 22, 256^3 36 / 23
-//   3D FP32        64^3 31 / 31, 72^3 41 / 36, 80^3 49 / 41, 101x90x77 50 / 42, 128^3 61 / 42, 256^3 75 / 46
+//   3D fixed point 67^3 22 / 19, 101x90x77 26 / 20, 126^3 30 / 22, 256^3 36 / 23
+//   3D FP32        72^3 42 / 48, 87^3 46 / 48, 93^3 51 / 45, 101x90x77 49 / 51, 106^3 53 / 42, 126^3 57 / 43, 256^3 75 / 46
+// 2D grids of 0.2M to 0.45M nodes are one wave of few blocks per SM, as long as the
+// fullest SM's: us per step, march / sweep, fixed point 526^2 (4 blocks on every SM)
+// 4.8 / 5.7, 263 x 1052 (5 on some) 6.15 / 5.6, 448^2 4.8 / 4.7; FP32 427^2 2.9 / 2.7, 6036 x
+// 30 4.1 / 2.95, 526^2 3.3 / 3.5 (the smaller ones mostly fit tiles, faster than either).
+// In 3D a few planes, or rows that fill the sweep's warps, favour the sweeps: FP32
+// 126x31x126 10.3 / 8.0, 234x234x15 20.8 / 16.8, 50x200x50 10.6 / 13.2; fixed point
+// 169x169x11 14.3 / 13.6, 27x106x106 12.3 / 19.9.  The 3D costs are fitted to 70 grids of
+// 0.3M to 2M nodes; none of them is slower by the rule.
 cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth)
 {
     *plan = MarchPlan{};
     *worth = false;
     if (c->geom.mirror) return cudaSuccess;
     if (c->d == 2) {
-        if (c->precision == LB_FX64) return March2Fx::setup(c, 200000, 0.45, plan, worth);
-        if (c->precision == LB_FP32_SHIFTED) return March2F::setup(c, 180000, 0.45, plan, worth);
-        return March2D::setup(c, 1800000, 0.8, plan, worth);
+        if (c->precision == LB_FX64) return March2Fx::setup(c, {240000, 0.45, 0.47}, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March2F::setup(c, {240000, 0.45}, plan, worth);
+        return March2D::setup(c, {1800000, 0.8}, plan, worth);
     }
     if (c->d == 3) {
-        if (c->precision == LB_FX64) return March3Fx::setup(c, 300000, 0.4, plan, worth);
-        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, 350000, 0.3, plan, worth);
+        if (c->precision == LB_FX64) return March3Fx::setup(c, {300000, 0.4, 0.0, 1.9, 0.026, 0.017}, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, {350000, 0.3, 0.0, 1.57, 0.009, 0.0069, 0.014}, plan, worth);
     }
     return cudaSuccess;
 }

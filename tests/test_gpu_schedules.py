@@ -134,3 +134,18 @@ def test_batches_march_where_the_windows_pay(count, N, precision, eps, march, tm
                  torch.zeros(2 * nodes, dtype=torch.float64, device="cuda"))
     assert ("march_batch" in _steps(b, stream, 10, tmp_path)) == march
     b.close()
+
+
+@pytest.mark.parametrize("N,precision,want", [
+    ((512, 512), "fx64", "march"), ((526, 526), "fx64", "march"), ((263, 1052), "fx64", "sweep"),
+    ((448, 448), "fx64", "batch_tb"), ((526, 526), "fp32s", "march"), ((6036, 30), "fp32s", "batch_tb"),
+    ((427, 427), "fp32s", "batch_tb"), ((126, 31, 126), "fp32s", "sweep"), ((234, 234, 15), "fp32s", "sweep"),
+    ((50, 200, 50), "fp32s", "march"), ((106, 106, 106), "fp32s", "march"), ((169, 169, 11), "fx64", "sweep"),
+    ((72, 72, 72), "fx64", "march"), ((1408, 1408), "fp64", "march")])
+def test_grids_march_where_the_windows_pay(N, precision, want, tmp_path):
+    stream = torch.cuda.Stream()
+    s = _solver(N, precision, stream=stream)
+    s.set_theta0(*_inputs(N))
+    names = set(_steps(s, stream, 30, tmp_path))
+    assert want in names and (want != "sweep" or names == {"sweep"})
+    s.close()
