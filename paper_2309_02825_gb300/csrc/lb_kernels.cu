@@ -228,7 +228,10 @@ __device__ __forceinline__ void init_node(T *__restrict__ dst, const Geom &g, co
             long long v[1 + D];
             unsigned emax;
             constexpr int PB = 7;
-            if (K.ints && f64_align_round<1 + D, PB>(x, v, emax) && emax - 983u <= 140u) {
+            // (a theta so near its reference that bits of its own terms would be lost
+            // beside the gradient's, zero included, takes the FP64 form)
+            const unsigned e0 = ((unsigned)__double2hiint(dth) >> 20) & 0x7ffu;
+            if (K.ints && f64_align_round<1 + D, PB>(x, v, emax) && emax - 983u <= 140u && emax - e0 <= 20u) {
                 const int k = (int)emax - 1075 - PB;  // the unit's exponent, -99 .. 41
                 init_fx<L>(v, K, [](long long a, long long c) { return mulfx_c(a, c); },
                            [&](auto I, long long f) { put(I, i64_to_f32_rn(f, k)); });
