@@ -149,3 +149,104 @@ def test_grids_march_where_the_windows_pay(N, precision, want, tmp_path):
     names = set(_steps(s, stream, 30, tmp_path))
     assert want in names and (want != "sweep" or names == {"sweep"})
     s.close()
+
+
+def _rough(N, seed=7):
+    """Random theta in [1, 2) and a random gradient: FP64 nodes of both forms."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    shape = tuple(reversed(N))
+    return (1.0 + torch.rand(shape, dtype=torch.float64, device="cuda", generator=g),
+            torch.randn((len(N),) + shape, dtype=torch.float64, device="cuda", generator=g))
+
+
+# windows of 60, 120 and 126 columns (fixed point, FP32, FP64), 30 and 28 in 3D: whole
+# windows, one column more (a column fewer each and a narrow last one) and one less; last
+# chunks of any number of rows
+@pytest.mark.parametrize("precision,N", [
+    ("fx64", (60, 8000)), ("fx64", (600, 800)), ("fx64", (601, 801)), ("fx64", (599, 803)), ("fx64", (1501, 443)),
+    ("fp32s", (120, 4000)), ("fp32s", (1200, 400)), ("fp32s", (1201, 401)), ("fp32s", (1199, 403)),
+    ("fp32s", (2113, 301)), ("fp64", (126, 15000)), ("fp64", (1512, 1300)), ("fp64", (1511, 1303)),
+    ("fp64", (251, 7503)), ("fx64", (60, 44, 200)), ("fx64", (61, 45, 201)), ("fx64", (59, 43, 203)),
+    ("fx64", (30, 33, 500)), ("fx64", (29, 23, 700)), ("fp32s", (56, 48, 300)), ("fp32s", (57, 49, 301)),
+    ("fp32s", (55, 47, 299)), ("fp32s", (85, 61, 201)), ("fp32s", (57, 25, 900))])
+def test_marching_windows_give_the_bits_of_single_sweeps(precision, N, tmp_path):
+    th, gr = _rough(N)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    s = _solver(N, precision, stream=stream)
+    one = _solver(N, precision)
+    if len(N) == 2:
+        one.set_blocking(0)
+    s.set_theta0(th, gr)
+    assert "march" in _steps(s, stream, 13, tmp_path)
+    s.set_theta0(th, gr)
+    one.set_theta0(th, gr)
+    for n in (13, 1, 6):
+        s.step(n)
+        for _ in range(n):  # one step per call: one sweep per launch
+            one.step(1)
+    torch.cuda.synchronize()
+    assert s.sum_theta() == one.sum_theta()
+    got = s.macros()
+    torch.cuda.synchronize()
+    for a, b in zip(got, one.macros()):
+        assert torch.equal(a, b)
+    s.check()
+    s.close()
+    one.close()
+
+
+@pytest.mark.parametrize("precision", ["fx64", "fp32s", "fp64"])
+def test_marching_batches_give_the_bits_of_one_launch_per_step(precision, tmp_path):
+    """Instances smaller than a window, of one to three rows, and a column more or
+    less than one, two and three windows (60, 56 and 126 columns), beside ones
+    large enough for the batch to march."""
+    edge = {"fx64": 60, "fp32s": 56, "fp64": 126}[precision]
+    sizes = [(1, 1), (2, 3), (5, 1), (7, 2), (edge, 3), (edge - 1, 40), (edge + 1, 41), (2 * edge, 9), (2 * edge + 1, 17),
+             (2 * edge - 1, 16), (3 * edge + 1, 8), (33, 500), (1500, 1100)]
+    ins = [_rough(N, 3 + k) for k, N in enumerate(sizes)]
+    th = torch.cat([t.reshape(-1) for t, _ in ins])
+    gr = torch.cat([g.reshape(-1) for _, g in ins])
+    dx = [1.0 / N[0] for N in sizes]
+    kw = {"theta_ref": [1.5] * len(sizes)} if precision == "fp32s" else {}
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    out = []
+    for own in (True, False):
+        b = lb.Batch(sizes, [NU] * len(sizes), dx, [EPS[2] * h * h / NU for h in dx], precision=precision, stream=stream,
+                     **kw)
+        if not own:
+            b.set_schedule(1e18, 128)
+        b.set_theta0(th, gr)
+        assert ("march_batch" in _steps(b, stream, 13, tmp_path)) == own
+        b.set_theta0(th, gr)
+        for n in (13, 1, 6):
+            b.step(n)
+        out.append(b.macros())
+        torch.cuda.synchronize()
+        b.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("single", [False, True])
+def test_resident_1d_reports_an_unstable_relaxation_set(single, tmp_path):
+    """w1 = 0.7 with s2 = 0.6 grows by 1.37 a step (largest eigenvalue over the wave
+    numbers): reported whatever the schedule."""
+    stream = torch.cuda.Stream()
+    s = lb.Solver(1, (200,), NU, 0.005, 0.16 * 0.005**2 / NU, relax={"s1": 1.5, "s2x": 0.6, "w1": 0.7}, precision="fx64",
+                  stream=stream)
+    if single:
+        s.set_blocking(0)
+    x = torch.ones(200, dtype=torch.float64, device="cuda")
+    x[::2] = 2.0
+    torch.cuda.synchronize()
+    s.set_theta0(x, torch.zeros(1, 200, dtype=torch.float64, device="cuda"))
+    assert _steps(s, stream, 5, tmp_path) == (["sweep"] * 5 if single else ["line"])
+    # (the captured call did not run, and an odd number of launches ends in the other buffer)
+    s.set_theta0(x, torch.zeros(1, 200, dtype=torch.float64, device="cuda"))
+    s.step(400)
+    with pytest.raises(lb.LBError) as ei:
+        s.check()
+    assert ei.value.status == lb.LB_EINVAL
+    s.close()
