@@ -48,11 +48,16 @@ typedef enum {
 } lb_status;
 
 typedef enum {
-    LB_FP64 = 0,         /* distributions stored in IEEE double; for d > 1 a
-                            collision forms its sums exactly on the integer
-                            pipes where the node's values allow it and rounds
-                            each result once, else in double arithmetic */
-    LB_FP32_SHIFTED = 1, /* stored and updated in float as f - w*theta_ref */
+    LB_FP64 = 0,         /* distributions stored in IEEE double; for d > 1 and
+                            for 1D rows of more than 160 nodes a collision
+                            forms its sums exactly on the integer pipes where
+                            the node's values allow it and rounds each result
+                            once, else in double arithmetic */
+    LB_FP32_SHIFTED = 1, /* stored and updated in float as f - w*theta_ref; the
+                            initialisation forms a node's values in 60 bits
+                            of the larger of theta0 - theta_ref and dx grad
+                            (in double arithmetic where the former is below
+                            2^-20 of the latter) and rounds each once */
     LB_FX64 = 2          /* stored as 64-bit fixed point round(f * 2^F), with F
                             chosen by lb_set_theta0 so that max|theta0| * 2^F <
                             2^59 (sums up to 16 max|theta0| fit); moment
@@ -202,9 +207,10 @@ lb_status lb_step(lb_ctx *ctx, int64_t nsteps);
  * whole state every step, so it is bound by HBM bandwidth.  A new context runs
  * the library's own choice: on periodic 2D and 3D grids large enough to fill
  * the device, launches of two to five steps that march windows of the grid
- * along its slowest axis; on small periodic 2D grids, launches of eight steps on
- * square tiles; on 1D grids of up to 4096 nodes (2048 for LB_FP64), all the
- * steps of a call in one launch; one sweep per launch elsewhere.  This call selects
+ * along its slowest axis, where these cost less than the sweeps; on small
+ * periodic 2D grids, launches of eight steps on square tiles; on 1D grids of up
+ * to 4096 nodes (2048 for LB_FP64), all the steps of a call in one launch; one
+ * sweep per launch elsewhere, and for calls (or remainders) of one or two steps.  This call selects
  * one sweep per launch or, on periodic 2D grids, launches of K steps on square
  * tiles: a block loads one tile of
  * the grid with a K-node periodic halo into shared memory, runs the same

@@ -34,11 +34,13 @@ typedef struct lb_adj lb_adj;
  * Adjoint workspace for `ctx` (any precision; d = 1, 2, 3; periodic axes or
  * mirror walls, lb_set_boundary).
  * The forward states are read in their storage type.  The reverse pass
- * computes in FP64 for LB_FP64 contexts, in FP32 for LB_FP32_SHIFTED contexts
+ * computes in FP64 for LB_FP64 contexts (on periodic grids of d > 1 a node's
+ * values are rounded at 2^-59 of their largest, 2^-58 for d = 3, summed exactly
+ * and each result rounded once, where the node's state allows it), in FP32 for LB_FP32_SHIFTED contexts
  * (whose forward map is FP32-accurate), and for LB_FX64 contexts in 64-bit
  * fixed point: the adjoint field is held as round(phi 2^G), G chosen from
  * the seed so that max|phi_T| 2^G < 2^56, K^T is formed from exact integer
- * sums and rounded products, and the dL/dnu term from exact 128-bit
+ * sums and rounded products (two in the rest channel), and the dL/dnu term from exact 128-bit
  * dot products (FP64 instead when the collision constants are too large for
  * that range: see lb_adjoint.cu).
  * The seed, the initialisation adjoint and the dL/dnu accumulation are FP64

@@ -22,8 +22,8 @@
  *    K steps instead of every step.  Blocks never wait on one another.
  *  - marching: each launch advances every instance two to five steps; a block
  *    marches a window of columns of one instance along its rows with the steps
- *    as pipeline stages.  A new batch takes these launches by itself where the
- *    batch is large enough for them to pay.
+ *    as pipeline stages.  A new batch takes these launches by itself where they
+ *    cost less than one launch per step.
  * The launches of the first two kinds are recorded once into CUDA graphs and
  * replayed; every instance evolves bit for bit as the same grid would alone.
  * lb_batch_autotune times all kinds (budgets, block sizes, steps per

@@ -7,9 +7,9 @@
 // instance descriptor once and then runs the same pull + collide as the
 // single-grid sweep.  Groups are sized so that their two buffers stay in
 // L2 while the group runs all its steps back to back; the launches are
-// replayed from CUDA graphs.  Batches large enough to fill the device take
+// replayed from CUDA graphs.  Batches where it costs less take
 // several steps per launch instead: marching windows over all instances
-// (lb_march.cu; march_worth says from which size), or, where asked for or found
+// (lb_march.cu; march_worth weighs them), or, where asked for or found
 // faster by lb_batch_autotune, square tiles in shared memory (batch_tb_kernel).
 #include <math.h>
 #include <string.h>
@@ -1186,7 +1186,8 @@ lb_status lb_batch_autotune(lb_batch *b, int trial_steps, double *choice)
         }
     if (b->precision == LB_FP64) {
         // the trials step whatever the buffers hold: one normal double everywhere
-        // (0x3f3f...), whose collisions take the integer form as a run's do
+        // (0x3f3f...), which the warm-up relaxes towards w_i theta, so that the timed
+        // collisions take the form a run's do (the first steps' equal values do not align)
         const size_t bytes = b->elem * (size_t)b->total_elems;
         for (void *p : b->buf)
             if (cudaMemsetAsync(p, 0x3f, bytes, b->stream) != cudaSuccess) return bfail(b, LB_ECUDA, "lb_batch_autotune: fill");

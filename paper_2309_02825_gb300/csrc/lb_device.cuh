@@ -1021,17 +1021,19 @@ __device__ __forceinline__ float f64_to_f32_rn(double v)
 {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const unsigned e = (hi >> 20) & 0x7ffu;
-    if (e - 897u > 253u) {  // below 2^-126, or 2^127 and more (volatile: not computed beside the usual path)
+    if (e - 897u > 253u) {  // below 2^-126, or 2^128 and more (volatile: not computed beside the usual path)
         float r;
         asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(v));
         return r;
     }
+    // (rounding up from the largest float carries into infinity)
     const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29), rem = lo << 3;
     const unsigned up = (rem > 0x80000000u || (rem == 0x80000000u && (m & 1u))) ? 1u : 0u;
     return __uint_as_float(((hi & 0x80000000u) | m) + up);
 }
 
-// Threads per block of the sweep: more, smaller blocks balance the SMs better.
+// Threads per block of the sweep, for every storage type: more, smaller blocks
+// balance the SMs better.
 template <typename T> __host__ __device__ constexpr int sweep_threads() { return 128; }
 
 // K is the collision-constant type; the matching collide() overload (float,
