@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_sweep_kernel(const Ins
         T n[L::Q];
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) n[i] = f[i][v];
-        collide(L{}, n, D.k);
+        collide_at<T>(L{}, n, D.k, x0 + V * lane + v, D.g.N0);
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) f[i][v] = n[i];
     }

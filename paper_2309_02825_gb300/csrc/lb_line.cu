@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const T *__restrict_
         }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            collide(D1Q3{}, f[v], k);
+            collide_at<T>(D1Q3{}, f[v], k, x0 + v, N);
 #pragma unroll
             for (int i = 0; i < 3; ++i) p[v][i] = f[v][i];
             if constexpr (std::is_same<K, CollFxR>::value) {
