@@ -475,8 +475,8 @@ cudaError_t upload_inst(lb_batch *b)
 // warps, its warps' row segments and its nodes.  Marching: the rows that a block's stages
 // process, each a fixed cost and one per warp with columns, as if the blocks filled
 // a wave.  The costs are fitted to 46 batches of equal instances (2 to 2000 columns,
-// 1 to 1024 rows, 0.24M to 4.2M nodes; FP32 from 0.04M) per precision; the schedule that they pick was
-// within 7 % of the faster one.  Windows of few rows or mostly idle columns do not pay: us
+// 1 to 1024 rows, 0.24M to 4.2M nodes; FP32 from 0.04M) per precision; the schedule
+// that they pick was within 7 % of the faster one (FP64 of 8 columns: 14 %).  Windows of few rows or mostly idle columns do not pay: us
 // per step, marching / one launch per step, 976 x (512 x 2) FP32 12.8 / 8.8, 1953 x (512
 // x 1) fixed point 30.8 / 22.1, 200 x 64^2 FP64 34.9 / 25.6; 122 x (512 x 16) FP32 6.5 /
 // 8.8, 31 x (2000 x 16) fixed point 13.1 / 21.5, 4 x 1024^2 FP64 96.6 / 121.  FP64
@@ -490,7 +490,7 @@ bool march_worth(const lb_batch *b, const std::vector<lbk::MarchBlock> &blocks, 
     };
     const Cost k = b->precision == LB_FP32_SHIFTED ? Cost{40000, 3180.0, 1.06, 0.35, 0.0017, 0.0355, 0.0033}
                    : b->precision == LB_FX64       ? Cost{200000, 0.0, 1.36, 0.48, 0.0118, 0.149, 0.0206}
-                                                   : Cost{350000, 0.0, 3.65, 1.64, 0.0, 0.426, 0.212};
+                                                   : Cost{350000, 0.0, 3.0, 0.85, 0.011, 0.426, 0.212};
     if (b->total_nodes < k.least) return false;
     const int ring = steps - 1;
     std::vector<char> direct(b->count, 0);
