@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(TH, TH <= 512 ? 2 : 1) batch_tb_kernel(const I
         }
     }
     if constexpr (std::is_same<T, long long>::value) {
-        if (range && __any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) raise_flag(range, 1);
+        if (range && __any_sync(0xffffffffu, acc >= 0x40000000u) && lane == 0) raise_flag_call(range, 1);
     }
 }
 

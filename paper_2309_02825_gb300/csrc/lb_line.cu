@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const T *__restrict_
         for (int i = 0; i < 3; ++i)
             if (x0 + v < N) dst[(int64_t)i * g.slab + x0 + v] = p[v][i];
     if constexpr (std::is_same<K, CollFxR>::value) {
-        if (acc >= 0x40000000u) raise_flag(k.range, 1);
+        if (acc >= 0x40000000u) raise_flag_call(k.range, 1);
     }
 }
 

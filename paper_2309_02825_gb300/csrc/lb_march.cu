@@ -242,7 +242,7 @@ __device__ __forceinline__ void march_body(const T *__restrict__ src, T *__restr
         w4 = r4;
     }
     if constexpr (std::is_same<K, CollFxR>::value) {
-        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && (tid & 31) == 0) raise_flag(k.range, 1);
+        if (__any_sync(0xffffffffu, acc >= 0x40000000u) && (tid & 31) == 0) raise_flag_call(k.range, 1);
     }
 }
 
