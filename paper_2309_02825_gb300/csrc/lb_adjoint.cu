@@ -1384,7 +1384,8 @@ lb_status lb_adjoint_forward(lb_adj *a, const double *theta0, double *theta, dou
                 cudaSuccess)
                 return acuda(a, e, "lb_adjoint_forward: checkpoint");
             const int64_t n = std::min<int64_t>(a->C, a->T - k * a->C);
-            if (n < a->C || c->run != lbk::kSchedSweeps || stream_capturing(c->stream)) {
+            const bool sweeps = c->run == lbk::kSchedSweeps || (c->run == lbk::kSchedMarch && c->march_short);
+            if (n < a->C || !sweeps || stream_capturing(c->stream)) {
                 if ((st = lb_step(c, n)) != LB_OK) return st;
                 continue;
             }

@@ -257,6 +257,7 @@ cudaError_t choose_schedule(lb_ctx *c)
     c->run = lbk::kSchedSweeps;
     lbk::blocked_release(c);
     c->march = lbk::MarchPlan{};
+    c->march_short = false;
     if (lbk::line_fits(c)) {
         c->run = lbk::kSchedLine;
         return cudaSuccess;
@@ -266,13 +267,13 @@ cudaError_t choose_schedule(lb_ctx *c)
     // recomputed nodes only load further: us per step, marching / one sweep per
     // launch at eps = 0.01, 1400^2 139 / 122, 2048^2 285 / 254, 4096^2 1062 / 1005.
     const bool direct = c->precision == LB_FP64 && !lbk::coll_f64_aligns(*c);
-    bool worth = false;
+    lbk::MarchWorth worth = lbk::kMarchNo;
     cudaError_t e = lbk::march_setup(c, &c->march, &worth);
     if (e != cudaSuccess) return e;
-    if (worth && !direct) {
-        c->run = lbk::kSchedMarch;
-        return cudaSuccess;
-    }
+    if (direct) worth = lbk::kMarchNo;
+    c->march_short = worth == lbk::kMarchShort;
+    if (worth != lbk::kMarchNo) c->run = lbk::kSchedMarch;
+    if (worth == lbk::kMarchYes) return cudaSuccess;
     if (c->d == 2) {
         // The smallest square tile, from 8 nodes in steps of 4, that leaves at
         // most one tile per SM; 8 steps per launch.  us per step (fixed point,
@@ -593,10 +594,11 @@ lb_status lb_autotune(lb_ctx *c, int trial_steps, double *choice)
     };
     std::vector<Cand> cands = {{lbk::kSchedSweeps, 0, 0, 0}};
     lbk::MarchPlan plan{};
-    bool worth = false;
+    lbk::MarchWorth worth = lbk::kMarchNo;
     if ((e = lbk::march_setup(c, &plan, &worth)) != cudaSuccess) return cuda_fail(c, e, "lb_autotune");
     if (plan.steps) cands.push_back({lbk::kSchedMarch, plan.steps, plan.bx, plan.threads});
     c->march = plan;
+    c->march_short = false;
     int optin = 0;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device)) != cudaSuccess)
         return cuda_fail(c, e, "lb_autotune");
@@ -764,7 +766,20 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
             nsteps -= n;
         }
     }
-    if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps) {
+    const auto replay = [&]() {  // recorded sweeps
+        while (cap == cudaStreamCaptureStatusNone && nsteps >= kGraphSteps) {
+            cudaError_t e = cudaSuccess;
+            if (!c->graph[c->cur]) e = record_sweeps(c, c->cur);
+            if (e == cudaSuccess) e = cudaGraphLaunch(c->graph[c->cur], c->stream);
+            if (e != cudaSuccess) return e;
+            nsteps -= kGraphSteps;
+            c->step += kGraphSteps;
+        }
+        return cudaSuccess;
+    };
+    cudaError_t er = cudaSuccess;
+    if (c->run == lbk::kSchedMarch && c->march_short && (er = replay()) != cudaSuccess) return cuda_fail(c, er, "lb_step: graph");
+    if (c->run == lbk::kSchedMarch && nsteps >= c->march.steps && !(c->march_short && held)) {
         // marching launches; the remainder below, one sweep per launch
         int64_t launches = nsteps / c->march.steps;
         if (held && c->march.steps % 2 == 0) launches -= launches % 2;
@@ -826,14 +841,7 @@ lb_status lb_step(lb_ctx *c, int64_t nsteps)
             if (!one()) return cuda_fail(c, e, "lb_step: sweep launch");
         return LB_OK;
     }
-    while (cap == cudaStreamCaptureStatusNone && nsteps >= kGraphSteps) {
-        cudaError_t e = cudaSuccess;
-        if (!c->graph[c->cur]) e = record_sweeps(c, c->cur);
-        if (e == cudaSuccess) e = cudaGraphLaunch(c->graph[c->cur], c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: graph");
-        nsteps -= kGraphSteps;
-        c->step += kGraphSteps;
-    }
+    if ((er = replay()) != cudaSuccess) return cuda_fail(c, er, "lb_step: graph");
     for (int64_t s = 0; s < nsteps; ++s) {
         cudaError_t e = lbk::launch_sweep(c, c->f[c->cur], c->f[c->cur ^ 1]);
         if (e != cudaSuccess) return cuda_fail(c, e, "lb_step: sweep launch");

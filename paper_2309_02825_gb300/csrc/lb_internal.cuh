@@ -315,6 +315,7 @@ struct lb_ctx {
     int tb_k = 0, tb_tile = 0, tb_threads = 0, tb_ntiles = 0, tb_tx = 0, tb_ty = 0;
     cudaGraphExec_t tb_graph[2] = {nullptr, nullptr};  // recorded tiled launches, by starting buffer
     lbk::MarchPlan march{};
+    bool march_short = false;  // marching only the steps of a call that no graph of sweeps covers (kMarchShort)
     std::string err;
 };
 
@@ -395,7 +396,12 @@ void blocked_release(lb_ctx *c);
 // Marching sweeps of a periodic 2D or 3D grid (lb_march.cu): the cut of the
 // grid (steps = 0 where they are not built), whether the rule takes them over
 // one sweep per launch, and one launch of plan.steps steps.
-cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth);
+enum MarchWorth {
+    kMarchNo = 0,
+    kMarchShort = 1,  // over sweeps launched one by one (calls too short for a recorded graph) only
+    kMarchYes = 2
+};
+cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, MarchWorth *worth);
 cudaError_t march_launch(lb_ctx *c, const void *src, void *dst, cudaStream_t s);
 // The same for batched 2D instances: variants of a storage type (the first is
 // the default), the blocks of a launch over `count` instances with the steps,

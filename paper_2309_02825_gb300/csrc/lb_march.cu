@@ -285,11 +285,12 @@ static void cut(int n, int most, int &parts, int &size)
 
 // What marching has to offer against one sweep per launch (march_setup).
 struct MarchRule {
-    int64_t nodes;  // at least so many nodes
+    int64_t least, nodes;  // at least so many nodes, for short calls and for all
     double use;     // of a launch's thread-iterations at least this share ends in stored nodes
-    double full;    // 2D, below 450000 nodes: the same with as many blocks on every SM as on the fullest
+    double full;    // 2D, below 450000 nodes, all calls: the same with as many blocks on every SM as on the fullest
     // 3D: us per step and unit of the plan's model, less than the sweeps' us per 1000
-    // nodes, lanes of the rows' warps, and nodes beyond 650000 (no longer in L2)
+    // nodes, lanes of the rows' warps, and nodes beyond 650000 (no longer in L2), replayed
+    // from a graph; launched one by one a sweep takes about 2.5 us more
     double unit, node, lane, far;
 };
 
@@ -305,11 +306,11 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
     // room for, in blocks of fewer warps, where they fill the SMs better
     // (101 x 90 x 77 FP32: 36 windows of 10 rows by 4 chunks on 152 SMs instead of
     // 32 of 12, 50 GLUPS against 44).
-    static void plan(const lb_ctx *c, const MarchRule &rule, MarchPlan *out, bool *worth)
+    static void plan(const lb_ctx *c, const MarchRule &rule, MarchPlan *out, MarchWorth *worth)
     {
         const Geom &g = c->geom;
         *out = MarchPlan{};
-        *worth = false;
+        *worth = kMarchNo;
         if (g.slab >= (1ll << 30)) return;  // offsets within a population are int
         const int NR = L::D == 3 ? g.N2 : g.N1, high = TH / kMarchW;
         MarchPlan p{};
@@ -349,16 +350,16 @@ template <class L, typename T, int KS, int TH, int MINB, bool SKIP> struct March
         const int64_t blocks = (int64_t)out->nx * out->ny * out->nc, waves = (blocks + slots - 1) / slots;
         const int64_t filled = (blocks + waves * c->sms - 1) / (waves * c->sms) * waves * c->sms;
         const double each = (double)out->threads * (out->chunk + 3 * kRing), nodes = (double)c->nodes;
-        *worth = c->nodes >= rule.nodes && nodes / (blocks * each) >= rule.use;
-        if (L::D == 2 && c->nodes < 450000) *worth = *worth && nodes / (filled * each) >= rule.full;
-        if (L::D == 3) {
-            const double lanes = (double)g.nseg * 32 * lane_width<L, T>();
-            *worth = *worth && rule.unit * least / KS < 1e-3 * (rule.node * nodes + rule.lane * lanes +
-                                                               rule.far * std::max(0.0, nodes - 650000));
-        }
+        if (c->nodes < rule.least || nodes / (blocks * each) < rule.use) return;
+        const double lanes = (double)g.nseg * 32 * lane_width<L, T>();
+        const double less = L::D == 3 ? 1e-3 * (rule.node * nodes + rule.lane * lanes + rule.far * std::max(0.0, nodes - 650000)) -
+                                            rule.unit * least / KS
+                                      : 0.0;  // us per step
+        const bool full = L::D == 3 || c->nodes >= 450000 || nodes / (filled * each) >= rule.full;
+        *worth = c->nodes >= rule.nodes && full && less >= 0.0 ? kMarchYes : (less > -2.5 ? kMarchShort : kMarchNo);
     }
     static const void *kernel() { return (const void *)march_kernel<L, T, KT, KS, TH, MINB, SKIP>; }
-    static cudaError_t setup(lb_ctx *c, const MarchRule &rule, MarchPlan *out, bool *worth)
+    static cudaError_t setup(lb_ctx *c, const MarchRule &rule, MarchPlan *out, MarchWorth *worth)
     {
         plan(c, rule, out, worth);
         return cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -403,20 +404,22 @@ using March3F = March<D3Q19, float, 3, 512, 1, false>;
 // In 3D a few planes, or rows that fill the sweep's warps, favour the sweeps: FP32
 // 126x31x126 10.3 / 8.0, 234x234x15 20.8 / 16.8, 50x200x50 10.6 / 13.2; fixed point
 // 169x169x11 14.3 / 13.6, 27x106x106 12.3 / 19.9.  The 3D costs are fitted to 70 grids of
-// 0.3M to 2M nodes; none of them is slower by the rule.
-cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, bool *worth)
+// 0.3M to 2M nodes; none of them is slower by the rule.  Sweeps of calls shorter than
+// a graph cost 2 us more each, and there the windows still pay on many of these (FP32
+// 101x90x77 14.2 / 16.4, 79^3 10.3 / 12.3; fixed point 169x169x11 14.3 / 16.4, 263 x 1052 6.15 / 7.7).
+cudaError_t march_setup(lb_ctx *c, MarchPlan *plan, MarchWorth *worth)
 {
     *plan = MarchPlan{};
-    *worth = false;
+    *worth = kMarchNo;
     if (c->geom.mirror) return cudaSuccess;
     if (c->d == 2) {
-        if (c->precision == LB_FX64) return March2Fx::setup(c, {240000, 0.45, 0.47}, plan, worth);
-        if (c->precision == LB_FP32_SHIFTED) return March2F::setup(c, {240000, 0.45}, plan, worth);
-        return March2D::setup(c, {1800000, 0.8}, plan, worth);
+        if (c->precision == LB_FX64) return March2Fx::setup(c, {200000, 240000, 0.45, 0.47}, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March2F::setup(c, {180000, 240000, 0.45}, plan, worth);
+        return March2D::setup(c, {1800000, 1800000, 0.8}, plan, worth);
     }
     if (c->d == 3) {
-        if (c->precision == LB_FX64) return March3Fx::setup(c, {300000, 0.4, 0.0, 1.9, 0.026, 0.017}, plan, worth);
-        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, {350000, 0.3, 0.0, 1.57, 0.009, 0.0069, 0.014}, plan, worth);
+        if (c->precision == LB_FX64) return March3Fx::setup(c, {300000, 300000, 0.4, 0.0, 1.9, 0.026, 0.017}, plan, worth);
+        if (c->precision == LB_FP32_SHIFTED) return March3F::setup(c, {350000, 350000, 0.3, 0.0, 1.57, 0.009, 0.0069, 0.014}, plan, worth);
     }
     return cudaSuccess;
 }

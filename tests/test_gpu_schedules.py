@@ -250,3 +250,33 @@ def test_resident_1d_reports_an_unstable_relaxation_set(single, tmp_path):
         s.check()
     assert ei.value.status == lb.LB_EINVAL
     s.close()
+
+
+@pytest.mark.parametrize("precision,N", [("fx64", (263, 1052)), ("fp32s", (101, 90, 77)), ("fp32s", (79, 79, 79)),
+                                         ("fx64", (169, 169, 11))])
+def test_graphs_of_sweeps_with_marching_remainders_give_the_same_bits(precision, N, tmp_path):
+    """Grids whose windows pay only against sweeps launched one by one: calls of a
+    graph's 32 steps and more replay sweeps and march the rest; captured calls sweep."""
+    th, gr = _rough(N)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    s = _solver(N, precision, stream=stream)
+    one = _solver(N, precision)
+    s.set_theta0(th, gr)
+    assert set(_steps(s, stream, 30, tmp_path)) == {"sweep"}
+    s.set_theta0(th, gr)
+    one.set_theta0(th, gr)
+    for n in (13, 45, 2, 64, 31):
+        s.step(n)
+        for _ in range(n):
+            one.step(1)
+    assert s.nsteps == one.nsteps
+    torch.cuda.synchronize()
+    assert s.sum_theta() == one.sum_theta()
+    got = s.macros()
+    torch.cuda.synchronize()
+    for a, b in zip(got, one.macros()):
+        assert torch.equal(a, b)
+    s.check()
+    s.close()
+    one.close()
