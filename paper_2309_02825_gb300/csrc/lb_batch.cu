@@ -398,6 +398,7 @@ struct lb_batch {
     // library's own choice rather than the autotuner's
     int mv = 0, m_steps = 0, m_threads = 0, m_cols = 0, m_blocks = 0;
     bool m_auto = false;
+    bool m_short = false;  // march only the steps of a call that no recorded graph covers
     lbk::MarchBlock *d_march = nullptr;
     // one launch for all instances' initialisation and recovery: the table, whether the constants have
     // changed since it was uploaded, and whether they all admit the batched initialisation
@@ -450,7 +451,7 @@ void free_march(lb_batch *b)
     cudaFree(b->d_march);
     b->d_march = nullptr;
     b->m_steps = b->m_blocks = 0;
-    b->m_auto = false;
+    b->m_auto = b->m_short = false;
 }
 
 // Bring the table of initialisation and recovery constants up to date (stream order).
@@ -482,16 +483,19 @@ cudaError_t upload_inst(lb_batch *b)
 // 8.8, 31 x (2000 x 16) fixed point 13.1 / 21.5, 4 x 1024^2 FP64 96.6 / 121.  FP64
 // instances whose collisions take the direct form load the FP64 pipe with
 // the recomputed nodes too (eps = 0.01: 10 x 512^2 221 / 180, 200 x 64^2 96 / 59).
-bool march_worth(const lb_batch *b, const std::vector<lbk::MarchBlock> &blocks, int steps, int resident)
+// Launched one by one, not replayed, a group's step costs 2 us more: batches that march
+// at no more than that march only calls (and remainders) shorter than a graph (11 of 32 to
+// 128 columns FP32, a call of 16 steps 48.5 / 68.3).
+lbk::MarchWorth march_worth(const lb_batch *b, const std::vector<lbk::MarchBlock> &blocks, int steps, int resident)
 {
     struct Cost {
         int64_t least;
         double launch, block, segment, node, row, warp_row;
     };
     const Cost k = b->precision == LB_FP32_SHIFTED ? Cost{40000, 3180.0, 1.06, 0.35, 0.0017, 0.0355, 0.0033}
-                   : b->precision == LB_FX64       ? Cost{200000, 0.0, 1.36, 0.48, 0.0118, 0.149, 0.0206}
+                   : b->precision == LB_FX64       ? Cost{200000, 1000.0, 1.32, 0.495, 0.0107, 0.152, 0.0188}
                                                    : Cost{350000, 0.0, 3.0, 0.85, 0.011, 0.426, 0.212};
-    if (b->total_nodes < k.least) return false;
+    if (b->total_nodes < k.least) return lbk::kMarchNo;
     const int ring = steps - 1;
     std::vector<char> direct(b->count, 0);
     double one = k.launch, march = 0.0;
@@ -504,7 +508,8 @@ bool march_worth(const lb_batch *b, const std::vector<lbk::MarchBlock> &blocks, 
     for (const lbk::MarchBlock &m : blocks)
         march += (direct[m.inst] ? 4.0 : 1.0) * steps * (m.nr + ring) *
                  (k.row + k.warp_row * ((m.nx + 2 * ring + 31) / 32));
-    return march * std::max(1.0, (double)resident / (double)blocks.size()) < one;
+    march *= std::max(1.0, (double)resident / (double)blocks.size());
+    return march < one ? lbk::kMarchYes : (march < one + 2000.0 * b->groups.size() ? lbk::kMarchShort : lbk::kMarchNo);
 }
 
 // Take marching launches of variant `v` (tables of the blocks); own: the library's
@@ -519,7 +524,8 @@ cudaError_t build_march(lb_batch *b, int v, bool own)
     int steps, threads, cols, resident;
     lbk::march_batch_plan(b->inst.data(), b->count, b->precision, v, sms, &blocks, &steps, &threads, &cols, &resident);
     if (blocks.empty() || blocks.size() > 0x7fffffff) return cudaSuccess;
-    if (own && !march_worth(b, blocks, steps, resident)) return cudaSuccess;
+    const lbk::MarchWorth worth = own ? march_worth(b, blocks, steps, resident) : lbk::kMarchYes;
+    if (worth == lbk::kMarchNo) return cudaSuccess;
     if ((e = cudaMalloc(&b->d_march, sizeof(lbk::MarchBlock) * blocks.size())) != cudaSuccess ||
         (e = cudaMemcpy(b->d_march, blocks.data(), sizeof(lbk::MarchBlock) * blocks.size(), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
@@ -530,6 +536,7 @@ cudaError_t build_march(lb_batch *b, int v, bool own)
     b->m_cols = cols;
     b->m_blocks = (int)blocks.size();
     b->m_auto = own;
+    b->m_short = worth == lbk::kMarchShort;
     return cudaSuccess;
 }
 
@@ -771,11 +778,40 @@ cudaError_t record_graph(lb_batch *b, Group &g, int from)
 cudaError_t run_steps(lb_batch *b, int64_t n)
 {
     cudaError_t e = cudaSuccess;
-    if (b->m_steps > 0) {  // marching launches; the remainder below, one launch per step
+    const auto one_per_step = [&](int64_t k) {  // k steps, group by group
+        for (Group &g : b->groups) {
+            int p = b->cur;
+            int64_t left = k;
+            if (b->use_graph) {
+                while (left >= kGraphSteps) {
+                    if (!g.graph[p]) {
+                        e = record_graph(b, g, p);
+                        if (e != cudaSuccess) return e;
+                    }
+                    e = cudaGraphLaunch(g.graph[p], b->stream);
+                    if (e != cudaSuccess) return e;
+                    left -= kGraphSteps;  // even: parity unchanged
+                }
+            }
+            for (; left > 0; --left) {
+                e = launch_group(b, g, p, b->stream);
+                if (e != cudaSuccess) return e;
+                p ^= 1;
+            }
+        }
+        if (k & 1) b->cur ^= 1;
+        return e;
+    };
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (b->m_steps > 0 && cudaStreamIsCapturing(b->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+    if (b->m_steps > 0 && !(b->m_short && cap != cudaStreamCaptureStatusNone)) {
+        // marching launches; the remainder below, one launch per step
+        if (b->m_short && b->use_graph && n >= kGraphSteps) {
+            if ((e = one_per_step(n / kGraphSteps * kGraphSteps)) != cudaSuccess) return e;
+            n %= kGraphSteps;
+        }
         // inside the caller's capture an even number of steps ends in the buffer it
         // began in, as one launch per step does: replays go on from one another
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(b->stream, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
         int64_t launches = n / b->m_steps;
         if (cap != cudaStreamCaptureStatusNone && b->m_steps % 2 == 0) launches -= launches % 2;
         n -= launches * b->m_steps;
@@ -807,28 +843,7 @@ cudaError_t run_steps(lb_batch *b, int64_t n)
         }
         return cudaSuccess;
     }
-    for (Group &g : b->groups) {
-        int p = b->cur;
-        int64_t left = n;
-        if (b->use_graph) {
-            while (left >= kGraphSteps) {
-                if (!g.graph[p]) {
-                    e = record_graph(b, g, p);
-                    if (e != cudaSuccess) return e;
-                }
-                e = cudaGraphLaunch(g.graph[p], b->stream);
-                if (e != cudaSuccess) return e;
-                left -= kGraphSteps;  // even: parity unchanged
-            }
-        }
-        for (; left > 0; --left) {
-            e = launch_group(b, g, p, b->stream);
-            if (e != cudaSuccess) return e;
-            p ^= 1;
-        }
-    }
-    if (n & 1) b->cur ^= 1;
-    return e;
+    return one_per_step(n);
 }
 
 }  // namespace

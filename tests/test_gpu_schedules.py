@@ -280,3 +280,27 @@ def test_graphs_of_sweeps_with_marching_remainders_give_the_same_bits(precision,
     s.check()
     s.close()
     one.close()
+
+
+@pytest.mark.parametrize("precision,count,edge", [("fp32s", 11, 68), ("fx64", 43, 69), ("fp64", 90, 64)])
+def test_batches_mix_graphs_and_marching_remainders_bit_for_bit(precision, count, edge):
+    """Batches near where marching pays: calls shorter and longer than a recorded graph of
+    one launch per step, against one launch per step throughout."""
+    sizes = [(edge + 3 * (j % 5) - 6, edge + 2 * (j % 7) - 6) for j in range(count)]
+    ins = [_rough(N, 3 + k) for k, N in enumerate(sizes)]
+    th = torch.cat([t.reshape(-1) for t, _ in ins])
+    gr = torch.cat([g.reshape(-1) for _, g in ins])
+    dx = [1.0 / N[0] for N in sizes]
+    kw = {"theta_ref": [1.5] * count} if precision == "fp32s" else {}
+    out = []
+    for own in (True, False):
+        b = lb.Batch(sizes, [NU] * count, dx, [EPS[2] * h * h / NU for h in dx], precision=precision, **kw)
+        if not own:
+            b.set_schedule(1e18, 128)
+        b.set_theta0(th, gr)
+        for n in (13, 45, 2, 64, 31):
+            b.step(n)
+        out.append(b.macros())
+        b.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
